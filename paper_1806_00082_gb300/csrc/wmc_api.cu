@@ -41,7 +41,8 @@ Layout layout(const wmc_params& p) {
   L.header = o; o = align256(o + sizeof(DevHeader));
   L.T = o; o = align256(o + sizeof(unsigned long long) * nx);
   L.R = o; o = align256(o + sizeof(unsigned long long) * (nx + 1));
-  L.IP = o; o = align256(o + sizeof(int) * (nx + 1));
+  L.U = o; o = align256(o + sizeof(uint32_t) * (nx + 1));
+  L.bp = o; o = align256(o + sizeof(uint32_t) * nx * ((nM + 31) / 32));
   L.reach = o; o = align256(o + nx);
   L.occ = o; o = align256(o + sizeof(int) * nx);
   L.row_map = o; o = align256(o + sizeof(int) * nx);
@@ -52,15 +53,14 @@ Layout layout(const wmc_params& p) {
   L.gthr = o; o = align256(o + sizeof(unsigned long long) * nx);
   L.thr_cell = o; o = align256(o + sizeof(unsigned long long) * nx);
   L.D = o; o = align256(o + sizeof(float) * nM);
-  L.xlo = o; o = align256(o + sizeof(uint32_t) * nM);
-  L.xhi = o; o = align256(o + sizeof(uint32_t) * nM);
+  L.xm = o; o = align256(o + sizeof(uint32_t) * nM);
+  L.nbk = o; o = align256(o + nx);
   L.max_items = kMaxItemsBase + 2 * (long long)nx;
-  L.items = o; o = align256(o + sizeof(int2) * (size_t)L.max_items);
-  // pair queue: one entry per created pair of a step (events beyond it are
-  // processed inside the step kernel instead)
+  // pair queue: one entry per quad that may hold a pair event (if they are
+  // more, the pair kernel walks the ids again instead)
   {
     const size_t want = nx * nM / 8;
-    L.pair_cap = (unsigned)(want < (1u << 16) ? (1u << 16) : (want > (1u << 21) ? (1u << 21) : want));
+    L.pair_cap = (unsigned)(want < (1u << 19) ? (1u << 19) : (want > (1u << 22) ? (1u << 22) : want));
   }
   L.pairs = o; o = align256(o + sizeof(uint4) * (size_t)L.pair_cap);
   L.B = o; o = align256(o + sizeof(float) * (size_t)L.Kp * (size_t)L.Np);
@@ -79,7 +79,8 @@ View view(const wmc_params& p, void* ws) {
   v.hdr = reinterpret_cast<DevHeader*>(b + L.header);
   v.T = reinterpret_cast<unsigned long long*>(b + L.T);
   v.R = reinterpret_cast<unsigned long long*>(b + L.R);
-  v.IP = reinterpret_cast<int*>(b + L.IP);
+  v.U = reinterpret_cast<uint32_t*>(b + L.U);
+  v.bp = reinterpret_cast<uint32_t*>(b + L.bp);
   v.reach = reinterpret_cast<unsigned char*>(b + L.reach);
   v.occ = reinterpret_cast<int*>(b + L.occ);
   v.row_map = reinterpret_cast<int*>(b + L.row_map);
@@ -89,10 +90,9 @@ View view(const wmc_params& p, void* ws) {
   v.gamma = reinterpret_cast<double*>(b + L.gamma);
   v.gthr = reinterpret_cast<unsigned long long*>(b + L.gthr);
   v.D = reinterpret_cast<float*>(b + L.D);
-  v.xlo = reinterpret_cast<uint32_t*>(b + L.xlo);
-  v.xhi = reinterpret_cast<uint32_t*>(b + L.xhi);
+  v.xm = reinterpret_cast<uint32_t*>(b + L.xm);
+  v.nbk = reinterpret_cast<unsigned char*>(b + L.nbk);
   v.thr_cell = reinterpret_cast<unsigned long long*>(b + L.thr_cell);
-  v.items = reinterpret_cast<int2*>(b + L.items);
   v.pairs = reinterpret_cast<uint4*>(b + L.pairs);
   v.B = reinterpret_cast<float*>(b + L.B);
   v.B2 = reinterpret_cast<float*>(b + L.B2);
@@ -470,7 +470,7 @@ wmc_status wmc_init(const wmc_params* p, void* ws, size_t ws_bytes, wmc_stream_t
   if (ws_bytes < L.total) return WMC_ERR_ARG;
   const View v = view(*p, ws);
   (void)num_sms();
-  prepare_step(*p);
+  prepare_step();
   cudaError_t e = launch_init_tables(*p, v, (cudaStream_t)stream);
   if (e == cudaSuccess) e = launch_init_tc_images(*p, v.tc, (cudaStream_t)stream);
   return cuda_status(e);

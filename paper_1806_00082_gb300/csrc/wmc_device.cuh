@@ -297,29 +297,6 @@ __device__ __forceinline__ int sample_coarse_row(const float* __restrict__ v, co
   return k1 - 1;  // not reached: block blk's sum exceeds the target
 }
 
-// The same draw with sequential loads and few registers (for the rare calls
-// from inside the particle-step kernel).
-__device__ __forceinline__ int sample_coarse_row_seq(const float* __restrict__ v, const long long* __restrict__ cc,
-                                                     int s, int Q, int r0, int n_M, unsigned long long U2) {
-  const unsigned long long Qtot = (unsigned long long)__ldg(cc + kCdfBlocks - 1);
-  const long long target = (long long)((__umul64hi(U2, Qtot) << 11) | ((U2 * Qtot) >> 53));
-  int lo = 0, hi = kCdfBlocks - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi) >> 1;
-    if (__ldg(cc + mid) > target) hi = mid; else lo = mid + 1;
-  }
-  const int E = (n_M + kCdfBlocks - 1) / kCdfBlocks;
-  const int k0 = min(lo * E, n_M), k1 = min(k0 + E, n_M);
-  long long run = lo ? __ldg(cc + lo - 1) : 0ll;
-  int rr = (r0 + k0) % Q;
-  for (int k = k0; k < k1; ++k) {
-    run += quantise(positive_part(v, Q, rr), s);
-    if (run > target) return k;
-    if (++rr == Q) rr = 0;
-  }
-  return k1 - 1;
-}
-
 // Smallest j in [0, 2^24] with fl32(j 2^-24 + d) >= edge (2^24 if none); the
 // predicate is monotone in j because rounding is.
 __device__ __forceinline__ int first_offset_reaching(float d, float edge) {

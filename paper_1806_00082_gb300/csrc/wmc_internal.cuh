@@ -32,19 +32,19 @@ constexpr uint32_t kPurposeGen = 1u;
 constexpr uint32_t kPurposeRepos = 2u;
 constexpr uint32_t kPurposePick = 3u;
 
-// Step work decomposition: the survivors of cell i (ids R[i] .. R[i] + T[i] - 1)
-// are cut into work items on a grid of kChunk ids aligned to A = R[i] rounded
-// down to a multiple of 4: item c of cell i holds the ids in
-// [A + c kChunk, A + (c+1) kChunk) that belong to the cell, so every Philox
-// call (four consecutive ids) stays within one item.  A cell has
-// ceil((T[i] + 3) / kChunk) items (the last may be empty).  A warp of the
-// particle-step kernel takes one item at a time, each lane a quad-aligned run
-// of at most kChunk / 32 consecutive ids.
+// The particle step walks the survivor ids in windows of 128, each window in
+// one cell (wmc_walk.cuh), so every Philox call (four consecutive ids) stays
+// within one window.  Its work is cut in units: a window is one unit, an
+// occupied cell costs kCellCost more, and one for every kBlocksPerUnit of its
+// non-empty 32-column blocks (latencies of dependent loads, in the time a busy
+// SM gives a warp for a window).  A work item, as counted in n_items and
+// bounded by max_items, is up to kChunk ids of one cell.
+constexpr uint32_t kCellCost = 4, kBlocksPerUnit = 2;
 constexpr int kStepThreads = 256;
 constexpr int kStepWarps = kStepThreads / 32;
 constexpr int kChunk = 2048;
 constexpr int kMaxStepBlocks = 8192;
-constexpr long long kMaxItemsBase = 1ll << 20;   // item descriptors: 2^32 / kChunk + n_x
+constexpr long long kMaxItemsBase = 1ll << 20;   // work items: 2^32 / kChunk + n_x
 // Lane blocks of the coarse momentum CDF: a row's n_M columns are cut into 32
 // blocks of E = ceil(n_M / 32) consecutive columns (block l is [l E, (l+1) E)).
 constexpr int kCdfBlocks = 32;
@@ -67,26 +67,24 @@ struct DevHeader {
   unsigned int flags;
   unsigned int step;    // device step counter (wmc_run)
   unsigned int magic;
-  unsigned int item_ticket;  // next work item of the running step launch
+  unsigned int item_ticket;  // id ranges handed out by the running step launch
   unsigned int blocks_done;  // step blocks finished (the last one resets both)
   unsigned int rows_by_cell; // 1: the kernel stage wrote its rows at the cell index, 0: at the occupied-list index
-  unsigned int pair_count;   // pair events queued by the particle-step kernel (reset by the pair kernel)
+  unsigned int pair_count;   // quads queued by the particle-step kernel (reset by the pair kernel)
   unsigned int pairs_done;   // pair-kernel blocks finished (the last one resets the queue and the ticket)
   unsigned int plan_epoch;   // launches of the plan so far (tags its blocks' published prefixes)
   unsigned int plan_ticket;  // logical block index of the running plan launch (reset by its last block)
-  unsigned int chunk;        // ids per work item of the current plan (0: kChunk)
+  unsigned int pad0;
   unsigned long long id_base;  // number of the first survivor (a sub-domain numbers after the cells before it)
-  unsigned int chunk_next;   // the plan's choice for the next step (the pair kernel makes it current)
-  unsigned int pad1;
 };
 
 // Totals of a run of cells in the plan's scan: survivors (64 bits), work
-// items, needed cells, and whether a cell held 2^31 survivors or more.
+// items, needed cells, whether a cell held 2^31 survivors or more, work units.
 struct PlanSums {
   unsigned long long T;
   int I, N;
   int big;
-  int pad;
+  unsigned int U;
 };
 
 // One block of the plan's scan publishes its own totals (agg) and then the
@@ -100,7 +98,7 @@ struct PlanStatus {
 
 // Byte offsets of the workspace regions (all 256-aligned).
 struct Layout {
-  size_t header, T, R, IP, reach, occ, row_map, VWh, ccdf, scale, gamma, gthr, thr_cell, D, xlo, xhi, items, pairs, B,
+  size_t header, T, R, U, bp, reach, occ, row_map, VWh, ccdf, scale, gamma, gthr, thr_cell, D, xm, nbk, pairs, B,
       B2, tc, plan, dft, total;
   long long max_items;
   unsigned pair_cap;  // entries of the pair queue
@@ -118,7 +116,8 @@ struct View {
   DevHeader* hdr;
   unsigned long long* T;   // [n_x] survivors per cell
   unsigned long long* R;   // [n_x + 1] first id of each cell (exclusive prefix of T)
-  int* IP;                 // [n_x + 1] first work item of each cell
+  uint32_t* U;             // [n_x + 1] first work unit of each cell
+  uint32_t* bp;            // [n_x][ceil(n_M / 32)] inclusive survivor prefixes of the row's 32-column blocks
   unsigned char* reach;    // [n_x] bit0 occupied, bit1 some drift right, bit2 some drift left
   int* occ;                // [n_x] occupied-cell list (ascending)
   int* row_map;            // [n_x] cell -> row of occ, or -1
@@ -129,10 +128,9 @@ struct View {
   unsigned long long* gthr;// [n_x] event threshold by occ row: word < gthr <=> word 2^-32 < gamma dt
   unsigned long long* thr_cell;  // [n_x] the same by cell (0 for cells without a kernel row)
   float* D;                // [n_M] drift per step in cells
-  uint32_t* xlo;           // [n_M] offset word w crosses left iff w < xlo[k]
-  uint32_t* xhi;           // [n_M] ... crosses right iff w > xhi[k]
-  int2* items;             // [max_items] work items (cell, chunk)
-  uint4* pairs;            // [pair_cap] pair events (id, cell, column, sign < 0) queued by the step
+  uint32_t* xm;            // [n_M] move entries (crossing threshold and direction, wmc_walk.cuh)
+  unsigned char* nbk;      // [n_x] non-empty 32-column blocks of the row
+  uint4* pairs;            // [pair_cap] quads that may hold pair events, queued by the step
   float* B;                // [Kp][Np] sine matrix S[m][r], m = kk + 1
   float* B2;               // [Kp2][Np] folded matrix of the N = 2 network, pair offset u
   void* tc;                // tensor-core operand images of S (BF16, FP16 hi, FP16 lo)
@@ -219,18 +217,16 @@ __device__ __forceinline__ uint4 philox4x32_10k(uint4 c, const PhiloxKeys& K) {
   return c;
 }
 
-// Work items of a cell holding t survivors (an upper bound when its first id
-// is not a multiple of 4; surplus items are empty).
-__host__ __device__ __forceinline__ int items_of_cell(unsigned long long t, unsigned int chunk = kChunk) {
-  return t ? (int)((t + 3 + chunk - 1) / chunk) : 0;
+// Work items of a cell holding t survivors.
+__host__ __device__ __forceinline__ int items_of_cell(unsigned long long t) {
+  return t ? (int)((t + 3 + kChunk - 1) / kChunk) : 0;
 }
 
-// Ids per work item: the header's current choice (kChunk until a step has
-// chosen); a power of two in [kMinChunk, kChunk].
-constexpr unsigned int kMinChunk = 512;
-__device__ __forceinline__ unsigned int work_chunk(const DevHeader* hdr) {
-  const unsigned int c = *(const volatile unsigned int*)&hdr->chunk;
-  return c ? c : (unsigned int)kChunk;
+// Windows of a cell holding t survivors (t < 2^31; its first id may be up to 3
+// places into its first window), and its work units with nb non-empty blocks.
+__host__ __device__ __forceinline__ uint32_t windows_of_cell(uint32_t t) { return (t + 3u + 127u) >> 7; }
+__host__ __device__ __forceinline__ uint32_t units_of_cell(unsigned long long t, uint32_t nb) {
+  return t ? windows_of_cell((uint32_t)t) + kCellCost + nb / kBlocksPerUnit : 0u;
 }
 
 // ---------------------------------------------------------------- launchers
@@ -242,7 +238,7 @@ cudaError_t launch_plan(const wmc_params& p, const View& v, const int32_t* hist,
 cudaError_t launch_rows(const wmc_params& p, const View& v, const int32_t* hist, int64_t* rho, cudaStream_t s,
                         int32_t* zero_out);
 cudaError_t launch_plan_scan(const wmc_params& p, const View& v, int advance_step, int clear_thr, cudaStream_t s);
-int step_grid(int n_M);
+int step_grid();
 // (net 1: the N = 1 network with B = the sine matrix; net 2: the N = 2
 // network with B = its folded matrix B2)
 cudaError_t launch_kernel_eval(const wmc_params& p, const float* V, const int* occ, const int* n_occ_dev,
@@ -300,6 +296,6 @@ cudaError_t step_timing_record(cudaStream_t s, bool end);
 // Whether step timing is on (part of the key of the cached step graphs).
 int step_timing_on();
 // Caches the step kernel's launch shape for this device (call outside graph capture).
-void prepare_step(const wmc_params& p);
+void prepare_step();
 
 }  // namespace wmc

@@ -2,20 +2,20 @@
 // kernel, density (rule 1), constant tables and the Philox check kernel.
 #include <math.h>
 
-#include "wmc_device.cuh"
+#include "wmc_walk.cuh"
 
 namespace wmc {
 
 // ---------------------------------------------------------------- constant tables
 // D[k] = fl32(M * d1), d1 = hbar pi dt / (m Q dx^2), M = k - n_M/2: the free
-// drift of momentum M dp over dt, in cells.  Crossing thresholds on the offset
-// word w (f = (w >> 8) 2^-24): a particle of column k moves right iff
-// fl32(f + D) >= 1 iff w > xhi[k], left iff fl32(f + D) < 0 iff w < xlo[k].
+// drift of momentum M dp over dt, in cells, and its move entry: a particle of
+// column k with offset word w (f = (w >> 8) 2^-24) moves right iff
+// fl32(f + D) >= 1, left iff fl32(f + D) < 0, decided by a threshold on w.
 // B[kk][r] = sin(2 pi ((kk+1) r mod Q) / Q) for kk < h-1, r < h (zero padding
 // elsewhere): the integer-indexed sine matrix of the network's hidden layer
 // (Sec. 2.2); B2[u][r] the folded matrix of the N = 2 network (Sec. 2.3).
-__global__ void k_init_tables(int n_M, int Q, double d1, float* __restrict__ D, uint32_t* __restrict__ xlo,
-                              uint32_t* __restrict__ xhi, float* __restrict__ B, int Kp, int Np,
+__global__ void k_init_tables(int n_M, int Q, double d1, float* __restrict__ D, uint32_t* __restrict__ xm,
+                              float* __restrict__ B, int Kp, int Np,
                               float* __restrict__ B2, int Kp2, DevHeader* hdr) {
   const long long tid = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   const long long nthreads = (long long)gridDim.x * blockDim.x;
@@ -27,11 +27,7 @@ __global__ void k_init_tables(int n_M, int Q, double d1, float* __restrict__ D, 
   for (long long k = tid; k < n_M; k += nthreads) {
     const float d = __double2float_rn((double)(k - n_M / 2) * d1);
     D[k] = d;
-    uint32_t lo = 0u, hi = 0xffffffffu;
-    if (d > 0.f) hi = (uint32_t)(((unsigned long long)first_offset_reaching(d, 1.f) << 8) - 1ull);
-    if (d < 0.f) lo = (uint32_t)((unsigned long long)first_offset_reaching(d, 0.f) << 8);
-    xlo[k] = lo;
-    xhi[k] = hi;
+    xm[k] = move_entry(d);
   }
   for (long long q = tid; q < (long long)Kp * Np; q += nthreads) B[q] = sine_entry_n1(Q, (int)(q / Np), (int)(q % Np));
   for (long long q = tid; q < (long long)Kp2 * Np; q += nthreads) B2[q] = sine_entry_n2(Q, (int)(q / Np), (int)(q % Np));
@@ -40,7 +36,7 @@ __global__ void k_init_tables(int n_M, int Q, double d1, float* __restrict__ D, 
 cudaError_t launch_init_tables(const wmc_params& p, const View& v, cudaStream_t s) {
   const Layout L = layout(p);
   const double d1 = ((kHbarJs * kPi) * p.dt_s) / ((p.mass_kg * (double)p.Q) * (p.dx_m * p.dx_m));
-  k_init_tables<<<256, 256, 0, s>>>(p.n_M, p.Q, d1, v.D, v.xlo, v.xhi, v.B, L.Kp, L.Np, v.B2, L.Kp2, v.hdr);
+  k_init_tables<<<256, 256, 0, s>>>(p.n_M, p.Q, d1, v.D, v.xm, v.B, L.Kp, L.Np, v.B2, L.Kp2, v.hdr);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   // no stale publication may carry a tag of a coming plan launch
@@ -49,8 +45,8 @@ cudaError_t launch_init_tables(const wmc_params& p, const View& v, cudaStream_t 
 
 // ---------------------------------------------------------------- per-cell scan and plan
 // The plan: exclusive prefix sums over the cells of survivors (the first id
-// R[i] of each cell), work items (the first item IP[i]) and needed cells (the
-// occupied list and its row map), then the item descriptors; with clear_thr
+// R[i] of each cell) and needed cells (the occupied list and its row map), and
+// the number of work items; with clear_thr
 // the per-cell event thresholds are cleared (a kernel stage over the occupied
 // list then fills the occupied cells).  One thread per cell, kPlanCells cells
 // per block; the blocks chain their prefixes by a decoupled look-back: each
@@ -69,7 +65,7 @@ __device__ __forceinline__ PlanSums plan_add(const PlanSums& a, const PlanSums& 
   r.I = a.I + b.I;
   r.N = a.N + b.N;
   r.big = a.big | b.big;
-  r.pad = 0;
+  r.U = a.U + b.U;
   return r;
 }
 
@@ -79,7 +75,7 @@ __device__ __forceinline__ PlanSums plan_load(const volatile PlanSums* p) {
   r.I = p->I;
   r.N = p->N;
   r.big = p->big;
-  r.pad = 0;
+  r.U = p->U;
   return r;
 }
 
@@ -88,15 +84,17 @@ __device__ __forceinline__ void plan_store(volatile PlanSums* p, const PlanSums&
   p->I = v.I;
   p->N = v.N;
   p->big = v.big;
+  p->U = v.U;
 }
 
 __global__ __launch_bounds__(kPlanCells) void k_plan(int n_x, const unsigned long long* __restrict__ T,
                                                      const unsigned char* __restrict__ reach,
-                                                     unsigned long long* __restrict__ R, int* __restrict__ IP,
+                                                     const unsigned char* __restrict__ nbk,
+                                                     unsigned long long* __restrict__ R, uint32_t* __restrict__ U,
                                                      int* __restrict__ occ, int* __restrict__ row_map,
-                                                     int2* __restrict__ items, long long max_items,
+                                                     long long max_items,
                                                      unsigned long long* __restrict__ thr_cell, DevHeader* hdr,
-                                                     PlanStatus* st, int advance_step, int clear_thr, int step_warps) {
+                                                     PlanStatus* st, int advance_step, int clear_thr) {
   __shared__ PlanSums w_s[kPlanCells / 32];
   __shared__ PlanSums s_ex;
   __shared__ int s_blk;
@@ -111,13 +109,12 @@ __global__ __launch_bounds__(kPlanCells) void k_plan(int n_x, const unsigned lon
   const unsigned int epoch = s_epoch;
   const int i = blk * kPlanCells + tid;
   const unsigned long long t = i < n_x ? __ldg(T + i) : 0ull;
-  const unsigned int chunk = work_chunk(hdr);  // (changed only after the step, by the pair kernel)
   PlanSums mine;
   mine.T = t;
-  mine.I = items_of_cell(t, chunk);
+  mine.I = items_of_cell(t);
   mine.N = i < n_x ? cell_needs_kernel(reach, i, n_x) : 0;
   mine.big = t > 0x7fffffffull;
-  mine.pad = 0;
+  mine.U = units_of_cell(t, i < n_x ? __ldg(nbk + i) : 0u);
   // block-wide inclusive scan
   PlanSums inc = mine;
 #pragma unroll
@@ -127,6 +124,7 @@ __global__ __launch_bounds__(kPlanCells) void k_plan(int n_x, const unsigned lon
     u.I = __shfl_up_sync(0xffffffffu, inc.I, off);
     u.N = __shfl_up_sync(0xffffffffu, inc.N, off);
     u.big = __shfl_up_sync(0xffffffffu, inc.big, off);
+    u.U = __shfl_up_sync(0xffffffffu, inc.U, off);
     if (lane >= off) inc = plan_add(inc, u);
   }
   if (lane == 31) w_s[wid] = inc;
@@ -140,6 +138,7 @@ __global__ __launch_bounds__(kPlanCells) void k_plan(int n_x, const unsigned lon
       u.I = __shfl_up_sync(0xffffffffu, w.I, off);
       u.N = __shfl_up_sync(0xffffffffu, w.N, off);
       u.big = __shfl_up_sync(0xffffffffu, w.big, off);
+      u.U = __shfl_up_sync(0xffffffffu, w.U, off);
       if (lane >= off) w = plan_add(w, u);
     }
     w_s[lane] = w;
@@ -188,6 +187,7 @@ __global__ __launch_bounds__(kPlanCells) void k_plan(int n_x, const unsigned lon
         u.I = __shfl_down_sync(0xffffffffu, mineb.I, off);
         u.N = __shfl_down_sync(0xffffffffu, mineb.N, off);
         u.big = __shfl_down_sync(0xffffffffu, mineb.big, off);
+        u.U = __shfl_down_sync(0xffffffffu, mineb.U, off);
         mineb = plan_add(mineb, u);
       }
       ex = plan_add(ex, mineb);  // (lane 0 holds the window's sum)
@@ -209,12 +209,9 @@ __global__ __launch_bounds__(kPlanCells) void k_plan(int n_x, const unsigned lon
   const unsigned long long id_base = hdr->id_base;
   if (i < n_x) {
     const unsigned long long r = id_base + ex.T + inc.T - mine.T;
-    const int baseI = ex.I + inc.I - mine.I;
     const int baseN = ex.N + inc.N - mine.N;
     R[i] = r;
-    IP[i] = baseI;
-    for (int c = 0; c < mine.I; ++c)
-      if ((long long)baseI + c < max_items) items[baseI + c] = make_int2(i, c);
+    U[i] = ex.U + inc.U - mine.U;
     if (clear_thr) thr_cell[i] = 0ull;
     if (mine.N) {
       occ[baseN] = i;
@@ -227,102 +224,126 @@ __global__ __launch_bounds__(kPlanCells) void k_plan(int n_x, const unsigned lon
     // totals of every cell
     const bool ok = !tot.big && id_base + tot.T < (1ull << 32) && (long long)tot.I <= max_items;
     R[n_x] = id_base + tot.T;
-    IP[n_x] = tot.I;
+    U[n_x] = tot.U;
     hdr->population = tot.T;
     hdr->n_items = ok ? tot.I : 0;
     hdr->n_occ = tot.N;
     if (!ok) atomicOr(&hdr->flags, WMC_FLAG_CAPACITY);
     if (advance_step) hdr->step += 1u;
-    // items for the next step: about four per step warp at this population,
-    // at least kMinChunk ids, at most kChunk (work distribution only: results
-    // do not depend on it)
-    {
-      const unsigned long long per = tot.T / (4ull * (unsigned long long)(step_warps > 0 ? step_warps : 1));
-      unsigned int c = kMinChunk;
-      while (c < per && c < (unsigned int)kChunk) c <<= 1;
-      hdr->chunk_next = c;
-    }
     hdr->plan_ticket = 0u;
     hdr->plan_epoch = (epoch + 1u) & 0x3fffffffu;
     __threadfence();
   }
 }
 
-// One warp per cell: survivors T[i] = sum_k |n(i,k)|, reach bits (bit0 cell
-// occupied, bit1 a momentum that drifts right is present, bit2 one that drifts
-// left), optionally the density rho[i] = sum_k n(i,k), and optionally a zeroed
-// row of the next histogram.
+// One warp per cell: survivors T[i] = sum_k |n(i,k)|, the inclusive survivor
+// prefixes of the row's 32-column blocks, reach bits (bit0 cell occupied, bit1
+// a momentum that drifts right is present, bit2 one that drifts left),
+// optionally the density rho[i] = sum_k n(i,k), and optionally a zeroed row of
+// the next histogram.
 constexpr int kRowsWarps = 8;
 
 __global__ __launch_bounds__(kRowsWarps * 32) void k_rows(const int32_t* __restrict__ hist, int n_x, int n_M,
                                                           const float* __restrict__ D,
                                                           unsigned long long* __restrict__ T,
-                                                          unsigned char* __restrict__ reach,
+                                                          uint32_t* __restrict__ bp, unsigned char* __restrict__ reach,
+                                                          unsigned char* __restrict__ nbk,
                                                           long long* __restrict__ rho, int32_t* __restrict__ zero_out) {
   const int warp = (int)((blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5);
   const int lane = threadIdx.x & 31;
-  if (warp < n_x) {
-    const int32_t* row = hist + (size_t)warp * n_M;
-    unsigned long long a = 0;
-    long long sn = 0;
-    unsigned bits = 0;
-    if ((n_M & 3) == 0) {
-      const int4* row4 = reinterpret_cast<const int4*>(row);
-      const float4* D4 = reinterpret_cast<const float4*>(D);
-      int4* z4 = zero_out ? reinterpret_cast<int4*>(zero_out + (size_t)warp * n_M) : nullptr;
-      for (int q = lane; q < n_M / 4; q += 32) {
-        const int4 n = row4[q];
-        const float4 d = D4[q];
-        if (z4) z4[q] = make_int4(0, 0, 0, 0);
-        const int nv[4] = {n.x, n.y, n.z, n.w};
-        const float dv[4] = {d.x, d.y, d.z, d.w};
+  if (warp >= n_x) return;
+  const int32_t* row = hist + (size_t)warp * n_M;
+  const int NB = (n_M + 31) >> 5;
+  uint32_t* bpr = bp + (size_t)warp * NB;
+  unsigned long long a = 0;
+  long long sn = 0;
+  unsigned bits = 0;
+  int nb = 0;            // non-empty blocks
+  uint32_t before = 0u;  // survivors of the blocks done (modulo 2^32: a larger cell is refused by the plan)
+  if ((n_M & 3) == 0) {
+    const int4* row4 = reinterpret_cast<const int4*>(row);
+    int4* z4 = zero_out ? reinterpret_cast<int4*>(zero_out + (size_t)warp * n_M) : nullptr;
+    const int nq = n_M >> 2;
+    for (int q0 = 0; q0 < nq; q0 += 128) {
+      int4 v[4];  // 512 columns, four loads in flight per lane
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          if (nv[e]) {
-            a += (unsigned long long)(nv[e] < 0 ? -(long long)nv[e] : (long long)nv[e]);
-            sn += nv[e];
-            bits |= 1u | (dv[e] > 0.f ? 2u : 0u) | (dv[e] < 0.f ? 4u : 0u);
-          }
-        }
+      for (int u = 0; u < 4; ++u) {
+        const int q = q0 + 32 * u + lane;
+        v[u] = q < nq ? row4[q] : make_int4(0, 0, 0, 0);
+        if (z4 && q < nq) z4[q] = make_int4(0, 0, 0, 0);
       }
-    } else {
-      for (int k = lane; k < n_M; k += 32) {
-        const int n = row[k];
-        if (zero_out) zero_out[(size_t)warp * n_M + k] = 0;
-        if (n) {
-          a += (unsigned long long)(n < 0 ? -(long long)n : (long long)n);
-          sn += n;
-          bits |= 1u | (D[k] > 0.f ? 2u : 0u) | (D[k] < 0.f ? 4u : 0u);
-        }
-      }
-    }
 #pragma unroll
-    for (int off = 16; off; off >>= 1) {
-      a += __shfl_down_sync(0xffffffffu, a, off);
-      sn += __shfl_down_sync(0xffffffffu, sn, off);
-      bits |= __shfl_down_sync(0xffffffffu, bits, off);
+      for (int u = 0; u < 4; ++u) {
+        const int q = q0 + 32 * u + lane;
+        if (q0 + 32 * u >= nq) break;
+        const int b = (q0 + 32 * u + lane) >> 3;  // eight lanes hold one 32-column block
+        uint32_t p = 0u;
+        if (__any_sync(0xffffffffu, (v[u].x | v[u].y | v[u].z | v[u].w) != 0)) {
+          const int nv[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
+#pragma unroll
+          for (int e = 0; e < 4; ++e)
+            if (nv[e]) {
+              const uint32_t m = nv[e] < 0 ? 0u - (uint32_t)nv[e] : (uint32_t)nv[e];
+              a += m;
+              p += m;
+              sn += nv[e];
+              const float d = __ldg(D + 4 * q + e);
+              bits |= 1u | (d > 0.f ? 2u : 0u) | (d < 0.f ? 4u : 0u);
+            }
+#pragma unroll
+          for (int o = 1; o < 8; o <<= 1) p += __shfl_xor_sync(0xffffffffu, p, o);
+          nb += __popc(__ballot_sync(0xffffffffu, p != 0u && (lane & 7) == 0));
+          uint32_t w = __shfl_up_sync(0xffffffffu, p, 8);
+          if (lane >= 8) p += w;
+          w = __shfl_up_sync(0xffffffffu, p, 16);
+          if (lane >= 16) p += w;
+        }
+        if ((lane & 7) == 0 && b < NB) bpr[b] = before + p;
+        before += __shfl_sync(0xffffffffu, p, 31);
+      }
     }
-    if (lane == 0) {
-      T[warp] = a;
-      reach[warp] = (unsigned char)bits;
-      if (rho) rho[warp] = sn;
+  } else {
+    for (int k0 = 0; k0 < n_M; k0 += 32) {
+      const int k = k0 + lane;
+      const int n = k < n_M ? row[k] : 0;
+      if (zero_out && k < n_M) zero_out[(size_t)warp * n_M + k] = 0;
+      const uint32_t m = n < 0 ? 0u - (uint32_t)n : (uint32_t)n;
+      if (n) {
+        a += m;
+        sn += n;
+        bits |= 1u | (D[k] > 0.f ? 2u : 0u) | (D[k] < 0.f ? 4u : 0u);
+      }
+      before += __reduce_add_sync(0xffffffffu, m);
+      nb += __any_sync(0xffffffffu, n != 0);
+      if (lane == 0) bpr[k0 >> 5] = before;
     }
+  }
+#pragma unroll
+  for (int off = 16; off; off >>= 1) {
+    a += __shfl_down_sync(0xffffffffu, a, off);
+    sn += __shfl_down_sync(0xffffffffu, sn, off);
+    bits |= __shfl_down_sync(0xffffffffu, bits, off);
+  }
+  if (lane == 0) {
+    T[warp] = a;
+    reach[warp] = (unsigned char)bits;
+    nbk[warp] = (unsigned char)nb;
+    if (rho) rho[warp] = sn;
   }
 }
 
 cudaError_t launch_rows(const wmc_params& p, const View& v, const int32_t* hist, int64_t* rho, cudaStream_t s,
                         int32_t* zero_out) {
   const int blocks = (p.n_x + kRowsWarps - 1) / kRowsWarps;
-  k_rows<<<blocks, kRowsWarps * 32, 0, s>>>(hist, p.n_x, p.n_M, v.D, v.T, v.reach,
+  k_rows<<<blocks, kRowsWarps * 32, 0, s>>>(hist, p.n_x, p.n_M, v.D, v.T, v.bp, v.reach, v.nbk,
                                             reinterpret_cast<long long*>(rho), zero_out);
   return cudaGetLastError();
 }
 
 cudaError_t launch_plan_scan(const wmc_params& p, const View& v, int advance_step, int clear_thr, cudaStream_t s) {
   const int blocks = (p.n_x + kPlanCells - 1) / kPlanCells;
-  k_plan<<<blocks, kPlanCells, 0, s>>>(p.n_x, v.T, v.reach, v.R, v.IP, v.occ, v.row_map, v.items,
-                                       layout(p).max_items, v.thr_cell, v.hdr, v.plan, advance_step, clear_thr,
-                                       step_grid(p.n_M) * kStepWarps);
+  k_plan<<<blocks, kPlanCells, 0, s>>>(p.n_x, v.T, v.reach, v.nbk, v.R, v.U, v.occ, v.row_map,
+                                       layout(p).max_items, v.thr_cell, v.hdr, v.plan, advance_step, clear_thr);
   return cudaGetLastError();
 }
 

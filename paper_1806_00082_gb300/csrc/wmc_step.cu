@@ -7,42 +7,33 @@
 // (i, M) carries the same cell, momentum and sign, and its offset is a Philox
 // draw of its id, so the histogram and the id prefix describe the ensemble
 // exactly.  Two kernels:
-//   k_step   -- each warp takes work items (at most kChunk ids of one cell)
-//               from a ticket counter, stages the cell's row prefix in its own
-//               shared memory (no block barriers), and gives each lane a
-//               quad-aligned run of ids: one Philox call per four ids for the
-//               offsets (REPOS, step t - 1) and one for the pair-creation words
-//               (GEN, step t) under a shared key schedule; a particle moves iff
-//               its offset word passes the integer threshold of its momentum
-//               column.  Parents are counted per bucket and added to the next
-//               histogram with one reduction per bucket run; pair events are
-//               queued in shared memory and appended to a global queue;
-//   k_pairs  -- one thread per queued event: the PICK draw, p' from the coarse
-//               CDF of the cell's kernel row, and the two children.
-// Events beyond the queue's capacity are completed inside k_step (same
-// arithmetic), so any rate is handled.
-#include "wmc_device.cuh"
+//   k_step   -- each warp takes ranges of consecutive ids (RangeSchedule) and
+//               walks them cell by cell (walk_ids): parents are counted per
+//               bucket and added to the next histogram with one reduction per
+//               bucket run; quads that may hold a pair event are queued;
+//   k_pairs  -- one thread per queued quad: its words again, the event tests,
+//               and per event the PICK draw, p' from the coarse CDF of the
+//               cell's kernel row, and the two children.
+// When the quads do not fit the queue, k_pairs finds them by a second walk, so
+// any rate is handled.
+#include "wmc_walk.cuh"
 
 namespace wmc {
 
-constexpr int kPairQ = 256;  // per-warp event queue (one quad iteration adds at most 128)
-// a queue entry packs the id's offset in its item (13 bits), the column (12),
-// the event cell relative to i - 1 (2) and the sign (1)
-static_assert(kChunk <= 8192, "item offsets take 13 bits of a queue entry");
-
+constexpr int kStepBlocks = 4;
 struct StepArgs {
   const int32_t* hist_in;
   int32_t* hist_out;
   const unsigned long long* R;
-  const int2* items;
+  const uint32_t* U;          // prefix of the cells' work units
+  const uint32_t* bp;         // id prefixes of the rows' 32-column blocks
   const int* row_map;
   const float* VWh;           // kernel rows [rows][Q/2]
   const long long* ccdf;      // coarse CDF [rows][kCdfBlocks]
   const int* scale;           // fixed-point scale of each row
   const unsigned long long* thr_cell;
-  const uint32_t* xlo;
-  const uint32_t* xhi;
-  uint4* pairs;               // queued events (id, cell, column, sign < 0)
+  const uint32_t* xm;         // move entries of the columns
+  uint4* pairs;               // queued quads (quad_events)
   unsigned pair_cap;
   DevHeader* hdr;
   int n_x, n_M, Q, r0, child_wrap;
@@ -54,7 +45,6 @@ struct StepArgs {
 // p' of the pair created by particle id (column k, sign sgn) in cell c and the
 // children c (k + M', +sgn), (k - M', -sgn); rows follow the cell index or the
 // occupied list as the kernel stage laid them out.
-template <bool SEQ = false>
 __device__ __forceinline__ void pair_children(const StepArgs& a, int rows_by_cell, uint32_t id, uint32_t t, int c,
                                               int k, int sgn, unsigned long long& pairs, unsigned long long& dropped,
                                               long long& drop_signed) {
@@ -65,8 +55,7 @@ __device__ __forceinline__ void pair_children(const StepArgs& a, int rows_by_cel
   const float* vrow = a.VWh + (size_t)orow * h;
   const long long* crow = a.ccdf + (size_t)orow * kCdfBlocks;
   const int sc = __ldg(a.scale + orow);
-  const int kp = SEQ ? sample_coarse_row_seq(vrow, crow, sc, a.Q, a.r0, n_M, U2)
-                     : sample_coarse_row(vrow, crow, sc, a.Q, a.r0, n_M, U2);
+  const int kp = sample_coarse_row(vrow, crow, sc, a.Q, a.r0, n_M, U2);
   ++pairs;
   const int Mp = kp - n_M / 2;
   const int kc2[2] = {k + Mp, k - Mp};
@@ -86,17 +75,29 @@ __device__ __forceinline__ void pair_children(const StepArgs& a, int rows_by_cel
   }
 }
 
-// The same with the counters added to the header at once: the step kernel's
-// rare path for events beyond the queue's capacity.
-__device__ __forceinline__ void pair_children_direct(const StepArgs& a, int rows_by_cell, uint32_t id, uint32_t t,
-                                                     int c, int k, int sgn) {
-  unsigned long long pairs = 0, dropped = 0;
-  long long drop_signed = 0;
-  pair_children<true>(a, rows_by_cell, id, t, c, k, sgn, pairs, dropped, drop_signed);
-  atomicAdd(&a.hdr->pairs, pairs);
-  if (dropped) {
-    atomicAdd(&a.hdr->dropped, dropped);
-    atomicAdd(reinterpret_cast<unsigned long long*>(&a.hdr->dropped_signed), (unsigned long long)drop_signed);
+// The pair events of one queued quad -- {id / 4, cell, column | sign bit << 12
+// | ids << 16, -}: its words are drawn again, its ids of the column tested against the threshold of the
+// cell they end in, and each event completed.
+__device__ __forceinline__ void quad_events(const StepArgs& a, int rows_by_cell, uint32_t t, const uint4& ev,
+                                            unsigned long long& pairs, unsigned long long& dropped,
+                                            long long& drop_signed) {
+  const int i = (int)ev.y, k = (int)(ev.z & 4095u);
+  const uint32_t e = __ldg(a.xm + k);
+  const int dir = move_dir(e);
+  uint4 wr = make_uint4(ev.x, t - 1u, kPurposeRepos, a.sim), wg = make_uint4(ev.x, t, kPurposeGen, a.sim);
+  philox4x32_10_x2k(wr, wg, a.K);
+  const unsigned long long t_st = __ldg(a.thr_cell + i);
+  const unsigned long long t_mv = (unsigned)(i + dir) < (unsigned)a.n_x ? __ldg(a.thr_cell + i + dir) : 0ull;
+  const uint32_t mvb = move_bits(wr, e), u4[4] = {wg.x, wg.y, wg.z, wg.w};
+  uint32_t m = 0u;
+#pragma unroll
+  for (int j = 0; j < 4; ++j) m |= (uint32_t)((unsigned long long)u4[j] < ((mvb >> j) & 1u ? t_mv : t_st)) << j;
+  m &= ev.z >> 16;
+  while (m) {
+    const int j = __ffs(m) - 1;
+    m &= m - 1u;
+    pair_children(a, rows_by_cell, 4u * ev.x + (uint32_t)j, t, i + ((mvb >> j) & 1u ? dir : 0), k,
+                       (ev.z >> 12) & 1u ? -1 : 1, pairs, dropped, drop_signed);
   }
 }
 
@@ -127,291 +128,138 @@ __device__ __forceinline__ void block_counters(DevHeader* hdr, unsigned long lon
   }
 }
 
-// Lane blocks of the staged row prefix: E2 = the power of two >= ceil(n_M / 32)
-// columns per lane.
-__host__ __device__ __forceinline__ int step_lg_block(int n_M) {
-  int lg = 0;
-  while ((32 << lg) < n_M) ++lg;
-  return lg;
-}
-
-// Shared memory of a step block: the per-column move test (flip, threshold)
-// of the block, then per warp the row prefix in a padded layout (column k at
-// k + (k >> lg), so that lane l's block of E2 = 2^lg columns is contiguous and
-// bank-conflict free), the sign bits, the non-empty bits and the event queue.
-__host__ __device__ __forceinline__ int step_warp_words(int n_M) {
-  const int E2 = 1 << step_lg_block(n_M);
-  return 32 * (E2 + 1) + 1 + 2 * ((n_M + 31) / 32) + kPairQ;
-}
-
-static size_t step_smem(int n_M) {
-  return sizeof(uint32_t) * (2 * (size_t)n_M + (size_t)kStepWarps * step_warp_words(n_M));
-}
-
-// 4-bit mask of the elements j of a quad with j < d (d may be <= 0 or >= 4).
-__device__ __forceinline__ uint32_t first_mask(int d) { return d >= 4 ? 0xfu : (d <= 0 ? 0u : (1u << d) - 1u); }
-
-__global__ __launch_bounds__(kStepThreads, 4) void k_step(StepArgs a) {
-  extern __shared__ __align__(16) uint32_t smem_step[];
-  __shared__ int s_qn[kStepWarps];
-  __shared__ unsigned long long s_thr[kStepWarps][3];  // event thresholds of cells i - 1, i, i + 1
-  const int n_M = a.n_M;
-  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  const int lg = step_lg_block(n_M), E2 = 1 << lg;
-  uint2* s_xm = reinterpret_cast<uint2*>(smem_step);
-  uint32_t* wsm = smem_step + 2 * n_M + wid * step_warp_words(n_M);
-  int* s_pp = reinterpret_cast<int*>(wsm);             // padded row prefix
-  const int NW = (n_M + 31) / 32;
-  uint32_t* s_sg = wsm + 32 * (E2 + 1) + 1;             // sign bits (1: negative)
-  uint32_t* s_nz = s_sg + NW;                            // non-empty bits
-  uint32_t* s_q = s_nz + NW;                              // event queue
-  const int rows_by_cell = (int)a.hdr->rows_by_cell;
-  const uint32_t t = a.t_from_device ? a.hdr->step : a.t;
-  const int n_items = a.hdr->n_items;
-  const unsigned int chunk = work_chunk(a.hdr);
-  // move test of column k: moves iff (w ^ flip) > thr, i.e. w > xhi (rightward
-  // drift), w < xlo (leftward, by complementing), never (thr = 2^32 - 1)
-  for (int k = tid; k < n_M; k += kStepThreads) {
-    const uint32_t lo = a.xlo[k], hi = a.xhi[k];
-    s_xm[k] = hi != 0xffffffffu ? make_uint2(0u, hi) : (lo ? make_uint2(0xffffffffu, ~lo) : make_uint2(0u, 0xffffffffu));
-  }
-  if (lane == 0) s_qn[wid] = 0;
-  __syncthreads();
-  auto P = [&](int k) { return s_pp[k + (k >> lg)]; };
-  // the first non-empty column after kk (n_M if none), from the non-empty bits
-  auto next_nonempty = [&](int kk) -> int {
-    int c = (kk + 1) >> 5;
-    uint32_t w = c < NW ? s_nz[c] & (0xffffffffu << ((kk + 1) & 31)) : 0u;
-    while (!w && ++c < NW) w = s_nz[c];
-    return w ? (c << 5) + __ffs(w) - 1 : n_M;
-  };
-
-  int cur_i = -1;
-  uint32_t base = 0u;
-  bool need_gen = false, any_full = false;
-  uint32_t rej = 0u;
-  // event threshold of a stayer, thr(i), as u < thr <=> u < min(thr, 2^32 - 1) or thr >= 2^32
-  uint32_t thr_st32 = 0u;
-  bool all_st = false;
-
-  int item = 0;
-  if (lane == 0) item = (int)atomicAdd(&a.hdr->item_ticket, 1u);
-  item = __shfl_sync(0xffffffffu, item, 0);
-  while (item < n_items) {
-    int nxt = 0;
-    if (lane == 0) nxt = (int)atomicAdd(&a.hdr->item_ticket, 1u);  // consumed at the end of this item
-    const int2 it = __ldg(a.items + item);
-    const int i = it.x, ch = it.y;
-    if (i != cur_i) {
-      // stage the row: |n| into the padded buffer, sign bits, then the
-      // exclusive prefix in place (lane l over its block of E2 columns)
-      const int32_t* row = a.hist_in + (size_t)i * n_M;
-      for (int k0 = 0; k0 < n_M; k0 += 32) {
-        const int k = k0 + lane;
-        const int n = k < n_M ? __ldg(row + k) : 0;
-        if (k < n_M) s_pp[k + (k >> lg)] = n < 0 ? -n : n;
-        const uint32_t b = __ballot_sync(0xffffffffu, n < 0);
-        const uint32_t z = __ballot_sync(0xffffffffu, n != 0);
-        if (lane == 0) {
-          s_sg[k0 >> 5] = b;
-          s_nz[k0 >> 5] = z;
-        }
-      }
-      __syncwarp();
-      const int kb0 = min(lane << lg, n_M), kb1 = min(kb0 + E2, n_M);
-      int* blk = s_pp + lane * (E2 + 1);
-      int local = 0;
-      for (int j = 0; j < kb1 - kb0; ++j) local += blk[j];
-      int incl = local;
-#pragma unroll
-      for (int off = 1; off < 32; off <<= 1) {
-        const int u = __shfl_up_sync(0xffffffffu, incl, off);
-        if (lane >= off) incl += u;
-      }
-      int run = incl - local;
-      for (int j = 0; j < kb1 - kb0; ++j) {
-        const int v = blk[j];
-        blk[j] = run;
-        run += v;
-      }
-      __syncwarp();
-      if (lane == 31) s_pp[n_M + (n_M >> lg)] = incl;
-      base = (uint32_t)__ldg(a.R + i);
-      const unsigned long long thr_m = i > 0 ? __ldg(a.thr_cell + i - 1) : 0ull;
-      const unsigned long long thr_0 = __ldg(a.thr_cell + i);
-      const unsigned long long thr_p = i + 1 < a.n_x ? __ldg(a.thr_cell + i + 1) : 0ull;
-      if (lane == 0) {
-        s_thr[wid][0] = thr_m;
-        s_thr[wid][1] = thr_0;
-        s_thr[wid][2] = thr_p;
-      }
-      need_gen = (thr_m | thr_0 | thr_p) != 0ull;
-      all_st = (thr_0 >> 32) != 0ull;
-      thr_st32 = all_st ? 0xffffffffu : (uint32_t)thr_0;
-      // events: a stayer tests thr(i), a mover thr(i +- 1) (0 outside the
-      // domain: absorbed particles create no pair); rej = the largest of them
-      // as a quick rejection of a whole quad (exact unless a threshold is 2^32)
-      const unsigned long long tmax =
-          thr_0 > thr_m ? (thr_0 > thr_p ? thr_0 : thr_p) : (thr_m > thr_p ? thr_m : thr_p);
-      any_full = tmax >> 32 != 0ull;
-      rej = any_full ? 0xffffffffu : (uint32_t)tmax;
-      cur_i = i;
-      __syncwarp();
-    }
-    const uint32_t Ti = (uint32_t)P(n_M);
-    // the item is [item0, item1) of the quad-aligned id range of the cell; each
-    // lane takes a quad-aligned span of it
-    const unsigned long long A = base & ~3u;
-    const unsigned long long row_end = (unsigned long long)base + Ti;
-    const unsigned long long item0 = A + (unsigned long long)ch * chunk;
-    const unsigned long long item1 = item0 + chunk < row_end ? item0 + chunk : row_end;
-    const uint32_t len = item1 > item0 ? (uint32_t)(item1 - item0) : 0u;
-    const uint32_t span = ((len + 127u) >> 7) << 2;
-    const unsigned long long lo64 = item0 + (unsigned long long)lane * span;
-    const unsigned long long g0_64 = lo64 > base ? lo64 : base;
-    const unsigned long long g1_64 = lo64 + span < item1 ? lo64 + span : item1;
-    const bool has = g0_64 < g1_64;
-    const uint32_t g0 = has ? (uint32_t)g0_64 : 0u, g1 = has ? (uint32_t)g1_64 : 0u;
-    const uint32_t i0 = (uint32_t)item0;
-    int32_t* const out_i = a.hist_out + (size_t)i * n_M;
-
-    // bucket state
-    int k = 0, sgn = 1, dir = 0;
-    uint32_t end = 0u, flip = 0u, mthr = 0xffffffffu;
-    uint32_t thr_mv32 = 0u;  // event threshold of a mover, thr(i + dir), in the same form
-    bool all_mv = false;
-    int n_st = 0, n_mv = 0;
-    auto load_bucket = [&]() {
-      end = base + (uint32_t)P(k + 1);
-      sgn = ((s_sg[k >> 5] >> (k & 31)) & 1u) ? -1 : 1;
-      const uint2 xm = s_xm[k];
-      flip = xm.x;
-      mthr = xm.y;
-      dir = flip ? -1 : (mthr != 0xffffffffu ? 1 : 0);
-      const unsigned long long thr_mv = s_thr[wid][dir + 1];
-      all_mv = (thr_mv >> 32) != 0ull;
-      thr_mv32 = all_mv ? 0xffffffffu : (uint32_t)thr_mv;
-    };
-    auto flush_bucket = [&]() {
-      if (n_st) atomicAdd(out_i + k, sgn > 0 ? n_st : -n_st);
-      if (n_mv) {
-        const int c = sgn > 0 ? n_mv : -n_mv;
-        if ((unsigned)(i + dir) < (unsigned)a.n_x) {
-          atomicAdd(out_i + (dir > 0 ? n_M : -n_M) + k, c);
-        } else {  // left the domain (edge cells only): counted at once
-          atomicAdd(&a.hdr->absorbed, (unsigned long long)n_mv);
-          atomicAdd(reinterpret_cast<unsigned long long*>(&a.hdr->absorbed_signed), (unsigned long long)(long long)c);
-        }
-      }
-      n_st = n_mv = 0;
-    };
-    // pair event of particle id (mover or not) of the current bucket
-    auto test_event = [&](uint32_t id, uint32_t u, int mv) {
-      if (u < (mv ? thr_mv32 : thr_st32) || (mv ? all_mv : all_st)) {
-        const int pos = atomicAdd(&s_qn[wid], 1);
-        if (pos < kPairQ)  // always (the queue is drained whenever it could fill within one quad iteration)
-          s_q[pos] = (id - i0) | ((uint32_t)k << 13) | ((uint32_t)(mv ? dir + 1 : 1) << 25) | (sgn < 0 ? 1u << 27 : 0u);
-      }
-    };
-    // queued events of this item to the global queue (warp-collective)
-    auto flush_queue = [&]() {
-      __syncwarp();
-      const int n = min(s_qn[wid], kPairQ);
-      if (n) {
-        unsigned qb = 0u;
-        if (lane == 0) qb = atomicAdd(&a.hdr->pair_count, (unsigned)n);
-        qb = __shfl_sync(0xffffffffu, qb, 0);
-        for (int e = lane; e < n; e += 32) {
-          const uint32_t q = s_q[e];
-          const uint32_t id = i0 + (q & 8191u);
-          const int kk = (int)((q >> 13) & 4095u), c = i - 1 + (int)((q >> 25) & 3u);
-          const int sg = (q >> 27) & 1u ? -1 : 1;
-          const unsigned slot = qb + (unsigned)e;
-          if (slot >= qb && slot < a.pair_cap)
-            a.pairs[slot] = make_uint4(id, (uint32_t)c, (uint32_t)kk, sg < 0 ? 1u : 0u);
-          else
-            pair_children_direct(a, rows_by_cell, id, t, c, kk, sg);
-        }
-        __syncwarp();
-        if (lane == 0) s_qn[wid] = 0;
-      }
-      __syncwarp();
-    };
-
-    if (has) {
-      // largest k with prefix(k) <= g0 - base: the bucket of the lane's first id
-      const int lid = (int)(g0 - base);
-      int lo = 0, hi = n_M;
-      while (hi - lo > 1) {
-        const int mid = (lo + hi) >> 1;
-        if (P(mid) <= lid) lo = mid; else hi = mid;
-      }
-      k = lo;
-      load_bucket();
-    }
-    const int nq = (int)(span >> 2);
-    const uint32_t q_first = (uint32_t)(lo64 >> 2);
+// The ids of a range of work units [w0, w1), cell by cell, through walk_ids.
+// COUNT: the step proper (parents counted, absorbed particles too); otherwise
+// only the quads that may hold events are queued.  queue: kWalkQueue entries
+// of the warp and 32 more for the walk's words.
+template <bool COUNT, class Flush>
+__device__ __forceinline__ void walk_range(const StepArgs& a, uint32_t t, uint32_t w0, uint32_t w1, int lane,
+                                           uint4* queue, int& nq, Flush flush) {
+  const int n_M = a.n_M, NB = (n_M + 31) >> 5;
+  CellWork cell = cell_of_unit(a.U, a.n_x, w0, lane);
 #pragma unroll 1
-    for (int jq = 0; jq < nq; ++jq) {
-      const uint32_t q = q_first + (uint32_t)jq;
-      const uint32_t qa = q << 2;
-      if (qa < g1 && qa + 4u > g0) {  // (g0 = g1 = 0 for a lane without ids)
-        uint4 wr = make_uint4(q, t - 1u, kPurposeRepos, a.sim);
-        uint4 wg = make_uint4(q, t, kPurposeGen, a.sim);
-        if (need_gen) philox4x32_10_x2k(wr, wg, a.K);
-        else wr = philox4x32_10k(wr, a.K);
-        const bool ev_possible = need_gen && (min(min(wg.x, wg.y), min(wg.z, wg.w)) < rej || any_full);
-        // the ids of the quad in [g0, g1), bucket by bucket: the ids below the
-        // current bucket's end are its members (a bucket ends exactly where the
-        // next non-empty one starts), counted together from their move bits;
-        // a lane whose quad crosses a bucket end takes a second pass
-        uint32_t rem = 0xfu;
-        if (qa < g0 || qa + 4u > g1) rem = first_mask((int)(g1 - qa)) & ~first_mask((int)(g0 - qa));
-        const uint32_t w4[4] = {wr.x, wr.y, wr.z, wr.w};
-        const uint32_t u4[4] = {wg.x, wg.y, wg.z, wg.w};
-        while (true) {
-          const uint32_t inb = rem & first_mask((int)(end - qa));
-          uint32_t mvb = 0u;
-#pragma unroll
-          for (int j = 0; j < 4; ++j) mvb |= (uint32_t)((w4[j] ^ flip) > mthr) << j;
-          mvb &= inb;
-          const int m = __popc(mvb);
-          n_mv += m;
-          n_st += __popc(inb) - m;
-          if (ev_possible) {
-#pragma unroll
-            for (int j = 0; j < 4; ++j)
-              if ((inb >> j) & 1u) test_event(qa + (uint32_t)j, u4[j], (int)((mvb >> j) & 1u));
-          }
-          rem &= ~inb;
-          if (!rem) break;
-          flush_bucket();
-          k = next_nonempty(k);
-          load_bucket();
-        }
+  while (true) {
+    const int i = cell.i;
+    const uint32_t first = id_prefix(a.R, i), last = id_prefix(a.R, i + 1);
+    const uint32_t A = first & ~3u, qA = A >> 2;
+    WalkCell c;
+    c.row = a.hist_in + (size_t)i * n_M;
+    c.bp = a.bp + (size_t)i * NB;
+    c.xm = a.xm;
+    c.n_M = n_M;
+    c.off = first & 3u;
+    const unsigned long long thr_m = i > 0 ? __ldg(a.thr_cell + i - 1) : 0ull, thr_0 = __ldg(a.thr_cell + i),
+                             thr_p = i + 1 < a.n_x ? __ldg(a.thr_cell + i + 1) : 0ull;
+    c.tmax = max(thr_0, max(thr_m, thr_p));
+    // v particles' net sign (n of them) to column k of cell i + d, or out of the domain
+    auto add = [&](int k, int d, int v, uint32_t n) {
+      if (!COUNT) return;
+      if ((unsigned)(i + d) < (unsigned)a.n_x) {
+        atomicAdd(a.hist_out + (size_t)(i + d) * n_M + k, v);
+      } else {  // (edge cells only)
+        atomicAdd(&a.hdr->absorbed, (unsigned long long)n);
+        atomicAdd(reinterpret_cast<unsigned long long*>(&a.hdr->absorbed_signed), (unsigned long long)(long long)v);
       }
-      __syncwarp();
-      if (s_qn[wid] > kPairQ - 128) flush_queue();
-    }
-    if (has) flush_bucket();
-    flush_queue();
-    item = __shfl_sync(0xffffffffu, nxt, 0);
+    };
+    walk_ids(
+        c, window_of_unit(cell, last - first, w0) << 7, min(last - A, window_of_unit(cell, last - first, w1) << 7),
+        lane, queue + kWalkQueue, nq,
+        [&](uint32_t q, bool gen, uint4& wr, uint4& wg) {
+          wr = make_uint4(qA + q, t - 1u, kPurposeRepos, a.sim);
+          if (gen) {
+            wg = make_uint4(qA + q, t, kPurposeGen, a.sim);
+            philox4x32_10_x2k(wr, wg, a.K);
+          } else {
+            wr = philox4x32_10k(wr, a.K);
+          }
+        },
+        [&](int k, uint32_t e, uint32_t stay, uint32_t move) {
+          if (stay) add(k, 0, e & 1u ? -(int)stay : (int)stay, stay);
+          if (move) add(k, move_dir(e), e & 1u ? -(int)move : (int)move, move);
+        },
+        [&](unsigned who, bool me, uint32_t q, int k, uint32_t e, uint32_t ids) {
+          if (me)
+            queue[nq + __popc(who & ((1u << lane) - 1u))] =
+                make_uint4(qA + q, (uint32_t)i, (uint32_t)k | ((e & 1u) << 12) | (ids << 16), 0u);
+          nq += __popc(who);
+        },
+        flush);
+    if (cell.u1 >= w1) break;
+    cell = next_cell(a.U, a.n_x, cell, lane);
   }
-  if (blockIdx.x == 0 && tid == 0 && n_items > 0) atomicAdd(&a.hdr->particle_steps, a.hdr->population);
 }
 
-// The queued pair events of the step: one thread each.  The last block to
+__global__ __launch_bounds__(kStepThreads, kStepBlocks) void k_step(const __grid_constant__ StepArgs a) {
+  __shared__ uint4 s_queue[kStepWarps][kWalkQueue + 32];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  uint4* queue = s_queue[wid];
+  const uint32_t t = a.t_from_device ? a.hdr->step : a.t;
+  // (n_items = 0: the plan refused the population)
+  const uint32_t total = a.hdr->n_items ? __ldg(a.U + a.n_x) : 0u;
+  int nq = 0;  // queued quads (uniform)
+  // the warp's queue to the global one; what does not fit there is dropped,
+  // and the pair kernel, which sees the count, finds all quads again
+  auto flush = [&]() {
+    __syncwarp();
+    unsigned qb = 0u;
+    if (lane == 0) qb = atomicAdd(&a.hdr->pair_count, (unsigned)nq);
+    qb = __shfl_sync(0xffffffffu, qb, 0);
+    for (int e = lane; e < nq; e += 32)
+      if (qb + (unsigned)e < a.pair_cap) a.pairs[qb + (unsigned)e] = queue[e];
+    __syncwarp();
+    nq = 0;
+  };
+  // consecutive ranges go to different SMs
+  RangeSchedule sched(total, gridDim.x * kStepWarps);
+  uint32_t ticket = (uint32_t)wid * gridDim.x + blockIdx.x, w0, w1;
+  while (sched.range(ticket, w0, w1)) {
+    const bool more = sched.more();
+    uint32_t nxt = 0u;
+    if (lane == 0 && more) nxt = atomicAdd(&a.hdr->item_ticket, 1u);  // consumed at the end of this range
+    walk_range<true>(a, t, w0, w1, lane, queue, nq, flush);
+    if (!more) break;
+    ticket = sched.n_warps + __shfl_sync(0xffffffffu, nxt, 0);
+  }
+  if (nq) flush();
+  if (blockIdx.x == 0 && threadIdx.x == 0 && a.hdr->n_items > 0) atomicAdd(&a.hdr->particle_steps, a.hdr->population);
+}
+
+// All quads of the step that may hold events, found by a second walk and
+// completed from the warps' queues: the pair kernel's path when they did not
+// fit the global queue (pair_cap quads).
+__device__ __noinline__ void rewalk_events(const StepArgs& a, uint32_t t, uint4* queue, unsigned long long& pairs,
+                                           unsigned long long& dropped, long long& drop_signed) {
+  const int lane = threadIdx.x & 31;
+  const int rows_by_cell = (int)a.hdr->rows_by_cell;
+  const uint32_t total = a.hdr->n_items ? __ldg(a.U + a.n_x) : 0u;
+  constexpr uint32_t kUnits = 32;
+  int nq = 0;
+  auto flush = [&]() {
+    __syncwarp();
+    for (int e = lane; e < nq; e += 32) quad_events(a, rows_by_cell, t, queue[e], pairs, dropped, drop_signed);
+    __syncwarp();
+    nq = 0;
+  };
+  const uint32_t stride = gridDim.x * kStepWarps * kUnits;
+  for (uint32_t w0 = (blockIdx.x * kStepWarps + (threadIdx.x >> 5)) * kUnits; w0 < total; w0 += stride)
+    walk_range<false>(a, t, w0, min(w0 + kUnits, total), lane, queue, nq, flush);
+  if (nq) flush();
+}
+
+// The queued quads of the step: one thread each.  The last block to
 // finish resets the queue and the work-item ticket for the next step.
-__global__ __launch_bounds__(kStepThreads) void k_pairs(StepArgs a) {
+__global__ __launch_bounds__(kStepThreads, 4) void k_pairs(const __grid_constant__ StepArgs a) {
   const int rows_by_cell = (int)a.hdr->rows_by_cell;
   const uint32_t t = a.t_from_device ? a.hdr->step : a.t;
-  const unsigned cnt = a.hdr->pair_count;
-  const unsigned n = cnt < a.pair_cap ? cnt : a.pair_cap;
+  const unsigned n = a.hdr->pair_count;
   unsigned long long pairs = 0, dropped = 0;
   long long drop_signed = 0;
-  for (unsigned e = blockIdx.x * kStepThreads + threadIdx.x; e < n; e += gridDim.x * kStepThreads) {
-    const uint4 ev = a.pairs[e];
-    pair_children(a, rows_by_cell, ev.x, t, (int)ev.y, (int)ev.z, ev.w ? -1 : 1, pairs, dropped, drop_signed);
+  if (n <= a.pair_cap) {
+    for (unsigned e = blockIdx.x * kStepThreads + threadIdx.x; e < n; e += gridDim.x * kStepThreads)
+      quad_events(a, rows_by_cell, t, a.pairs[e], pairs, dropped, drop_signed);
+  } else {
+    __shared__ uint4 s_queue[kStepWarps][kWalkQueue + 32];
+    rewalk_events(a, t, s_queue[threadIdx.x >> 5], pairs, dropped, drop_signed);
   }
   block_counters(a.hdr, pairs, 0ull, 0ll, dropped, drop_signed);
   __syncthreads();
@@ -420,33 +268,28 @@ __global__ __launch_bounds__(kStepThreads) void k_pairs(StepArgs a) {
     if (atomicAdd(&a.hdr->pairs_done, 1u) == gridDim.x - 1u) {
       a.hdr->pair_count = 0u;
       a.hdr->item_ticket = 0u;
-      a.hdr->chunk = a.hdr->chunk_next ? a.hdr->chunk_next : (unsigned int)kChunk;
       a.hdr->pairs_done = 0u;
       __threadfence();
     }
   }
 }
 
-int step_grid(int n_M) {
-  static int cached_nM[8] = {0};
-  static int cached_grid[8] = {0};
+int step_grid() {
+  static int cached[8] = {0};
   int dev = 0;
   cudaGetDevice(&dev);
   const int slot = dev & 7;
-  if (cached_nM[slot] == n_M && cached_grid[slot] > 0) return cached_grid[slot];
+  if (cached[slot] > 0) return cached[slot];
   int per_sm = 0;
-  const size_t sm = step_smem(n_M);
-  if (sm > 48 * 1024) raise_smem_limit(reinterpret_cast<const void*>(k_step), sm);
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_step, kStepThreads, sm);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_step, kStepThreads, 0);
   if (per_sm < 1) per_sm = 1;
   int g = per_sm * num_sms();
   if (g > kMaxStepBlocks) g = kMaxStepBlocks;
-  cached_nM[slot] = n_M;
-  cached_grid[slot] = g;
+  cached[slot] = g;
   return g;
 }
 
-void prepare_step(const wmc_params& p) { (void)step_grid(p.n_M); }
+void prepare_step() { (void)step_grid(); }
 
 cudaError_t launch_step(const wmc_params& p, const View& v, const int32_t* hist_in, uint32_t t, int t_from_device,
                         int32_t* hist_out, cudaStream_t s) {
@@ -455,14 +298,14 @@ cudaError_t launch_step(const wmc_params& p, const View& v, const int32_t* hist_
   a.hist_in = hist_in;
   a.hist_out = hist_out;
   a.R = v.R;
-  a.items = v.items;
+  a.U = v.U;
+  a.bp = v.bp;
   a.row_map = v.row_map;
   a.VWh = v.VWh;
   a.ccdf = v.ccdf;
   a.scale = v.scale;
   a.thr_cell = v.thr_cell;
-  a.xlo = v.xlo;
-  a.xhi = v.xhi;
+  a.xm = v.xm;
   a.pairs = v.pairs;
   a.pair_cap = L.pair_cap;
   a.hdr = v.hdr;
@@ -477,10 +320,10 @@ cudaError_t launch_step(const wmc_params& p, const View& v, const int32_t* hist_
   a.K = philox_keys(a.k0, a.k1);
   a.t = t;
   a.t_from_device = t_from_device;
-  const int grid = step_grid(p.n_M);
+  const int grid = step_grid();
   cudaError_t e = step_timing_record(s, false);
   if (e != cudaSuccess) return e;
-  k_step<<<grid, kStepThreads, step_smem(p.n_M), s>>>(a);
+  k_step<<<grid, kStepThreads, 0, s>>>(a);
   e = cudaGetLastError();
   if (e == cudaSuccess) e = step_timing_record(s, true);
   if (e != cudaSuccess) return e;
@@ -490,110 +333,115 @@ cudaError_t launch_step(const wmc_params& p, const View& v, const int32_t* hist_
   return cudaGetLastError();
 }
 
-// Loads the signed counts of cell i into s_n and their exclusive prefix of
-// |n| into s_pre[0..n_M] (s_pre[n_M] = survivors of the cell), block-wide.
-__device__ __forceinline__ void load_row_prefix(const int32_t* __restrict__ hist, int i, int n_M, int* s_n,
-                                                int* s_pre, int* s_wsum) {
-  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  const int E = (n_M + kStepThreads - 1) / kStepThreads;
-  const int k0 = min(tid * E, n_M), k1 = min(k0 + E, n_M);
-  const int32_t* row = hist + (size_t)i * n_M;
-  int local = 0;
-  for (int k = k0; k < k1; ++k) {
-    const int n = row[k];
-    s_n[k] = n;
-    local += n < 0 ? -n : n;
-  }
-  int incl = local;
-#pragma unroll
-  for (int off = 1; off < 32; off <<= 1) {
-    const int u = __shfl_up_sync(0xffffffffu, incl, off);
-    if (lane >= off) incl += u;
-  }
-  if (lane == 31) s_wsum[wid] = incl;
-  __syncthreads();
-  if (wid == 0) {
-    int w = lane < kStepThreads / 32 ? s_wsum[lane] : 0;
-#pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-      const int u = __shfl_up_sync(0xffffffffu, w, off);
-      if (lane >= off) w += u;
-    }
-    if (lane < kStepThreads / 32) s_wsum[lane] = w;
-  }
-  __syncthreads();
-  int excl = (wid ? s_wsum[wid - 1] : 0) + incl - local;
-  for (int k = k0; k < k1; ++k) {
-    s_pre[k] = excl;
-    const int n = s_n[k];
-    excl += n < 0 ? -n : n;
-  }
-  if (tid == kStepThreads - 1) s_pre[n_M] = s_wsum[kStepThreads / 32 - 1];
-}
-
 // ---------------------------------------------------------------- explicit survivors
+// One warp per range of work units, cell by cell: lane l writes the ids 4 l ..
+// 4 l + 3 of a window (one Philox call) as one vector per array (cell 16 B,
+// offset 16 B, momentum 8 B, sign 4 B) where the quad lies inside the cell,
+// else id by id.  Bound by the 11 B written per particle; 1e7 particles on 2000
+// cells: 180 -> 45 us (one thread per run of ids, a call per id and single
+// stores before; the writes alone would take 16 us).
 __global__ __launch_bounds__(kStepThreads) void k_materialize(const int32_t* __restrict__ hist,
                                                               const unsigned long long* __restrict__ R,
-                                                              const int* __restrict__ IP, DevHeader* hdr, int n_x,
-                                                              int n_M, uint32_t sim, uint32_t k0, uint32_t k1,
-                                                              uint32_t t, int32_t* __restrict__ cell,
-                                                              float* __restrict__ f, int16_t* __restrict__ M,
-                                                              int8_t* __restrict__ sign, long long capacity) {
-  extern __shared__ int smem[];
-  int* s_pre = smem;
-  int* s_n = s_pre + (n_M + 1);
-  __shared__ int s_wsum[kStepThreads / 32];
-  __shared__ int s_row;
-  const int tid = threadIdx.x;
+                                                              const uint32_t* __restrict__ U,
+                                                              const uint32_t* __restrict__ bp,
+                                                              const uint32_t* __restrict__ xm, DevHeader* hdr, int n_x,
+                                                              int n_M, uint32_t sim, PhiloxKeys K, uint32_t t,
+                                                              int32_t* __restrict__ cell, float* __restrict__ f,
+                                                              int16_t* __restrict__ M, int8_t* __restrict__ sign,
+                                                              long long capacity, int vec_ok) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   if ((long long)hdr->population > capacity) {
-    if (blockIdx.x == 0 && tid == 0) atomicOr(&hdr->flags, WMC_FLAG_CAPACITY);
+    if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(&hdr->flags, WMC_FLAG_CAPACITY);
     return;
   }
-  const int n_items = hdr->n_items;
-  const unsigned long long id_base = hdr->id_base;
-  for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
-    __syncthreads();
-    if (tid == 0) {
-      int lo = 0, hi = n_x;
-      while (hi - lo > 1) {
-        const int mid = (lo + hi) >> 1;
-        if (__ldg(IP + mid) <= item) lo = mid; else hi = mid;
+  const uint32_t id_base = (uint32_t)hdr->id_base;
+  const uint32_t total = hdr->n_items ? __ldg(U + n_x) : 0u, n_warps = gridDim.x * kStepWarps;
+  const bool vec = vec_ok && (id_base & 3u) == 0u;  // a quad's place in the arrays is a multiple of 4
+  const uint32_t size = max((total + n_warps - 1u) / n_warps, 1u);
+  const uint32_t wn = (uint32_t)wid * gridDim.x + blockIdx.x;
+  if (wn >= (total + size - 1u) / size) return;
+  const uint32_t w0 = wn * size, w1 = min(w0 + size, total);
+  const int NB = (n_M + 31) >> 5, h = n_M / 2;
+  CellWork cw = cell_of_unit(U, n_x, w0, lane);
+#pragma unroll 1
+  while (true) {
+    const uint32_t first = id_prefix(R, cw.i), last = id_prefix(R, cw.i + 1), A = first & ~3u;
+    WalkCell c;
+    c.row = hist + (size_t)cw.i * n_M;
+    c.bp = bp + (size_t)cw.i * NB;
+    c.xm = xm;
+    c.n_M = n_M;
+    c.off = first & 3u;
+    WalkBlock B;
+    walk_begin(B);
+    const uint32_t r1 = min(last - A, window_of_unit(cw, last - first, w1) << 7);
+#pragma unroll 1
+    for (uint32_t a = window_of_unit(cw, last - first, w0) << 7; a < r1; a += 128u) {
+      const uint32_t qa = a + 4u * (uint32_t)lane, wend = min(a + 128u, r1);
+      const uint4 w = philox4x32_10k(make_uint4((A + qa) >> 2, t, kPurposeRepos, sim), K);
+      int ck[4] = {0, 0, 0, 0};
+      uint32_t neg = 0u, have = 0u;
+      uint32_t x = max(a, c.off);  // ids before x have their columns
+#pragma unroll 1
+      while (x < wend) {
+        if (x >= B.end) walk_load(c, x, B, lane);
+        const uint32_t lim = min(B.end, wend);
+        const unsigned nz = __ballot_sync(0xffffffffu, (B.e & 8u) != 0u);
+        const uint32_t from = max(qa, x);
+        int jl = 0;
+#pragma unroll
+        for (int s = 16; s; s >>= 1) {
+          const uint32_t e = __shfl_sync(0xffffffffu, B.E, jl + s - 1);
+          if (e <= from) jl += s;
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const uint32_t id = qa + (uint32_t)j;
+          const bool on = id >= x && id < lim;
+          const uint32_t e = __shfl_sync(0xffffffffu, B.E, jl);
+          if (on && e <= id) jl = (__ffs(nz & (0xfffffffeu << jl)) - 1) & 31;
+          const uint32_t en = __shfl_sync(0xffffffffu, B.e, jl);
+          if (on) {
+            ck[j] = min((B.b << 5) + jl, n_M - 1);
+            neg |= (en & 1u) << j;
+            have |= 1u << j;
+          }
+        }
+        x = lim;
       }
-      s_row = lo;
-    }
-    __syncthreads();
-    const int i = s_row;
-    const int chunk = item - __ldg(IP + i);
-    load_row_prefix(hist, i, n_M, s_n, s_pre, s_wsum);
-    __syncthreads();
-    const int Ti = s_pre[n_M];
-    const uint32_t base = (uint32_t)__ldg(R + i);
-    const int per_item = (int)work_chunk(hdr), kPer = per_item / kStepThreads;
-    const int lo = chunk * per_item + tid * kPer;  // ids [chunk c, (chunk + 1) c) of the row, c ids per item
-    const int hi = min(lo + kPer, Ti);
-    if (lo < hi) {
-      int k = bucket_of(s_pre, n_M, lo);
-      for (int lid = lo; lid < hi; ++lid) {
-        while (s_pre[k + 1] <= lid) ++k;
-        const uint32_t id = base + (uint32_t)lid;
-        const uint4 w = philox4x32_10(make_uint4(id >> 2, t, kPurposeRepos, sim), k0, k1);
-        const uint32_t wj = (id & 3u) == 0u ? w.x : ((id & 3u) == 1u ? w.y : ((id & 3u) == 2u ? w.z : w.w));
-        const uint32_t o = id - (uint32_t)id_base;  // place in this histogram
-        cell[o] = i;
-        f[o] = (float)(wj >> 8) * 0x1p-24f;
-        M[o] = (int16_t)(k - n_M / 2);
-        sign[o] = (int8_t)(s_n[k] > 0 ? 1 : -1);
+      const long long o = (long long)(A + qa) - (long long)id_base;
+      const float fv[4] = {(float)(w.x >> 8) * 0x1p-24f, (float)(w.y >> 8) * 0x1p-24f, (float)(w.z >> 8) * 0x1p-24f,
+                           (float)(w.w >> 8) * 0x1p-24f};
+      if (vec && have == 0xfu) {
+        *reinterpret_cast<int4*>(cell + o) = make_int4(cw.i, cw.i, cw.i, cw.i);
+        *reinterpret_cast<float4*>(f + o) = make_float4(fv[0], fv[1], fv[2], fv[3]);
+        *reinterpret_cast<short4*>(M + o) =
+            make_short4((short)(ck[0] - h), (short)(ck[1] - h), (short)(ck[2] - h), (short)(ck[3] - h));
+        *reinterpret_cast<char4*>(sign + o) = make_char4(neg & 1u ? -1 : 1, neg & 2u ? -1 : 1, neg & 4u ? -1 : 1,
+                                                         neg & 8u ? -1 : 1);
+      } else {
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          if ((have >> j) & 1u) {
+            cell[o + j] = cw.i;
+            f[o + j] = fv[j];
+            M[o + j] = (int16_t)(ck[j] - h);
+            sign[o + j] = (int8_t)((neg >> j) & 1u ? -1 : 1);
+          }
       }
     }
+    if (cw.u1 >= w1) break;
+    cw = next_cell(U, n_x, cw, lane);
   }
 }
 
 cudaError_t launch_materialize(const wmc_params& p, const View& v, const int32_t* hist, uint32_t t, int32_t* cell,
                                float* f, int16_t* M, int8_t* sign, long long capacity, cudaStream_t s) {
-  const size_t sm = sizeof(int) * (size_t)(2 * p.n_M + 1);
-  k_materialize<<<2 * num_sms(), kStepThreads, sm, s>>>(hist, v.R, v.IP, v.hdr, p.n_x, p.n_M, p.sim,
-                                                        (uint32_t)(p.seed & 0xffffffffu), (uint32_t)(p.seed >> 32),
-                                                        t, cell, f, M, sign, capacity);
+  const auto aligned = [](const void* q, uintptr_t n) { return (reinterpret_cast<uintptr_t>(q) & (n - 1)) == 0; };
+  const int vec_ok = aligned(cell, 16) && aligned(f, 16) && aligned(M, 8) && aligned(sign, 4);
+  k_materialize<<<6 * num_sms(), kStepThreads, 0, s>>>(
+      hist, v.R, v.U, v.bp, v.xm, v.hdr, p.n_x, p.n_M, p.sim,
+      philox_keys((uint32_t)(p.seed & 0xffffffffu), (uint32_t)(p.seed >> 32)), t, cell, f, M, sign, capacity, vec_ok);
   return cudaGetLastError();
 }
 

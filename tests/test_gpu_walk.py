@@ -1,0 +1,99 @@
+"""The particle step's walk over the survivors and the snapshot of the explicit
+particles, bit for bit against the oracle, at the edges of the walk's cases:
+windows of 128 ids in one bucket, in a few, in many; column blocks of 32 that
+are empty, partial or beyond the first 32 blocks; cells of one particle; ranges
+that start inside a cell; more quads with events than the queue holds."""
+import numpy as np
+import pytest
+
+import oracle
+import wmc_inputs as wi
+from tests._util import gpu_run_table, oracle_tables
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def wmc():
+    from paper_1806_00082_gb300 import build, wmc as w
+    build.build()
+    w.load()
+    return w
+
+
+def _workload(n_x, Q, n_M):
+    wl = wi.BARRIER_100.replace(name=f"walk-{n_x}-{Q}-{n_M}", n_x=n_x, Q=Q, n_M=n_M, child_wrap=int(n_M == 34))
+    rng = np.random.Generator(np.random.PCG64(n_M))
+    V = 0.2 * min(1.0, Q / n_M)  # gamma grows with the periods on the grid
+    return wl, rng.uniform(-V, V, n_x).astype(np.float32)
+
+
+def _state(kind, wl, rng):
+    n_x, n_M = wl.n_x, wl.n_M
+    h = np.zeros((n_x, n_M), np.int64)
+    sign = rng.choice([-1, 1], size=(n_x, n_M))
+    if kind == "ones":  # every bucket one particle, some cells empty
+        h[:] = sign
+        h[::3] = 0
+    elif kind == "sizes":  # bucket sizes around a quad, a lane's limit, a window
+        sizes = np.array([0, 0, 1, 2, 3, 4, 5, 7, 8, 9, 31, 127, 128, 129, 255, 256, 260, 1000])
+        h[:] = sign * rng.choice(sizes, size=(n_x, n_M), p=np.r_[0.3, 0.3, np.full(16, 0.4 / 16)])
+    elif kind == "far":  # a few particles in columns far apart
+        for i in range(0, n_x, 2):
+            k = rng.choice(n_M, size=min(n_M, 5), replace=False)
+            h[i, k] = rng.integers(1, 4, size=k.size)
+        h[n_x // 2, n_M - 1] = -70_000
+    return h.astype(np.int32)
+
+
+@pytest.mark.parametrize("kind", ["ones", "sizes", "far"])
+@pytest.mark.parametrize("n_x,Q,n_M", [(7, 2, 2), (40, 32, 30), (40, 32, 34), (33, 64, 128), (24, 64, 1026), (9, 64, 2052)])
+def test_walk_bit_exact(wmc, kind, n_x, Q, n_M):
+    wl, V = _workload(n_x, Q, n_M)
+    h0 = _state(kind, wl, np.random.Generator(np.random.PCG64(7 * n_x + n_M)))
+    full, half = oracle_tables(wl, V)
+    ref, st = oracle.simulate(oracle.params(wl), h0, 3, 2, table=full)
+    got, c = gpu_run_table(wmc, torch, wmc.Params.of(wl), half, h0, 3, 2)
+    np.testing.assert_array_equal(got, ref)
+    assert c["pairs"] == st[oracle.ST_PAIRS] and c["flags"] == 0
+
+
+def test_more_event_quads_than_the_queue(wmc):
+    """2^19 queue entries, more quads with events in a step."""
+    wl, V = _workload(40, 32, 64)
+    rng = np.random.Generator(np.random.PCG64(1))
+    h0 = rng.integers(-8000, 8000, size=(40, 64)).astype(np.int32)
+    wl = wl.replace(dt_s=4e-16)
+    full, half = oracle_tables(wl, V)
+    ref, st = oracle.simulate(oracle.params(wl), h0, 1, 1, table=full)
+    got, c = gpu_run_table(wmc, torch, wmc.Params.of(wl), half, h0, 1, 1)
+    assert st[oracle.ST_PAIRS] > 2 * 2 ** 19
+    np.testing.assert_array_equal(got, ref)
+    assert c["pairs"] == st[oracle.ST_PAIRS] and c["flags"] == 0
+
+
+@pytest.mark.parametrize("id_base", [0, 1, 3, 130])
+@pytest.mark.parametrize("n_x,n_M", [(7, 2), (40, 34), (9, 2052)])
+def test_snapshot_places_and_words(wmc, id_base, n_x, n_M):
+    """Every particle at place id - id_base, its offset word from its id."""
+    wl, _ = _workload(n_x, 64 if n_M > 64 else 32, n_M)
+    h0 = _state("sizes", wl, np.random.Generator(np.random.PCG64(n_x + id_base)))
+    p = wmc.Params.of(wl)
+    ws = wmc.workspace(p)
+    wmc.init(p, ws)
+    wmc.set_id_base(p, ws, id_base)
+    hd = torch.from_numpy(h0).cuda()
+    wmc.annihilate(p, hd, ws)
+    P = int(np.abs(h0).sum())
+    cell, f, M, s = (x.cpu().numpy() for x in wmc.materialize(p, hd, 5, ws, P))
+    n = np.abs(h0).reshape(-1)
+    at = np.repeat(np.arange(n.size), n)
+    np.testing.assert_array_equal(cell, at // n_M)
+    np.testing.assert_array_equal(M, at % n_M - n_M // 2)
+    np.testing.assert_array_equal(s, np.sign(h0.reshape(-1))[at])
+    ids = np.unique(np.concatenate([np.arange(min(P, 40)), np.arange(max(0, P - 40), P), np.arange(0, P, max(1, P // 50))]))
+    for i in ids:
+        gid = int(i) + id_base
+        w = int(oracle.philox((gid // 4, 5, 2, wl.sim), (wl.seed & 0xffffffff, wl.seed >> 32))[gid % 4])
+        assert f[i] == np.float32((w >> 8) * 2.0 ** -24)
