@@ -6,19 +6,19 @@
 //
 // Cells of all simulations are concatenated (global cell c = cell_off[s] + i);
 // per-cell arrays (survivors, id prefix, reach bits, row map, thresholds) are
-// indexed by global cell, and the survivor-id prefix, work items and occupied
+// indexed by global cell, and the survivor-id prefix, work units and occupied
 // list come from one scan over all cells (three passes: block sums, a scan of
 // the block sums, and the final block scan).  Ids restart at 0 in every
 // simulation: id = G[c] - G[cell_off[s]] + (offset within the cell).
 //
-// The work-item size (threads x ids per thread) is a run-time parameter chosen
-// by wmc_batch_autotune; the results do not depend on it.
+// The largest range of ids a warp takes at a time is a run-time parameter
+// (ids per lane) chosen by wmc_batch_autotune; the results do not depend on it.
 #include <string.h>
 
 #include <mutex>
 #include <vector>
 
-#include "wmc_device.cuh"
+#include "wmc_walk.cuh"
 
 namespace wmc {
 
@@ -37,12 +37,14 @@ constexpr int kScanCells = 1024;  // cells per block of the batch scan
 constexpr int kScanThreads = 256;
 constexpr int kBatchMaxH = 128;   // warp-per-row kernel: Q <= 256
 constexpr int kBatchRowWarps = 8;
+constexpr int kScanned = 4;       // counters of the scan: survivors, work items, needed cells, work units
 
 struct BatchLayout {
-  size_t header, descs, sim_base, cell_sim, T, G, reach, row_map, thr_cell, occ, items, blk, VWh, cdf, gamma, gthr,
-      D, xlo, xhi, sine, total;
+  size_t header, descs, sim_base, cell_sim, T, G, U, bp, nbk, reach, row_map, thr_cell, occ, pairs, blk, VWh, cdf,
+      gamma, gthr, xm, sine, total;
   long long n_cells, hist_elems, tab_elems, sine_elems, max_items;
-  int n_blk, H, NM;
+  unsigned pair_cap;
+  int n_blk, H, NM, NB;  // NB: 32-column blocks of the widest row
 };
 
 int ceil_log2_host(int n) {
@@ -91,19 +93,27 @@ BatchLayout batch_layout(const wmc_params* ps, int n) {
   L.cell_sim = o; o = al256(o + sizeof(int) * nc);
   L.T = o; o = al256(o + sizeof(unsigned long long) * nc);
   L.G = o; o = al256(o + sizeof(unsigned long long) * (nc + 1));
+  L.U = o; o = al256(o + sizeof(uint32_t) * (nc + 1));
+  L.NB = (L.NM + 31) / 32;
+  L.bp = o; o = al256(o + sizeof(uint32_t) * nc * (size_t)L.NB);
+  L.nbk = o; o = al256(o + nc);
   L.reach = o; o = al256(o + nc);
   L.row_map = o; o = al256(o + sizeof(int) * nc);
   L.thr_cell = o; o = al256(o + sizeof(unsigned long long) * nc);
   L.occ = o; o = al256(o + sizeof(int) * nc);
-  L.items = o; o = al256(o + sizeof(int2) * (size_t)L.max_items);
-  L.blk = o; o = al256(o + sizeof(unsigned long long) * 3 * (size_t)(L.n_blk + 1));
+  // one entry per quad that may hold a pair event (if they are more, the pair
+  // kernel walks the ids again instead)
+  {
+    const long long want = L.hist_elems / 8;
+    L.pair_cap = (unsigned)(want < (1ll << 19) ? (1ll << 19) : (want > (1ll << 22) ? (1ll << 22) : want));
+  }
+  L.pairs = o; o = al256(o + sizeof(uint4) * (size_t)L.pair_cap);
+  L.blk = o; o = al256(o + sizeof(unsigned long long) * kScanned * (size_t)(L.n_blk + 1));
   L.VWh = o; o = al256(o + sizeof(float) * nc * (size_t)L.H);
   L.cdf = o; o = al256(o + sizeof(long long) * nc * (size_t)L.NM);
   L.gamma = o; o = al256(o + sizeof(double) * nc);
   L.gthr = o; o = al256(o + sizeof(unsigned long long) * nc);
-  L.D = o; o = al256(o + sizeof(float) * (size_t)L.tab_elems);
-  L.xlo = o; o = al256(o + sizeof(uint32_t) * (size_t)L.tab_elems);
-  L.xhi = o; o = al256(o + sizeof(uint32_t) * (size_t)L.tab_elems);
+  L.xm = o; o = al256(o + sizeof(uint32_t) * (size_t)L.tab_elems);
   L.sine = o; o = al256(o + sizeof(float) * (size_t)L.sine_elems);
   L.total = o;
   return L;
@@ -114,12 +124,12 @@ struct BatchView {
   SimDesc* descs;
   unsigned long long *sim_base, *T, *G, *thr_cell, *gthr, *blk;
   int *cell_sim, *row_map, *occ;
-  unsigned char* reach;
-  int2* items;
-  float *VWh, *D, *sine;
+  unsigned char *reach, *nbk;
+  uint4* pairs;
+  float *VWh, *sine;
   long long* cdf;
   double* gamma;
-  uint32_t *xlo, *xhi;
+  uint32_t *U, *bp, *xm;
 };
 
 BatchView batch_view(const BatchLayout& L, void* ws) {
@@ -135,15 +145,16 @@ BatchView batch_view(const BatchLayout& L, void* ws) {
   v.row_map = reinterpret_cast<int*>(b + L.row_map);
   v.thr_cell = reinterpret_cast<unsigned long long*>(b + L.thr_cell);
   v.occ = reinterpret_cast<int*>(b + L.occ);
-  v.items = reinterpret_cast<int2*>(b + L.items);
+  v.U = reinterpret_cast<uint32_t*>(b + L.U);
+  v.bp = reinterpret_cast<uint32_t*>(b + L.bp);
+  v.nbk = reinterpret_cast<unsigned char*>(b + L.nbk);
+  v.pairs = reinterpret_cast<uint4*>(b + L.pairs);
   v.blk = reinterpret_cast<unsigned long long*>(b + L.blk);
   v.VWh = reinterpret_cast<float*>(b + L.VWh);
   v.cdf = reinterpret_cast<long long*>(b + L.cdf);
   v.gamma = reinterpret_cast<double*>(b + L.gamma);
   v.gthr = reinterpret_cast<unsigned long long*>(b + L.gthr);
-  v.D = reinterpret_cast<float*>(b + L.D);
-  v.xlo = reinterpret_cast<uint32_t*>(b + L.xlo);
-  v.xhi = reinterpret_cast<uint32_t*>(b + L.xhi);
+  v.xm = reinterpret_cast<uint32_t*>(b + L.xm);
   v.sine = reinterpret_cast<float*>(b + L.sine);
   return v;
 }
@@ -161,9 +172,8 @@ __device__ __forceinline__ int owner(const SimDesc* __restrict__ d, int n, long 
 
 // ---------------------------------------------------------------- set-up
 __global__ void k_b_init(const SimDesc* __restrict__ d, int n, long long n_cells, long long tab_elems,
-                         long long sine_elems, int* __restrict__ cell_sim, float* __restrict__ D,
-                         uint32_t* __restrict__ xlo, uint32_t* __restrict__ xhi, float* __restrict__ sine,
-                         DevHeader* hdr) {
+                         long long sine_elems, int* __restrict__ cell_sim, uint32_t* __restrict__ xm,
+                         float* __restrict__ sine, DevHeader* hdr) {
   const long long tid = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   const long long nt = (long long)gridDim.x * blockDim.x;
   if (tid == 0) {
@@ -175,13 +185,7 @@ __global__ void k_b_init(const SimDesc* __restrict__ d, int n, long long n_cells
   for (long long e = tid; e < tab_elems; e += nt) {
     const SimDesc& s = d[owner(d, n, e, 1)];
     const int k = (int)(e - s.tab_off);
-    const float dd = __double2float_rn((double)(k - s.n_M / 2) * s.d1);
-    D[e] = dd;
-    uint32_t lo = 0u, hi = 0xffffffffu;
-    if (dd > 0.f) hi = (uint32_t)(((unsigned long long)first_offset_reaching(dd, 1.f) << 8) - 1ull);
-    if (dd < 0.f) lo = (uint32_t)((unsigned long long)first_offset_reaching(dd, 0.f) << 8);
-    xlo[e] = lo;
-    xhi[e] = hi;
+    xm[e] = move_entry(__double2float_rn((double)(k - s.n_M / 2) * s.d1));
   }
   for (long long e = tid; e < sine_elems; e += nt) {
     const SimDesc& s = d[owner(d, n, e, 2)];
@@ -191,9 +195,12 @@ __global__ void k_b_init(const SimDesc* __restrict__ d, int n, long long n_cells
 }
 
 // ---------------------------------------------------------------- per-cell scan
+// One warp per cell: survivors, survivor prefixes of the row's 32-column
+// blocks and the number of non-empty ones, reach bits.
 __global__ void k_b_rows(const int32_t* __restrict__ hist, const SimDesc* __restrict__ d,
-                         const int* __restrict__ cell_sim, const float* __restrict__ D, long long n_cells,
-                         unsigned long long* __restrict__ T, unsigned char* __restrict__ reach) {
+                         const int* __restrict__ cell_sim, long long n_cells, int NB,
+                         unsigned long long* __restrict__ T, uint32_t* __restrict__ bp,
+                         unsigned char* __restrict__ nbk, unsigned char* __restrict__ reach) {
   const long long c = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (c >= n_cells) return;
@@ -201,33 +208,65 @@ __global__ void k_b_rows(const int32_t* __restrict__ hist, const SimDesc* __rest
   const long long i = c - s.cell_off;
   const int n_M = s.n_M;
   const int32_t* row = hist + s.hist_off + i * n_M;
+  uint32_t* bpr = bp + (size_t)c * NB;
   // the drift D[M] = fl32(M d1), d1 > 0, has the sign of M: a column right of
   // the centre drifts right, left of it left (a D that rounds to zero only
   // marks a neighbour that needs its kernel anyway, which changes no result)
   unsigned long long a = 0;
   unsigned bits = 0;
+  int nb = 0;
+  uint32_t before = 0u;  // survivors of the blocks done (modulo 2^32: a larger cell is refused by the scan)
   if ((n_M & 3) == 0 && (reinterpret_cast<uintptr_t>(row) & 15) == 0) {
     const int4* row4 = reinterpret_cast<const int4*>(row);
-    for (int q = lane; q < n_M / 4; q += 32) {
-      const int4 n4 = __ldg(row4 + q);
-      const int nv[4] = {n4.x, n4.y, n4.z, n4.w};
+    const int nq = n_M >> 2;
+    for (int q0 = 0; q0 < nq; q0 += 64) {
+      int4 v[2];
 #pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        if (nv[e]) {
-          const int M = 4 * q + e - n_M / 2;
-          a += (unsigned long long)(nv[e] < 0 ? -(long long)nv[e] : (long long)nv[e]);
-          bits |= 1u | (M > 0 ? 2u : 0u) | (M < 0 ? 4u : 0u);
+      for (int u = 0; u < 2; ++u) {
+        const int q = q0 + 32 * u + lane;
+        v[u] = q < nq ? __ldg(row4 + q) : make_int4(0, 0, 0, 0);
+      }
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const int q = q0 + 32 * u + lane;
+        if (q0 + 32 * u >= nq) break;
+        uint32_t p = 0u;
+        if (__any_sync(0xffffffffu, (v[u].x | v[u].y | v[u].z | v[u].w) != 0)) {
+          const int nv[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
+#pragma unroll
+          for (int e = 0; e < 4; ++e)
+            if (nv[e]) {
+              const int M = 4 * q + e - n_M / 2;
+              const uint32_t m = nv[e] < 0 ? 0u - (uint32_t)nv[e] : (uint32_t)nv[e];
+              a += m;
+              p += m;
+              bits |= 1u | (M > 0 ? 2u : 0u) | (M < 0 ? 4u : 0u);
+            }
+#pragma unroll
+          for (int o = 1; o < 8; o <<= 1) p += __shfl_xor_sync(0xffffffffu, p, o);
+          nb += __popc(__ballot_sync(0xffffffffu, p != 0u && (lane & 7) == 0));
+          uint32_t w = __shfl_up_sync(0xffffffffu, p, 8);
+          if (lane >= 8) p += w;
+          w = __shfl_up_sync(0xffffffffu, p, 16);
+          if (lane >= 16) p += w;
         }
+        if ((lane & 7) == 0 && q < nq) bpr[q >> 3] = before + p;
+        before += __shfl_sync(0xffffffffu, p, 31);
       }
     }
   } else {
-    for (int k = lane; k < n_M; k += 32) {
-      const int nv = __ldg(row + k);
+    for (int k0 = 0; k0 < n_M; k0 += 32) {
+      const int k = k0 + lane;
+      const int nv = k < n_M ? __ldg(row + k) : 0;
+      const uint32_t m = nv < 0 ? 0u - (uint32_t)nv : (uint32_t)nv;
       if (nv) {
         const int M = k - n_M / 2;
-        a += (unsigned long long)(nv < 0 ? -(long long)nv : (long long)nv);
+        a += m;
         bits |= 1u | (M > 0 ? 2u : 0u) | (M < 0 ? 4u : 0u);
       }
+      before += __reduce_add_sync(0xffffffffu, m);
+      nb += __any_sync(0xffffffffu, nv != 0);
+      if (lane == 0) bpr[k0 >> 5] = before;
     }
   }
 #pragma unroll
@@ -238,6 +277,7 @@ __global__ void k_b_rows(const int32_t* __restrict__ hist, const SimDesc* __rest
   if (lane == 0) {
     T[c] = a;
     reach[c] = (unsigned char)bits;
+    nbk[c] = (unsigned char)nb;
   }
 }
 
@@ -254,106 +294,84 @@ __device__ __forceinline__ int b_items(unsigned long long t, int chunk) {
   return t ? (int)((t + 3 + chunk - 1) / chunk) : 0;
 }
 
-// block-wide exclusive scan of three counters (256 threads)
-__device__ __forceinline__ void block_scan3(unsigned long long& a, unsigned long long& b, unsigned long long& c,
-                                            unsigned long long* sh /*3 x 8*/, unsigned long long tot[3]) {
+// block-wide exclusive scan of kScanned counters (256 threads)
+__device__ __forceinline__ void block_scan(unsigned long long (&x)[kScanned], unsigned long long* sh /*kScanned x 8*/,
+                                           unsigned long long (&tot)[kScanned]) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  unsigned long long ia = a, ib = b, ic = c;
 #pragma unroll
-  for (int off = 1; off < 32; off <<= 1) {
-    const unsigned long long ua = __shfl_up_sync(0xffffffffu, ia, off);
-    const unsigned long long ub = __shfl_up_sync(0xffffffffu, ib, off);
-    const unsigned long long uc = __shfl_up_sync(0xffffffffu, ic, off);
-    if (lane >= off) {
-      ia += ua;
-      ib += ub;
-      ic += uc;
+  for (int j = 0; j < kScanned; ++j) {
+    unsigned long long in = x[j];
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+      const unsigned long long u = __shfl_up_sync(0xffffffffu, in, off);
+      if (lane >= off) in += u;
     }
-  }
-  if (lane == 31) {
-    sh[wid] = ia;
-    sh[8 + wid] = ib;
-    sh[16 + wid] = ic;
+    if (lane == 31) sh[8 * j + wid] = in;
+    x[j] = in - x[j];
   }
   __syncthreads();
-  unsigned long long pa = 0, pb = 0, pc = 0, ta = 0, tb = 0, tc = 0;
-  for (int w = 0; w < 8; ++w) {
-    if (w < wid) {
-      pa += sh[w];
-      pb += sh[8 + w];
-      pc += sh[16 + w];
+#pragma unroll
+  for (int j = 0; j < kScanned; ++j) {
+    tot[j] = 0;
+    for (int w = 0; w < 8; ++w) {
+      if (w == wid) x[j] += tot[j];
+      tot[j] += sh[8 * j + w];
     }
-    ta += sh[w];
-    tb += sh[8 + w];
-    tc += sh[16 + w];
   }
-  a = pa + ia - a;
-  b = pb + ib - b;
-  c = pc + ic - c;
-  tot[0] = ta;
-  tot[1] = tb;
-  tot[2] = tc;
 }
 
 constexpr int kCellsPerThread = kScanCells / kScanThreads;
 
+// the counters of cell c added to x
+__device__ __forceinline__ void scan_cell(unsigned long long t, int need, uint32_t nb, int chunk,
+                                          unsigned long long (&x)[kScanned]) {
+  x[0] += t;
+  x[1] += b_items(t, chunk);
+  x[2] += need;
+  x[3] += units_of_cell(t, nb);
+}
+
 __global__ __launch_bounds__(kScanThreads) void k_b_scan1(const unsigned long long* __restrict__ T,
                                                           const unsigned char* __restrict__ reach,
+                                                          const unsigned char* __restrict__ nbk,
                                                           const SimDesc* __restrict__ d,
                                                           const int* __restrict__ cell_sim, long long n_cells,
                                                           int chunk, unsigned long long* __restrict__ blk) {
-  __shared__ unsigned long long sh[24];
+  __shared__ unsigned long long sh[8 * kScanned];
   const long long c0 = (long long)blockIdx.x * kScanCells + threadIdx.x * kCellsPerThread;
-  unsigned long long a = 0, b = 0, c = 0;
+  unsigned long long x[kScanned] = {}, tot[kScanned];
   for (int q = 0; q < kCellsPerThread; ++q) {
     const long long cc = c0 + q;
     if (cc >= n_cells) break;
-    const unsigned long long t = T[cc];
-    a += t;
-    b += b_items(t, chunk);
-    c += b_needs(reach, d, cell_sim, cc);
+    scan_cell(T[cc], b_needs(reach, d, cell_sim, cc), nbk[cc], chunk, x);
   }
-  unsigned long long tot[3];
-  block_scan3(a, b, c, sh, tot);
-  if (threadIdx.x == 0) {
-    blk[3 * blockIdx.x] = tot[0];
-    blk[3 * blockIdx.x + 1] = tot[1];
-    blk[3 * blockIdx.x + 2] = tot[2];
-  }
+  block_scan(x, sh, tot);
+  if (threadIdx.x == 0)
+    for (int j = 0; j < kScanned; ++j) blk[kScanned * blockIdx.x + j] = tot[j];
 }
 
 // single block: exclusive scan of the block sums, totals to the header
 __global__ __launch_bounds__(kScanThreads) void k_b_scan2(unsigned long long* __restrict__ blk, int n_blk,
                                                           long long max_items, DevHeader* hdr, int advance_step) {
-  __shared__ unsigned long long sh[24];
-  __shared__ unsigned long long carry[3];
-  if (threadIdx.x == 0) carry[0] = carry[1] = carry[2] = 0;
+  __shared__ unsigned long long sh[8 * kScanned];
+  __shared__ unsigned long long carry[kScanned];
+  if (threadIdx.x < kScanned) carry[threadIdx.x] = 0;
   __syncthreads();
   for (int base = 0; base < n_blk; base += kScanThreads) {
     const int q = base + threadIdx.x;
-    unsigned long long a = 0, b = 0, c = 0;
-    if (q < n_blk) {
-      a = blk[3 * q];
-      b = blk[3 * q + 1];
-      c = blk[3 * q + 2];
-    }
-    unsigned long long tot[3];
-    block_scan3(a, b, c, sh, tot);
-    if (q < n_blk) {
-      blk[3 * q] = a + carry[0];
-      blk[3 * q + 1] = b + carry[1];
-      blk[3 * q + 2] = c + carry[2];
-    }
+    unsigned long long x[kScanned] = {}, tot[kScanned];
+    if (q < n_blk)
+      for (int j = 0; j < kScanned; ++j) x[j] = blk[kScanned * q + j];
+    block_scan(x, sh, tot);
+    if (q < n_blk)
+      for (int j = 0; j < kScanned; ++j) blk[kScanned * q + j] = x[j] + carry[j];
     __syncthreads();
-    if (threadIdx.x == 0) {
-      carry[0] += tot[0];
-      carry[1] += tot[1];
-      carry[2] += tot[2];
-    }
+    if (threadIdx.x == 0)
+      for (int j = 0; j < kScanned; ++j) carry[j] += tot[j];
     __syncthreads();
   }
   if (threadIdx.x == 0) {
-    const int ok = (long long)carry[1] <= max_items;
+    const int ok = (long long)carry[1] <= max_items && carry[3] < (1ull << 32);
     hdr->n_items = ok ? (int)carry[1] : 0;
     hdr->n_occ = (int)carry[2];
     hdr->population = 0;  // summed per simulation by k_b_simbase
@@ -363,51 +381,46 @@ __global__ __launch_bounds__(kScanThreads) void k_b_scan2(unsigned long long* __
 }
 
 __global__ __launch_bounds__(kScanThreads) void k_b_scan3(
-    const unsigned long long* __restrict__ T, const unsigned char* __restrict__ reach, const SimDesc* __restrict__ d,
-    const int* __restrict__ cell_sim, long long n_cells, int chunk, const unsigned long long* __restrict__ blk,
-    unsigned long long* __restrict__ G, int2* __restrict__ items, int* __restrict__ occ, int* __restrict__ row_map,
+    const unsigned long long* __restrict__ T, const unsigned char* __restrict__ reach,
+    const unsigned char* __restrict__ nbk, const SimDesc* __restrict__ d, const int* __restrict__ cell_sim,
+    long long n_cells, int chunk, const unsigned long long* __restrict__ blk, unsigned long long* __restrict__ G,
+    uint32_t* __restrict__ U, int* __restrict__ occ, int* __restrict__ row_map,
     unsigned long long* __restrict__ thr_cell, DevHeader* hdr) {
-  __shared__ unsigned long long sh[24];
+  __shared__ unsigned long long sh[8 * kScanned];
   const long long c0 = (long long)blockIdx.x * kScanCells + threadIdx.x * kCellsPerThread;
-  unsigned long long a = 0, b = 0, c = 0;
+  unsigned long long x[kScanned] = {}, tot[kScanned];
   for (int q = 0; q < kCellsPerThread; ++q) {
     const long long cc = c0 + q;
     if (cc >= n_cells) break;
-    const unsigned long long t = T[cc];
-    a += t;
-    b += b_items(t, chunk);
-    c += b_needs(reach, d, cell_sim, cc);
+    scan_cell(T[cc], b_needs(reach, d, cell_sim, cc), nbk[cc], chunk, x);
   }
-  unsigned long long tot[3];
-  block_scan3(a, b, c, sh, tot);
-  a += blk[3 * blockIdx.x];
-  b += blk[3 * blockIdx.x + 1];
-  c += blk[3 * blockIdx.x + 2];
-  const bool write_items = hdr->n_items > 0;
+  block_scan(x, sh, tot);
+#pragma unroll
+  for (int j = 0; j < kScanned; ++j) x[j] += blk[kScanned * blockIdx.x + j];
   for (int q = 0; q < kCellsPerThread; ++q) {
     const long long cc = c0 + q;
     if (cc >= n_cells) break;
     const unsigned long long t = T[cc];
-    G[cc] = a;
+    const int need = b_needs(reach, d, cell_sim, cc);
+    G[cc] = x[0];
+    U[cc] = (uint32_t)x[3];
     if (t > 0x7fffffffull) {  // a cell's ids must fit the 31-bit row-local offsets
       atomicOr(&hdr->flags, WMC_FLAG_CAPACITY);
       hdr->n_items = 0;
     }
-    const int ni = b_items(t, chunk);
-    if (write_items)
-      for (int k = 0; k < ni; ++k) items[b + k] = make_int2((int)cc, k);
-    if (b_needs(reach, d, cell_sim, cc)) {
-      occ[c] = (int)cc;
-      row_map[cc] = (int)c;
-      ++c;
+    if (need) {
+      occ[x[2]] = (int)cc;
+      row_map[cc] = (int)x[2];
     } else {
       row_map[cc] = -1;
     }
     thr_cell[cc] = 0ull;
-    a += t;
-    b += ni;
+    scan_cell(t, need, nbk[cc], chunk, x);
   }
-  if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) G[n_cells] = blk[3 * blockIdx.x] + tot[0];
+  if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) {
+    G[n_cells] = blk[kScanned * blockIdx.x] + tot[0];
+    U[n_cells] = (uint32_t)(blk[kScanned * blockIdx.x + 3] + tot[3]);
+  }
 }
 
 // per simulation: first id offset and population
@@ -512,195 +525,262 @@ struct BatchStepArgs {
   const int* cell_sim;
   const unsigned long long* G;
   const unsigned long long* sim_base;
-  const int2* items;
+  const uint32_t* U;
+  const uint32_t* bp;
   const int* row_map;
   const long long* cdf;
   const unsigned long long* thr_cell;
-  const uint32_t* xlo;
-  const uint32_t* xhi;
+  const uint32_t* xm;
+  uint4* pairs;
+  unsigned pair_cap;
   DevHeader* hdr;
-  int NM, per_thread;
+  int NM, NB, n_cells;
+  uint32_t max_range;  // work units of the schedule's largest ranges
 };
 
-// One warp per work item: an item is a run of 32 x per_thread ids of one row
-// (quad-aligned to the global ids), so a sparse row costs one warp, not a
-// block.  Each warp owns its slice of shared memory (row prefix and signed
-// counts) and takes items from the global ticket without block-wide barriers;
-// parents and children go to the output histogram with global atomics, one
-// per run of ids in a bucket (lanes ending in the same bucket combine first),
-// so a sparse item touches only the buckets it holds.
+// The walk and the pair events of wmc_step.cu on the concatenated cells: the
+// work units of all simulations are one sequence, so a warp's range may run
+// from one simulation into the next.
 constexpr int kBStepWarps = 8;
 
-__global__ __launch_bounds__(kBStepWarps * 32, 4) void k_b_step(BatchStepArgs a) {
-  extern __shared__ int smem[];
-  const int NM = a.NM;
-  const int tid = threadIdx.x, lane = tid & 31;
-  int* s_pre = smem + (size_t)(tid >> 5) * (2 * NM + 1);
-  int* s_n = s_pre + (NM + 1);
-  __shared__ unsigned long long s_red[5][kBStepWarps];
-  const uint32_t t = a.hdr->step;
-  const int n_items = a.hdr->n_items;
-  const int PER = a.per_thread;
-  const int chunk = 32 * PER;
-  unsigned long long pairs = 0, absorbed = 0, dropped = 0;
-  long long abs_signed = 0, drop_signed = 0;
+// One thread's share of the step's counters.
+struct PairCounters {
+  unsigned long long pairs = 0, dropped = 0;
+  long long drop_signed = 0;
+};
 
-  for (;;) {
-    int item = 0;
-    if (lane == 0) item = (int)atomicAdd(&a.hdr->item_ticket, 1u);
-    item = __shfl_sync(0xffffffffu, item, 0);
-    if (item >= n_items) break;
-    const int2 it = __ldg(a.items + item);
-    const long long cg = it.x;
-    const int ch = it.y;
-    const int sidx = __ldg(a.cell_sim + cg);
-    const SimDesc& S = a.d[sidx];
-    const int n_M = S.n_M, n_x = S.n_x;
-    const int i = (int)(cg - S.cell_off);
-    const uint32_t base = (uint32_t)(__ldg(a.G + cg) - __ldg(a.sim_base + sidx));
-    const unsigned long long thr_m = i > 0 ? __ldg(a.thr_cell + cg - 1) : 0ull;
-    const unsigned long long thr_0 = __ldg(a.thr_cell + cg);
-    const unsigned long long thr_p = i + 1 < n_x ? __ldg(a.thr_cell + cg + 1) : 0ull;
-    const uint32_t sim = S.sim, k0 = S.k0, k1 = S.k1;
-    const int32_t* hrow = a.hist_in + S.hist_off;
-    int32_t* hout = a.hist_out + S.hist_off + (size_t)(i - 1) * n_M;  // rows i-1, i, i+1 at hout + d n_M
-    const uint32_t* xlo = a.xlo + S.tab_off;
-    const uint32_t* xhi = a.xhi + S.tab_off;
-    warp_row_prefix(hrow, i, n_M, s_n, s_pre, lane);
-    __syncwarp();
-
-    const uint32_t Ti = (uint32_t)s_pre[n_M];
-    // the item is [item0, item1) of the quad-aligned id range of the cell; its
-    // ids are spread over the 32 lanes in quad-aligned spans, so a sparse cell
-    // keeps every lane busy
-    const unsigned long long A = base & ~3u;
-    const unsigned long long row_end = (unsigned long long)base + Ti;
-    const unsigned long long item0 = A + (unsigned long long)ch * chunk;
-    const unsigned long long item1 = item0 + chunk < row_end ? item0 + chunk : row_end;
-    const unsigned long long len = item1 > item0 ? item1 - item0 : 0ull;
-    const unsigned long long span = ((len + 127ull) / 128ull) * 4ull;
-    const unsigned long long lo64 = item0 + (unsigned long long)lane * span;
-    const unsigned long long g0_64 = lo64 > base ? lo64 : base;
-    const unsigned long long g1_64 = lo64 + span < item1 ? lo64 + span : item1;
-    const uint32_t g0 = g0_64 < g1_64 ? (uint32_t)g0_64 : 0u;
-    const uint32_t g1 = g0_64 < g1_64 ? (uint32_t)g1_64 : 0u;
-    const bool need_gen = (thr_m | thr_0 | thr_p) != 0ull;
-
-    int k = 0, n_tot = 0, n_mov = 0, sgn = 1, dir = 0;
-    if (g0 < g1) {
-      k = bucket_of(s_pre, n_M, (int)(g0 - base));
-      uint32_t end_g = base + (uint32_t)s_pre[k + 1];
-      sgn = s_n[k] > 0 ? 1 : -1;
-      uint32_t lo = __ldg(xlo + k), hi = __ldg(xhi + k);
-      dir = drift_dir(lo, hi);
-      unsigned long long thr_move = dir > 0 ? thr_p : (dir < 0 ? thr_m : 0ull);
-      for (uint32_t q = g0 >> 2; q <= (g1 - 1u) >> 2; ++q) {
-        const uint32_t qa = q << 2;
-        const uint4 wr = philox4x32_10(make_uint4(q, t - 1u, kPurposeRepos, sim), k0, k1);
-        uint4 wg = make_uint4(0u, 0u, 0u, 0u);
-        if (need_gen) wg = philox4x32_10(make_uint4(q, t, kPurposeGen, sim), k0, k1);
-        const uint32_t w4[4] = {wr.x, wr.y, wr.z, wr.w};
-        const uint32_t u4[4] = {wg.x, wg.y, wg.z, wg.w};
+// The pair events of one queued quad {id / 4, cell, column | sign bit << 12 |
+// ids << 16, -}.
+__device__ __forceinline__ void b_quad_events(const BatchStepArgs& a, uint32_t t, const uint4& ev, PairCounters& pc) {
+  const int cg = (int)ev.y, k = (int)(ev.z & 4095u);
+  const SimDesc& S = a.d[__ldg(a.cell_sim + cg)];
+  const int n_M = S.n_M, i = (int)(cg - S.cell_off);
+  const uint32_t sim = S.sim, k0 = S.k0, k1 = S.k1;
+  const uint32_t e = __ldg(a.xm + S.tab_off + k);
+  const int dir = move_dir(e);
+  uint4 wr = make_uint4(ev.x, t - 1u, kPurposeRepos, sim), wg = make_uint4(ev.x, t, kPurposeGen, sim);
+  philox4x32_10_x2(wr, wg, k0, k1);
+  const unsigned long long t_st = __ldg(a.thr_cell + cg);
+  const unsigned long long t_mv = (unsigned)(i + dir) < (unsigned)S.n_x ? __ldg(a.thr_cell + cg + dir) : 0ull;
+  const uint32_t mvb = move_bits(wr, e), u4[4] = {wg.x, wg.y, wg.z, wg.w};
+  uint32_t m = 0u;
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const uint32_t id = qa + (uint32_t)j;
-          if (id < g0 || id >= g1) continue;
-          if (id >= end_g) {
-            const int stay = n_tot - n_mov;
-            if (stay) atomicAdd(hout + (size_t)n_M + k, sgn * stay);
-            if (n_mov) {
-              if ((unsigned)(i + dir) < (unsigned)n_x) {
-                atomicAdd(hout + (size_t)(dir + 1) * n_M + k, sgn * n_mov);
-              } else {
-                absorbed += n_mov;
-                abs_signed += sgn * n_mov;
-              }
-            }
-            n_tot = n_mov = 0;
-            do { ++k; } while (base + (uint32_t)s_pre[k + 1] <= id);
-            end_g = base + (uint32_t)s_pre[k + 1];
-            sgn = s_n[k] > 0 ? 1 : -1;
-            lo = __ldg(xlo + k);
-            hi = __ldg(xhi + k);
-            dir = drift_dir(lo, hi);
-            thr_move = dir > 0 ? thr_p : (dir < 0 ? thr_m : 0ull);
-          }
-          const int mv = (w4[j] > hi) | (w4[j] < lo);
-          n_mov += mv;
-          ++n_tot;
-          if (need_gen && (unsigned long long)u4[j] < (mv ? thr_move : thr_0)) {
-            // pair: p' from the PICK draw of this id, children into row d
-            const int dd = mv ? dir + 1 : 1;
-            const int orow = __ldg(a.row_map + cg - 1 + dd);
-            const uint4 wp = philox4x32_10(make_uint4(id, t, kPurposePick, sim), k0, k1);
-            const unsigned long long U2 =
-                ((unsigned long long)(wp.x >> 5) << 26) | (unsigned long long)(wp.y >> 6);
-            const int kp = sample_cdf_row(a.cdf + (size_t)orow * NM, n_M, U2);
-            ++pairs;
-            const int Mp = kp - n_M / 2;
-            const int kc2[2] = {k + Mp, k - Mp};
-            const int sc2[2] = {sgn, -sgn};
+  for (int j = 0; j < 4; ++j) m |= (uint32_t)((unsigned long long)u4[j] < ((mvb >> j) & 1u ? t_mv : t_st)) << j;
+  m &= ev.z >> 16;
+  while (m) {
+    const int j = __ffs(m) - 1;
+    m &= m - 1u;
+    // p' from the PICK draw of this id, children into the cell it ended in
+    const int dd = (mvb >> j) & 1u ? dir : 0;
+    const int orow = __ldg(a.row_map + cg + dd);
+    const uint4 wp = philox4x32_10(make_uint4(4u * ev.x + (uint32_t)j, t, kPurposePick, sim), k0, k1);
+    const unsigned long long U2 = ((unsigned long long)(wp.x >> 5) << 26) | (unsigned long long)(wp.y >> 6);
+    const int Mp = sample_cdf_row(a.cdf + (size_t)orow * a.NM, n_M, U2) - n_M / 2;
+    ++pc.pairs;
+    const int sgn = (ev.z >> 12) & 1u ? -1 : 1;
+    const int kc2[2] = {k + Mp, k - Mp}, sc2[2] = {sgn, -sgn};
+    int32_t* out = a.hist_out + S.hist_off + (size_t)(i + dd) * n_M;
 #pragma unroll
-            for (int qq = 0; qq < 2; ++qq) {
-              int kc = kc2[qq];
-              if (kc < 0 || kc >= n_M) {
-                if (!S.wrap) {
-                  ++dropped;
-                  drop_signed += sc2[qq];
-                  continue;
-                }
-                kc = ((kc % n_M) + n_M) % n_M;
-              }
-              atomicAdd(hout + (size_t)dd * n_M + kc, sc2[qq]);
-            }
-          }
+    for (int q = 0; q < 2; ++q) {
+      int kc = kc2[q];
+      if (kc < 0 || kc >= n_M) {
+        if (!S.wrap) {
+          ++pc.dropped;
+          pc.drop_signed += sc2[q];
+          continue;
         }
+        kc = ((kc % n_M) + n_M) % n_M;
       }
+      atomicAdd(out + kc, sc2[q]);
     }
-    const int key = n_tot ? k : -1;
-    const unsigned peers = __match_any_sync(0xffffffffu, key);
-    const int stay = __reduce_add_sync(peers, n_tot - n_mov);
-    const int mov = __reduce_add_sync(peers, n_mov);
-    if (key >= 0 && lane == __ffs(peers) - 1) {
-      if (stay) atomicAdd(hout + (size_t)n_M + k, sgn * stay);
-      if (mov) {
-        if ((unsigned)(i + dir) < (unsigned)n_x) {
-          atomicAdd(hout + (size_t)(dir + 1) * n_M + k, sgn * mov);
-        } else {
-          absorbed += mov;
-          abs_signed += sgn * mov;
-        }
-      }
-    }
-    __syncwarp();
   }
-  const int wid = tid >> 5;
-  unsigned long long vals[5] = {pairs, absorbed, (unsigned long long)abs_signed, dropped,
-                                (unsigned long long)drop_signed};
+}
+
+// A cell of some simulation for the walk: its pointers in the warp's shared
+// memory, so that the draws keep their registers.
+struct BatchRow {
+  const int32_t* row;
+  const uint32_t* bp;
+  const uint32_t* xm;
+  int32_t* out;  // the cell's row of the next histogram
+  int n_M, i, n_x, cg;
+};
+
+struct BatchCell {
+  const BatchRow* r;
+  uint32_t off, rej;
+  bool gen;
+  __device__ __forceinline__ int n_M() const { return r->n_M; }
+  __device__ __forceinline__ int row(int col) const { return __ldg(r->row + col); }
+  __device__ __forceinline__ uint32_t bp(int b) const { return __ldg(r->bp + b); }
+  __device__ __forceinline__ uint32_t xm(int col) const { return __ldg(r->xm + col); }
+};
+
+// The ids of the work units [w0, w1), cell by cell.  COUNT: parents counted,
+// absorbed particles too; otherwise only the quads that may hold events are
+// queued.
+template <bool COUNT, class Flush>
+__device__ __forceinline__ void b_walk_range(const BatchStepArgs& a, uint32_t t, uint32_t w0, uint32_t w1, int lane,
+                                             uint4* queue, BatchRow* br, int& nq, Flush flush) {
+  CellWork cell = cell_of_unit(a.U, a.n_cells, w0, lane);
+#pragma unroll 1
+  while (true) {
+    const int cg = cell.i, sidx = __ldg(a.cell_sim + cg);
+    const SimDesc& S = a.d[sidx];
+    const int i = (int)(cg - S.cell_off);
+    const uint32_t sim = S.sim, k0 = S.k0, k1 = S.k1;
+    const uint32_t sb = id_prefix(a.sim_base, sidx);
+    const uint32_t first = id_prefix(a.G, cg) - sb, last = id_prefix(a.G, cg + 1) - sb;
+    const uint32_t A = first & ~3u, qA = A >> 2;
+    __syncwarp();
+    if (lane == 0) {
+      const int n_M = S.n_M;
+      const long long at = S.hist_off + (long long)i * n_M;
+      br->row = a.hist_in + at;
+      br->bp = a.bp + (size_t)cg * a.NB;
+      br->xm = a.xm + S.tab_off;
+      br->out = a.hist_out + at;
+      br->n_M = n_M;
+      br->i = i;
+      br->n_x = S.n_x;
+      br->cg = cg;
+    }
+    __syncwarp();
+    BatchCell c{br, first & 3u};
+    const unsigned long long thr_m = i > 0 ? __ldg(a.thr_cell + cg - 1) : 0ull, thr_0 = __ldg(a.thr_cell + cg),
+                             thr_p = i + 1 < S.n_x ? __ldg(a.thr_cell + cg + 1) : 0ull;
+    const unsigned long long tmax = max(thr_0, max(thr_m, thr_p));
+    c.gen = tmax != 0ull;
+    c.rej = (uint32_t)(tmax - 1ull);
+    auto add = [&](int k, int dd, int v, uint32_t n) {
+      if (!COUNT) return;
+      if ((unsigned)(br->i + dd) < (unsigned)br->n_x) {
+        atomicAdd(br->out + dd * br->n_M + k, v);
+      } else {  // (edge cells only)
+        atomicAdd(&a.hdr->absorbed, (unsigned long long)n);
+        atomicAdd(reinterpret_cast<unsigned long long*>(&a.hdr->absorbed_signed), (unsigned long long)(long long)v);
+      }
+    };
+    walk_ids(
+        c, window_of_unit(cell, last - first, w0) << 7, min(last - A, window_of_unit(cell, last - first, w1) << 7),
+        lane, queue + kWalkQueue, nq,
+        [&](uint32_t q, bool gen, uint4& wr, uint4& wg) {
+          wr = make_uint4(qA + q, t - 1u, kPurposeRepos, sim);
+          if (gen) {
+            wg = make_uint4(qA + q, t, kPurposeGen, sim);
+            philox4x32_10_x2(wr, wg, k0, k1);
+          } else {
+            wr = philox4x32_10(wr, k0, k1);
+          }
+        },
+        [&](int k, uint32_t e, uint32_t stay, uint32_t move) {
+          if (stay) add(k, 0, e & 1u ? -(int)stay : (int)stay, stay);
+          if (move) add(k, move_dir(e), e & 1u ? -(int)move : (int)move, move);
+        },
+        [&](unsigned who, bool me, uint32_t q, int k, uint32_t e, uint32_t ids) {
+          if (me)
+            queue[nq + __popc(who & ((1u << lane) - 1u))] =
+                make_uint4(qA + q, (uint32_t)br->cg, (uint32_t)k | ((e & 1u) << 12) | (ids << 16), 0u);
+          nq += __popc(who);
+        },
+        flush);
+    if (cell.u1 >= w1) break;
+    cell = next_cell(a.U, a.n_cells, cell, lane);
+  }
+}
+
+__global__ __launch_bounds__(kBStepWarps * 32, 4) void k_b_step(const __grid_constant__ BatchStepArgs a) {
+  __shared__ uint4 s_queue[kBStepWarps][kWalkQueue + 32];
+  __shared__ BatchRow s_row[kBStepWarps];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  uint4* queue = s_queue[wid];
+  const uint32_t t = a.hdr->step;
+  const uint32_t total = a.hdr->n_items ? __ldg(a.U + a.n_cells) : 0u;
+  int nq = 0;
+  auto flush = [&]() {  // (what does not fit is found again by the pair kernel)
+    __syncwarp();
+    unsigned qb = 0u;
+    if (lane == 0) qb = atomicAdd(&a.hdr->pair_count, (unsigned)nq);
+    qb = __shfl_sync(0xffffffffu, qb, 0);
+    for (int e = lane; e < nq; e += 32)
+      if (qb + (unsigned)e < a.pair_cap) a.pairs[qb + (unsigned)e] = queue[e];
+    __syncwarp();
+    nq = 0;
+  };
+  RangeSchedule sched(total, gridDim.x * kBStepWarps, a.max_range);
+  uint32_t ticket = (uint32_t)wid * gridDim.x + blockIdx.x, w0, w1;
+  while (sched.range(ticket, w0, w1)) {
+    const bool more = sched.more();
+    uint32_t nxt = 0u;
+    if (lane == 0 && more) nxt = atomicAdd(&a.hdr->item_ticket, 1u);  // consumed at the end of this range
+    b_walk_range<true>(a, t, w0, w1, lane, queue, s_row + wid, nq, flush);
+    if (!more) break;
+    ticket = sched.n_warps + __shfl_sync(0xffffffffu, nxt, 0);
+  }
+  if (nq) flush();
+  if (blockIdx.x == 0 && threadIdx.x == 0 && a.hdr->n_items > 0) atomicAdd(&a.hdr->particle_steps, a.hdr->population);
+}
+
+// All quads that may hold events, by a second walk (they did not fit the queue).
+__device__ __noinline__ void b_rewalk_events(const BatchStepArgs& a, uint32_t t, uint4* queue, BatchRow* br, PairCounters& pc) {
+  const int lane = threadIdx.x & 31;
+  const uint32_t total = a.hdr->n_items ? __ldg(a.U + a.n_cells) : 0u;
+  constexpr uint32_t kUnits = 32;
+  int nq = 0;
+  auto flush = [&]() {
+    __syncwarp();
+    for (int e = lane; e < nq; e += 32) b_quad_events(a, t, queue[e], pc);
+    __syncwarp();
+    nq = 0;
+  };
+  const uint32_t stride = gridDim.x * kBStepWarps * kUnits;
+  for (uint32_t w0 = (blockIdx.x * kBStepWarps + (threadIdx.x >> 5)) * kUnits; w0 < total; w0 += stride)
+    b_walk_range<false>(a, t, w0, min(w0 + kUnits, total), lane, queue, br, nq, flush);
+  if (nq) flush();
+}
+
+// The queued quads of the step: one thread each.  The last block to finish
+// resets the queue and the range ticket for the next step.
+__global__ __launch_bounds__(kBStepWarps * 32, 4) void k_b_pairs(const __grid_constant__ BatchStepArgs a) {
+  __shared__ uint4 s_queue[kBStepWarps][kWalkQueue + 32];
+  __shared__ BatchRow s_row[kBStepWarps];
+  __shared__ unsigned long long s_red[3][kBStepWarps];
+  const uint32_t t = a.hdr->step;
+  const unsigned n = a.hdr->pair_count;
+  // (blocks without work leave at once and are not counted)
+  const unsigned blocks = n > a.pair_cap ? gridDim.x : min(gridDim.x, max(1u, (n + blockDim.x - 1) / blockDim.x));
+  if (blockIdx.x >= blocks) return;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  PairCounters pc;
+  if (n <= a.pair_cap) {
+    for (unsigned e = blockIdx.x * blockDim.x + threadIdx.x; e < n; e += blocks * blockDim.x)
+      b_quad_events(a, t, a.pairs[e], pc);
+  } else {
+    b_rewalk_events(a, t, s_queue[wid], s_row + wid, pc);
+  }
+  const unsigned long long vals[3] = {pc.pairs, pc.dropped, (unsigned long long)pc.drop_signed};
 #pragma unroll
-  for (int j = 0; j < 5; ++j) {
+  for (int j = 0; j < 3; ++j) {
     unsigned long long v = vals[j];
 #pragma unroll
     for (int off = 16; off; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
     if (lane == 0) s_red[j][wid] = v;
   }
   __syncthreads();
-  if (tid < 5) {
+  if (threadIdx.x < 3) {
     unsigned long long v = 0;
-    for (int w = 0; w < kBStepWarps; ++w) v += s_red[tid][w];
-    if (v) {
-      unsigned long long* dst[5] = {&a.hdr->pairs, &a.hdr->absorbed,
-                                    reinterpret_cast<unsigned long long*>(&a.hdr->absorbed_signed), &a.hdr->dropped,
-                                    reinterpret_cast<unsigned long long*>(&a.hdr->dropped_signed)};
-      atomicAdd(dst[tid], v);
-    }
+    for (int w = 0; w < kBStepWarps; ++w) v += s_red[threadIdx.x][w];
+    unsigned long long* dst[3] = {&a.hdr->pairs, &a.hdr->dropped,
+                                  reinterpret_cast<unsigned long long*>(&a.hdr->dropped_signed)};
+    if (v) atomicAdd(dst[threadIdx.x], v);
   }
-  if (blockIdx.x == 0 && tid == 0 && n_items > 0) atomicAdd(&a.hdr->particle_steps, a.hdr->population);
-  if (tid == 0) {
+  __syncthreads();
+  if (threadIdx.x == 0) {
     __threadfence();
-    if (atomicAdd(&a.hdr->blocks_done, 1u) == gridDim.x - 1) {
+    if (atomicAdd(&a.hdr->pairs_done, 1u) == blocks - 1u) {
+      a.hdr->pair_count = 0u;
       a.hdr->item_ticket = 0u;
-      a.hdr->blocks_done = 0u;
+      a.hdr->pairs_done = 0u;
       __threadfence();
     }
   }
@@ -709,13 +789,9 @@ __global__ __launch_bounds__(kBStepWarps * 32, 4) void k_b_step(BatchStepArgs a)
 __global__ void k_b_set_step(DevHeader* hdr, uint32_t step) { hdr->step = step; }
 
 // ---------------------------------------------------------------- host driver
-size_t b_step_smem(int NM) { return sizeof(int) * (size_t)kBStepWarps * (2 * NM + 1); }
-
-int b_step_grid(int NM) {
+int b_step_grid() {
   int per_sm = 0;
-  const size_t sm = b_step_smem(NM);
-  if (sm > 48 * 1024) raise_smem_limit(reinterpret_cast<const void*>(k_b_step), sm);
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_b_step, kBStepWarps * 32, sm);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_b_step, kBStepWarps * 32, 0);
   if (per_sm < 1) per_sm = 1;
   return per_sm * num_sms();
 }
@@ -723,11 +799,12 @@ int b_step_grid(int NM) {
 cudaError_t b_one_step(const BatchLayout& L, const BatchView& v, int n, const float* V, const int32_t* in,
                        int32_t* out, int per_thread, int grid, cudaStream_t s) {
   const long long nc = L.n_cells;
-  const int chunk = 32 * per_thread;  // ids per warp item
-  k_b_rows<<<(unsigned)((nc * 32 + 255) / 256), 256, 0, s>>>(in, v.descs, v.cell_sim, v.D, nc, v.T, v.reach);
-  k_b_scan1<<<L.n_blk, kScanThreads, 0, s>>>(v.T, v.reach, v.descs, v.cell_sim, nc, chunk, v.blk);
+  const int chunk = 32 * per_thread;  // ids per work item as counted in n_items
+  k_b_rows<<<(unsigned)((nc * 32 + 255) / 256), 256, 0, s>>>(in, v.descs, v.cell_sim, nc, L.NB, v.T, v.bp,
+                                                               v.nbk, v.reach);
+  k_b_scan1<<<L.n_blk, kScanThreads, 0, s>>>(v.T, v.reach, v.nbk, v.descs, v.cell_sim, nc, chunk, v.blk);
   k_b_scan2<<<1, kScanThreads, 0, s>>>(v.blk, L.n_blk, L.max_items, v.hdr, 1);
-  k_b_scan3<<<L.n_blk, kScanThreads, 0, s>>>(v.T, v.reach, v.descs, v.cell_sim, nc, chunk, v.blk, v.G, v.items, v.occ,
+  k_b_scan3<<<L.n_blk, kScanThreads, 0, s>>>(v.T, v.reach, v.nbk, v.descs, v.cell_sim, nc, chunk, v.blk, v.G, v.U, v.occ,
                                              v.row_map, v.thr_cell, v.hdr);
   k_b_simbase<<<(n + 127) / 128, 128, 0, s>>>(v.descs, n, v.G, v.sim_base, v.hdr);
   const int rows_blocks = (int)((nc + kBatchRowWarps - 1) / kBatchRowWarps);
@@ -750,16 +827,25 @@ cudaError_t b_one_step(const BatchLayout& L, const BatchView& v, int n, const fl
   a.cell_sim = v.cell_sim;
   a.G = v.G;
   a.sim_base = v.sim_base;
-  a.items = v.items;
+  a.U = v.U;
+  a.bp = v.bp;
   a.row_map = v.row_map;
   a.cdf = v.cdf;
   a.thr_cell = v.thr_cell;
-  a.xlo = v.xlo;
-  a.xhi = v.xhi;
+  a.xm = v.xm;
+  a.pairs = v.pairs;
+  a.pair_cap = L.pair_cap;
   a.hdr = v.hdr;
   a.NM = L.NM;
-  a.per_thread = per_thread;
-  k_b_step<<<grid, kBStepWarps * 32, b_step_smem(L.NM), s>>>(a);
+  a.NB = L.NB;
+  a.n_cells = (int)nc;
+  // 32 per_thread ids in windows of 128; shorter ranges than the single
+  // simulation's only add their own cost
+  a.max_range = per_thread / 4 > (int)kMaxRange ? (uint32_t)per_thread / 4u : kMaxRange;
+  k_b_step<<<grid, kBStepWarps * 32, 0, s>>>(a);
+  const unsigned pair_blocks = (L.pair_cap + kBStepWarps * 32 - 1) / (kBStepWarps * 32);
+  const unsigned pair_most = 8u * (unsigned)num_sms();
+  k_b_pairs<<<pair_blocks < pair_most ? pair_blocks : pair_most, kBStepWarps * 32, 0, s>>>(a);
   return cudaGetLastError();
 }
 
@@ -843,9 +929,9 @@ wmc_status wmc_batch_init(const wmc_params* ps, int32_t n_sims, void* ws, size_t
   if (cudaMemcpyAsync(v.descs, d.data(), sizeof(SimDesc) * n_sims, cudaMemcpyHostToDevice, s) != cudaSuccess)
     return WMC_ERR_CUDA;
   if (cudaStreamSynchronize(s) != cudaSuccess) return WMC_ERR_CUDA;
-  k_b_init<<<512, 256, 0, s>>>(v.descs, n_sims, L.n_cells, L.tab_elems, L.sine_elems, v.cell_sim, v.D, v.xlo, v.xhi,
-                               v.sine, v.hdr);
-  (void)b_step_grid(L.NM);
+  k_b_init<<<512, 256, 0, s>>>(v.descs, n_sims, L.n_cells, L.tab_elems, L.sine_elems, v.cell_sim, v.xm, v.sine,
+                               v.hdr);
+  (void)b_step_grid();
   return cudaGetLastError() == cudaSuccess ? WMC_OK : WMC_ERR_CUDA;
 }
 
@@ -861,7 +947,7 @@ wmc_status wmc_batch_run(const wmc_params* ps, int32_t n_sims, const float* V, i
   const BatchLayout L = batch_layout(ps, n_sims);
   const BatchView v = batch_view(L, ws);
   cudaStream_t s = (cudaStream_t)stream;
-  const int grid = b_step_grid(L.NM);
+  const int grid = b_step_grid();
   k_b_set_step<<<1, 1, 0, s>>>(v.hdr, t_first - 1u);
   if (cudaGetLastError() != cudaSuccess) return WMC_ERR_CUDA;
   const int pairs = n_steps / 2;
@@ -925,7 +1011,7 @@ wmc_status wmc_batch_autotune(const wmc_params* ps, int32_t n_sims, const float*
   const BatchLayout L = batch_layout(ps, n_sims);
   const BatchView v = batch_view(L, ws);
   cudaStream_t s = (cudaStream_t)stream;
-  const int grid = b_step_grid(L.NM);
+  const int grid = b_step_grid();
   const int cands[5] = {16, 32, 64, 128, 256};
   cudaEvent_t e0, e1;
   if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess) return WMC_ERR_CUDA;

@@ -182,51 +182,11 @@ __device__ __forceinline__ unsigned long long event_threshold(double g, double d
   return (unsigned long long)ceil(gd * 4294967296.0);
 }
 
-// Loads the signed counts of cell i into s_n and the exclusive prefix of |n|
-// into s_pre[0..n_M] (s_pre[n_M] = survivors of the cell), by one warp: 32
-// columns at a time (lane l takes column k0 + l, so the loads coalesce and the
-// shared-memory stores hit distinct banks), a warp scan per chunk and a carry.
-__device__ __forceinline__ void warp_row_prefix(const int32_t* __restrict__ hist, int i, int n_M, int* s_n,
-                                                int* s_pre, int lane) {
-  const int32_t* row = hist + (size_t)i * n_M;
-  int carry = 0;
-  for (int k0 = 0; k0 < n_M; k0 += 32) {
-    const int k = k0 + lane;
-    const int n = k < n_M ? __ldg(row + k) : 0;
-    const int v = n < 0 ? -n : n;
-    int incl = v;
-#pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-      const int u = __shfl_up_sync(0xffffffffu, incl, off);
-      if (lane >= off) incl += u;
-    }
-    if (k < n_M) {
-      s_n[k] = n;
-      s_pre[k] = carry + incl - v;
-    }
-    carry += __shfl_sync(0xffffffffu, incl, 31);
-  }
-  if (lane == 0) s_pre[n_M] = carry;
-}
-
 // Cell i needs its kernel row this step: occupied, or a neighbour drifts into
 // it (reach bits: 1 occupied, 2 has a rightward momentum, 4 a leftward one).
 __device__ __forceinline__ int cell_needs_kernel(const unsigned char* reach, int i, int n_x) {
   return (reach[i] & 1) || (i > 0 && (reach[i - 1] & 2)) || (i + 1 < n_x && (reach[i + 1] & 4));
 }
-
-// Largest k with s_pre[k] <= lid (so s_pre[k] <= lid < s_pre[k+1]).
-__device__ __forceinline__ int bucket_of(const int* s_pre, int n_M, int lid) {
-  int lo = 0, hi = n_M;
-  while (hi - lo > 1) {
-    const int mid = (lo + hi) >> 1;
-    if (s_pre[mid] <= lid) lo = mid; else hi = mid;
-  }
-  return lo;
-}
-
-// Drift direction of column k from its thresholds: +1, -1, or 0 (never moves).
-__device__ __forceinline__ int drift_dir(uint32_t lo, uint32_t hi) { return hi != 0xffffffffu ? 1 : (lo ? -1 : 0); }
 
 // Index of p' for the 53-bit uniform integer U2 in a fixed-point CDF row c of
 // n_M columns: target = floor(U2 Qtot / 2^53), Qtot = c[n_M - 1], and the

@@ -128,6 +128,20 @@ __device__ __forceinline__ void block_counters(DevHeader* hdr, unsigned long lon
   }
 }
 
+// A cell of one simulation for the walk.
+struct StepCell {
+  const int32_t* hist;
+  const uint32_t* bpa;
+  const uint32_t* xma;
+  int nM, i;
+  uint32_t off, rej;
+  bool gen;
+  __device__ __forceinline__ int n_M() const { return nM; }
+  __device__ __forceinline__ int row(int col) const { return __ldg(hist + (size_t)i * nM + col); }
+  __device__ __forceinline__ uint32_t bp(int b) const { return __ldg(bpa + (size_t)i * ((nM + 31) >> 5) + b); }
+  __device__ __forceinline__ uint32_t xm(int col) const { return __ldg(xma + col); }
+};
+
 // The ids of a range of work units [w0, w1), cell by cell, through walk_ids.
 // COUNT: the step proper (parents counted, absorbed particles too); otherwise
 // only the quads that may hold events are queued.  queue: kWalkQueue entries
@@ -135,22 +149,19 @@ __device__ __forceinline__ void block_counters(DevHeader* hdr, unsigned long lon
 template <bool COUNT, class Flush>
 __device__ __forceinline__ void walk_range(const StepArgs& a, uint32_t t, uint32_t w0, uint32_t w1, int lane,
                                            uint4* queue, int& nq, Flush flush) {
-  const int n_M = a.n_M, NB = (n_M + 31) >> 5;
+  const int n_M = a.n_M;
   CellWork cell = cell_of_unit(a.U, a.n_x, w0, lane);
 #pragma unroll 1
   while (true) {
     const int i = cell.i;
     const uint32_t first = id_prefix(a.R, i), last = id_prefix(a.R, i + 1);
     const uint32_t A = first & ~3u, qA = A >> 2;
-    WalkCell c;
-    c.row = a.hist_in + (size_t)i * n_M;
-    c.bp = a.bp + (size_t)i * NB;
-    c.xm = a.xm;
-    c.n_M = n_M;
-    c.off = first & 3u;
+    StepCell c{a.hist_in, a.bp, a.xm, n_M, i, first & 3u};
     const unsigned long long thr_m = i > 0 ? __ldg(a.thr_cell + i - 1) : 0ull, thr_0 = __ldg(a.thr_cell + i),
                              thr_p = i + 1 < a.n_x ? __ldg(a.thr_cell + i + 1) : 0ull;
-    c.tmax = max(thr_0, max(thr_m, thr_p));
+    const unsigned long long tmax = max(thr_0, max(thr_m, thr_p));
+    c.gen = tmax != 0ull;
+    c.rej = (uint32_t)(tmax - 1ull);
     // v particles' net sign (n of them) to column k of cell i + d, or out of the domain
     auto add = [&](int k, int d, int v, uint32_t n) {
       if (!COUNT) return;
@@ -252,10 +263,14 @@ __global__ __launch_bounds__(kStepThreads, 4) void k_pairs(const __grid_constant
   const int rows_by_cell = (int)a.hdr->rows_by_cell;
   const uint32_t t = a.t_from_device ? a.hdr->step : a.t;
   const unsigned n = a.hdr->pair_count;
+  // the blocks that have work (or block 0) count themselves done; the others
+  // leave at once, whether they see the count or its reset
+  const unsigned blocks = n > a.pair_cap ? gridDim.x : min(gridDim.x, max(1u, (n + kStepThreads - 1) / kStepThreads));
+  if (blockIdx.x >= blocks) return;
   unsigned long long pairs = 0, dropped = 0;
   long long drop_signed = 0;
   if (n <= a.pair_cap) {
-    for (unsigned e = blockIdx.x * kStepThreads + threadIdx.x; e < n; e += gridDim.x * kStepThreads)
+    for (unsigned e = blockIdx.x * kStepThreads + threadIdx.x; e < n; e += blocks * kStepThreads)
       quad_events(a, rows_by_cell, t, a.pairs[e], pairs, dropped, drop_signed);
   } else {
     __shared__ uint4 s_queue[kStepWarps][kWalkQueue + 32];
@@ -265,7 +280,7 @@ __global__ __launch_bounds__(kStepThreads, 4) void k_pairs(const __grid_constant
   __syncthreads();
   if (threadIdx.x == 0) {
     __threadfence();
-    if (atomicAdd(&a.hdr->pairs_done, 1u) == gridDim.x - 1u) {
+    if (atomicAdd(&a.hdr->pairs_done, 1u) == blocks - 1u) {
       a.hdr->pair_count = 0u;
       a.hdr->item_ticket = 0u;
       a.hdr->pairs_done = 0u;
@@ -361,17 +376,12 @@ __global__ __launch_bounds__(kStepThreads) void k_materialize(const int32_t* __r
   const uint32_t wn = (uint32_t)wid * gridDim.x + blockIdx.x;
   if (wn >= (total + size - 1u) / size) return;
   const uint32_t w0 = wn * size, w1 = min(w0 + size, total);
-  const int NB = (n_M + 31) >> 5, h = n_M / 2;
+  const int h = n_M / 2;
   CellWork cw = cell_of_unit(U, n_x, w0, lane);
 #pragma unroll 1
   while (true) {
     const uint32_t first = id_prefix(R, cw.i), last = id_prefix(R, cw.i + 1), A = first & ~3u;
-    WalkCell c;
-    c.row = hist + (size_t)cw.i * n_M;
-    c.bp = bp + (size_t)cw.i * NB;
-    c.xm = xm;
-    c.n_M = n_M;
-    c.off = first & 3u;
+    const StepCell c{hist, bp, xm, n_M, cw.i, first & 3u, 0u, false};
     WalkBlock B;
     walk_begin(B);
     const uint32_t r1 = min(last - A, window_of_unit(cw, last - first, w1) << 7);

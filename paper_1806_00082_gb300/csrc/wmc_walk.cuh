@@ -58,18 +58,17 @@ __device__ __forceinline__ uint32_t move_bits(const uint4& w, uint32_t e) {
 }
 
 // 4-bit mask of the elements j of a quad with j < d (d may be <= 0 or >= 4).
-__device__ __forceinline__ uint32_t first_mask(int d) { return d >= 4 ? 0xfu : (d <= 0 ? 0u : (1u << d) - 1u); }
+__device__ __forceinline__ uint32_t first_mask(int d) { return (1u << min(max(d, 0), 4)) - 1u; }
 
-// One cell's row and tables as the walk needs them.  Id offsets are relative
-// to A, the cell's first id rounded down to a multiple of 4; off = first id - A.
-struct WalkCell {
-  const int32_t* row;   // signed counts [n_M]
-  const uint32_t* bp;   // inclusive id prefixes of the 32-column blocks, [ceil(n_M / 32)]
-  const uint32_t* xm;   // move entries of the columns (move_entry)
-  int n_M;
-  uint32_t off;
-  unsigned long long tmax;  // largest event threshold of cells i - 1, i, i + 1
-};
+// The walk takes a cell as a type C with
+//   row(col), xm(col): signed count and move entry of a column;
+//   bp(b): inclusive id prefix of 32-column block b;
+//   n_M(): columns;  off: first id - A, where A is the first id rounded down to
+//   a multiple of 4 (id offsets are relative to A);
+//   gen, rej: whether any of the cells i - 1, i, i + 1 has an event threshold,
+//   and the largest such threshold less one.
+// (Accessors, so that a cell's pointers need not stay in registers during the
+// draws.)
 
 // The column block a warp holds: lane l's column 32 b + l.
 struct WalkBlock {
@@ -91,30 +90,31 @@ __device__ __forceinline__ void walk_begin(WalkBlock& k) {
 // Moves on to the block holding the id at offset x (at or after k.end, before
 // the cell's last).  In a sparse row the ids of one window lie in many blocks:
 // the block prefixes stay in the warp and the next block is always under way.
-__device__ __forceinline__ void walk_load(const WalkCell& c, uint32_t x, WalkBlock& k, int lane) {
-  const int NB = (c.n_M + 31) >> 5;
+template <class C>
+__device__ __forceinline__ void walk_load(const C& c, uint32_t x, WalkBlock& k, int lane) {
+  const int n_M = c.n_M(), NB = (n_M + 31) >> 5;
   const uint32_t rel = x - c.off;
   int g = k.b & ~31;
   unsigned above;
   while (!(above = __ballot_sync(0xffffffffu, k.grp > rel))) {
     g += 32;
-    k.grp = g + lane < NB ? __ldg(c.bp + g + lane) : 0xffffffffu;
+    k.grp = g + lane < NB ? c.bp(g + lane) : 0xffffffffu;
   }
   const int j = __ffs(above) - 1, nb = g + j;
   k.end = c.off + __shfl_sync(0xffffffffu, k.grp, j);
   uint32_t start = __shfl_sync(0xffffffffu, k.grp, j ? j - 1 : 0);
-  if (j == 0) start = g ? __ldg(c.bp + g - 1) : 0u;
+  if (j == 0) start = g ? c.bp(g - 1) : 0u;
   int col = (nb << 5) + lane;
   int n = k.pn;
   uint32_t e = k.pe;
   if (k.b < 0 || nb != k.b + 1) {
-    n = col < c.n_M ? __ldg(c.row + col) : 0;
-    e = col < c.n_M ? __ldg(c.xm + col) : kMoveNever;
+    n = col < n_M ? c.row(col) : 0;
+    e = col < n_M ? c.xm(col) : kMoveNever;
   }
   k.b = nb;
   col += 32;
-  k.pn = col < c.n_M ? __ldg(c.row + col) : 0;
-  k.pe = col < c.n_M ? __ldg(c.xm + col) : kMoveNever;
+  k.pn = col < n_M ? c.row(col) : 0;
+  k.pe = col < n_M ? c.xm(col) : kMoveNever;
   uint32_t incl = n < 0 ? 0u - (uint32_t)n : (uint32_t)n;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
@@ -194,9 +194,9 @@ struct RangeSchedule {
   uint32_t n_warps;
   uint32_t start, size, ticket;  // current round: first unit, units a range, first ticket
 
-  __device__ __forceinline__ RangeSchedule(uint32_t units, uint32_t warps)
+  __device__ __forceinline__ RangeSchedule(uint32_t units, uint32_t warps, uint32_t most = kMaxRange)
       : total(units), n_warps(warps), start(0u), ticket(0u) {
-    size = units <= kSingleRound * warps ? (units + warps - 1u) / warps : kMaxRange;
+    size = units <= kSingleRound * warps ? (units + warps - 1u) / warps : most;
     if (units > kSingleRound * warps) fit();
   }
   // halves the range size while a round of it would take more than half of what is left
@@ -234,13 +234,13 @@ constexpr int kWalkQueue = 160;
 // push(who, me, offset / 4, k, e, ids) queues the quads of the lanes `who`
 // (warp-collective; adds to nq); flush() empties the queue; words: 32 uint4 of
 // the warp's shared memory.
-template <class Draw, class Count, class Push, class Flush>
-__device__ __forceinline__ void walk_ids(const WalkCell& c, uint32_t r0, uint32_t r1, int lane, uint4* words,
+template <class C, class Draw, class Count, class Push, class Flush>
+__device__ __forceinline__ void walk_ids(const C& c, uint32_t r0, uint32_t r1, int lane, uint4* words,
                                          const int& nq, Draw draw, Count count, Push push, Flush flush) {
   const uint32_t g0 = r0 > c.off ? r0 : c.off;
   if (g0 >= r1) return;
-  const bool gen = c.tmax != 0ull;
-  const uint32_t rej = (uint32_t)(c.tmax - 1ull);  // gen: a word above it creates no pair anywhere
+  const bool gen = c.gen;
+  const uint32_t rej = c.rej;  // gen: a word above it creates no pair anywhere
   WalkBlock B;
   walk_begin(B);
   uint32_t a = r0;
@@ -255,7 +255,7 @@ __device__ __forceinline__ void walk_ids(const WalkCell& c, uint32_t r0, uint32_
     if (x == a && stop - a >= 128u) {
       // whole windows of one bucket
       const uint32_t e = __shfl_sync(0xffffffffu, B.e, j), th = e | 255u;
-      const int k = min((B.b << 5) + j, c.n_M - 1);
+      const int k = min((B.b << 5) + j, c.n_M() - 1);
       const uint32_t end = a + ((stop - a) & ~127u), from = a;
       uint32_t above = 0u;
       if (gen) {
@@ -315,7 +315,7 @@ __device__ __forceinline__ void walk_ids(const WalkCell& c, uint32_t r0, uint32_
         const uint32_t f = __shfl_sync(0xffffffffu, from, j), t = __shfl_sync(0xffffffffu, to, j),
                        e = __shfl_sync(0xffffffffu, B.e, j);
         const uint32_t inb = first_mask((int)(t - qa)) & ~first_mask((int)(f - qa));
-        const int k = min((B.b << 5) + j, c.n_M - 1);
+        const int k = min((B.b << 5) + j, c.n_M() - 1);
         const uint32_t mv = __reduce_add_sync(0xffffffffu, (uint32_t)__popc(move_bits(wr, e) & inb));
         if (cand) {
           const bool me = (cand >> lane) & 1u && inb != 0u;
@@ -327,7 +327,7 @@ __device__ __forceinline__ void walk_ids(const WalkCell& c, uint32_t r0, uint32_
       if (most) {
         const uint32_t* w = reinterpret_cast<const uint32_t*>(words) + (from - a);
         const uint32_t th = B.e | 255u;
-        const int k = min((B.b << 5) + lane, c.n_M - 1);
+        const int k = min((B.b << 5) + lane, c.n_M() - 1);
         uint32_t above = 0u;
 #pragma unroll
         for (uint32_t t = 0; t < kLaneBucket / 2; ++t)
