@@ -115,7 +115,11 @@ int num_sms() {
   return cached[dev];
 }
 
-__global__ void k_set_step(DevHeader* hdr, uint32_t step) { hdr->step = step; }
+// Start of a run: the step number, and nothing known about the caller's buffers.
+__global__ void k_set_step(DevHeader* hdr, uint32_t step) {
+  hdr->step = step;
+  hdr->rows_known = 0u;
+}
 
 __global__ void k_set_id_base(DevHeader* hdr, unsigned long long base) { hdr->id_base = base; }
 

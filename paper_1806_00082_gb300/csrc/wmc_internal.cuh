@@ -74,6 +74,11 @@ struct DevHeader {
   unsigned int pairs_done;   // pair-kernel blocks finished (the last one resets the queue and the ticket)
   unsigned int plan_epoch;   // launches of the plan so far (tags its blocks' published prefixes)
   unsigned int plan_ticket;  // logical block index of the running plan launch (reset by its last block)
+  // 1 between the steps of one wmc_run / wmc_batch_run call: the state about to
+  // be scanned can hold particles only in the last step's needed cells, and the
+  // other buffer only in the cells that were occupied then
+  unsigned int rows_known;
+  int n_live;      // batched form: needed cells with a row that is not exactly zero
   unsigned int pad0;
   unsigned long long id_base;  // number of the first survivor (a sub-domain numbers after the cells before it)
 };

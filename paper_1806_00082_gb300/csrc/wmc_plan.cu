@@ -229,7 +229,10 @@ __global__ __launch_bounds__(kPlanCells) void k_plan(int n_x, const unsigned lon
     hdr->n_items = ok ? tot.I : 0;
     hdr->n_occ = tot.N;
     if (!ok) atomicOr(&hdr->flags, WMC_FLAG_CAPACITY);
-    if (advance_step) hdr->step += 1u;
+    if (advance_step) {
+      hdr->step += 1u;
+      hdr->rows_known = 1u;
+    }
     hdr->plan_ticket = 0u;
     hdr->plan_epoch = (epoch + 1u) & 0x3fffffffu;
     __threadfence();
@@ -240,7 +243,14 @@ __global__ __launch_bounds__(kPlanCells) void k_plan(int n_x, const unsigned lon
 // prefixes of the row's 32-column blocks, reach bits (bit0 cell occupied, bit1
 // a momentum that drifts right is present, bit2 one that drifts left),
 // optionally the density rho[i] = sum_k n(i,k), and optionally a zeroed row of
-// the next histogram.
+// the next histogram.  Between the steps of a run (rows_known) only the rows
+// that can hold particles are read -- the cells the last step needed, by its
+// row map -- and only the rows that were occupied are zeroed: at 16384 cells
+// with 3555 occupied, 18.5 -> 10 us (64 MB read and 64 MB written otherwise).
+// States under kKnownRowsState columns are scanned whole (hdr null): they stay
+// in L2, and the look at the flags first costs a load's latency (2000 cells x
+// 256 columns: 302 against 305 us per 20 steps).
+constexpr long long kKnownRowsState = 1ll << 21;
 constexpr int kRowsWarps = 8;
 
 __global__ __launch_bounds__(kRowsWarps * 32) void k_rows(const int32_t* __restrict__ hist, int n_x, int n_M,
@@ -248,10 +258,21 @@ __global__ __launch_bounds__(kRowsWarps * 32) void k_rows(const int32_t* __restr
                                                           unsigned long long* __restrict__ T,
                                                           uint32_t* __restrict__ bp, unsigned char* __restrict__ reach,
                                                           unsigned char* __restrict__ nbk,
-                                                          long long* __restrict__ rho, int32_t* __restrict__ zero_out) {
+                                                          long long* __restrict__ rho, int32_t* __restrict__ zero_out,
+                                                          const int* __restrict__ row_map, const DevHeader* hdr) {
   const int warp = (int)((blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5);
   const int lane = threadIdx.x & 31;
   if (warp >= n_x) return;
+  if (zero_out && hdr && hdr->rows_known) {
+    if (T[warp] == 0ull) zero_out = nullptr;  // the row is zero
+    if (row_map[warp] < 0) {                  // no particle can be here (nor was one: zero_out is null)
+      if (lane == 0) {
+        T[warp] = 0ull;
+        reach[warp] = 0;
+      }
+      return;
+    }
+  }
   const int32_t* row = hist + (size_t)warp * n_M;
   const int NB = (n_M + 31) >> 5;
   uint32_t* bpr = bp + (size_t)warp * NB;
@@ -336,7 +357,8 @@ cudaError_t launch_rows(const wmc_params& p, const View& v, const int32_t* hist,
                         int32_t* zero_out) {
   const int blocks = (p.n_x + kRowsWarps - 1) / kRowsWarps;
   k_rows<<<blocks, kRowsWarps * 32, 0, s>>>(hist, p.n_x, p.n_M, v.D, v.T, v.bp, v.reach, v.nbk,
-                                            reinterpret_cast<long long*>(rho), zero_out);
+                                            reinterpret_cast<long long*>(rho), zero_out, v.row_map,
+                                            (long long)p.n_x * p.n_M >= kKnownRowsState ? v.hdr : nullptr);
   return cudaGetLastError();
 }
 
