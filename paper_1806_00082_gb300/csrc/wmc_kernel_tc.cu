@@ -13,9 +13,9 @@
 //     ring of shared-memory stages, M = N = 128, two TMEM accumulator buffers
 //     so that the epilogue of one column tile overlaps the MMAs of the next
 //     (K <= 512);
-//   - k_kernel_eval_tc_ws_split<FP16 | TF32>: the hi/lo split forms, three MMAs
-//     per K step (hi x hi, hi x lo, lo x hi), A resident in shared memory per
-//     K pass, each K block's main product in its own accumulator;
+//   - k_rows_split<FP16 | TF32>: the hi/lo split forms, three MMAs per K step
+//     (hi x hi, hi x lo, lo x hi), A through a ring of TMEM stages, each K
+//     block's main product in its own accumulator;
 //   - k_kernel_eval_tc: a per-tile kernel with both operands streamed, for
 //     BF16 / FP16 windows wider than the tensor-memory form holds.
 // Shared-memory operands use the K-major 128-byte swizzled layout: rows of
@@ -128,16 +128,6 @@ __device__ __forceinline__ void mma_f16(uint32_t d_tmem, uint64_t adesc, uint64_
       "{\n\t.reg .pred p;\n\t"
       "setp.ne.b32 p, %4, 0;\n\t"
       "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-      : "memory");
-}
-
-__device__ __forceinline__ void mma_tf32(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
-                                         uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
       "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
       : "memory");
 }
@@ -313,28 +303,24 @@ __global__ void k_init_tc_images32(int Q, int KB32, int NT, uint32_t* __restrict
 // from it without branches.
 constexpr int kStages = 2;
 
-__host__ __device__ constexpr size_t tc_smem_bytes(bool split, int h) {
-  return kSmemAlignPad + (size_t)(split ? 8 : 4) * kTileBytes + sizeof(float) * (size_t)(TM + 2 * h);
+__host__ __device__ constexpr size_t tc_smem_bytes(int h) {
+  return kSmemAlignPad + (size_t)4 * kTileBytes + sizeof(float) * (size_t)(TM + 2 * h);
 }
 
 template <int PREC>
 __global__ __launch_bounds__(128, 1) void k_kernel_eval_tc(const float* __restrict__ V, int n_x, int bc, int Q,
                                                            const int* __restrict__ occ,
                                                            const int* __restrict__ n_occ_dev, int n_occ_host,
-                                                           const uint16_t* __restrict__ img_b,
-                                                           const uint16_t* __restrict__ img_lo, int KB, float c,
+                                                           const uint16_t* __restrict__ img_b, int KB, float c,
                                                            float* __restrict__ VWh, unsigned int* __restrict__ flags) {
-  constexpr bool SPLIT = PREC == WMC_FP16_SPLIT;
   constexpr int kind_fmt = PREC == WMC_BF16 ? 1 : 0;
-  constexpr uint32_t kCols = SPLIT ? 512u : 256u;
+  constexpr uint32_t kCols = 256u;
   constexpr uint32_t idesc = idesc_f16(kind_fmt);
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t* smem = align_smem(smem_raw);
   uint8_t* sA[kStages] = {smem, smem + kTileBytes};
   uint8_t* sB[kStages] = {smem + 2 * kTileBytes, smem + 3 * kTileBytes};
-  uint8_t* sAl[kStages] = {smem + 4 * kTileBytes, smem + 5 * kTileBytes};  // split form only
-  uint8_t* sBl[kStages] = {smem + 6 * kTileBytes, smem + 7 * kTileBytes};
-  float* sV = reinterpret_cast<float*>(smem + (SPLIT ? 8 : 4) * kTileBytes);
+  float* sV = reinterpret_cast<float*>(smem + 4 * kTileBytes);
   __shared__ __align__(8) uint64_t bar_tma[kStages];
   __shared__ __align__(8) uint64_t bar_mma[kStages];
   __shared__ uint32_t tmem_slot;
@@ -368,7 +354,7 @@ __global__ __launch_bounds__(128, 1) void k_kernel_eval_tc(const float* __restri
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = tmem_slot;
-  const uint32_t accA = tmem, accB = tmem + (uint32_t)TN, accX = tmem + 2u * (uint32_t)TN;
+  const uint32_t accA = tmem, accB = tmem + (uint32_t)TN;
   const int pot0 = (occ || row0 >= n_rows) ? 0 : row0 / n_x;
   const bool contig = __syncthreads_and(valid && cell == s_cell0 + tid && pot_idx == pot0) != 0;
   if (contig) {
@@ -377,24 +363,21 @@ __global__ __launch_bounds__(128, 1) void k_kernel_eval_tc(const float* __restri
   }
 
   const int half_kb = (KB + 1) / 2;
-  const uint32_t tx_bytes = SPLIT ? 2u * kTileBytes : kTileBytes;
   const uint16_t* imgB_tile = img_b + (size_t)blockIdx.y * KB * (kTileBytes / 2);
-  const uint16_t* imgL_tile = SPLIT ? img_lo + (size_t)blockIdx.y * KB * (kTileBytes / 2) : nullptr;
 
   auto issue_copy = [&](int kb, int st) {
-    mbar_expect_tx(&bar_tma[st], tx_bytes);
+    mbar_expect_tx(&bar_tma[st], kTileBytes);
     bulk_g2s(sB[st], imgB_tile + (size_t)kb * (kTileBytes / 2), kTileBytes, &bar_tma[st]);
-    if (SPLIT) bulk_g2s(sBl[st], imgL_tile + (size_t)kb * (kTileBytes / 2), kTileBytes, &bar_tma[st]);
   };
   // this thread's A row of K block kb: window terms m = kb*64 + k + 1
   auto build_A = [&](int kb, int st) {
     if (contig) __syncthreads();  // the window is staged (first use) / keeps warps aligned
 #pragma unroll
     for (int k8 = 0; k8 < TK / 8; ++k8) {
-      uint32_t hw[4], lw[4];
+      uint32_t hw[4];
 #pragma unroll
       for (int e = 0; e < 8; e += 2) {
-        uint16_t hb[2], lb[2];
+        uint16_t hb[2];
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
           const int m = kb * TK + k8 * 8 + e + u + 1;
@@ -404,15 +387,12 @@ __global__ __launch_bounds__(128, 1) void k_kernel_eval_tc(const float* __restri
             else if (valid)
               dv = __fsub_rn(potential_at(Vr, n_x, bc, (long long)cell + m), potential_at(Vr, n_x, bc, (long long)cell - m));
           }
-          hb[u] = to_bits(dv, SPLIT ? WMC_FP16 : PREC);
-          if (SPLIT) lb[u] = to_bits(__fmul_rn(__fsub_rn(dv, from_bits(hb[u], WMC_FP16)), 2048.f), WMC_FP16);
+          hb[u] = to_bits(dv, PREC);
         }
         hw[e / 2] = (uint32_t)hb[0] | ((uint32_t)hb[1] << 16);
-        if (SPLIT) lw[e / 2] = (uint32_t)lb[0] | ((uint32_t)lb[1] << 16);
       }
       const uint32_t off = core_offset(tid, k8 * 8);
       *reinterpret_cast<uint4*>(sA[st] + off) = make_uint4(hw[0], hw[1], hw[2], hw[3]);
-      if (SPLIT) *reinterpret_cast<uint4*>(sAl[st] + off) = make_uint4(lw[0], lw[1], lw[2], lw[3]);
     }
   };
 
@@ -437,12 +417,6 @@ __global__ __launch_bounds__(128, 1) void k_kernel_eval_tc(const float* __restri
           const uint64_t a_hi = smem_desc(smem_u32(sA[st]) + s * kKStepBytes);
           const uint64_t b_hi = smem_desc(smem_u32(sB[st]) + s * kKStepBytes);
           mma_f16(acc, a_hi, b_hi, idesc, (first && s == 0) ? 0u : 1u);
-          if (SPLIT) {
-            const uint64_t a_lo = smem_desc(smem_u32(sAl[st]) + s * kKStepBytes);
-            const uint64_t b_lo = smem_desc(smem_u32(sBl[st]) + s * kKStepBytes);
-            mma_f16(accX, a_hi, b_lo, idesc, (kb == 0 && s == 0) ? 0u : 1u);
-            mma_f16(accX, a_lo, b_hi, idesc, 1u);
-          }
         }
         mma_commit(&bar_mma[st]);
         // the other stage is free once the MMAs of block kb - 1 are done
@@ -476,10 +450,9 @@ __global__ __launch_bounds__(128, 1) void k_kernel_eval_tc(const float* __restri
     const uint32_t lane_base = (uint32_t)(warp * 32) << 16;
     const bool has_B = KB > half_kb;
     for (int cc = 0; cc < TN; cc += 16) {
-      float a[16], b[16], x[16];
+      float a[16], b[16];
       tmem_ld16(accA + lane_base + (uint32_t)cc, a);
       if (has_B) tmem_ld16(accB + lane_base + (uint32_t)cc, b);
-      if (SPLIT) tmem_ld16(accX + lane_base + (uint32_t)cc, x);
       if (row < n_rows) {
         float* out = VWh + (size_t)row * h + col0 + cc;
 #pragma unroll
@@ -487,7 +460,6 @@ __global__ __launch_bounds__(128, 1) void k_kernel_eval_tc(const float* __restri
           if (col0 + cc + q >= h) break;
           float v = a[q];
           if (has_B) v = __fadd_rn(v, b[q]);
-          if (SPLIT) v = __fadd_rn(v, __fmul_rn(x[q], 0x1p-11f));
           out[q] = __fmul_rn(c, v);
         }
       }
@@ -811,26 +783,47 @@ __global__ __launch_bounds__(kWsThreads, 1) void k_kernel_eval_tc_ta(const float
   }
 }
 
-// ---------------------------------------------------------------- warp-specialised split forms
+// ---------------------------------------------------------------- split forms
 // FP16 hi/lo split: A = A_hi + 2^-11 A_lo, B = B_hi + 2^-11 B_lo, and
 //   A B ~ A_hi B_hi + 2^-11 (A_hi B_lo + A_lo B_hi)
 // (the A_lo B_lo term is below FP32 rounding).  3xTF32 (TF32 = true) is the
 // same with TF32 parts and no scaling (TF32 keeps the FP32 exponent range):
-// A = A_hi + A_lo with A_hi = tf32(A), A_lo = tf32(A - A_hi).  A 16 KB operand
-// block holds 128 rows x 64 FP16 or x 32 TF32 values.  One CTA per 128 rows
-// and one column tile.  K runs in passes of `bp` blocks (the A_hi / A_lo
-// blocks of a pass stay in shared memory while B_hi / B_lo stream through a
-// 2-stage ring).  The tensor core's FP32 accumulation does not round to
-// nearest: its error grows with the number of MMAs accumulated into one
-// TMEM accumulator.  So the A_hi B_hi product of every K block goes to its own
-// accumulator (three rotating 128-column TMEM buffers), which the epilogue
-// warps drain into FP32 registers (round to nearest) as each block completes;
-// the cross terms, 2^-11 smaller, share a fourth accumulator over all of K.
-// Roles as in k_kernel_eval_tc_ta; the builders build a pass, then drain its
-// blocks, and the drain of its last block (all MMAs before it complete) frees
-// A for the next pass.
-constexpr int kSpStages = 2;
-constexpr int kSpMaxHalf = 4;  // blocks resident per pass
+// A = A_hi + A_lo with A_hi = tf32(A), A_lo = tf32(A - A_hi).  An operand block
+// holds 128 rows x 64 FP16 or x 32 TF32 values.  The tensor core's FP32
+// accumulation does not round to nearest: its error grows with the number of
+// MMAs accumulated into one TMEM accumulator.  So the A_hi B_hi product of
+// every K block goes to an accumulator of its own, drained into FP32 registers
+// (round to nearest); the cross terms, 2^-11 smaller, share one over all of K.
+//
+// One persistent CTA per SM takes a run of consecutive 128 x 128 tiles (the
+// column tiles of a row tile follow each other) and keeps four stages working
+// at once across K blocks and tiles:
+//   - warps 0-7 build A, one row and half a K block per thread, into a ring of
+//     two TMEM stages (32 columns hi, 32 lo);
+//   - warp 17 streams the (hi, lo) blocks of B through kSpStages of shared
+//     memory;
+//   - warps 16 and 18 issue 12 MMAs per K block (N = 128, A from TMEM): the
+//     main products into two alternating TMEM accumulators, the cross terms into
+//     a third;
+//   - warps 8-15 drain the main accumulator of each K block, 64 columns per
+//     warp, and write the tile.
+// What bounds it: the MMA pipe and its hand-overs.  An MMA of this shape takes
+// 82 cycles with A in TMEM (86 with A in shared memory, where the builders'
+// stores, the copies and the MMA's own reads would also exceed the 128 B/cycle
+// of shared memory), and each commit holds up the MMAs behind it by about 165,
+// so a K block takes about 1860 cycles here.  The form before built passes of
+// four K blocks in shared memory and drained each pass before it built the
+// next, 3400 cycles a block: 16384 cells at Q = 1024 (3xTF32) 111 -> 63 us, 3600
+// occupied cells in the step 47 -> 22 us, 262144 rows at Q = 256 155 -> 78 us,
+// the adjoint contraction over the same rows 277 -> 192 us.
+constexpr int kSpStages = 5;
+// K blocks whose barriers are in use at once: more than the longest look-back,
+// kSpStages blocks, so that no waiter meets a barrier two phases on.
+constexpr int kSpRing = 8;
+static_assert(kSpRing > kSpStages, "a barrier comes round only after every waiter has seen it");
+constexpr int kSpSpan = 640;                 // cells a tile's rows may span for its window to be staged
+constexpr int kSpBuilders = 256, kSpThreads = 19 * 32;
+constexpr uint32_t kSpAccX = 2 * TN, kSpA = 3 * TN;  // TMEM columns: main 0, main 1, cross, A ring
 
 // NET = 3, the adjoint contraction Abar = c Gbar S^T of the differentiation
 // form: A is Gbar[row][r] = gVW[row][r] + g_gamma[row] dgamma/dVWh[row][r]
@@ -850,373 +843,457 @@ __device__ __forceinline__ int grid_count_tc(int r, int Q, int a, int b, int r0)
   return a + (off < b ? 1 : 0);
 }
 
-__device__ __forceinline__ float gbar_entry(const DenseA& g, int Q, int h, int row, int r) {
-  if (r >= h) return 0.f;
-  float v = g.gVW ? __ldg(g.gVW + (size_t)row * h + r) : 0.f;
-  const float gg = g.g_gamma ? __ldg(g.g_gamma + row) : 0.f;
-  if (gg != 0.f && r > 0) {
-    const float w = __ldg(g.VWh + (size_t)row * h + r);
-    const int dg = w > 0.f ? grid_count_tc(r, Q, g.ca, g.cb, g.cr0) : (w < 0.f ? -grid_count_tc(Q - r, Q, g.ca, g.cb, g.cr0) : 0);
-    v = __fadd_rn(v, __fmul_rn(gg, (float)dg));
+__host__ __device__ constexpr size_t split_window_floats(int h) { return (size_t)kSpSpan + 2 * (size_t)h + 4; }
+
+__host__ __device__ constexpr size_t split_smem_bytes(int h) {
+  return kSmemAlignPad + (size_t)kSpStages * 2 * kTileBytes + sizeof(float) * 8 * kWsStageFloats +
+         sizeof(float) * 2 * split_window_floats(h);
+}
+
+__device__ __forceinline__ void mma_tf32_ta(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc, uint32_t idesc,
+                                            uint32_t accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::1.kind::tf32 [%0], [%1], %2, %3, p;\n\t}" ::"r"(d_tmem),
+      "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(accumulate)
+      : "memory");
+}
+
+__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
+
+// Four bytes of global memory to shared memory, zero if not in; waited for by
+// cp_async_wait.
+__device__ __forceinline__ void cp_async4(float* dst, const float* src, bool in) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(in ? 4 : 0)
+               : "memory");
+}
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+// Reductions over the kSpBuilders builder threads (named barrier 1; every
+// builder thread takes part).
+__device__ __forceinline__ void sp_builders_sync() {
+  asm volatile("barrier.cta.sync 1, %0;" ::"n"(kSpBuilders) : "memory");
+}
+
+// The row tile a CTA builds from: whether its window is staged, and the row of
+// this thread.
+struct SplitRows {
+  bool window;
+  int cell0;   // first cell of the window's rows
+  int cell;    // this thread's row: cell and potential (clamped to a valid row)
+  int pot;
+};
+
+// N consecutive terms kk = k0 .. of the A operand of one row.  w[m] = V(cell + m).
+template <int NET, int N>
+__device__ __forceinline__ void a_run_window(const float* w, int h, int cell, int k0, float (&dv)[N]) {
+  if (NET == 1) {
+    if (k0 + N <= h - 1) {
+#pragma unroll
+      for (int e = 0; e < N; ++e) dv[e] = __fsub_rn(w[k0 + e + 1], w[-(k0 + e + 1)]);
+    } else {
+#pragma unroll
+      for (int e = 0; e < N; ++e) {
+        const int m = k0 + e + 1;
+        dv[e] = 0.f;
+        if (m <= h - 1) dv[e] = __fsub_rn(w[m], w[-m]);
+      }
+    }
+  } else {
+    // a pair to the right of the cell where i + u is even, else its mirror to the left
+#pragma unroll
+    for (int e = 0; e < N; ++e) {
+      const int u = k0 + e;
+      dv[e] = 0.f;
+      if (u <= h - 1) {
+        const bool right = ((cell + u) & 1) == 0;
+        const int at = right ? u : -u - 1;
+        const float s = __fadd_rn(w[at], w[at + 1]);
+        dv[e] = right ? s : -s;
+      }
+    }
   }
-  return v;
-}
-constexpr int kSpParts = 3;    // per-K-block accumulators (the cross-term accumulator is a fourth)
-
-// blocks per pass: half of K for FP16 (one or two passes), 4 for TF32
-__host__ __device__ constexpr int split_pass_blocks(int KB, bool tf32) {
-  return tf32 ? 4 : ((KB + 1) / 2 < 4 ? (KB + 1) / 2 : 4);
-}
-
-__host__ __device__ constexpr size_t ws_split_smem_bytes(int KB, int h, bool tf32 = false) {
-  return kSmemAlignPad + (size_t)2 * split_pass_blocks(KB, tf32) * kTileBytes + (size_t)kSpStages * 2 * kTileBytes +
-         sizeof(float) * (size_t)((TM + 2 * h) > (kWsBuilders / 32) * kWsStageFloats
-                                      ? (TM + 2 * h)
-                                      : (kWsBuilders / 32) * kWsStageFloats);
 }
 
 template <bool TF32, int NET>
-__global__ __launch_bounds__(kWsThreads, 1) void k_kernel_eval_tc_ws_split(
+__global__ __launch_bounds__(kSpThreads, 1) void k_rows_split(
     const float* __restrict__ V, int n_x, int bc, int Q, const int* __restrict__ occ,
     const int* __restrict__ n_occ_dev, int n_occ_host, const void* __restrict__ img_hi_v,
-    const void* __restrict__ img_lo_v, int KB, float c, float* __restrict__ VWh, unsigned int* __restrict__ flags,
-    DenseA dense) {
+    const void* __restrict__ img_lo_v, int KB, int NT, float c, float* __restrict__ VWh,
+    unsigned int* __restrict__ flags, DenseA dense) {
   // FP16 x FP16 -> FP32 (format 0) or TF32 x TF32 -> FP32 (format 2)
   constexpr uint32_t idesc = idesc_f16(TF32 ? 2u : 0u);
   constexpr int KBLK = TF32 ? 32 : TK;   // K values per operand block
-  constexpr int EPC = KBLK / 8;          // values per 16-byte chunk
+  constexpr int EPT = KBLK / 2;          // values a builder thread makes of one block
   constexpr float kLoScale = TF32 ? 1.f : 0x1p-11f;
   const uint8_t* img_hi = static_cast<const uint8_t*>(img_hi_v);
   const uint8_t* img_lo = static_cast<const uint8_t*>(img_lo_v);
   extern __shared__ __align__(1024) uint8_t smem_raw[];
-  uint8_t* smem = align_smem(smem_raw);
-  const int bp = split_pass_blocks(KB, TF32);                 // blocks per pass
-  uint8_t* sAh = smem;                                        // bp blocks of A_hi
-  uint8_t* sAl = smem + (size_t)bp * kTileBytes;               // bp blocks of A_lo
-  uint8_t* sB = smem + (size_t)2 * bp * kTileBytes;            // stages of (B_hi, B_lo)
-  float* sV = reinterpret_cast<float*>(sB + (size_t)kSpStages * 2 * kTileBytes);  // shared with the staging
-  __shared__ __align__(8) uint64_t a_ready[kSpMaxHalf];
-  __shared__ __align__(8) uint64_t b_full[kSpStages], b_empty[kSpStages];
-  __shared__ __align__(8) uint64_t acc_full[kSpParts], acc_empty[kSpParts], drain;
+  uint8_t* sB = align_smem(smem_raw);                                             // stages of (B_hi, B_lo)
+  float* s_stage = reinterpret_cast<float*>(sB + (size_t)kSpStages * 2 * kTileBytes);  // output staging, per drain warp
+  float* s_win = s_stage + 8 * kWsStageFloats;                                    // two windows
+  // of K block g, index g % kSpRing: its operands are there; its MMAs are complete
+  __shared__ __align__(8) uint64_t full[kSpRing], done[kSpRing];
+  __shared__ __align__(8) uint64_t acc_empty[2], x_empty, drain[2];
   __shared__ uint32_t tmem_slot;
   __shared__ volatile int s_abort;
+  __shared__ int s_min[8], s_max[8];
+  __shared__ float s_cnt[NET == 3 ? 2 * kAdjMaxH : 1];
 
   const int n_rows = n_occ_dev ? *n_occ_dev : n_occ_host;
-  const int row0 = blockIdx.x * TM;
   const int h = Q / 2;
-  if (row0 >= n_rows) return;
+  const long long n_tiles = (long long)((n_rows + TM - 1) / TM) * NT;
+  // this CTA's tiles [t0, t0 + n_my); row tile t / NT, column tile t % NT
+  const long long t0 = n_tiles * blockIdx.x / gridDim.x;
+  const int n_my = (int)(n_tiles * (blockIdx.x + 1) / gridDim.x - t0);
+  if (n_my <= 0) return;  // uniform over the CTA, before any allocation
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int nt = blockIdx.y;
-  const int n_pass = (KB + bp - 1) / bp;
-  const int n_tiles = KB;  // B tiles streamed: one per K block
 
   if (warp == 0) tmem_alloc(&tmem_slot, 512u);
   if (tid == 0) {
-    for (int q = 0; q < kSpMaxHalf; ++q) mbar_init(&a_ready[q], kWsBuilders);
-    for (int q = 0; q < kSpStages; ++q) {
-      mbar_init(&b_full[q], 1);
-      mbar_init(&b_empty[q], 1);
+    for (int q = 0; q < kSpRing; ++q) {
+      mbar_init(&full[q], kSpBuilders / 32 + 1);  // the builder warps, and the B producer with its bytes
+      mbar_init(&done[q], 2);                     // both MMA threads
     }
-    for (int q = 0; q < kSpParts; ++q) {
-      mbar_init(&acc_full[q], 1);
-      mbar_init(&acc_empty[q], kWsBuilders / 32);  // one arrival per epilogue warp
+    for (int q = 0; q < 2; ++q) {
+      mbar_init(&acc_empty[q], 8);
+      mbar_init(&drain[q], 1);
     }
-    mbar_init(&drain, 1);
+    mbar_init(&x_empty, 8);
     fence_mbar_init();
     s_abort = 0;
   }
+  if (NET == 3)
+    for (int r = tid; r < h; r += kSpThreads) {
+      s_cnt[r] = r ? (float)grid_count_tc(r, Q, dense.ca, dense.cb, dense.cr0) : 0.f;
+      s_cnt[kAdjMaxH + r] = r ? (float)grid_count_tc(Q - r, Q, dense.ca, dense.cb, dense.cr0) : 0.f;
+    }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = tmem_slot;
-  const uint32_t acc_x = tmem + (uint32_t)(kSpParts * TN);  // cross terms; block buffers at tmem + TN b
+  const int n_blocks = n_my * KB;  // K blocks of this CTA, numbered through its tiles
+  // a failed wait (about a second): every role stops working
+  auto give_up = [&]() {
+    atomicOr(flags, WMC_FLAG_TIMEOUT);
+    s_abort = 1;
+  };
+  auto wait_full = [&](int g) { return mbar_wait(&full[g % kSpRing], (uint32_t)((g / kSpRing) & 1)); };
+  auto wait_done = [&](int g) { return mbar_wait(&done[g % kSpRing], (uint32_t)((g / kSpRing) & 1)); };
 
-  if (warp == kWsBuilders / 32 + 1) {
-    // ---- B producer: tile kb of column tile nt, hi and lo, in K order
+  if (warp == 17) {
+    // ---- B producer
     if (lane == 0) {
       int issued = 0;
-      for (int t = 0; t < n_tiles && !s_abort; ++t) {
-        const int st = t % kSpStages;
-        if (t >= kSpStages && !mbar_wait(&b_empty[st], (uint32_t)(((t / kSpStages) - 1) & 1))) {
-          atomicOr(flags, WMC_FLAG_TIMEOUT);
-          s_abort = 1;
+      for (int g = 0; g < n_blocks && !s_abort; ++g) {
+        const int st = g % kSpStages;
+        if (g >= kSpStages && !wait_done(g - kSpStages)) {
+          give_up();
           break;
         }
         uint8_t* dst = sB + (size_t)st * 2 * kTileBytes;
-        const size_t off = ((size_t)nt * KB + t) * kTileBytes;  // bytes
-        mbar_expect_tx(&b_full[st], 2 * kTileBytes);
-        bulk_g2s(dst, img_hi + off, kTileBytes, &b_full[st]);
-        bulk_g2s(dst + kTileBytes, img_lo + off, kTileBytes, &b_full[st]);
-        issued = t + 1;
+        const int ct = (int)((t0 + g / KB) % NT);
+        const size_t off = ((size_t)ct * KB + g % KB) * kTileBytes;  // bytes
+        mbar_expect_tx(&full[g % kSpRing], 2 * kTileBytes);
+        bulk_g2s(dst, img_hi + off, kTileBytes, &full[g % kSpRing]);
+        bulk_g2s(dst + kTileBytes, img_lo + off, kTileBytes, &full[g % kSpRing]);
+        issued = g + 1;
       }
-      if (s_abort)
-        for (int t = max(0, issued - kSpStages); t < issued; ++t)
-          (void)mbar_wait(&b_full[t % kSpStages], (uint32_t)((t / kSpStages) & 1));
+      if (s_abort)  // let the copies still in flight land before the CTA exits (bounded: the builders,
+                    // who give up too, may leave their arrivals out)
+        for (int g = max(0, issued - kSpStages); g < issued; ++g) (void)wait_full(g);
     }
-  } else if (warp == kWsBuilders / 32) {
-    // ---- MMA issuer
+  } else if (warp == 16 || warp == 18) {
+    // ---- MMA issuers: one thread the main products, one the cross terms.  An
+    // MMA holds its thread for 65 cycles and more, and a wait on a barrier that
+    // is ready takes 130: one thread for both needed 2100 cycles a block for
+    // 1000 cycles of MMAs.
+    const bool is_main = warp == 16;
     if (lane == 0) {
-      for (int pass = 0; pass < n_pass && !s_abort; ++pass) {
-        const int kb0 = pass * bp, kb1 = min(KB, kb0 + bp);
-        for (int kb = kb0; kb < kb1; ++kb) {
-          const int kbl = kb - kb0, st = kb % kSpStages, buf = kb % kSpParts;
-          if (!mbar_wait(&a_ready[kbl], (uint32_t)(pass & 1)) ||
-              !mbar_wait(&b_full[st], (uint32_t)((kb / kSpStages) & 1)) ||
-              (kb >= kSpParts && !mbar_wait(&acc_empty[buf], (uint32_t)(((kb / kSpParts) - 1) & 1)))) {
-            atomicOr(flags, WMC_FLAG_TIMEOUT);
-            s_abort = 1;
-            break;
-          }
-          tc_fence_after();
-          const uint32_t acc_m = tmem + (uint32_t)(buf * TN);
-          const uint32_t ah = smem_u32(sAh + (size_t)kbl * kTileBytes), al = smem_u32(sAl + (size_t)kbl * kTileBytes);
-          const uint32_t bh = smem_u32(sB + (size_t)st * 2 * kTileBytes), bl = bh + kTileBytes;
-#pragma unroll
-          for (int s4 = 0; s4 < TK / 16; ++s4) {
-            const uint32_t o = s4 * kKStepBytes;
-            const uint64_t dah = smem_desc(ah + o), dbh = smem_desc(bh + o);
-            const bool first_m = s4 == 0;
-            if (TF32) {
-              mma_tf32(acc_m, dah, dbh, idesc, first_m ? 0u : 1u);
-              mma_tf32(acc_x, dah, smem_desc(bl + o), idesc, (kb == 0 && s4 == 0) ? 0u : 1u);
-              mma_tf32(acc_x, smem_desc(al + o), dbh, idesc, 1u);
-            } else {
-              mma_f16(acc_m, dah, dbh, idesc, first_m ? 0u : 1u);
-              mma_f16(acc_x, dah, smem_desc(bl + o), idesc, (kb == 0 && s4 == 0) ? 0u : 1u);
-              mma_f16(acc_x, smem_desc(al + o), dbh, idesc, 1u);
-            }
-          }
-          mma_commit(&b_empty[st]);
-          mma_commit(&acc_full[buf]);
-        }
-      }
-      if (s_abort) {
-        mma_commit(&drain);
-        (void)mbar_wait(&drain, 0u);
-      }
-    }
-  } else {
-    // ---- A builders (warps 0-15): both passes, then the epilogue
-    const int rc = tid & (TM - 1);
-    const int rowc = row0 + rc;
-    const bool validc = rowc < n_rows;
-    const int cellc = validc ? (occ ? __ldg(occ + rowc) : rowc % n_x) : 0;
-    const int potc = (occ || !validc) ? 0 : rowc / n_x;
-    const int cell0 = occ ? __ldg(occ + row0) : row0 % n_x;
-    const int pot0 = occ ? 0 : row0 / n_x;
-    const bool contig = NET != 3 && builders_and(validc && cellc == cell0 + rc && potc == pot0);
-    if (contig) {
-      const float* V0 = V + (size_t)pot0 * n_x;
-      constexpr int kU = 4;
-      for (int q0 = tid; q0 < TM + 2 * h; q0 += kU * kWsBuilders) {
-        float v[kU];
-#pragma unroll
-        for (int u = 0; u < kU; ++u) {
-          const int q = q0 + u * kWsBuilders;
-          v[u] = q < TM + 2 * h ? potential_at(V0, n_x, bc, (long long)cell0 - h + q) : 0.f;
-        }
-#pragma unroll
-        for (int u = 0; u < kU; ++u)
-          if (q0 + u * kWsBuilders < TM + 2 * h) sV[q0 + u * kWsBuilders] = v[u];
-      }
-      builders_sync();
-    }
-    const int rg = tid & 31, k8 = (tid >> 5) & 7, par = tid >> 8;
-    int cell_d[4];
-    bool valid_d[4];
-    const float* V_d[4];
-#pragma unroll
-    for (int d = 0; d < 4; ++d) {
-      const int row = row0 + 4 * rg + d;
-      valid_d[d] = row < n_rows;
-      cell_d[d] = (contig || !valid_d[d]) ? 0 : (occ ? __ldg(occ + row) : row % n_x);
-      V_d[d] = V + (size_t)((occ || !valid_d[d]) ? 0 : row / n_x) * n_x;
-    }
-    const bool fast = contig && (h & 3) == 0;
-    // epilogue slice of warp w: TMEM lanes 32 (w % 4) .. + 31, columns 32 (w / 4) .. + 31
-    const int quad = warp & 3, cq = warp >> 2;
-    const uint32_t lane_base = (uint32_t)(quad * 32) << 16;
-    float sacc[32];  // sum over the K blocks drained so far of A_hi B_hi
-#pragma unroll
-    for (int q = 0; q < 32; ++q) sacc[q] = 0.f;
-    bool drained_all = true;
-    for (int pass = 0; pass < n_pass; ++pass) {
-      const int kb0 = pass * bp, kb1 = min(KB, kb0 + bp), cnt = kb1 - kb0;
-      for (int kbl = 1 - par; kbl < cnt; kbl += 2)
-        asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&a_ready[kbl])) : "memory");
-#pragma unroll 1
-      for (int kbl = par; kbl < cnt; kbl += 2) {
-        const int kb = kb0 + kbl;
-        const int m0 = kb * KBLK + k8 * EPC + 1;
-        float dv[4][EPC];
-        if (NET == 1 && fast && m0 + EPC - 1 <= h - 1) {
-          // P[j] = V at offset m0 - 1 + j right of row 4 rg, N[j] = V at offset m0 + EPC - 1 - j left of it
-          constexpr int NW = EPC + 4;
-          float P[NW], N[NW];
-          const float* pp = sV + 4 * rg + h + m0 - 1;
-          const float* pn = sV + 4 * rg + h - m0 - (EPC - 1);
-#pragma unroll
-          for (int q = 0; q < NW / 4; ++q) {
-            const float4 a = *reinterpret_cast<const float4*>(pp + 4 * q);
-            const float4 b = *reinterpret_cast<const float4*>(pn + 4 * q);
-            P[4 * q] = a.x, P[4 * q + 1] = a.y, P[4 * q + 2] = a.z, P[4 * q + 3] = a.w;
-            N[4 * q] = b.x, N[4 * q + 1] = b.y, N[4 * q + 2] = b.z, N[4 * q + 3] = b.w;
-          }
-#pragma unroll
-          for (int d = 0; d < 4; ++d)
-#pragma unroll
-            for (int e = 0; e < EPC; ++e) dv[d][e] = __fsub_rn(P[d + e + 1], N[d - e + EPC - 1]);
-        } else if (NET == 3) {
-          const int r0 = m0 - 1;
-          if ((h & 3) == 0 && EPC == 4 && r0 + 3 < h) {
-            // four consecutive columns of each row: one 16-byte load per operand
-            float4 gv[4], wv[4];
-            float gg[4];
-#pragma unroll
-            for (int d = 0; d < 4; ++d) {
-              const size_t o = (size_t)(row0 + 4 * rg + d) * h + r0;
-              gv[d] = (valid_d[d] && dense.gVW) ? __ldg(reinterpret_cast<const float4*>(dense.gVW + o))
-                                                : make_float4(0.f, 0.f, 0.f, 0.f);
-              gg[d] = (valid_d[d] && dense.g_gamma) ? __ldg(dense.g_gamma + row0 + 4 * rg + d) : 0.f;
-              wv[d] = (valid_d[d] && gg[d] != 0.f) ? __ldg(reinterpret_cast<const float4*>(dense.VWh + o))
-                                                   : make_float4(0.f, 0.f, 0.f, 0.f);
-            }
-#pragma unroll
-            for (int d = 0; d < 4; ++d) {
-              const float g4[4] = {gv[d].x, gv[d].y, gv[d].z, gv[d].w};
-              const float w4[4] = {wv[d].x, wv[d].y, wv[d].z, wv[d].w};
-#pragma unroll
-              for (int e = 0; e < EPC; ++e) {
-                const int r = r0 + e;
-                float v = g4[e];
-                if (gg[d] != 0.f && r > 0) {
-                  const int dg = w4[e] > 0.f ? grid_count_tc(r, Q, dense.ca, dense.cb, dense.cr0)
-                                             : (w4[e] < 0.f ? -grid_count_tc(Q - r, Q, dense.ca, dense.cb, dense.cr0) : 0);
-                  v = __fadd_rn(v, __fmul_rn(gg[d], (float)dg));
-                }
-                dv[d][e] = valid_d[d] ? v : 0.f;
-              }
-            }
-          } else {
-#pragma unroll
-            for (int d = 0; d < 4; ++d)
-#pragma unroll
-              for (int e = 0; e < EPC; ++e)
-                dv[d][e] = valid_d[d] ? gbar_entry(dense, Q, h, row0 + 4 * rg + d, m0 - 1 + e) : 0.f;
-          }
-        } else {
-#pragma unroll
-          for (int d = 0; d < 4; ++d)
-#pragma unroll
-            for (int e = 0; e < EPC; ++e) {
-              const int kk = m0 - 1 + e;
-              dv[d][e] = 0.f;
-              if (contig) dv[d][e] = a_entry_window<NET == 3 ? 1 : NET>(sV + 4 * rg + d, h, cell0 + 4 * rg + d, kk);
-              else if (valid_d[d]) dv[d][e] = a_term<NET == 3 ? 1 : NET>(V_d[d], n_x, bc, h, cell_d[d], kk);
-            }
-        }
-        uint4 wh[4], wl[4];
-#pragma unroll
-        for (int d = 0; d < 4; ++d) {
-          uint32_t hw[4], lw[4];
-          if (TF32) {
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-              hw[e] = to_tf32(dv[d][e]);
-              lw[e] = to_tf32(__fsub_rn(dv[d][e], __uint_as_float(hw[e])));
-            }
-          } else {
-#pragma unroll
-            for (int e = 0; e < 8; e += 2) {
-              const uint16_t h0 = to_bits(dv[d][e], WMC_FP16), h1 = to_bits(dv[d][e + 1], WMC_FP16);
-              const uint16_t l0 = to_bits(__fmul_rn(__fsub_rn(dv[d][e], from_bits(h0, WMC_FP16)), 2048.f), WMC_FP16);
-              const uint16_t l1 =
-                  to_bits(__fmul_rn(__fsub_rn(dv[d][e + 1], from_bits(h1, WMC_FP16)), 2048.f), WMC_FP16);
-              hw[e / 2] = (uint32_t)h0 | ((uint32_t)h1 << 16);
-              lw[e / 2] = (uint32_t)l0 | ((uint32_t)l1 << 16);
-            }
-          }
-          wh[d] = make_uint4(hw[0], hw[1], hw[2], hw[3]);
-          wl[d] = make_uint4(lw[0], lw[1], lw[2], lw[3]);
-        }
-        uint8_t* bh = sAh + (size_t)kbl * kTileBytes;
-        uint8_t* bl = sAl + (size_t)kbl * kTileBytes;
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const int x = (i + (rg >> 1)) & 3;
-          const uint32_t off = core_offset(4 * rg + x, k8 * 8);
-          *reinterpret_cast<uint4*>(bh + off) = x == 0 ? wh[0] : x == 1 ? wh[1] : x == 2 ? wh[2] : wh[3];
-          *reinterpret_cast<uint4*>(bl + off) = x == 0 ? wl[0] : x == 1 ? wl[1] : x == 2 ? wl[2] : wl[3];
-        }
-        fence_proxy_async_smem();
-        asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&a_ready[kbl])) : "memory");
-      }
-      // drain the pass's K blocks in order; after the last one every MMA that
-      // reads this pass's A has completed, so the next pass may overwrite it
-      for (int kb = kb0; kb < kb1 && drained_all; ++kb) {
-        const int buf = kb % kSpParts;
-        int okw = 1;
-        if (lane == 0) okw = !s_abort && mbar_wait(&acc_full[buf], (uint32_t)((kb / kSpParts) & 1));
-        if (__shfl_sync(0xffffffffu, okw, 0) == 0) {  // warp-uniform: the TMEM loads are warp-collective
-          if (lane == 0) atomicOr(flags, WMC_FLAG_TIMEOUT);
-          s_abort = 1;
-          drained_all = false;
+      int kb = 0, tile = 0;
+      for (int g = 0; g < n_blocks && !s_abort; ++g) {
+        const int ab = g & 1;
+        if (!wait_full(g) || (is_main ? g >= 2 && !mbar_wait(&acc_empty[ab], (uint32_t)(((g >> 1) & 1) ^ 1))
+                                      : kb == 0 && tile > 0 && !mbar_wait(&x_empty, (uint32_t)((tile - 1) & 1)))) {
+          give_up();
           break;
         }
         tc_fence_after();
-        uint32_t r0[16], r1[16];
-        const uint32_t ta = tmem + (uint32_t)(buf * TN) + lane_base + (uint32_t)(cq * 32);
-        tmem_ld16_issue(ta, r0);
-        tmem_ld16_issue(ta + 16u, r1);
-        tmem_wait16(r0);
-        tmem_wait16(r1);
+        const uint32_t ah = tmem + kSpA + (uint32_t)(ab * 64), al = ah + 32u;
+        const uint32_t bh = smem_u32(sB + (size_t)(g % kSpStages) * 2 * kTileBytes), bl = bh + kTileBytes;
+        if (is_main) {
+          const uint32_t acc_m = tmem + (uint32_t)(ab * TN);
 #pragma unroll
-        for (int q = 0; q < 16; ++q) {
-          sacc[q] = __fadd_rn(sacc[q], __uint_as_float(r0[q]));
-          sacc[16 + q] = __fadd_rn(sacc[16 + q], __uint_as_float(r1[q]));
-        }
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0)
-          asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&acc_empty[buf])) : "memory");
-      }
-      if (!drained_all) break;
-    }
-    // epilogue: v = c (sum of the block products + 2^-11 x cross)
-    float* stg = sV + warp * kWsStageFloats;
-    const bool vec_ok = (h & 3) == 0 && (reinterpret_cast<uintptr_t>(VWh) & 15) == 0;
-    if (drained_all) {
+          for (int s4 = 0; s4 < 4; ++s4) {
+            const uint64_t d = smem_desc(bh + s4 * kKStepBytes);
+            if (TF32) mma_tf32_ta(acc_m, ah + s4 * 8, d, idesc, s4 ? 1u : 0u);
+            else mma_f16_ta(acc_m, ah + s4 * 8, d, idesc, s4 ? 1u : 0u);
+          }
+        } else {
+          const uint32_t acc_x = tmem + kSpAccX;
 #pragma unroll
-      for (int hf = 0; hf < 2; ++hf) {
-        const int cc = cq * 32 + hf * 16;
-        const int col0 = nt * TN + cc;
-        float a[16], x[16];
-        tmem_ld16(acc_x + lane_base + (uint32_t)cc, x);
-#pragma unroll
-        for (int q = 0; q < 16; ++q) a[q] = __fmul_rn(c, __fadd_rn(sacc[hf * 16 + q], __fmul_rn(x[q], kLoScale)));
-#pragma unroll
-        for (int g = 0; g < 4; ++g)
-          *reinterpret_cast<float4*>(stg + lane * 16 + 4 * (g ^ ((lane >> 1) & 3))) =
-              make_float4(a[4 * g], a[4 * g + 1], a[4 * g + 2], a[4 * g + 3]);
-        __syncwarp();
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const int rr = 8 * i + (lane >> 2), g = lane & 3;
-          const float4 v = *reinterpret_cast<const float4*>(stg + rr * 16 + 4 * (g ^ ((rr >> 1) & 3)));
-          const int grow = row0 + quad * 32 + rr, gcol = col0 + 4 * g;
-          if (grow < n_rows && gcol < h) {
-            float* out = VWh + (size_t)grow * h + gcol;
-            if (vec_ok) {
-              *reinterpret_cast<float4*>(out) = v;
+          for (int s4 = 0; s4 < 4; ++s4) {
+            const uint64_t dh = smem_desc(bh + s4 * kKStepBytes), dl = smem_desc(bl + s4 * kKStepBytes);
+            const uint32_t more = (kb == 0 && s4 == 0) ? 0u : 1u;
+            if (TF32) {
+              mma_tf32_ta(acc_x, ah + s4 * 8, dl, idesc, more);
+              mma_tf32_ta(acc_x, al + s4 * 8, dh, idesc, 1u);
             } else {
-              out[0] = v.x;
-              if (gcol + 1 < h) out[1] = v.y;
-              if (gcol + 2 < h) out[2] = v.z;
-              if (gcol + 3 < h) out[3] = v.w;
+              mma_f16_ta(acc_x, ah + s4 * 8, dl, idesc, more);
+              mma_f16_ta(acc_x, al + s4 * 8, dh, idesc, 1u);
             }
           }
         }
+        mma_commit(&done[g % kSpRing]);
+        if (++kb == KB) {
+          kb = 0;
+          ++tile;
+        }
+      }
+      if (s_abort) {  // drain the MMAs already issued before TMEM is freed (bounded)
+        uint64_t* mine = &drain[is_main ? 0 : 1];
+        mma_commit(mine);
+        (void)mbar_wait(mine, 0u);
+      }
+    }
+  } else if (warp < 8) {
+    // ---- A builders: thread = row 32 (warp % 4) + lane of the tile, K half warp / 4
+    const int quad = warp & 3, half = warp >> 2;
+    const int rr = 32 * quad + lane;
+    const uint32_t a_base = tmem + kSpA + ((uint32_t)(quad * 32) << 16) + (uint32_t)(half * 16);
+    bool ok = true;  // (a thread that gave up keeps to the barriers)
+    // the rows of a row tile: this thread's cell and whether the tile's window
+    // can be staged; starts the copies of the window (every builder thread)
+    auto rows_of = [&](int rt, float* win) {
+      SplitRows r;
+      const int row = min(rt * TM + rr, n_rows - 1);
+      r.cell = occ ? __ldg(occ + row) : row % n_x;
+      r.pot = occ ? 0 : row / n_x;
+      r.window = false;
+      r.cell0 = 0;
+      if (NET != 3) {
+        int lo = r.cell, hi = r.cell;
+        if (occ) {
+          lo = __reduce_min_sync(0xffffffffu, lo);
+          hi = __reduce_max_sync(0xffffffffu, hi);
+          if (lane == 0) {
+            s_min[warp] = lo;
+            s_max[warp] = hi;
+          }
+          sp_builders_sync();
+          lo = min(min(s_min[0], s_min[1]), min(s_min[2], s_min[3]));
+          hi = max(max(s_max[0], s_max[1]), max(s_max[2], s_max[3]));
+          sp_builders_sync();
+          r.window = hi - lo < kSpSpan;
+        } else {
+          lo = (rt * TM) % n_x;
+          const int last = min(rt * TM + TM, n_rows) - 1;
+          hi = last % n_x;
+          r.window = (rt * TM) / n_x == last / n_x;  // one potential
+        }
+        r.cell0 = lo;
+        if (r.window) {
+          const float* Vp = V + (size_t)((occ ? 0 : (rt * TM) / n_x)) * n_x;
+          const int n = hi - lo + 1 + 2 * h;
+          for (int q = tid; q < n; q += kSpBuilders) {
+            const long long l = (long long)lo - h + q;
+            const bool in = l >= 0 && l < n_x;
+            cp_async4(win + q, Vp + (in ? l : (l < 0 ? 0 : n_x - 1)), in || bc);
+          }
+        }
+      }
+      return r;
+    };
+    const size_t wf = split_window_floats(h);
+    SplitRows cur = rows_of((int)(t0 / NT), s_win);
+    cp_async_wait();
+    sp_builders_sync();
+    int wb = 0;
+    // NET = 3: the next block's entries of gVW and VWh, asked for ahead
+    constexpr int RAW = NET == 3 ? EPT : 1;
+    float graw[RAW], vraw[RAW], gg = 0.f;
+    auto load_dense = [&](int g) {
+      const int row = (int)((t0 + g / KB) / NT) * TM + rr, k0 = (g % KB) * KBLK + half * EPT;
+      const bool on = g < n_blocks && row < n_rows;
+      gg = on && dense.g_gamma ? __ldg(dense.g_gamma + row) : 0.f;
+      const size_t o = (size_t)row * h + k0;
+      if ((h & 3) == 0) {
+#pragma unroll
+        for (int q = 0; q < RAW / 4; ++q) {
+          const bool in = on && k0 + 4 * q < h;
+          const float4 a = in && dense.gVW ? __ldg(reinterpret_cast<const float4*>(dense.gVW + o + 4 * q))
+                                           : make_float4(0.f, 0.f, 0.f, 0.f);
+          const float4 b = in && dense.g_gamma ? __ldg(reinterpret_cast<const float4*>(dense.VWh + o + 4 * q))
+                                               : make_float4(0.f, 0.f, 0.f, 0.f);
+          graw[4 * q] = a.x, graw[4 * q + 1] = a.y, graw[4 * q + 2] = a.z, graw[4 * q + 3] = a.w;
+          vraw[4 * q] = b.x, vraw[4 * q + 1] = b.y, vraw[4 * q + 2] = b.z, vraw[4 * q + 3] = b.w;
+        }
+      } else {
+#pragma unroll
+        for (int e = 0; e < RAW; ++e) {
+          const bool in = on && k0 + e < h;
+          graw[e] = in && dense.gVW ? __ldg(dense.gVW + o + e) : 0.f;
+          vraw[e] = in && dense.g_gamma ? __ldg(dense.VWh + o + e) : 0.f;
+        }
+      }
+    };
+    if (NET == 3) load_dense(0);
+    for (int tile = 0; tile < n_my; ++tile) {
+      const int rt = (int)((t0 + tile) / NT);
+      // the next tile's window on its way while this tile is built
+      const bool last = tile + 1 == n_my, same = last || (int)((t0 + tile + 1) / NT) == rt;
+      SplitRows nxt = cur;
+      if (!same) nxt = rows_of(rt + 1, s_win + (wb ^ 1) * wf);
+      const float* w = s_win + wb * wf + h + (cur.cell - cur.cell0);
+      const float* Vr = NET == 3 ? nullptr : V + (size_t)cur.pot * n_x;
+#pragma unroll 1
+      for (int kb = 0; kb < KB; ++kb) {
+        const int g = tile * KB + kb, ab = g & 1;
+        const int k0 = kb * KBLK + half * EPT;
+        float dv[EPT];
+        if (NET == 3) {
+#pragma unroll
+          for (int e = 0; e < EPT; ++e) {
+            const int r = k0 + e;
+            float v = graw[NET == 3 ? e : 0];
+            if (gg != 0.f && r > 0 && r < h) {
+              const float x = vraw[NET == 3 ? e : 0];
+              const float dg = x > 0.f ? s_cnt[NET == 3 ? r : 0] : (x < 0.f ? -s_cnt[NET == 3 ? kAdjMaxH + r : 0] : 0.f);
+              v = __fadd_rn(v, __fmul_rn(gg, dg));
+            }
+            dv[e] = v;
+          }
+          load_dense(g + 1);
+        } else if (cur.window) {
+          a_run_window<NET == 3 ? 1 : NET, EPT>(w, h, cur.cell, k0, dv);
+        } else {
+#pragma unroll
+          for (int e = 0; e < EPT; ++e) dv[e] = a_term<NET == 3 ? 1 : NET>(Vr, n_x, bc, h, cur.cell, k0 + e);
+        }
+        uint32_t hi[16], lo[16];
+        if (TF32) {
+#pragma unroll
+          for (int e = 0; e < 16; ++e) {
+            hi[e] = to_tf32(dv[e]);
+            lo[e] = to_tf32(__fsub_rn(dv[e], __uint_as_float(hi[e])));
+          }
+        } else {
+#pragma unroll
+          for (int e = 0; e < 16; ++e) {
+            const float x = dv[TF32 ? 0 : 2 * e], y = dv[TF32 ? 0 : 2 * e + 1];
+            hi[e] = pack2<WMC_FP16>(x, y);
+            lo[e] = pack2<WMC_FP16>(__fmul_rn(__fsub_rn(x, from_bits((uint16_t)(hi[e] & 0xffffu), WMC_FP16)), 2048.f),
+                                    __fmul_rn(__fsub_rn(y, from_bits((uint16_t)(hi[e] >> 16), WMC_FP16)), 2048.f));
+          }
+        }
+        if (ok && g >= 2) {
+          ok = !s_abort && wait_done(g - 2);
+          if (!ok) give_up();
+        }
+        ok = __all_sync(0xffffffffu, ok);  // (the TMEM stores are warp-collective)
+        if (ok) {
+          tc_fence_after();
+          tmem_st16(a_base + (uint32_t)(ab * 64), hi);
+          tmem_st16(a_base + (uint32_t)(ab * 64 + 32), lo);
+          tmem_wait_st();
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&full[g % kSpRing]);
+        }
+      }
+      if (!same) {
+        cp_async_wait();
+        sp_builders_sync();
+        wb ^= 1;
+        cur = nxt;
+      }
+    }
+  } else {
+    // ---- drain and output: warp 8 + w reads lanes 32 (w % 4) .. + 31, columns 64 (w / 4) .. + 63
+    const int dw = warp - 8, quad = dw & 3, ch = dw >> 2;
+    const uint32_t t_base = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(ch * 64);
+    float* stg = s_stage + dw * kWsStageFloats;
+    const bool vec_ok = (h & 3) == 0 && (reinterpret_cast<uintptr_t>(VWh) & 15) == 0;
+    bool ok = true;
+    for (int tile = 0; tile < n_my && ok; ++tile) {
+      float sacc[64];  // sum over the K blocks drained so far of A_hi B_hi
+#pragma unroll
+      for (int q = 0; q < 64; ++q) sacc[q] = 0.f;
+      for (int kb = 0; kb < KB; ++kb) {
+        const int g = tile * KB + kb, ab = g & 1;
+        int okw = 1;
+        if (lane == 0) okw = !s_abort && wait_done(g);
+        if (__shfl_sync(0xffffffffu, okw, 0) == 0) {  // warp-uniform: the TMEM loads are warp-collective
+          if (lane == 0) give_up();
+          ok = false;
+          break;
+        }
+        tc_fence_after();
+        uint32_t r[2][16];
+        tmem_ld16_issue(t_base + (uint32_t)(ab * TN), r[0]);
+        tmem_ld16_issue(t_base + (uint32_t)(ab * TN) + 16u, r[1]);
+        tmem_wait16(r[0]);
+        tmem_wait16(r[1]);
+#pragma unroll
+        for (int q = 0; q < 32; ++q) sacc[q] = __fadd_rn(sacc[q], __uint_as_float(r[q >> 4][q & 15]));
+        tmem_ld16_issue(t_base + (uint32_t)(ab * TN) + 32u, r[0]);
+        tmem_ld16_issue(t_base + (uint32_t)(ab * TN) + 48u, r[1]);
+        tmem_wait16(r[0]);
+        tmem_wait16(r[1]);
+        tc_fence_before();
         __syncwarp();
+        if (lane == 0) mbar_arrive(&acc_empty[ab]);
+#pragma unroll
+        for (int q = 0; q < 32; ++q) sacc[32 + q] = __fadd_rn(sacc[32 + q], __uint_as_float(r[q >> 4][q & 15]));
+      }
+      if (!ok) break;
+      // v = c (sum of the block products + 2^-11 x cross); every MMA of the tile is complete
+#pragma unroll
+      for (int p = 0; p < 4; ++p) {
+        float x[16];
+        tmem_ld16(t_base + kSpAccX + (uint32_t)(16 * p), x);
+#pragma unroll
+        for (int q = 0; q < 16; ++q)
+          sacc[16 * p + q] = __fmul_rn(c, __fadd_rn(sacc[16 * p + q], __fmul_rn(x[q], kLoScale)));
+      }
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&x_empty);
+      const int row0 = (int)((t0 + tile) / NT) * TM + quad * 32;
+      const int col00 = (int)((t0 + tile) % NT) * TN + ch * 64;
+#pragma unroll
+      for (int p = 0; p < 4; ++p) {
+        const int col0 = col00 + 16 * p;
+        if (col0 < h) {  // uniform
+          // 32 rows x 16 columns through shared memory, so that stores are whole 64-byte row segments
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+            *reinterpret_cast<float4*>(stg + lane * 16 + 4 * (q ^ ((lane >> 1) & 3))) =
+                make_float4(sacc[16 * p + 4 * q], sacc[16 * p + 4 * q + 1], sacc[16 * p + 4 * q + 2],
+                            sacc[16 * p + 4 * q + 3]);
+          __syncwarp();
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const int r2 = 8 * i + (lane >> 2), q = lane & 3;
+            const float4 v = *reinterpret_cast<const float4*>(stg + r2 * 16 + 4 * (q ^ ((r2 >> 1) & 3)));
+            const int grow = row0 + r2, gcol = col0 + 4 * q;
+            if (grow < n_rows && gcol < h) {
+              float* out = VWh + (size_t)grow * h + gcol;
+              if (vec_ok) {
+                *reinterpret_cast<float4*>(out) = v;
+              } else {
+                out[0] = v.x;
+                if (gcol + 1 < h) out[1] = v.y;
+                if (gcol + 2 < h) out[2] = v.z;
+                if (gcol + 3 < h) out[3] = v.w;
+              }
+            }
+          }
+          __syncwarp();
+        }
       }
     }
   }
@@ -1285,6 +1362,21 @@ cudaError_t launch_init_tc_images(const wmc_params& p, void* images, cudaStream_
   return cudaGetLastError();
 }
 
+// One persistent CTA per SM, fewer if there are fewer tiles.
+template <bool TF32, int NET>
+static cudaError_t launch_split(const float* V, int n_x, int bc, int Q, const int* occ, const int* n_occ_dev,
+                                int n_occ_host, int max_rows, const void* img_hi, const void* img_lo, int KB, int NT,
+                                float c, float* out, unsigned int* flags, const DenseA& dense, cudaStream_t s) {
+  const size_t sm = split_smem_bytes(Q / 2);
+  const cudaError_t e = raise_smem_limit(reinterpret_cast<const void*>(k_rows_split<TF32, NET>), sm);
+  if (e != cudaSuccess) return e;
+  const long long tiles = (long long)((max_rows + TM - 1) / TM) * NT;
+  const unsigned grid = (unsigned)(tiles < num_sms() ? tiles : num_sms());
+  k_rows_split<TF32, NET><<<grid, kSpThreads, sm, s>>>(V, n_x, bc, Q, occ, n_occ_dev, n_occ_host, img_hi, img_lo, KB, NT,
+                                                       c, out, flags, dense);
+  return cudaGetLastError();
+}
+
 // Abar = c Gbar S^T on the 3xTF32 split kernel (NET = 3), rows = n_pot n_x
 // implicit rows; Q <= 256.
 cudaError_t launch_adjoint_abar_tc(const wmc_params& p, int rows, const float* VWh, const float* gVW,
@@ -1302,13 +1394,8 @@ cudaError_t launch_adjoint_abar_tc(const wmc_params& p, int rows, const float* V
   d.cb = p.n_M - d.ca * p.Q;
   d.cr0 = ((-(p.n_M / 2)) % p.Q + p.Q) % p.Q;
   const float c = (float)(-2.0 / (kHbarEVs * (double)p.Q));
-  const size_t sm = ws_split_smem_bytes(g.KBa, g_h(p), true);
-  const dim3 grid((rows + TM - 1) / TM, g.NT);
-  cudaError_t e = raise_smem_limit(reinterpret_cast<const void*>(k_kernel_eval_tc_ws_split<true, 3>), sm);
-  if (e != cudaSuccess) return e;
-  k_kernel_eval_tc_ws_split<true, 3><<<grid, kWsThreads, sm, s>>>(nullptr, rows, 0, p.Q, nullptr, nullptr, rows, ba,
-                                                                  ba + g.bytes_per_imagea, g.KBa, c, Abar, flags, d);
-  return cudaGetLastError();
+  return launch_split<true, 3>(nullptr, rows, 0, p.Q, nullptr, nullptr, rows, rows, ba, ba + g.bytes_per_imagea, g.KBa,
+                               g.NT, c, Abar, flags, d, s);
 }
 
 // The form behind a requested precision: WMC_FP32 takes the 3xTF32 split
@@ -1322,8 +1409,7 @@ int resolve_precision(const wmc_params& p, int prec, int net, long long rows) {
   if (prec == WMC_FP32_SIMT) return WMC_FP32;
   if (prec != WMC_FP32 || net != 1) return prec;
   if (p.Q <= 256 && !(p.Q >= 128 && rows >= (long long)TM * num_sms())) return prec;
-  const TcImages g = tc_geometry(p);
-  return ws_split_smem_bytes(g.KB32, g_h(p), true) <= 226 * 1024 ? WMC_TF32X3 : WMC_FP32;
+  return WMC_TF32X3;
 }
 
 // The N = 2 network (net = 2) runs on the warp-specialised BF16 / FP16 and
@@ -1354,28 +1440,19 @@ cudaError_t launch_kernel_eval_tc(const wmc_params& p, int prec, const float* V,
   const float c = (float)(-2.0 / (kHbarEVs * (double)p.Q));
   dim3 grid((max_rows + TM - 1) / TM, g.NT);
   if (prec == WMC_BF16) {
-    const size_t sm = tc_smem_bytes(false, g_h(p));
+    const size_t sm = tc_smem_bytes(g_h(p));
     raise_smem_limit(reinterpret_cast<const void*>(k_kernel_eval_tc<WMC_BF16>), sm);
     k_kernel_eval_tc<WMC_BF16><<<grid, 128, sm, s>>>(V, p.n_x, p.bc_potential, p.Q, occ, n_occ_dev, n_occ_host,
-                                                     base, nullptr, g.KB, c, VWh, flags);
+                                                     base, g.KB, c, VWh, flags);
   } else if (prec == WMC_FP16) {
-    const size_t sm = tc_smem_bytes(false, g_h(p));
+    const size_t sm = tc_smem_bytes(g_h(p));
     raise_smem_limit(reinterpret_cast<const void*>(k_kernel_eval_tc<WMC_FP16>), sm);
     k_kernel_eval_tc<WMC_FP16><<<grid, 128, sm, s>>>(V, p.n_x, p.bc_potential, p.Q, occ, n_occ_dev, n_occ_host,
-                                                     base + n16, nullptr, g.KB, c, VWh, flags);
-  } else if (prec == WMC_TF32X3 && ws_split_smem_bytes(g.KB32, g_h(p), true) <= 226 * 1024) {
-    const size_t sm = ws_split_smem_bytes(g.KB32, g_h(p), true);
+                                                     base + n16, g.KB, c, VWh, flags);
+  } else if (prec == WMC_TF32X3) {
     const uint8_t* b32 = reinterpret_cast<const uint8_t*>(images) + 3 * g.bytes_per_image;
-    raise_smem_limit(reinterpret_cast<const void*>(k_kernel_eval_tc_ws_split<true, 1>), sm);
-    k_kernel_eval_tc_ws_split<true, 1><<<grid, kWsThreads, sm, s>>>(V, p.n_x, p.bc_potential, p.Q, occ, n_occ_dev,
-                                                                 n_occ_host, b32, b32 + g.bytes_per_image32,
-                                                                 g.KB32, c, VWh, flags, DenseA{});
-  } else if (prec == WMC_FP16_SPLIT) {
-    const size_t sm = tc_smem_bytes(true, g_h(p));
-    raise_smem_limit(reinterpret_cast<const void*>(k_kernel_eval_tc<WMC_FP16_SPLIT>), sm);
-    k_kernel_eval_tc<WMC_FP16_SPLIT><<<grid, 128, sm, s>>>(V, p.n_x, p.bc_potential, p.Q, occ, n_occ_dev,
-                                                           n_occ_host, base + n16, base + 2 * n16, g.KB, c, VWh,
-                                                           flags);
+    return launch_split<true, 1>(V, p.n_x, p.bc_potential, p.Q, occ, n_occ_dev, n_occ_host, max_rows, b32,
+                                 b32 + g.bytes_per_image32, g.KB32, g.NT, c, VWh, flags, DenseA{}, s);
   } else {
     return cudaErrorInvalidValue;
   }
@@ -1421,15 +1498,9 @@ static cudaError_t launch_tc_net(const wmc_params& p, int prec, const float* V, 
                                                                       flags);
     return cudaGetLastError();
   }
-  if (prec == WMC_FP16_SPLIT && ws_split_smem_bytes(KB, g_h(p)) <= 226 * 1024) {
-    const size_t sm = ws_split_smem_bytes(KB, g_h(p));
-    const dim3 grid(row_tiles, g.NT);
-    raise_smem_limit(reinterpret_cast<const void*>(k_kernel_eval_tc_ws_split<false, NET>), sm);
-    k_kernel_eval_tc_ws_split<false, NET><<<grid, kWsThreads, sm, s>>>(V, p.n_x, p.bc_potential, p.Q, occ,
-                                                                       n_occ_dev, n_occ_host, base + n16,
-                                                                       base + 2 * n16, KB, c, VWh, flags, DenseA{});
-    return cudaGetLastError();
-  }
+  if (prec == WMC_FP16_SPLIT)
+    return launch_split<false, NET>(V, p.n_x, p.bc_potential, p.Q, occ, n_occ_dev, n_occ_host, max_rows, base + n16,
+                                    base + 2 * n16, KB, g.NT, c, VWh, flags, DenseA{}, s);
   return cudaErrorNotSupported;
 }
 

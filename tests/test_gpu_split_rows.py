@@ -1,0 +1,65 @@
+"""The hi/lo split contraction (3xTF32, FP16 split) at the edges of its tiles and
+of the window staging, against the FP64 oracle: row counts about a 128-row tile,
+windows that fill no column tile or K block, cell lists too scattered or out of
+order for one window, and rows over several potentials.  1e-6 normwise is the
+accuracy the split forms are stated for."""
+import numpy as np
+import pytest
+
+import oracle
+import wmc_inputs as wi
+from tests._util import normwise
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+TOL = 1e-6
+
+
+@pytest.fixture(scope="module")
+def wmc():
+    from paper_1806_00082_gb300 import build, wmc as w
+    build.build()
+    w.load()
+    return w
+
+
+def _cells(kind, n, n_x, rng):
+    if kind == "run":
+        return np.arange(n) + (n_x - n) // 2
+    if kind == "scattered":  # every tile spans more cells than one window holds
+        return np.sort(rng.choice(n_x, size=n, replace=False))
+    return rng.permutation(n_x)[:n]
+
+
+@pytest.mark.parametrize("form", ["tf32x3", "fp16_split"])
+@pytest.mark.parametrize("kind,n", [("run", 1), ("run", 129), ("run", 300), ("scattered", 127), ("scattered", 260),
+                                    ("shuffled", 128)])
+@pytest.mark.parametrize("Q", [4, 66, 258, 602, 1024])
+def test_split_rows(wmc, form, kind, n, Q):
+    wl = wi.DOUBLE_BARRIER_16384.replace(n_x=6001, Q=Q, n_M=Q, barriers=(wi.Barrier(0.25, 4e-9, 300e-9),))
+    V = wi.potential(wl)
+    cells = _cells(kind, n, wl.n_x, np.random.Generator(np.random.PCG64(n + Q))).astype(np.int32)
+    p = wmc.Params.of(wl)
+    ws = wmc.workspace(p)
+    wmc.init(p, ws)
+    got = wmc.kernel_eval(p, torch.from_numpy(V).cuda(), torch.from_numpy(cells).cuda(), ws,
+                          prec=wmc.PRECISIONS[form]).cpu().numpy()
+    pick = np.unique(np.r_[0, 1, n // 2, n - 2, n - 1, np.arange(0, n, 37)]).clip(0, n - 1)
+    ref = oracle.kernel_rows(oracle.params(wl.replace(n_M=Q)), V, cells[pick])[:, Q // 2:]
+    assert normwise(got[pick], ref) <= TOL
+    assert wmc.get_counters(p, ws)["flags"] == 0
+
+
+@pytest.mark.parametrize("n_pot,n_x", [(3, 50), (5, 333), (2, 128)])
+def test_split_rows_over_several_potentials(wmc, n_pot, n_x):
+    """Rows r over potential r / n_x: tiles that straddle two potentials or more."""
+    Q = 130
+    wl = wi.TANH_BARRIERS_4096.replace(n_x=n_x, Q=Q, n_M=Q)
+    V = np.random.Generator(np.random.PCG64(n_x)).uniform(-0.2, 0.2, (n_pot, n_x)).astype(np.float32)
+    p = wmc.Params.of(wl)
+    ws = wmc.workspace(p)
+    wmc.init(p, ws)
+    got = wmc.kernel_eval_rows(p, torch.from_numpy(V).cuda(), ws, wmc.TF32X3).cpu().numpy().reshape(n_pot, n_x, -1)
+    for b in range(n_pot):
+        ref = oracle.kernel_rows(oracle.params(wl), V[b], np.arange(n_x))[:, Q // 2:]
+        assert normwise(got[b], ref) <= TOL
