@@ -213,22 +213,6 @@ __device__ __forceinline__ float potential_at(const float* __restrict__ V, int n
   return __ldg(V + (l < 0 ? 0 : n_x - 1));
 }
 
-// Entry (row, kk) of the A operand: the N = 1 network's potential difference
-// V(i + m) - V(i - m), m = kk + 1 (zero beyond m = h - 1), or the N = 2
-// network's signed pair sum at offset u = kk: V(i+u) + V(i+u+1) if i + u is
-// even, else -(V(i-u-1) + V(i-u)) (zero beyond u = h - 1).  From a staged
-// window w (w[h + j] = V(i + j)) or from the potential itself.
-template <int NET>
-__device__ __forceinline__ float a_entry_window(const float* w, int h, int i, int kk) {
-  if (NET == 1) {
-    const int m = kk + 1;
-    return m <= h - 1 ? __fsub_rn(w[h + m], w[h - m]) : 0.f;
-  }
-  const int u = kk;
-  if (u > h - 1) return 0.f;
-  return ((i + u) & 1) == 0 ? __fadd_rn(w[h + u], w[h + u + 1]) : -__fadd_rn(w[h - u - 1], w[h - u]);
-}
-
 // Byte offset of element (row, k) of a 128 x 64 K-major operand block in the
 // 128-byte swizzled layout (row r at 128 r, chunk k / 8 stored at chunk
 // (k / 8) ^ (r % 8)); blocks of consecutive rows concatenate.
@@ -471,13 +455,12 @@ __global__ __launch_bounds__(128, 1) void k_kernel_eval_tc(const float* __restri
 }
 
 // ---------------------------------------------------------------- warp-specialised forms
-// Roles of the warp-specialised kernels below (576 threads): warps 0-15 build
+// Roles of the form below (608 threads): warps 0-15 build
 // the A operand and then run the epilogue, warp 16 has one thread issue the
 // MMAs, warp 17 one thread stream the B operand images.  The epilogue warp w
 // reads TMEM lane quadrant w % 4 and transposes each 32 x 16 piece through
 // shared memory, so that global stores are whole 64-byte row segments.
 constexpr int kWsBuilders = 512;
-constexpr int kWsThreads = kWsBuilders + 64;
 
 constexpr int kWsStageFloats = 32 * 16;  // epilogue staging per warp: 32 rows x 16 columns
 
@@ -508,6 +491,42 @@ __device__ __forceinline__ uint32_t pack2(float a, float b) {
   }
 }
 
+// Cells the rows of a 128-row tile may span for their potential window (span
+// + 2 h values) to be staged in shared memory; beyond, every term is read from
+// the potential itself.  Scattered lists of every second cell still fit.
+constexpr int kWindowSpan = 640;
+
+// N consecutive terms kk = k0 .. of the A operand of one row.  w[m] = V(cell + m).
+template <int NET, int N>
+__device__ __forceinline__ void a_run_window(const float* w, int h, int cell, int k0, float (&dv)[N]) {
+  if (NET == 1) {
+    if (k0 + N <= h - 1) {
+#pragma unroll
+      for (int e = 0; e < N; ++e) dv[e] = __fsub_rn(w[k0 + e + 1], w[-(k0 + e + 1)]);
+    } else {
+#pragma unroll
+      for (int e = 0; e < N; ++e) {
+        const int m = k0 + e + 1;
+        dv[e] = 0.f;
+        if (m <= h - 1) dv[e] = __fsub_rn(w[m], w[-m]);
+      }
+    }
+  } else {
+    // a pair to the right of the cell where i + u is even, else its mirror to the left
+#pragma unroll
+    for (int e = 0; e < N; ++e) {
+      const int u = k0 + e;
+      dv[e] = 0.f;
+      if (u <= h - 1) {
+        const bool right = ((cell + u) & 1) == 0;
+        const int at = right ? u : -u - 1;
+        const float s = __fadd_rn(w[at], w[at + 1]);
+        dv[e] = right ? s : -s;
+      }
+    }
+  }
+}
+
 // ---------------------------------------------------------------- A in tensor memory
 // BF16 / FP16, K <= 512: one CTA per 128 rows and a run of 128-column tiles.
 // The whole A operand of the row tile lives in tensor memory (up to 8 blocks
@@ -523,19 +542,24 @@ __device__ __forceinline__ uint32_t pack2(float a, float b) {
 // and a drained accumulator buffer, commits each stage and each tile.  Every
 // wait is bounded; on a timeout an abort flag makes all roles drain to the
 // final barrier, after which TMEM is freed.
-constexpr int kTaStages = 11;
+constexpr int kTaStages = 5;        // stages of two 64-K blocks
+constexpr int kTaThreads = kWsBuilders + 96;
+constexpr uint32_t kTaStageBytes = 2 * kTileBytes;
 constexpr int kTaMaxKB = 8;
 constexpr uint32_t kTaAccCol = 256;
 
+__host__ __device__ constexpr size_t ta_window_floats(int h) {
+  return (size_t)kWindowSpan + 2 * (size_t)h + 4 > (size_t)(kWsBuilders / 32) * kWsStageFloats
+             ? (size_t)kWindowSpan + 2 * (size_t)h + 4
+             : (size_t)(kWsBuilders / 32) * kWsStageFloats;
+}
+
 __host__ __device__ constexpr size_t ta_smem_bytes(int h) {
-  return kSmemAlignPad + (size_t)kTaStages * kTileBytes +
-         sizeof(float) * (size_t)((TM + 2 * h) > (kWsBuilders / 32) * kWsStageFloats
-                                      ? (TM + 2 * h)
-                                      : (kWsBuilders / 32) * kWsStageFloats);
+  return kSmemAlignPad + (size_t)kTaStages * kTaStageBytes + sizeof(float) * ta_window_floats(h);
 }
 
 template <int PREC, int NET>
-__global__ __launch_bounds__(kWsThreads, 1) void k_kernel_eval_tc_ta(const float* __restrict__ V, int n_x, int bc,
+__global__ __launch_bounds__(kTaThreads, 1) void k_kernel_eval_tc_ta(const float* __restrict__ V, int n_x, int bc,
                                                                      int Q, const int* __restrict__ occ,
                                                                      const int* __restrict__ n_occ_dev, int n_occ_host,
                                                                      const uint16_t* __restrict__ img_b, int KB,
@@ -547,12 +571,13 @@ __global__ __launch_bounds__(kWsThreads, 1) void k_kernel_eval_tc_ta(const float
   constexpr uint32_t n_cols = 512;
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t* smem = align_smem(smem_raw);
-  uint8_t* sB = smem;                                                     // STG stages of 128 x 64
-  float* sV = reinterpret_cast<float*>(sB + (size_t)STG * kTileBytes);  // window, then epilogue staging
+  uint8_t* sB = smem;                                                     // STG stages of two 128 x 64 blocks
+  float* sV = reinterpret_cast<float*>(sB + (size_t)STG * kTaStageBytes);  // window, then epilogue staging
   __shared__ __align__(8) uint64_t a_ready[kTaMaxKB];
   __shared__ __align__(8) uint64_t b_full[kTaStages], b_empty[kTaStages];
   __shared__ __align__(8) uint64_t acc_full[2], acc_empty[2];
-  __shared__ __align__(8) uint64_t drain;
+  __shared__ __align__(8) uint64_t drain[2];
+  __shared__ int s_min[kWsBuilders / 32], s_max[kWsBuilders / 32];
   __shared__ uint32_t tmem_slot;
   __shared__ volatile int s_abort;
 
@@ -564,7 +589,7 @@ __global__ __launch_bounds__(kWsThreads, 1) void k_kernel_eval_tc_ta(const float
   // this CTA's 128-column tiles: [nt_begin, nt_begin + n_my)
   const int nt_begin = (int)(((long long)blockIdx.y * NT) / n_split);
   const int n_my = (int)(((long long)(blockIdx.y + 1) * NT) / n_split) - nt_begin;
-  const int n_tiles = n_my * KB;
+  const int KP = (KB + 1) / 2, n_tiles = n_my * KP;  // stages of a column tile, and of all
 
   if (warp == 0) tmem_alloc(&tmem_slot, n_cols);
   if (tid == 0) {
@@ -577,7 +602,7 @@ __global__ __launch_bounds__(kWsThreads, 1) void k_kernel_eval_tc_ta(const float
       mbar_init(&acc_full[q], 1);
       mbar_init(&acc_empty[q], kWsBuilders / 32);  // one arrival per epilogue warp
     }
-    mbar_init(&drain, 1);
+    for (int q = 0; q < 2; ++q) mbar_init(&drain[q], 1);
     fence_mbar_init();
     s_abort = 0;
   }
@@ -597,21 +622,22 @@ __global__ __launch_bounds__(kWsThreads, 1) void k_kernel_eval_tc_ta(const float
           s_abort = 1;
           break;
         }
-        const int nt = nt_begin + t / KB, kb = t % KB;
-        mbar_expect_tx(&b_full[st], kTileBytes);
-        bulk_g2s(sB + (size_t)st * kTileBytes, img_b + ((size_t)nt * KB + kb) * (kTileBytes / 2), kTileBytes,
-                 &b_full[st]);
+        const int nt = nt_begin + t / KP, kb = 2 * (t % KP);
+        const uint32_t bytes = kb + 1 < KB ? kTaStageBytes : kTileBytes;
+        mbar_expect_tx(&b_full[st], bytes);
+        bulk_g2s(sB + (size_t)st * kTaStageBytes, img_b + ((size_t)nt * KB + kb) * (kTileBytes / 2), bytes, &b_full[st]);
         issued = t + 1;
       }
       if (s_abort)  // let the copies still in flight land before the CTA exits (bounded)
         for (int t = max(0, issued - STG); t < issued; ++t)
           (void)mbar_wait(&b_full[t % STG], (uint32_t)((t / STG) & 1));
     }
-  } else if (warp == kWsBuilders / 32) {
-    // ---- MMA issuer
+  } else if (warp == kWsBuilders / 32 || warp == kWsBuilders / 32 + 2) {
+    // ---- MMA issuers: one thread the even column tiles (accumulator 0), one the
+    // odd ones, so that one's waits and commits pass behind the other's MMAs
+    const int buf = warp == kWsBuilders / 32 ? 0 : 1;
     if (lane == 0) {
-      for (int j = 0; j < n_my && !s_abort; ++j) {
-        const int buf = j & 1;
+      for (int j = buf; j < n_my && !s_abort; j += 2) {
         if (j >= 2 && !mbar_wait(&acc_empty[buf], (uint32_t)(((j - 2) >> 1) & 1))) {
           atomicOr(flags, WMC_FLAG_TIMEOUT);
           s_abort = 1;
@@ -620,93 +646,83 @@ __global__ __launch_bounds__(kWsThreads, 1) void k_kernel_eval_tc_ta(const float
         tc_fence_after();
         const uint32_t acc = tmem + kTaAccCol + (uint32_t)(buf * TN);
         for (int kb = 0; kb < KB; ++kb) {
-          const int t = j * KB + kb, st = t % STG;
-          if ((j == 0 && !mbar_wait(&a_ready[kb], 0u)) ||
-              !mbar_wait(&b_full[st], (uint32_t)((t / STG) & 1))) {
+          const int t = j * KP + kb / 2, st = t % STG;
+          if ((j < 2 && !mbar_wait(&a_ready[kb], 0u)) ||
+              ((kb & 1) == 0 && !mbar_wait(&b_full[st], (uint32_t)((t / STG) & 1)))) {
             atomicOr(flags, WMC_FLAG_TIMEOUT);
             s_abort = 1;
             break;
           }
           tc_fence_after();
-          const uint32_t b_base = smem_u32(sB + (size_t)st * kTileBytes);
+          const uint32_t b_base = smem_u32(sB + (size_t)st * kTaStageBytes + (kb & 1) * kTileBytes);
 #pragma unroll
           for (int s4 = 0; s4 < TK / 16; ++s4)
             mma_f16_ta(acc, tmem + (uint32_t)(kb * (TK / 2) + s4 * 8), smem_desc(b_base + s4 * kKStepBytes), idesc,
                        (kb == 0 && s4 == 0) ? 0u : 1u);
-          mma_commit(&b_empty[st]);
+          if (((kb & 1) || kb + 1 == KB) && t + STG < n_tiles) mma_commit(&b_empty[st]);  // (a stage filled again)
         }
         if (s_abort) break;
         mma_commit(&acc_full[buf]);
       }
       if (s_abort) {  // drain the MMAs already issued before TMEM is freed (bounded)
-        mma_commit(&drain);
-        (void)mbar_wait(&drain, 0u);
+        mma_commit(&drain[buf]);
+        (void)mbar_wait(&drain[buf], 0u);
       }
     }
   } else {
     // ---- A builders (warps 0-15), then the epilogue
-    // contiguity of the tile's rows (row row0 + tid % 128, each checked by four threads)
-    const int rc = tid & (TM - 1);
-    const int rowc = row0 + rc;
-    const bool validc = rowc < n_rows;
-    const int cellc = validc ? (occ ? __ldg(occ + rowc) : rowc % n_x) : 0;
-    const int potc = (occ || !validc) ? 0 : rowc / n_x;
-    const int cell0 = occ ? __ldg(occ + row0) : row0 % n_x;
-    const int pot0 = occ ? 0 : row0 / n_x;
-    const bool contig = builders_and(validc && cellc == cell0 + rc && potc == pot0);
-    if (contig) {
+    // this thread's row of the tile = its TMEM lane (rows past the end repeat the last)
+    const int quad = warp & 3, kp = warp >> 2;
+    const int row = min(row0 + 32 * quad + lane, n_rows - 1);
+    const int cell = occ ? __ldg(occ + row) : row % n_x;
+    const int pot0 = occ ? 0 : row0 / n_x, pot_i = occ ? 0 : row / n_x;
+    // the cells of the tile's rows, and whether their window can be staged
+    int lo = __reduce_min_sync(0xffffffffu, cell), hi = __reduce_max_sync(0xffffffffu, cell);
+    if (lane == 0) {
+      s_min[warp] = lo;
+      s_max[warp] = hi;
+    }
+    const bool one_pot = builders_and(pot_i == pot0);
+    lo = min(min(s_min[0], s_min[1]), min(s_min[2], s_min[3]));
+    hi = max(max(s_max[0], s_max[1]), max(s_max[2], s_max[3]));
+    const bool window = one_pot && hi - lo < kWindowSpan;
+    if (window) {
       const float* V0 = V + (size_t)pot0 * n_x;
+      const int n = hi - lo + 1 + 2 * h;
       constexpr int kU = 4;  // loads issued together
-      for (int q0 = tid; q0 < TM + 2 * h; q0 += kU * kWsBuilders) {
+      for (int q0 = tid; q0 < n; q0 += kU * kWsBuilders) {
         float v[kU];
 #pragma unroll
         for (int u = 0; u < kU; ++u) {
           const int q = q0 + u * kWsBuilders;
-          v[u] = q < TM + 2 * h ? potential_at(V0, n_x, bc, (long long)cell0 - h + q) : 0.f;
+          v[u] = q < n ? potential_at(V0, n_x, bc, (long long)lo - h + q) : 0.f;
         }
 #pragma unroll
         for (int u = 0; u < kU; ++u)
-          if (q0 + u * kWsBuilders < TM + 2 * h) sV[q0 + u * kWsBuilders] = v[u];
+          if (q0 + u * kWsBuilders < n) sV[q0 + u * kWsBuilders] = v[u];
       }
       builders_sync();
     }
-    // this thread's row of the tile = its TMEM lane
-    const int quad = warp & 3, kp = warp >> 2;
-    const int rr = 32 * quad + lane;
-    const int row = row0 + rr;
-    const bool valid = row < n_rows;
-    const int cell = (contig || !valid) ? 0 : (occ ? __ldg(occ + row) : row % n_x);
-    const float* Vr = V + (size_t)((occ || !valid) ? 0 : row / n_x) * n_x;
+    const float* w = sV + h + (cell - lo);
+    const float* Vr = V + (size_t)pot_i * n_x;
     const uint32_t lane_base = (uint32_t)(quad * 32) << 16;
 #pragma unroll 1
     for (int kb = kp; kb < KB; kb += 4) {
-      uint32_t wv[32];
-      const int k0 = kb * TK;  // K index of the block's first value
-      if (NET == 1 && contig && k0 + TK <= h - 1) {
-        // m = k0 + 1 .. k0 + 64, all inside the sum: wp[m] = V(i + m), wp[-m] = V(i - m)
-        const float* wp = sV + rr + h;
+#pragma unroll 1
+      for (int hf = 0; hf < 2; ++hf) {  // 32 K values, 16 columns
+        float dv[32];
+        const int k0 = kb * TK + 32 * hf;
+        if (window) {
+          a_run_window<NET, 32>(w, h, cell, k0, dv);
+        } else {
 #pragma unroll
-        for (int e = 0; e < 32; ++e) {
-          const int m = k0 + 2 * e + 1;
-          wv[e] = pack2<PREC>(__fsub_rn(wp[m], wp[-m]), __fsub_rn(wp[m + 1], wp[-m - 1]));
+          for (int e = 0; e < 32; ++e) dv[e] = a_term<NET>(Vr, n_x, bc, h, cell, k0 + e);
         }
-      } else {
+        uint32_t wv[16];
 #pragma unroll
-        for (int e = 0; e < 32; ++e) {
-          const int kk = k0 + 2 * e;
-          float a = 0.f, b = 0.f;
-          if (contig) {
-            a = a_entry_window<NET>(sV + rr, h, cell0 + rr, kk);
-            b = a_entry_window<NET>(sV + rr, h, cell0 + rr, kk + 1);
-          } else if (valid) {
-            a = a_term<NET>(Vr, n_x, bc, h, cell, kk);
-            b = a_term<NET>(Vr, n_x, bc, h, cell, kk + 1);
-          }
-          wv[e] = pack2<PREC>(a, b);
-        }
+        for (int e = 0; e < 16; ++e) wv[e] = pack2<PREC>(dv[2 * e], dv[2 * e + 1]);
+        tmem_st16(tmem + lane_base + (uint32_t)(kb * (TK / 2) + 16 * hf), wv);
       }
-      tmem_st16(tmem + lane_base + (uint32_t)(kb * (TK / 2)), wv);
-      tmem_st16(tmem + lane_base + (uint32_t)(kb * (TK / 2) + 16), wv + 16);
       tmem_wait_st();
       tc_fence_before();
       __syncwarp();
@@ -821,7 +837,6 @@ constexpr int kSpStages = 5;
 // kSpStages blocks, so that no waiter meets a barrier two phases on.
 constexpr int kSpRing = 8;
 static_assert(kSpRing > kSpStages, "a barrier comes round only after every waiter has seen it");
-constexpr int kSpSpan = 640;                 // cells a tile's rows may span for its window to be staged
 constexpr int kSpBuilders = 256, kSpThreads = 19 * 32;
 constexpr uint32_t kSpAccX = 2 * TN, kSpA = 3 * TN;  // TMEM columns: main 0, main 1, cross, A ring
 
@@ -843,7 +858,7 @@ __device__ __forceinline__ int grid_count_tc(int r, int Q, int a, int b, int r0)
   return a + (off < b ? 1 : 0);
 }
 
-__host__ __device__ constexpr size_t split_window_floats(int h) { return (size_t)kSpSpan + 2 * (size_t)h + 4; }
+__host__ __device__ constexpr size_t split_window_floats(int h) { return (size_t)kWindowSpan + 2 * (size_t)h + 4; }
 
 __host__ __device__ constexpr size_t split_smem_bytes(int h) {
   return kSmemAlignPad + (size_t)kSpStages * 2 * kTileBytes + sizeof(float) * 8 * kWsStageFloats +
@@ -886,37 +901,6 @@ struct SplitRows {
   int cell;    // this thread's row: cell and potential (clamped to a valid row)
   int pot;
 };
-
-// N consecutive terms kk = k0 .. of the A operand of one row.  w[m] = V(cell + m).
-template <int NET, int N>
-__device__ __forceinline__ void a_run_window(const float* w, int h, int cell, int k0, float (&dv)[N]) {
-  if (NET == 1) {
-    if (k0 + N <= h - 1) {
-#pragma unroll
-      for (int e = 0; e < N; ++e) dv[e] = __fsub_rn(w[k0 + e + 1], w[-(k0 + e + 1)]);
-    } else {
-#pragma unroll
-      for (int e = 0; e < N; ++e) {
-        const int m = k0 + e + 1;
-        dv[e] = 0.f;
-        if (m <= h - 1) dv[e] = __fsub_rn(w[m], w[-m]);
-      }
-    }
-  } else {
-    // a pair to the right of the cell where i + u is even, else its mirror to the left
-#pragma unroll
-    for (int e = 0; e < N; ++e) {
-      const int u = k0 + e;
-      dv[e] = 0.f;
-      if (u <= h - 1) {
-        const bool right = ((cell + u) & 1) == 0;
-        const int at = right ? u : -u - 1;
-        const float s = __fadd_rn(w[at], w[at + 1]);
-        dv[e] = right ? s : -s;
-      }
-    }
-  }
-}
 
 template <bool TF32, int NET>
 __global__ __launch_bounds__(kSpThreads, 1) void k_rows_split(
@@ -1087,7 +1071,7 @@ __global__ __launch_bounds__(kSpThreads, 1) void k_rows_split(
           lo = min(min(s_min[0], s_min[1]), min(s_min[2], s_min[3]));
           hi = max(max(s_max[0], s_max[1]), max(s_max[2], s_max[3]));
           sp_builders_sync();
-          r.window = hi - lo < kSpSpan;
+          r.window = hi - lo < kWindowSpan;
         } else {
           lo = (rt * TM) % n_x;
           const int last = min(rt * TM + TM, n_rows) - 1;
@@ -1489,11 +1473,11 @@ static cudaError_t launch_tc_net(const wmc_params& p, int prec, const float* V, 
     if (e != cudaSuccess) return e;
     const dim3 grid(row_tiles, n_split);
     if (prec == WMC_BF16)
-      k_kernel_eval_tc_ta<WMC_BF16, NET><<<grid, kWsThreads, sm, s>>>(V, p.n_x, p.bc_potential, p.Q, occ, n_occ_dev,
+      k_kernel_eval_tc_ta<WMC_BF16, NET><<<grid, kTaThreads, sm, s>>>(V, p.n_x, p.bc_potential, p.Q, occ, n_occ_dev,
                                                                       n_occ_host, img, KB, g.NT, n_split, c, VWh,
                                                                       flags);
     else
-      k_kernel_eval_tc_ta<WMC_FP16, NET><<<grid, kWsThreads, sm, s>>>(V, p.n_x, p.bc_potential, p.Q, occ, n_occ_dev,
+      k_kernel_eval_tc_ta<WMC_FP16, NET><<<grid, kTaThreads, sm, s>>>(V, p.n_x, p.bc_potential, p.Q, occ, n_occ_dev,
                                                                       n_occ_host, img, KB, g.NT, n_split, c, VWh,
                                                                       flags);
     return cudaGetLastError();

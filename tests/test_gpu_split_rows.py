@@ -50,6 +50,49 @@ def test_split_rows(wmc, form, kind, n, Q):
     assert wmc.get_counters(p, ws)["flags"] == 0
 
 
+def _operands(V, cells, Q, net):
+    """FP32 window terms [n, h] and matrix [h, h] of the N = 1 or N = 2 network, V = 0 outside."""
+    h = Q // 2
+    Vp = np.pad(V, h + 1).astype(np.float32)
+    u = np.arange(h)[None, :]
+    i = cells[:, None].astype(np.int64)
+    at = lambda l: Vp[l + h + 1]
+    r = np.arange(h)
+    if net == 1:
+        A = at(i + u + 1) - at(i - u - 1)
+        A[:, h - 1] = 0
+        S = np.sin(2 * np.pi * (((r[:, None] + 1) * r[None, :]) % Q) / Q)
+    else:
+        A = np.where((i + u) % 2 == 0, at(i + u) + at(i + u + 1), -(at(i - u - 1) + at(i - u)))
+        S = np.cos(np.pi * r / Q) * np.sin(np.pi * (((2 * r[:, None] + 1) * r[None, :]) % (2 * Q)) / Q)
+    return A.astype(np.float32), S.astype(np.float32)
+
+
+@pytest.mark.parametrize("form", ["bf16", "fp16"])
+@pytest.mark.parametrize("kind,n", [("run", 1), ("run", 300), ("scattered", 260), ("shuffled", 128)])
+@pytest.mark.parametrize("Q", [4, 258, 602, 1024])
+def test_one_pass_forms_and_n2(wmc, form, kind, n, Q):
+    """BF16 and FP16 rows of both networks against the FP64 product of the rounded
+    operands: what is left is the FP32 accumulation, one truncation of the running
+    sum per MMA of 16 terms and of each product's alignment, at most
+    (K / 16 + 2) 2^-22 of the sum of the terms' magnitudes."""
+    wl = wi.DOUBLE_BARRIER_16384.replace(n_x=6001, Q=Q, n_M=Q, barriers=(wi.Barrier(0.25, 4e-9, 300e-9),))
+    V = wi.potential(wl)
+    cells = _cells(kind, n, wl.n_x, np.random.Generator(np.random.PCG64(n + Q))).astype(np.int32)
+    p = wmc.Params.of(wl)
+    ws = wmc.workspace(p)
+    wmc.init(p, ws)
+    Vd, cd = torch.from_numpy(V).cuda(), torch.from_numpy(cells).cuda()
+    c = 2.0 / (6.582119569e-16 * Q)
+    for net, f in ((1, wmc.kernel_eval), (2, wmc.kernel_eval_n2)):
+        got = f(p, Vd, cd, ws, prec=wmc.PRECISIONS[form]).cpu().numpy().astype(np.float64)
+        A, S = (torch.from_numpy(x).to(torch.bfloat16 if form == "bf16" else torch.float16).double().numpy()
+                for x in _operands(V, cells, Q, net))
+        bound = c * ((Q // 32 + 2) * 2.0 ** -22 * (np.abs(A) @ np.abs(S))) + 1e-6 * np.abs(A @ S) * c + 1e-30
+        assert np.all(np.abs(got + c * (A @ S)) <= bound)
+    assert wmc.get_counters(p, ws)["flags"] == 0
+
+
 @pytest.mark.parametrize("n_pot,n_x", [(3, 50), (5, 333), (2, 128)])
 def test_split_rows_over_several_potentials(wmc, n_pot, n_x):
     """Rows r over potential r / n_x: tiles that straddle two potentials or more."""
