@@ -82,6 +82,22 @@ __device__ __forceinline__ long long quantise(float x, int s) {
   return (long long)(q + ((rem > half || (rem == half && (q & 1u))) ? 1u : 0u));
 }
 
+// The same with the scale as a factor sf = 2^s (scale_factor; 0 where it is no
+// normal FP32 number): from 2^23 on the product is an integer, the mantissa
+// shifted; below, it is exact (a subnormal one is under half a unit either way)
+// and a 32-bit conversion rounds it to nearest even.
+__device__ __forceinline__ float scale_factor(int s) {
+  return s >= -126 && s <= 126 ? __uint_as_float((uint32_t)(s + 127) << 23) : 0.f;
+}
+__device__ __forceinline__ long long quantise(float x, int s, float sf) {
+  if (sf == 0.f) return quantise(x, s);
+  const uint32_t b = __float_as_uint(x);
+  const int sh = (int)(b >> 23) - 150 + s;  // (negative for a subnormal x)
+  const unsigned long long big = (unsigned long long)((b & 0x7fffffu) | 0x800000u) << (sh & 63);
+  const uint32_t small = __float2uint_rn(__fmul_rn(x, sf));
+  return (long long)(sh >= 0 ? big : (unsigned long long)small);
+}
+
 __device__ __forceinline__ int floor_log2_pos(float x) {  // x > 0
   const uint32_t b = __float_as_uint(x);
   const uint32_t E = b >> 23;
@@ -146,9 +162,10 @@ __device__ __forceinline__ void warp_row_cdf(XRes xres, int Q, int r0, int n_M, 
     return;
   }
   const int s = 61 - log2_nM - floor_log2_pos(__uint_as_float(mx));
+  const float sf = scale_factor(s);
   long long local = 0;
   for (int k = k0, rr = rr0; k < k1; ++k) {
-    local += quantise(xres(rr), s);
+    local += quantise(xres(rr), s, sf);
     if (++rr == Q) rr = 0;
   }
   long long incl = local;
@@ -162,7 +179,7 @@ __device__ __forceinline__ void warp_row_cdf(XRes xres, int Q, int r0, int n_M, 
   if (out) {
     long long run = incl - local;
     for (int k = k0, rr = rr0; k < k1; ++k) {
-      run += quantise(xres(rr), s);
+      run += quantise(xres(rr), s, sf);
       out[k] = run;
       if (++rr == Q) rr = 0;
     }
@@ -236,6 +253,7 @@ __device__ __forceinline__ int sample_coarse_row(const float* __restrict__ v, co
   const int k0 = min(blk * E, n_M), k1 = min(k0 + E, n_M);
   const int h = Q / 2;
   int rr = (r0 + k0) % Q;
+  const float sf = scale_factor(s);
   for (int kb = k0; kb < k1; kb += 8) {
     float x[8];
 #pragma unroll
@@ -248,7 +266,7 @@ __device__ __forceinline__ int sample_coarse_row(const float* __restrict__ v, co
     }
 #pragma unroll
     for (int e = 0; e < 8; ++e) {
-      run += quantise(x[e], s);
+      run += quantise(x[e], s, sf);
       if (kb + e < k1 && run > target) return kb + e;
     }
     rr += 8;
