@@ -102,6 +102,8 @@ _lock = threading.Lock()
 def load(path: str | None = None):
     """Loads libwmc.so (built by ``paper_1806_00082_gb300.build``); raises if absent."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is not None:
             return _lib
@@ -158,18 +160,26 @@ def load(path: str | None = None):
         return lib
 
 
-def _stream():
-    return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+# The current device's current stream as an integer handle.  The raw accessors
+# build no Stream object (a call's marshalling takes about as long as a small
+# kernel); the public call is used where they are missing.
+if hasattr(torch._C, "_cuda_getCurrentRawStream") and hasattr(torch._C, "_cuda_getDevice"):
+    def _stream():
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+else:
+    def _stream():
+        return torch.cuda.current_stream().cuda_stream
 
 
 def _ptr(t):
+    """Address of a device tensor (the argtypes turn it into a pointer)."""
     if t is None:
         return None
     if not t.is_cuda:
         raise ValueError("libwmc device arguments must be CUDA tensors")
     if not t.is_contiguous():
         raise ValueError("libwmc device arguments must be contiguous")
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
 def _check(name: str, code: int):
