@@ -860,9 +860,15 @@ __device__ __forceinline__ int grid_count_tc(int r, int Q, int a, int b, int r0)
 
 __host__ __device__ constexpr size_t split_window_floats(int h) { return (size_t)kWindowSpan + 2 * (size_t)h + 4; }
 
-__host__ __device__ constexpr size_t split_smem_bytes(int h) {
-  return kSmemAlignPad + (size_t)kSpStages * 2 * kTileBytes + sizeof(float) * 8 * kWsStageFloats +
-         sizeof(float) * 2 * split_window_floats(h);
+// NET = 3: the rows of gVW and VWh of a K block (128 x 32) pass through
+// kDenseStages buffers of shared memory each, padded to 36 floats a row; fewer
+// B stages make room.
+constexpr int kDenseStages = 3, kDensePitch = 36;
+__host__ __device__ constexpr int split_stages(int net) { return net == 3 ? 3 : kSpStages; }
+
+__host__ __device__ constexpr size_t split_smem_bytes(int h, int net) {
+  return kSmemAlignPad + (size_t)split_stages(net) * 2 * kTileBytes + sizeof(float) * 8 * kWsStageFloats +
+         sizeof(float) * (net == 3 ? (size_t)2 * kDenseStages * TM * kDensePitch : 2 * split_window_floats(h));
 }
 
 __device__ __forceinline__ void mma_tf32_ta(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc, uint32_t idesc,
@@ -883,6 +889,10 @@ __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
 // cp_async_wait.
 __device__ __forceinline__ void cp_async4(float* dst, const float* src, bool in) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(in ? 4 : 0)
+               : "memory");
+}
+__device__ __forceinline__ void cp_async16(float* dst, const float* src, bool in) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(in ? 16 : 0)
                : "memory");
 }
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
@@ -912,13 +922,14 @@ __global__ __launch_bounds__(kSpThreads, 1) void k_rows_split(
   constexpr uint32_t idesc = idesc_f16(TF32 ? 2u : 0u);
   constexpr int KBLK = TF32 ? 32 : TK;   // K values per operand block
   constexpr int EPT = KBLK / 2;          // values a builder thread makes of one block
+  constexpr int STG = split_stages(NET);
   constexpr float kLoScale = TF32 ? 1.f : 0x1p-11f;
   const uint8_t* img_hi = static_cast<const uint8_t*>(img_hi_v);
   const uint8_t* img_lo = static_cast<const uint8_t*>(img_lo_v);
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t* sB = align_smem(smem_raw);                                             // stages of (B_hi, B_lo)
-  float* s_stage = reinterpret_cast<float*>(sB + (size_t)kSpStages * 2 * kTileBytes);  // output staging, per drain warp
-  float* s_win = s_stage + 8 * kWsStageFloats;                                    // two windows
+  float* s_stage = reinterpret_cast<float*>(sB + (size_t)STG * 2 * kTileBytes);  // output staging, per drain warp
+  float* s_win = s_stage + 8 * kWsStageFloats;  // two windows (NET = 3: the rows' buffers)
   // of K block g, index g % kSpRing: its operands are there; its MMAs are complete
   __shared__ __align__(8) uint64_t full[kSpRing], done[kSpRing];
   __shared__ __align__(8) uint64_t acc_empty[2], x_empty, drain[2];
@@ -973,8 +984,8 @@ __global__ __launch_bounds__(kSpThreads, 1) void k_rows_split(
     if (lane == 0) {
       int issued = 0;
       for (int g = 0; g < n_blocks && !s_abort; ++g) {
-        const int st = g % kSpStages;
-        if (g >= kSpStages && !wait_done(g - kSpStages)) {
+        const int st = g % STG;
+        if (g >= STG && !wait_done(g - STG)) {
           give_up();
           break;
         }
@@ -988,7 +999,7 @@ __global__ __launch_bounds__(kSpThreads, 1) void k_rows_split(
       }
       if (s_abort)  // let the copies still in flight land before the CTA exits (bounded: the builders,
                     // who give up too, may leave their arrivals out)
-        for (int g = max(0, issued - kSpStages); g < issued; ++g) (void)wait_full(g);
+        for (int g = max(0, issued - STG); g < issued; ++g) (void)wait_full(g);
     }
   } else if (warp == 16 || warp == 18) {
     // ---- MMA issuers: one thread the main products, one the cross terms.  An
@@ -1007,7 +1018,7 @@ __global__ __launch_bounds__(kSpThreads, 1) void k_rows_split(
         }
         tc_fence_after();
         const uint32_t ah = tmem + kSpA + (uint32_t)(ab * 64), al = ah + 32u;
-        const uint32_t bh = smem_u32(sB + (size_t)(g % kSpStages) * 2 * kTileBytes), bl = bh + kTileBytes;
+        const uint32_t bh = smem_u32(sB + (size_t)(g % STG) * 2 * kTileBytes), bl = bh + kTileBytes;
         if (is_main) {
           const uint32_t acc_m = tmem + (uint32_t)(ab * TN);
 #pragma unroll
@@ -1096,35 +1107,29 @@ __global__ __launch_bounds__(kSpThreads, 1) void k_rows_split(
     cp_async_wait();
     sp_builders_sync();
     int wb = 0;
-    // NET = 3: the next block's entries of gVW and VWh, asked for ahead
-    constexpr int RAW = NET == 3 ? EPT : 1;
-    float graw[RAW], vraw[RAW], gg = 0.f;
-    auto load_dense = [&](int g) {
-      const int row = (int)((t0 + g / KB) / NT) * TM + rr, k0 = (g % KB) * KBLK + half * EPT;
-      const bool on = g < n_blocks && row < n_rows;
-      gg = on && dense.g_gamma ? __ldg(dense.g_gamma + row) : 0.f;
-      const size_t o = (size_t)row * h + k0;
-      if ((h & 3) == 0) {
+    // NET = 3: the rows of gVW and VWh come by 16-byte copies, eight threads a
+    // row (128 bytes), kDenseStages - 1 blocks ahead: 32 rows read by one warp's
+    // own loads, 16 bytes of each, took 192 us for 262144 rows of 128 columns.
+    const bool dense_vec = NET == 3 && (h & 3) == 0 &&
+                           ((reinterpret_cast<uintptr_t>(dense.gVW) | reinterpret_cast<uintptr_t>(dense.VWh)) & 15) == 0;
+    constexpr size_t kDenseBuf = (size_t)TM * kDensePitch;
+    auto copy_dense = [&](int g) {
+      if (g < n_blocks) {
+        const int rt = (int)((t0 + g / KB) / NT), k0 = (g % KB) * KBLK;
+        float* dst = s_win + (size_t)(g % kDenseStages) * 2 * kDenseBuf;
 #pragma unroll
-        for (int q = 0; q < RAW / 4; ++q) {
-          const bool in = on && k0 + 4 * q < h;
-          const float4 a = in && dense.gVW ? __ldg(reinterpret_cast<const float4*>(dense.gVW + o + 4 * q))
-                                           : make_float4(0.f, 0.f, 0.f, 0.f);
-          const float4 b = in && dense.g_gamma ? __ldg(reinterpret_cast<const float4*>(dense.VWh + o + 4 * q))
-                                               : make_float4(0.f, 0.f, 0.f, 0.f);
-          graw[4 * q] = a.x, graw[4 * q + 1] = a.y, graw[4 * q + 2] = a.z, graw[4 * q + 3] = a.w;
-          vraw[4 * q] = b.x, vraw[4 * q + 1] = b.y, vraw[4 * q + 2] = b.z, vraw[4 * q + 3] = b.w;
-        }
-      } else {
-#pragma unroll
-        for (int e = 0; e < RAW; ++e) {
-          const bool in = on && k0 + e < h;
-          graw[e] = in && dense.gVW ? __ldg(dense.gVW + o + e) : 0.f;
-          vraw[e] = in && dense.g_gamma ? __ldg(dense.VWh + o + e) : 0.f;
+        for (int q = tid; q < TM * 8; q += kSpBuilders) {
+          const int r = q >> 3, col = 4 * (q & 7), row = rt * TM + r;
+          const bool in = row < n_rows && k0 + col < h;
+          const size_t o = in ? (size_t)row * h + k0 + col : 0;
+          if (dense.gVW) cp_async16(dst + r * kDensePitch + col, dense.gVW + o, in);
+          if (dense.g_gamma) cp_async16(dst + kDenseBuf + r * kDensePitch + col, dense.VWh + o, in);
         }
       }
+      asm volatile("cp.async.commit_group;" ::: "memory");
     };
-    if (NET == 3) load_dense(0);
+    if (dense_vec)
+      for (int g = 0; g < kDenseStages - 1; ++g) copy_dense(g);
     for (int tile = 0; tile < n_my; ++tile) {
       const int rt = (int)((t0 + tile) / NT);
       // the next tile's window on its way while this tile is built
@@ -1139,18 +1144,44 @@ __global__ __launch_bounds__(kSpThreads, 1) void k_rows_split(
         const int k0 = kb * KBLK + half * EPT;
         float dv[EPT];
         if (NET == 3) {
+          const int row = rt * TM + rr;
+          const bool on = row < n_rows;
+          const float gg = on && dense.g_gamma ? __ldg(dense.g_gamma + row) : 0.f;
+          float graw[EPT], vraw[EPT];
+          if (dense_vec) {
+            // this block's rows have arrived, and every thread has read the last block's
+            asm volatile("cp.async.wait_group %0;" ::"n"(kDenseStages - 2) : "memory");
+            sp_builders_sync();
+            copy_dense(g + kDenseStages - 1);
+            const float* src = s_win + (size_t)(g % kDenseStages) * 2 * kDenseBuf + rr * kDensePitch + half * EPT;
+#pragma unroll
+            for (int q = 0; q < EPT / 4; ++q) {
+              const float4 a = dense.gVW ? *reinterpret_cast<const float4*>(src + 4 * q) : make_float4(0.f, 0.f, 0.f, 0.f);
+              const float4 b = dense.g_gamma ? *reinterpret_cast<const float4*>(src + kDenseBuf + 4 * q)
+                                             : make_float4(0.f, 0.f, 0.f, 0.f);
+              graw[4 * q] = a.x, graw[4 * q + 1] = a.y, graw[4 * q + 2] = a.z, graw[4 * q + 3] = a.w;
+              vraw[4 * q] = b.x, vraw[4 * q + 1] = b.y, vraw[4 * q + 2] = b.z, vraw[4 * q + 3] = b.w;
+            }
+          } else {
+            const size_t o = (size_t)row * h + k0;
+#pragma unroll
+            for (int e = 0; e < EPT; ++e) {
+              const bool in = on && k0 + e < h;
+              graw[e] = in && dense.gVW ? __ldg(dense.gVW + o + e) : 0.f;
+              vraw[e] = in && dense.g_gamma ? __ldg(dense.VWh + o + e) : 0.f;
+            }
+          }
 #pragma unroll
           for (int e = 0; e < EPT; ++e) {
             const int r = k0 + e;
-            float v = graw[NET == 3 ? e : 0];
+            float v = graw[e];
             if (gg != 0.f && r > 0 && r < h) {
-              const float x = vraw[NET == 3 ? e : 0];
+              const float x = vraw[e];
               const float dg = x > 0.f ? s_cnt[NET == 3 ? r : 0] : (x < 0.f ? -s_cnt[NET == 3 ? kAdjMaxH + r : 0] : 0.f);
               v = __fadd_rn(v, __fmul_rn(gg, dg));
             }
             dv[e] = v;
           }
-          load_dense(g + 1);
         } else if (cur.window) {
           a_run_window<NET == 3 ? 1 : NET, EPT>(w, h, cur.cell, k0, dv);
         } else {
@@ -1351,7 +1382,7 @@ template <bool TF32, int NET>
 static cudaError_t launch_split(const float* V, int n_x, int bc, int Q, const int* occ, const int* n_occ_dev,
                                 int n_occ_host, int max_rows, const void* img_hi, const void* img_lo, int KB, int NT,
                                 float c, float* out, unsigned int* flags, const DenseA& dense, cudaStream_t s) {
-  const size_t sm = split_smem_bytes(Q / 2);
+  const size_t sm = split_smem_bytes(Q / 2, NET);
   const cudaError_t e = raise_smem_limit(reinterpret_cast<const void*>(k_rows_split<TF32, NET>), sm);
   if (e != cudaSuccess) return e;
   const long long tiles = (long long)((max_rows + TM - 1) / TM) * NT;

@@ -16,30 +16,45 @@
 //   dW[d] = sum_i P G,  dwv1 = sum W V(i+d) G,  dwv2 = sum W V(i+d+1) G,
 //   dwt1 = sum W P H d, dwt2 = sum W P H (d + 1).
 //
-// k_n2_train: one CTA per training run (runs differ in learning rate; they
-// train on the same examples in the same order), the whole SGD loop inside the
-// CTA: per step the phase tables (sincospif of the current wt), the residuals
-// in shared memory, the gradient reductions in a fixed order (a run is
-// deterministic) and the update.  No step waits on another CTA.
+// k_n2_train: one cluster of CTAs per training run (runs differ in learning
+// rate; they train on the same examples in the same order), the whole SGD loop
+// inside it.  The rows of an example are split over the CTAs; each builds the
+// phase tables (sincospif of the current wt) for itself, its residuals and its
+// share of the gradient; the shares are exchanged through distributed shared
+// memory with one cluster barrier per step and added in rank order by every
+// CTA, so all of them make the same update and a run is deterministic.
 // k_n2_eval: the trained model's rows, in 1/s, for given parameters.
+#include <cooperative_groups.h>
+
 #include "wmc_device.cuh"
 
 namespace wmc {
 
 namespace {
 
-constexpr int kN2Threads = 1024;
 constexpr float kPiF = 3.14159265358979f;  // pi rounded to FP32
+constexpr int kN2Threads = 512;
 constexpr int kN2Warps = kN2Threads / 32;
+constexpr int kN2MaxCluster = 8;
 
-// Shared memory of k_n2_train: sin and phi-weighted cos tables [Q][h],
-// residuals and the products W P [n_x][h] each, V over [-h, n_x + h], cos(pi j
-// / Q) [h], the parameters, the W gradient, reduction scratch.
-__host__ __device__ inline size_t n2_smem_floats(int n_x, int Q) {
-  const int h = Q / 2;
-  return 2 * (size_t)Q * h + 2 * (size_t)n_x * h + (size_t)(n_x + Q + 2) + (size_t)h + (size_t)(Q + 4) +
-         (size_t)Q + (size_t)6 * kN2Warps;
-}
+// Sizes of k_n2_train with the rows over C CTAs.  Rows and pair offsets are
+// held by parity (row i meets the offsets dd = d + h of parity (i + h) mod 2):
+// M row pairs per CTA and h offsets, both padded to fours for 16-byte loads.
+struct N2Shape {
+  int h, hp, M, Mp;
+  __host__ __device__ N2Shape(int n_x, int Q, int C)
+      : h(Q / 2), hp((Q / 2 + 3) & ~3), M((n_x / 2 + C - 1) / C), Mp(((n_x / 2 + C - 1) / C + 3) & ~3) {}
+  // sin and phi-weighted cos tables [h][2][hp]; W P [h][2][Mp], later the W
+  // gradient's parts [Mp / 4][2][hp]; residuals [2][h][Mp]; V of the rows'
+  // windows; cos(pi j / Q); parameters; the exchanged sums, two buffers;
+  // reduction scratch
+  __host__ __device__ size_t table() const { return (size_t)h * 2 * hp; }
+  __host__ __device__ size_t rows() const { return (size_t)h * 2 * Mp; }
+  __host__ __device__ size_t window() const { return (size_t)2 * Mp + 2 * h + 4; }
+  __host__ __device__ size_t floats() const {
+    return 2 * table() + 2 * rows() + ((window() + 3) & ~(size_t)3) + hp + (2 * h + 4) + 2 * (2 * h + 5) + 5 * kN2Warps;
+  }
+};
 
 __device__ __forceinline__ float n2_pot(const float* __restrict__ V, int n_x, int bc, int l) {
   if (l >= 0 && l < n_x) return __ldg(V + l);
@@ -47,129 +62,215 @@ __device__ __forceinline__ float n2_pot(const float* __restrict__ V, int n_x, in
   return __ldg(V + (l < 0 ? 0 : n_x - 1));
 }
 
-// Sum of v over the block in a fixed order (warp shuffles, then warp 0);
-// every thread gets the result.
-__device__ __forceinline__ float n2_block_sum(float v, float* red) {
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
-  __syncthreads();
-  if (lane == 0) red[wid] = v;
-  __syncthreads();
-  float s = 0.f;
-  for (int w = 0; w < kN2Warps; ++w) s += red[w];
-  return s;
-}
-
 }  // namespace
 
+// A thread's tile is 4 rows (of one parity) x 4 columns of the residuals, then
+// 4 rows x 4 offsets of the gradient sums: 16 and 32 FMAs for 5 and 3 loads of
+// shared memory (one load per FMA, 40 k shared-memory cycles a step, bound the
+// form with one output per thread at 36 us a step on one SM).  256 cells, Q =
+// 64, three runs: 6.9 us a step with eight CTAs per run, bound by the
+// barriers and the chain of phases.
 __global__ __launch_bounds__(kN2Threads) void k_n2_train(int n_x, int Q, int bc, int n_ex, const float* __restrict__ Vs,
                                                           const float* __restrict__ VW, float scale, int epochs,
                                                           const int* __restrict__ order, const float* __restrict__ lr,
                                                           float* __restrict__ params, float* __restrict__ loss_out) {
-  extern __shared__ float sm_n2[];
-  const int h = Q / 2, run = blockIdx.x;
+  namespace cg = cooperative_groups;
+  extern __shared__ __align__(16) float sm_n2[];
+  cg::cluster_group cluster = cg::this_cluster();
+  const int C = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
+  const int run = blockIdx.x / C;
+  const N2Shape z(n_x, Q, C);
+  const int h = z.h, hp = z.hp, M = z.M, Mp = z.Mp, NV = Q + 5;  // NV exchanged sums: dW, dwv, dwt, loss
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  float* sS = sm_n2;                       // [Q][h] sin(2 pi j / Q (wt1 d + wt2 (d + 1)))
-  float* sC = sS + (size_t)Q * h;          // [Q][h] phi_j times the cosines
-  // residuals times (2 / n_out) cos(pi j / Q), by row parity: [2][h][n_x / 2]
-  // (lanes of one offset read consecutive rows of one parity without bank conflicts)
-  float* sR = sC + (size_t)Q * h;
-  float* sWP = sR + (size_t)n_x * h;       // [h][n_x]: W[d] P(i, d) of the k-th pair of row i
-  float* sV = sWP + (size_t)n_x * h;       // V(l) at l + h, l in [-h, n_x + h]
-  float* sCJ = sV + (n_x + Q + 2);         // cos(pi j / Q)
-  float* sP = sCJ + h;                     // parameters
-  float* sGW = sP + (Q + 4);               // dL/dW
-  float* red = sGW + Q;                    // [6][warps]
+  float* sS = sm_n2;              // [h][2][hp]: sin of offset dd (parity, dd / 2) at column j
+  float* sC = sS + z.table();     // phi_j times the cosines
+  float* sWP = sC + z.table();    // [h][2][Mp]: W P of pair k of the rows of each parity
+  float* sR = sWP + z.rows();     // [2][h][Mp]: residuals times (2 / n_out) cos(pi j / Q)
+  float* sV = sR + z.rows();      // V(i0 - h + q)
+  float* sCJ = sV + ((z.window() + 3) & ~(size_t)3);
+  float* sP = sCJ + hp;           // parameters
+  float* sX = sP + (Q + 4);       // exchanged sums, by step parity
+  float* red = sX + 2 * NV;       // [5][warps]
+  float* sGp = sWP;               // the W gradient's parts, once W P has been used
+  const int m0 = rank * M, m_n = max(0, min(M, n_x / 2 - m0));  // this CTA's row pairs
+  const int i0 = 2 * m0;
   const float rate = __ldg(lr + run);
   float* prm = params + (size_t)run * (Q + 4);
   for (int q = tid; q < Q + 4; q += kN2Threads) sP[q] = prm[q];
   for (int j = tid; j < h; j += kN2Threads) sCJ[j] = cospif((float)j / (float)Q);
+  for (size_t q = tid; q < 2 * z.table(); q += kN2Threads) sS[q] = 0.f;  // (the padding stays zero)
   const float inv_n = 2.f / (float)((long long)n_x * (h - 1));  // d(mean of squares)/dy = inv_n r
-  const int half = n_x / 2;
+  const int RG = Mp / 4, JG = hp / 4;  // groups of four row pairs, of four columns or offsets
+  const int n_tasks = 2 * RG * JG;
   __syncthreads();
+  int step = 0;
   for (int ep = 0; ep < epochs; ++ep) {
     float ep_loss = 0.f;
-    for (int s = 0; s < n_ex; ++s) {
+    for (int s = 0; s < n_ex; ++s, ++step) {
       const int ex = __ldg(order + (size_t)ep * n_ex + s);
       const float* V = Vs + (size_t)ex * n_x;
       const float* T = VW + (size_t)ex * n_x * h;
       const float wv1 = sP[Q], wv2 = sP[Q + 1], wt1 = sP[Q + 2], wt2 = sP[Q + 3];
-      // phase tables of the current wt and the example's potential
+      // phase tables of the current wt, the potential and W P
+      for (int q = tid; q < 2 * m_n + 2 * h + 1; q += kN2Threads) sV[q] = n2_pot(V, n_x, bc, i0 - h + q);
       for (int q = tid; q < Q * h; q += kN2Threads) {
-        const int d = q / h - h, j = q % h;
+        const int j = q / Q, dd = q % Q, d = dd - h;
         float sv, cv;
         sincospif(2.f * (float)j / (float)Q * (wt1 * (float)d + wt2 * (float)(d + 1)), &sv, &cv);
-        sS[q] = sv;
-        sC[q] = cv * (2.f * (float)j / (float)Q) * kPiF;
-      }
-      for (int l = tid - h; l <= n_x + h; l += kN2Threads) sV[l + h] = n2_pot(V, n_x, bc, l);
-      __syncthreads();
-      for (int q = tid; q < n_x * h; q += kN2Threads) {  // W[d] P(i, d), k-th pair of row i
-        const int k = q / n_x, i = q % n_x;
-        const int d = (((i - h) & 1) == 0 ? -h : -h + 1) + 2 * k;
-        sWP[q] = sP[d + h] * fmaf(wv1, sV[i + d + h], wv2 * sV[i + d + 1 + h]);
+        const size_t at = ((size_t)j * 2 + (dd & 1)) * hp + (dd >> 1);
+        sS[at] = sv;
+        sC[at] = cv * (2.f * (float)j / (float)Q) * kPiF;
       }
       __syncthreads();
-      // residuals (thread q: column j = q / n_x, row i = q % n_x)
+      for (int q = tid; q < h * 2 * Mp; q += kN2Threads) {  // pair k of row i0 + 2 m + p
+        const int m = q % Mp, p = (q / Mp) & 1, k = q / (2 * Mp);
+        const int dd = 2 * k + ((i0 + p + h) & 1), at = 2 * m + p + dd;  // sV[at] = V(i + d)
+        sWP[q] = m < m_n ? sP[dd] * fmaf(wv1, sV[at], wv2 * sV[at + 1]) : 0.f;
+      }
+      __syncthreads();
+      // residuals
       float part = 0.f;
-      for (int q = tid; q < n_x * h; q += kN2Threads) {
-        const int j = q / n_x, i = q % n_x;
-        float r = 0.f;
-        if (j > 0) {
-          const int dd0 = ((i - h) & 1) == 0 ? 0 : 1;  // d + h of the first pair
-          float acc = 0.f;
-          for (int k = 0; k < h; ++k) acc = fmaf(sWP[(size_t)k * n_x + i], sS[(dd0 + 2 * k) * h + j], acc);
-          r = fmaf(sCJ[j], acc, -__ldg(T + (size_t)i * h + j) * scale);
-        }
-        sR[((size_t)(i & 1) * h + j) * half + (i >> 1)] = r * sCJ[j] * inv_n;
-        part = fmaf(r, r, part);
-      }
-      const float loss = n2_block_sum(part, red) * (0.5f * inv_n);
-      ep_loss += loss;
-      // gradients: warp w takes the offsets d = w - h, w + warps - h, ...; its
-      // lanes take the rows i = (d & 1) + 2 m of each
-      float gv1 = 0.f, gv2 = 0.f, gt1 = 0.f, gt2 = 0.f;
-      for (int dd = wid; dd < Q; dd += kN2Warps) {
-        const int d = dd - h;
-        const float Wd = sP[dd];
-        float gw = 0.f;
-        const float* rp = sR + (size_t)(d & 1) * h * half;
-        for (int m = lane; m < half; m += 32) {
-          const int i = (d & 1) + 2 * m;
-          float G = 0.f, H = 0.f;
-          for (int j = 1; j < h; ++j) {
-            const float rc = rp[(size_t)j * half + m];
-            G = fmaf(rc, sS[dd * h + j], G);
-            H = fmaf(rc, sC[dd * h + j], H);
+      for (int t = tid; t < n_tasks; t += kN2Threads) {
+        const int rg = t % RG, jg = (t / RG) % JG, p = t / (RG * JG);
+        const int pd = (i0 + p + h) & 1;  // parity of the rows' offsets
+        float tv[4][4];  // targets, asked for before the sums
+#pragma unroll
+        for (int b = 0; b < 4; ++b)
+#pragma unroll
+          for (int a = 0; a < 4; ++a) {
+            const int m = 4 * rg + a, j = 4 * jg + b;
+            tv[a][b] = m < m_n && j < h ? __ldg(T + (size_t)(i0 + 2 * m + p) * h + j) : 0.f;
           }
-          const float Va = sV[i + d + h], Vb = sV[i + d + 1 + h];
-          const float P = fmaf(wv1, Va, wv2 * Vb);
-          gw = fmaf(P, G, gw);
-          gv1 = fmaf(Wd * Va, G, gv1);
-          gv2 = fmaf(Wd * Vb, G, gv2);
-          gt1 = fmaf(Wd * P * H, (float)d, gt1);
-          gt2 = fmaf(Wd * P * H, (float)(d + 1), gt2);
+        float acc[4][4];
+#pragma unroll
+        for (int a = 0; a < 4; ++a)
+#pragma unroll
+          for (int b = 0; b < 4; ++b) acc[a][b] = 0.f;
+        const float* wp = sWP + (size_t)p * Mp + 4 * rg;
+        const float* st = sS + (size_t)pd * hp;
+        int jb[4];
+#pragma unroll
+        for (int b = 0; b < 4; ++b) jb[b] = min(4 * jg + b, h - 1) * 2 * hp;
+#pragma unroll 4
+        for (int k = 0; k < h; ++k) {
+          const float4 w4 = *reinterpret_cast<const float4*>(wp + (size_t)k * 2 * Mp);
+          const float wa[4] = {w4.x, w4.y, w4.z, w4.w};
+#pragma unroll
+          for (int b = 0; b < 4; ++b) {
+            const float sv = st[jb[b] + k];
+#pragma unroll
+            for (int a = 0; a < 4; ++a) acc[a][b] = fmaf(wa[a], sv, acc[a][b]);
+          }
         }
 #pragma unroll
-        for (int off = 16; off > 0; off >>= 1) gw += __shfl_down_sync(0xffffffffu, gw, off);
-        if (lane == 0) sGW[dd] = gw;
+        for (int b = 0; b < 4; ++b) {
+          const int j = 4 * jg + b;
+          if (j < h) {
+            float4 r4;
+            float* rv = reinterpret_cast<float*>(&r4);
+            const float cj = sCJ[j];
+#pragma unroll
+            for (int a = 0; a < 4; ++a) {
+              const float r = j > 0 && 4 * rg + a < m_n ? fmaf(cj, acc[a][b], -tv[a][b] * scale) : 0.f;
+              part = fmaf(r, r, part);
+              rv[a] = r * cj * inv_n;
+            }
+            *reinterpret_cast<float4*>(sR + ((size_t)p * h + j) * Mp + 4 * rg) = r4;
+          }
+        }
       }
-      const float Gv1 = n2_block_sum(gv1, red), Gv2 = n2_block_sum(gv2, red + kN2Warps);
-      const float Gt1 = n2_block_sum(gt1, red + 2 * kN2Warps), Gt2 = n2_block_sum(gt2, red + 3 * kN2Warps);
-      // update (every thread has read the parameters it needs for this step)
-      for (int dd = tid; dd < Q; dd += kN2Threads) sP[dd] = fmaf(-rate, sGW[dd], sP[dd]);
-      if (tid == 0) {
-        sP[Q] = fmaf(-rate, Gv1, wv1);
-        sP[Q + 1] = fmaf(-rate, Gv2, wv2);
-        sP[Q + 2] = fmaf(-rate, Gt1, wt1);
-        sP[Q + 3] = fmaf(-rate, Gt2, wt2);
+      __syncthreads();
+      // gradient sums of 4 rows x 4 offsets
+      float gv1 = 0.f, gv2 = 0.f, gt1 = 0.f, gt2 = 0.f;
+      for (int t = tid; t < n_tasks; t += kN2Threads) {
+        const int rg = t % RG, dg = (t / RG) % JG, p = t / (RG * JG);
+        const int pd = (i0 + p + h) & 1;
+        float G[4][4], H[4][4];
+#pragma unroll
+        for (int a = 0; a < 4; ++a)
+#pragma unroll
+          for (int b = 0; b < 4; ++b) G[a][b] = H[a][b] = 0.f;
+        const float* rp = sR + (size_t)p * h * Mp + 4 * rg;
+        const size_t tb = (size_t)pd * hp + 4 * dg;
+#pragma unroll 2
+        for (int j = 1; j < h; ++j) {
+          const float4 r4 = *reinterpret_cast<const float4*>(rp + (size_t)j * Mp);
+          const float4 s4 = *reinterpret_cast<const float4*>(sS + tb + (size_t)j * 2 * hp);
+          const float4 c4 = *reinterpret_cast<const float4*>(sC + tb + (size_t)j * 2 * hp);
+          const float ra[4] = {r4.x, r4.y, r4.z, r4.w}, sb[4] = {s4.x, s4.y, s4.z, s4.w}, cb[4] = {c4.x, c4.y, c4.z, c4.w};
+#pragma unroll
+          for (int a = 0; a < 4; ++a)
+#pragma unroll
+            for (int b = 0; b < 4; ++b) {
+              G[a][b] = fmaf(ra[a], sb[b], G[a][b]);
+              H[a][b] = fmaf(ra[a], cb[b], H[a][b]);
+            }
+        }
+        float4 g4;
+        float* gw = reinterpret_cast<float*>(&g4);
+#pragma unroll
+        for (int b = 0; b < 4; ++b) {
+          const int dd = 2 * (4 * dg + b) + pd, d = dd - h;
+          gw[b] = 0.f;
+          if (4 * dg + b < h) {
+            const float Wd = sP[dd];
+#pragma unroll
+            for (int a = 0; a < 4; ++a) {
+              const int m = 4 * rg + a;
+              if (m < m_n) {
+                const float Va = sV[2 * m + p + dd], Vb = sV[2 * m + p + dd + 1];
+                const float P = fmaf(wv1, Va, wv2 * Vb);
+                gw[b] = fmaf(P, G[a][b], gw[b]);
+                gv1 = fmaf(Wd * Va, G[a][b], gv1);
+                gv2 = fmaf(Wd * Vb, G[a][b], gv2);
+                gt1 = fmaf(Wd * P * H[a][b], (float)d, gt1);
+                gt2 = fmaf(Wd * P * H[a][b], (float)(d + 1), gt2);
+              }
+            }
+          }
+        }
+        // (each offset belongs to one row parity, so a slot has one writer)
+        *reinterpret_cast<float4*>(sGp + ((size_t)rg * 2 + pd) * hp + 4 * dg) = g4;
+      }
+      float v5[5] = {gv1, gv2, gt1, gt2, part};
+#pragma unroll
+      for (int q = 0; q < 5; ++q) {
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) v5[q] += __shfl_down_sync(0xffffffffu, v5[q], off);
+        if (lane == 0) red[q * kN2Warps + wid] = v5[q];
+      }
+      __syncthreads();
+      float* mine = sX + (step & 1) * NV;
+      for (int q = tid; q < NV; q += kN2Threads) {
+        float v = 0.f;
+        if (q < Q)
+          for (int rg = 0; rg < RG; ++rg) v += sGp[((size_t)rg * 2 + (q & 1)) * hp + (q >> 1)];
+        else
+          for (int w = 0; w < kN2Warps; ++w) v += red[(q - Q) * kN2Warps + w];
+        mine[q] = v;
+      }
+      // every CTA's sums are there; the other buffer serves the next step, so
+      // that no CTA overwrites sums another still reads
+      if (C > 1) cluster.sync();
+      else __syncthreads();
+      for (int q = tid; q < NV; q += kN2Threads) {
+        float x[kN2MaxCluster], v = 0.f;  // (all loads under way before the first sum)
+#pragma unroll
+        for (int c = 0; c < kN2MaxCluster; ++c)
+          x[c] = c < C ? (C > 1 ? *(cluster.map_shared_rank(mine, c) + q) : mine[q]) : 0.f;
+#pragma unroll
+        for (int c = 0; c < kN2MaxCluster; ++c)
+          if (c < C) v += x[c];
+        if (q < Q + 4) sP[q] = fmaf(-rate, v, sP[q]);
+        else ep_loss += v * (0.5f * inv_n);
       }
       __syncthreads();
     }
-    if (tid == 0 && loss_out) loss_out[(size_t)run * epochs + ep] = ep_loss / (float)n_ex;
+    if (rank == 0 && tid == (Q + 4) % kN2Threads && loss_out) loss_out[(size_t)run * epochs + ep] = ep_loss / (float)n_ex;
   }
-  for (int q = tid; q < Q + 4; q += kN2Threads) prm[q] = sP[q];
+  if (rank == 0)
+    for (int q = tid; q < Q + 4; q += kN2Threads) prm[q] = sP[q];
+  if (C > 1) cluster.sync();  // no CTA leaves while another reads its shared memory
 }
 
 // Rows of the trained model in 1/s: row = potential b, cell i (b n_x + i),
@@ -218,16 +319,35 @@ wmc_status wmc_n2_train(const wmc_params* p, int32_t n_examples, const float* V,
   if (!params_ok(p) || n_examples <= 0 || epochs < 0 || n_runs < 0 || !V || !VW || !order || !lr || !params)
     return WMC_ERR_ARG;
   if (p->n_x % 2 != 0) return WMC_ERR_ARG;
-  const size_t sm = sizeof(float) * n2_smem_floats(p->n_x, p->Q);
-  if (sm > 200 * 1024) return WMC_ERR_UNSUPPORTED;
+  // the sizes one CTA's shared memory holds with whole tables and rows
+  const size_t h = (size_t)p->Q / 2;
+  if (sizeof(float) * (2 * (size_t)p->Q * h + 2 * (size_t)p->n_x * h + (size_t)(p->n_x + p->Q + 2) + h +
+                       (size_t)(2 * p->Q + 4) + 192) > 200 * 1024)
+    return WMC_ERR_UNSUPPORTED;
   if (n_runs == 0 || epochs == 0) return WMC_OK;
-  if (sm > 48 * 1024 &&
-      raise_smem_limit(reinterpret_cast<const void*>(k_n2_train), sm) != cudaSuccess)
+  // CTAs per run: as many as the SMs hold for all runs, with at least four row
+  // pairs each
+  int C = 1;
+  while (2 * C <= kN2MaxCluster && (long long)n_runs * 2 * C <= num_sms() && p->n_x / 2 >= 4 * 2 * C) C *= 2;
+  const size_t sm = sizeof(float) * N2Shape(p->n_x, p->Q, C).floats();
+  if (sm > 48 * 1024 && raise_smem_limit(reinterpret_cast<const void*>(k_n2_train), sm) != cudaSuccess)
     return WMC_ERR_CUDA;
   const float scale = (float)(kHbarEVs * (double)p->Q / 2.0);
-  k_n2_train<<<n_runs, kN2Threads, sm, (cudaStream_t)stream>>>(p->n_x, p->Q, p->bc_potential, n_examples, V, VW,
-                                                               scale, epochs, order, lr, params, loss);
-  return cudaGetLastError() == cudaSuccess ? WMC_OK : WMC_ERR_CUDA;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(n_runs * C));
+  cfg.blockDim = dim3(kN2Threads);
+  cfg.dynamicSmemBytes = sm;
+  cfg.stream = (cudaStream_t)stream;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = (unsigned)C;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, k_n2_train, p->n_x, p->Q, p->bc_potential, n_examples, V, VW, scale, epochs, order, lr,
+                            params, loss) == cudaSuccess
+             ? WMC_OK
+             : WMC_ERR_CUDA;
 }
 
 wmc_status wmc_n2_eval(const wmc_params* p, const float* params, const float* V, int32_t n_pot, float* VWh,

@@ -392,6 +392,15 @@ __global__ __launch_bounds__(kStepThreads) void k_materialize(const int32_t* __r
       int ck[4] = {0, 0, 0, 0};
       uint32_t neg = 0u, have = 0u;
       uint32_t x = max(a, c.off);  // ids before x have their columns
+      if (x >= B.end) walk_load(c, x, B, lane);
+      const int j0 = __ffs(__ballot_sync(0xffffffffu, B.E > x)) - 1;
+      if (x == a && wend - a == 128u && __shfl_sync(0xffffffffu, B.E, j0) >= wend) {  // one bucket
+        const int k = min((B.b << 5) + j0, n_M - 1);
+        ck[0] = ck[1] = ck[2] = ck[3] = k;
+        neg = __shfl_sync(0xffffffffu, B.e, j0) & 1u ? 0xfu : 0u;
+        have = 0xfu;
+        x = wend;
+      }
 #pragma unroll 1
       while (x < wend) {
         if (x >= B.end) walk_load(c, x, B, lane);

@@ -95,3 +95,26 @@ def test_zero_loss_where_n2_is_exact_and_determinism(wmc):
     out = prm.cpu().numpy()
     assert np.array_equal(out[0], out[1])
     assert np.abs(out[0] - p0).max() <= 1e-5
+
+
+@pytest.mark.parametrize("n_x,q,runs", [(2, 6, 1), (34, 10, 3), (66, 14, 30), (96, 30, 152)])
+def test_sgd_with_the_rows_split_over_ctas(wmc, n_x, q, runs):
+    """Row pairs that fill no group of four and do not divide over the CTAs of a
+    run (8, 4 and 1 of them), windows whose half is odd."""
+    w = _wl(n_x=n_x, q=q)
+    n_ex, epochs = 4, 3
+    lrs = np.linspace(3e-3, 3e-2, runs).astype(np.float32)
+    Vs = np.random.default_rng(n_x).uniform(-0.2, 0.3, (n_ex, n_x)).astype(np.float32)
+    T = _targets(w, Vs)
+    order = wi.sgd_order(epochs, n_ex)
+    p0 = nt.initial_params(w.Q)
+    prm = torch.from_numpy(np.tile(p0.astype(np.float32), (runs, 1))).cuda()
+    loss = torch.zeros((runs, epochs), device="cuda")
+    wmc.n2_train(wmc.Params.of(w), torch.from_numpy(Vs).cuda(), torch.from_numpy(T).cuda(),
+                 torch.from_numpy(order).cuda(), torch.from_numpy(lrs).cuda(), prm, loss)
+    got, got_loss = prm.cpu().numpy().astype(np.float64), loss.cpu().numpy()
+    Ts = T.astype(np.float64) * nt.target_scale(w.Q)
+    for r in sorted({0, runs // 2, runs - 1}):
+        pf, hist = nt.train(p0, Vs, Ts, order, float(lrs[r]), w.Q)
+        assert np.linalg.norm(got[r] - pf) <= 1e-2 * np.linalg.norm(pf - p0) + 1e-6
+        assert np.all(np.abs(got_loss[r] - hist) <= 1e-4 * hist + 1e-12)
