@@ -831,7 +831,7 @@ __global__ __launch_bounds__(kTaThreads, 1) void k_kernel_eval_tc_ta(const float
 // four K blocks in shared memory and drained each pass before it built the
 // next, 3400 cycles a block: 16384 cells at Q = 1024 (3xTF32) 111 -> 63 us, 3600
 // occupied cells in the step 47 -> 22 us, 262144 rows at Q = 256 155 -> 78 us,
-// the adjoint contraction over the same rows 277 -> 192 us.
+// the adjoint contraction over the same rows 277 -> 130 us (half of it the builders and the stores).
 constexpr int kSpStages = 5;
 // K blocks whose barriers are in use at once: more than the longest look-back,
 // kSpStages blocks, so that no waiter meets a barrier two phases on.
@@ -936,7 +936,7 @@ __global__ __launch_bounds__(kSpThreads, 1) void k_rows_split(
   __shared__ uint32_t tmem_slot;
   __shared__ volatile int s_abort;
   __shared__ int s_min[8], s_max[8];
-  __shared__ float s_cnt[NET == 3 ? 2 * kAdjMaxH : 1];
+  __shared__ __align__(16) float s_cnt[NET == 3 ? 2 * kAdjMaxH : 4];
 
   const int n_rows = n_occ_dev ? *n_occ_dev : n_occ_host;
   const int h = Q / 2;
@@ -1113,17 +1113,25 @@ __global__ __launch_bounds__(kSpThreads, 1) void k_rows_split(
     const bool dense_vec = NET == 3 && (h & 3) == 0 &&
                            ((reinterpret_cast<uintptr_t>(dense.gVW) | reinterpret_cast<uintptr_t>(dense.VWh)) & 15) == 0;
     constexpr size_t kDenseBuf = (size_t)TM * kDensePitch;
+    int cd_rt = (int)(t0 / NT), cd_kb = 0, cd_ct = (int)(t0 % NT);  // the next block to copy
     auto copy_dense = [&](int g) {
       if (g < n_blocks) {
-        const int rt = (int)((t0 + g / KB) / NT), k0 = (g % KB) * KBLK;
-        float* dst = s_win + (size_t)(g % kDenseStages) * 2 * kDenseBuf;
+        const int r0 = tid >> 3, col = 4 * (tid & 7), k0 = cd_kb * KBLK;
+        float* dst = s_win + (size_t)(g % kDenseStages) * 2 * kDenseBuf + r0 * kDensePitch + col;
+        size_t o = (size_t)(cd_rt * TM + r0) * h + k0 + col;
+        const int left = k0 + col < h ? n_rows - cd_rt * TM - r0 : 0;  // rows from r0 on
 #pragma unroll
-        for (int q = tid; q < TM * 8; q += kSpBuilders) {
-          const int r = q >> 3, col = 4 * (q & 7), row = rt * TM + r;
-          const bool in = row < n_rows && k0 + col < h;
-          const size_t o = in ? (size_t)row * h + k0 + col : 0;
-          if (dense.gVW) cp_async16(dst + r * kDensePitch + col, dense.gVW + o, in);
-          if (dense.g_gamma) cp_async16(dst + kDenseBuf + r * kDensePitch + col, dense.VWh + o, in);
+        for (int q = 0; q < TM / 32; ++q, o += 32 * (size_t)h) {
+          const bool in = 32 * q < left;
+          if (dense.gVW) cp_async16(dst + 32 * q * kDensePitch, dense.gVW + (in ? o : 0), in);
+          if (dense.g_gamma) cp_async16(dst + kDenseBuf + 32 * q * kDensePitch, dense.VWh + (in ? o : 0), in);
+        }
+        if (++cd_kb == KB) {
+          cd_kb = 0;
+          if (++cd_ct == NT) {
+            cd_ct = 0;
+            ++cd_rt;
+          }
         }
       }
       asm volatile("cp.async.commit_group;" ::: "memory");
@@ -1171,16 +1179,37 @@ __global__ __launch_bounds__(kSpThreads, 1) void k_rows_split(
               vraw[e] = in && dense.g_gamma ? __ldg(dense.VWh + o + e) : 0.f;
             }
           }
+          if (gg == 0.f) {
 #pragma unroll
-          for (int e = 0; e < EPT; ++e) {
-            const int r = k0 + e;
-            float v = graw[e];
-            if (gg != 0.f && r > 0 && r < h) {
-              const float x = vraw[e];
-              const float dg = x > 0.f ? s_cnt[NET == 3 ? r : 0] : (x < 0.f ? -s_cnt[NET == 3 ? kAdjMaxH + r : 0] : 0.f);
-              v = __fadd_rn(v, __fmul_rn(gg, dg));
+            for (int e = 0; e < EPT; ++e) dv[e] = graw[e];
+          } else if (k0 + EPT <= h) {
+            // multiplicities four columns at a time (the same for every lane)
+#pragma unroll
+            for (int q = 0; q < EPT / 4; ++q) {
+              const int at = NET == 3 ? k0 + 4 * q : 0;
+              const float4 cp = *reinterpret_cast<const float4*>(s_cnt + at);
+              const float4 cn = *reinterpret_cast<const float4*>(s_cnt + (NET == 3 ? kAdjMaxH : 0) + at);
+              const float p4[4] = {cp.x, cp.y, cp.z, cp.w}, n4[4] = {cn.x, cn.y, cn.z, cn.w};
+#pragma unroll
+              for (int e = 0; e < 4; ++e) {
+                const float x = vraw[4 * q + e];
+                const float dg = x > 0.f ? p4[e] : (x < 0.f ? -n4[e] : 0.f);
+                dv[4 * q + e] = __fadd_rn(graw[4 * q + e], __fmul_rn(gg, dg));
+              }
             }
-            dv[e] = v;
+            if (k0 == 0) dv[0] = graw[0];  // (column 0 counts nowhere, whatever gg is)
+          } else {
+#pragma unroll
+            for (int e = 0; e < EPT; ++e) {
+              const int r = k0 + e;
+              float v = graw[e];
+              if (r > 0 && r < h) {
+                const float x = vraw[e];
+                const float dg = x > 0.f ? s_cnt[NET == 3 ? r : 0] : (x < 0.f ? -s_cnt[NET == 3 ? kAdjMaxH + r : 0] : 0.f);
+                v = __fadd_rn(v, __fmul_rn(gg, dg));
+              }
+              dv[e] = v;
+            }
           }
         } else if (cur.window) {
           a_run_window<NET == 3 ? 1 : NET, EPT>(w, h, cur.cell, k0, dv);
