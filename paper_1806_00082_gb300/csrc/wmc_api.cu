@@ -60,7 +60,7 @@ Layout layout(const wmc_params& p) {
   // more, the pair kernel walks the ids again instead)
   {
     const size_t want = nx * nM / 8;
-    L.pair_cap = (unsigned)(want < (1u << 19) ? (1u << 19) : (want > (1u << 22) ? (1u << 22) : want));
+    L.pair_cap = (unsigned)(want < (1u << 21) ? (1u << 21) : (want > (1u << 22) ? (1u << 22) : want));
   }
   L.pairs = o; o = align256(o + sizeof(uint4) * (size_t)L.pair_cap);
   L.B = o; o = align256(o + sizeof(float) * (size_t)L.Kp * (size_t)L.Np);

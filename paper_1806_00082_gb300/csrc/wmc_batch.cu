@@ -16,6 +16,7 @@
 #include <string.h>
 
 #include <mutex>
+#include <type_traits>
 #include <vector>
 
 #include "wmc_walk.cuh"
@@ -106,7 +107,7 @@ BatchLayout batch_layout(const wmc_params* ps, int n) {
   // kernel walks the ids again instead)
   {
     const long long want = L.hist_elems / 8;
-    L.pair_cap = (unsigned)(want < (1ll << 19) ? (1ll << 19) : (want > (1ll << 22) ? (1ll << 22) : want));
+    L.pair_cap = (unsigned)(want < (1ll << 21) ? (1ll << 21) : (want > (1ll << 23) ? (1ll << 23) : want));
   }
   L.pairs = o; o = al256(o + sizeof(uint4) * (size_t)L.pair_cap);
   L.blk = o; o = al256(o + sizeof(unsigned long long) * kScanned * (size_t)(L.n_blk + 1));
@@ -192,12 +193,15 @@ __global__ void k_b_init(const SimDesc* __restrict__ d, int n, long long n_cells
 // ---------------------------------------------------------------- per-cell scan
 // Per cell: survivors, survivor prefixes of the row's 32-column blocks and the
 // number of non-empty ones, reach bits, and a zeroed row of the next histogram.
-// A warp takes kRowsPerWarp cells; between the steps of a run (rows_known) it
-// passes over the cells that can hold no particle -- those the last step did
-// not need -- and zeroes only the rows that were occupied.  Memory-bound: 512
-// simulations, a third of the cells occupied, 240 us and 106 us for clearing
-// the next histograms before.
+// A warp takes RPW cells; between the steps of a run (rows_known) it passes over
+// the cells that can hold no particle -- those the last step did not need -- and
+// zeroes only the rows that were occupied.  Memory-bound for many cells: 512
+// simulations, 1.06e6 cells, a third of them occupied, 119 us (every row read
+// 240 us, and 106 us for clearing the next histograms).  Few cells are a chain
+// of latencies instead, eight rows of a warp one after the other 15 us for
+// 13000 to 19000 cells, so below kManyCells a warp takes one.
 constexpr int kRowsPerWarp = 8;
+constexpr long long kManyCells = 1ll << 16;
 
 __device__ __forceinline__ void b_row(const int32_t* __restrict__ hist, const SimDesc* __restrict__ d,
                                       const int* __restrict__ cell_sim, long long c, int NB,
@@ -286,17 +290,18 @@ __device__ __forceinline__ void b_row(const int32_t* __restrict__ hist, const Si
   }
 }
 
+template <int RPW>
 __global__ void k_b_rows(const int32_t* __restrict__ hist, const SimDesc* __restrict__ d,
                          const int* __restrict__ cell_sim, long long n_cells, int NB,
                          unsigned long long* __restrict__ T, uint32_t* __restrict__ bp,
                          unsigned char* __restrict__ nbk, unsigned char* __restrict__ reach,
                          int32_t* __restrict__ out, const int* __restrict__ row_map, const DevHeader* hdr) {
-  const long long c0 = ((blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5) * kRowsPerWarp;
+  const long long c0 = ((blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5) * RPW;
   const int lane = threadIdx.x & 31;
   if (c0 >= n_cells) return;
   const bool known = hdr->rows_known != 0u;
   const long long c = c0 + lane;
-  const bool in = lane < kRowsPerWarp && c < n_cells;
+  const bool in = lane < RPW && c < n_cells;
   const bool clear = in && (!known || T[c] != 0ull), read = in && (!known || row_map[c] >= 0);
   if (in && !read) {  // (its row of the next histogram is zero)
     T[c] = 0ull;
@@ -504,22 +509,25 @@ __global__ __launch_bounds__(256) void k_b_live(const float* __restrict__ V, con
   }
 }
 
-// One warp per such cell: FP32 contraction with the simulation's own window and
+// One warp per such cell (LIVE), or per needed cell with the same test inside
+// where there are few: FP32 contraction with the simulation's own window and
 // sine matrix (read through L1), then the fixed-point CDF and event threshold
-// of the row.  (With a warp per needed cell, most of them flat, the rows took
-// 171 us of 512 simulations' step, a chain of dependent loads each.)
-template <int C>
+// of the row.  With a warp per needed cell, most of them flat, the rows took
+// 171 us of 512 simulations' step, a chain of dependent loads each, 48 us by the
+// list; for 19000 cells the list's own kernel takes 13 us, so it is made from
+// kManyCells cells on.
+template <int C, bool LIVE>
 __global__ __launch_bounds__(kBatchRowWarps * 32) void k_b_kernel_rows(
     const float* __restrict__ V, const SimDesc* __restrict__ d, const int* __restrict__ cell_sim,
     const int* __restrict__ occ, const int* __restrict__ live, DevHeader* __restrict__ hdr,
     const float* __restrict__ sine, int NM, long long* __restrict__ cdf, unsigned long long* __restrict__ thr_cell) {
   __shared__ float s_buf[kBatchRowWarps][2 * 32 * C];
-  const int n_rows = hdr->n_live;
+  const int n_rows = LIVE ? hdr->n_live : hdr->n_occ;
   const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
   float* s_row = s_buf[wid];
   float* s_dv = s_buf[wid] + 32 * C;
   for (int l = blockIdx.x * kBatchRowWarps + wid; l < n_rows; l += gridDim.x * kBatchRowWarps) {
-    const int row = __ldg(live + l);
+    const int row = LIVE ? __ldg(live + l) : l;
     const int cg = __ldg(occ + row);
     const SimDesc& s = d[__ldg(cell_sim + cg)];
     const int i = (int)(cg - s.cell_off), h = s.h, Q = s.Q, n_M = s.n_M;
@@ -530,6 +538,12 @@ __global__ __launch_bounds__(kBatchRowWarps * 32) void k_b_kernel_rows(
       const int m = lane + 1 + 32 * q;
       s_dv[m - 1] = m <= h - 1 ? __fsub_rn(pot(Vs, s.n_x, s.bc, (long long)i + m), pot(Vs, s.n_x, s.bc, (long long)i - m))
                                : 0.f;
+    }
+    if (!LIVE) {
+      bool nz = false;
+#pragma unroll
+      for (int q = 0; q < C; ++q) nz |= s_dv[lane + 32 * q] != 0.f;
+      if (!__any_sync(0xffffffffu, nz)) continue;
     }
     __syncwarp();
     float sacc[C], eacc[C];
@@ -846,19 +860,31 @@ __global__ void k_b_set_step(DevHeader* hdr, uint32_t step) {
 
 // ---------------------------------------------------------------- host driver
 int b_step_grid() {
+  static int cached[8] = {0};
+  int dev = 0;
+  cudaGetDevice(&dev);
+  int& grid = cached[dev & 7];
+  if (grid > 0) return grid;
   int per_sm = 0;
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_b_step, kBStepWarps * 32, 0);
   if (per_sm < 1) per_sm = 1;
-  return per_sm * num_sms();
+  grid = per_sm * num_sms();
+  return grid;
 }
 
 cudaError_t b_one_step(const BatchLayout& L, const BatchView& v, int n, const float* V, const int32_t* in,
                        int32_t* out, int per_thread, int grid, cudaStream_t s) {
   const long long nc = L.n_cells;
   const int chunk = 32 * per_thread;  // ids per work item as counted in n_items
-  const long long row_warps = (nc + kRowsPerWarp - 1) / kRowsPerWarp;
-  k_b_rows<<<(unsigned)((row_warps * 32 + 255) / 256), 256, 0, s>>>(in, v.descs, v.cell_sim, nc, L.NB, v.T, v.bp, v.nbk,
-                                                                    v.reach, out, v.row_map, v.hdr);
+  const bool many = nc >= kManyCells;
+  const long long row_warps = many ? (nc + kRowsPerWarp - 1) / kRowsPerWarp : nc;
+  const unsigned row_blocks = (unsigned)((row_warps * 32 + 255) / 256);
+  if (many)
+    k_b_rows<kRowsPerWarp><<<row_blocks, 256, 0, s>>>(in, v.descs, v.cell_sim, nc, L.NB, v.T, v.bp, v.nbk, v.reach, out,
+                                                      v.row_map, v.hdr);
+  else
+    k_b_rows<1><<<row_blocks, 256, 0, s>>>(in, v.descs, v.cell_sim, nc, L.NB, v.T, v.bp, v.nbk, v.reach, out, v.row_map,
+                                           v.hdr);
   k_b_scan1<<<L.n_blk, kScanThreads, 0, s>>>(v.T, v.reach, v.nbk, v.descs, v.cell_sim, nc, chunk, v.blk);
   k_b_scan2<<<1, kScanThreads, 0, s>>>(v.blk, L.n_blk, L.max_items, v.hdr, 1);
   k_b_scan3<<<L.n_blk, kScanThreads, 0, s>>>(v.T, v.reach, v.nbk, v.descs, v.cell_sim, nc, chunk, v.blk, v.G, v.U, v.occ,
@@ -866,17 +892,18 @@ cudaError_t b_one_step(const BatchLayout& L, const BatchView& v, int n, const fl
   k_b_simbase<<<(n + 127) / 128, 128, 0, s>>>(v.descs, n, v.G, v.sim_base, v.hdr);
   const int rows_blocks = (int)((nc + kBatchRowWarps - 1) / kBatchRowWarps);
   const int rb = rows_blocks < 8 * num_sms() ? rows_blocks : 8 * num_sms();
-  const int live_blocks = (int)((nc + 255) / 256);
-  k_b_live<<<live_blocks < rb ? live_blocks : rb, 256, 0, s>>>(V, v.descs, v.cell_sim, v.occ, v.live, v.hdr);
-  if (L.H <= 32)
-    k_b_kernel_rows<1><<<rb, kBatchRowWarps * 32, 0, s>>>(V, v.descs, v.cell_sim, v.occ, v.live, v.hdr, v.sine, L.NM,
-                                                          v.cdf, v.thr_cell);
-  else if (L.H <= 64)
-    k_b_kernel_rows<2><<<rb, kBatchRowWarps * 32, 0, s>>>(V, v.descs, v.cell_sim, v.occ, v.live, v.hdr, v.sine, L.NM,
-                                                          v.cdf, v.thr_cell);
-  else
-    k_b_kernel_rows<4><<<rb, kBatchRowWarps * 32, 0, s>>>(V, v.descs, v.cell_sim, v.occ, v.live, v.hdr, v.sine, L.NM,
-                                                          v.cdf, v.thr_cell);
+  auto rows = [&](auto live) {
+    constexpr bool LIVE = decltype(live)::value;
+    const auto k = L.H <= 32 ? k_b_kernel_rows<1, LIVE> : (L.H <= 64 ? k_b_kernel_rows<2, LIVE> : k_b_kernel_rows<4, LIVE>);
+    k<<<rb, kBatchRowWarps * 32, 0, s>>>(V, v.descs, v.cell_sim, v.occ, v.live, v.hdr, v.sine, L.NM, v.cdf, v.thr_cell);
+  };
+  if (many) {
+    const int live_blocks = (int)((nc + 255) / 256);
+    k_b_live<<<live_blocks < rb ? live_blocks : rb, 256, 0, s>>>(V, v.descs, v.cell_sim, v.occ, v.live, v.hdr);
+    rows(std::true_type{});
+  } else {
+    rows(std::false_type{});
+  }
   BatchStepArgs a;
   a.hist_in = in;
   a.hist_out = out;
@@ -906,9 +933,14 @@ cudaError_t b_one_step(const BatchLayout& L, const BatchView& v, int n, const fl
   return cudaGetLastError();
 }
 
+// Executable graphs of the step pair a -> b -> a for the last few
+// configurations used, as in the single form: a caller that goes from one batch
+// to another and back does not recapture (a pass over 58 small simulations,
+// three batches in turn: most of its 430 us was capture and instantiation).
+constexpr int kBatchGraphs = 4;
 struct BatchGraph {
-  std::mutex mu;
   bool valid = false;
+  unsigned long long last_use = 0;
   std::vector<wmc_params> ps;
   const void *V, *a, *b, *ws;
   int per;
@@ -916,7 +948,12 @@ struct BatchGraph {
   int device;
   cudaGraphExec_t exec = nullptr;
 };
-BatchGraph g_bgraph;
+struct BatchGraphs {
+  std::mutex mu;
+  unsigned long long uses = 0;
+  BatchGraph slot[kBatchGraphs];
+};
+BatchGraphs g_bgraph;
 
 bool valid_per(int per) { return per == 4 || per == 8 || per == 16 || per == 32 || per == 64 || per == 128 || per == 256; }
 
@@ -1012,16 +1049,23 @@ wmc_status wmc_batch_run(const wmc_params* ps, int32_t n_sims, const float* V, i
     std::lock_guard<std::mutex> lock(g_bgraph.mu);
     int dev = 0;
     cudaGetDevice(&dev);
-    bool hit = g_bgraph.valid && (int)g_bgraph.ps.size() == n_sims && g_bgraph.V == V && g_bgraph.a == hist_a &&
-               g_bgraph.b == hist_b && g_bgraph.ws == ws && g_bgraph.per == per_thread && g_bgraph.stream == s &&
-               g_bgraph.device == dev;
-    if (hit) hit = memcmp(g_bgraph.ps.data(), ps, sizeof(wmc_params) * n_sims) == 0;
-    if (!hit) {
-      if (g_bgraph.exec) {
-        cudaGraphExecDestroy(g_bgraph.exec);
-        g_bgraph.exec = nullptr;
+    BatchGraph *hit = nullptr, *victim = &g_bgraph.slot[0];
+    for (BatchGraph& g : g_bgraph.slot) {
+      if (g.valid && (int)g.ps.size() == n_sims && g.V == V && g.a == hist_a && g.b == hist_b && g.ws == ws &&
+          g.per == per_thread && g.stream == s && g.device == dev &&
+          memcmp(g.ps.data(), ps, sizeof(wmc_params) * n_sims) == 0) {
+        hit = &g;
+        break;
       }
-      g_bgraph.valid = false;
+      if (!g.valid || (victim->valid && g.last_use < victim->last_use)) victim = &g;
+    }
+    if (!hit) {
+      BatchGraph& gs = *victim;
+      if (gs.exec) {
+        cudaGraphExecDestroy(gs.exec);
+        gs.exec = nullptr;
+      }
+      gs.valid = false;
       cudaGraph_t graph = nullptr;
       if (cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal) != cudaSuccess) return WMC_ERR_CUDA;
       cudaError_t e = b_one_step(L, v, n_sims, V, hist_a, hist_b, per_thread, grid, s);
@@ -1031,21 +1075,26 @@ wmc_status wmc_batch_run(const wmc_params* ps, int32_t n_sims, const float* V, i
         if (graph) cudaGraphDestroy(graph);
         return WMC_ERR_CUDA;
       }
-      e = cudaGraphInstantiate(&g_bgraph.exec, graph, 0);
+      e = cudaGraphInstantiate(&gs.exec, graph, 0);
       cudaGraphDestroy(graph);
-      if (e != cudaSuccess) return WMC_ERR_CUDA;
-      g_bgraph.valid = true;
-      g_bgraph.ps.assign(ps, ps + n_sims);
-      g_bgraph.V = V;
-      g_bgraph.a = hist_a;
-      g_bgraph.b = hist_b;
-      g_bgraph.ws = ws;
-      g_bgraph.per = per_thread;
-      g_bgraph.stream = s;
-      g_bgraph.device = dev;
+      if (e != cudaSuccess) {
+        gs.exec = nullptr;
+        return WMC_ERR_CUDA;
+      }
+      gs.valid = true;
+      gs.ps.assign(ps, ps + n_sims);
+      gs.V = V;
+      gs.a = hist_a;
+      gs.b = hist_b;
+      gs.ws = ws;
+      gs.per = per_thread;
+      gs.stream = s;
+      gs.device = dev;
+      hit = &gs;
     }
+    hit->last_use = ++g_bgraph.uses;
     for (int q = 0; q < pairs; ++q)
-      if (cudaGraphLaunch(g_bgraph.exec, s) != cudaSuccess) return WMC_ERR_CUDA;
+      if (cudaGraphLaunch(hit->exec, s) != cudaSuccess) return WMC_ERR_CUDA;
   } else {
     for (int q = 0; q < pairs; ++q) {
       if (b_one_step(L, v, n_sims, V, hist_a, hist_b, per_thread, grid, s) != cudaSuccess) return WMC_ERR_CUDA;

@@ -60,15 +60,15 @@ def test_walk_bit_exact(wmc, kind, n_x, Q, n_M):
 
 
 def test_more_event_quads_than_the_queue(wmc):
-    """2^19 queue entries, more quads with events in a step."""
+    """2^21 queue entries, more quads with events in a step."""
     wl, V = _workload(40, 32, 64)
     rng = np.random.Generator(np.random.PCG64(1))
-    h0 = rng.integers(-8000, 8000, size=(40, 64)).astype(np.int32)
+    h0 = rng.integers(-32000, 32000, size=(40, 64)).astype(np.int32)
     wl = wl.replace(dt_s=4e-16)
     full, half = oracle_tables(wl, V)
     ref, st = oracle.simulate(oracle.params(wl), h0, 1, 1, table=full)
     got, c = gpu_run_table(wmc, torch, wmc.Params.of(wl), half, h0, 1, 1)
-    assert st[oracle.ST_PAIRS] > 2 * 2 ** 19
+    assert st[oracle.ST_PAIRS] > 2 * 2 ** 21
     np.testing.assert_array_equal(got, ref)
     assert c["pairs"] == st[oracle.ST_PAIRS] and c["flags"] == 0
 
