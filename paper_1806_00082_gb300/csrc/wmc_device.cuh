@@ -207,15 +207,29 @@ __device__ __forceinline__ int cell_needs_kernel(const unsigned char* reach, int
 
 // Index of p' for the 53-bit uniform integer U2 in a fixed-point CDF row c of
 // n_M columns: target = floor(U2 Qtot / 2^53), Qtot = c[n_M - 1], and the
-// smallest k with c[k] > target (always exists, since target < Qtot).
+// smallest k with c[k] > target (always exists, since target < Qtot).  A chain
+// of dependent loads, so each step takes three at once and leaves a quarter of
+// the columns.
 __device__ __forceinline__ int sample_cdf_row(const long long* __restrict__ c, int n_M, unsigned long long U2) {
   const unsigned long long Qtot = (unsigned long long)__ldg(c + n_M - 1);
   const long long target = (long long)((__umul64hi(U2, Qtot) << 11) | ((U2 * Qtot) >> 53));
   int lo = 0, hi = n_M - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi) >> 1;
-    if (__ldg(c + mid) > target) hi = mid; else lo = mid + 1;
+  while (hi - lo > 3) {
+    const int q = (hi - lo) >> 2, m1 = lo + q, m2 = m1 + q, m3 = m2 + q;
+    const long long c1 = __ldg(c + m1), c2 = __ldg(c + m2), c3 = __ldg(c + m3);
+    if (c2 > target) {
+      hi = c1 > target ? m1 : m2;
+      if (c1 <= target) lo = m1 + 1;
+    } else {
+      lo = c3 > target ? m2 + 1 : m3 + 1;
+      if (c3 > target) hi = m3;
+    }
   }
+  int below = 0;
+#pragma unroll
+  for (int u = 0; u < 3; ++u)
+    if (lo + u < hi) below += __ldg(c + lo + u) <= target;
+  lo += below;
   return lo;
 }
 

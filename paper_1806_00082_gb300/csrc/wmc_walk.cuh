@@ -35,7 +35,11 @@
 
 namespace wmc {
 
-constexpr uint32_t kLaneBucket = 8;
+// With 4, 8, 16 and 32: 16384 cells, four steps 1320, 1238, 1207 and 1207 us; 2000
+// cells, twenty steps 306, 306, 305 and 312 us; 512 simulations, four steps 3346,
+// 3286, 3263 and 3300 us; 38 simulations of 2.5e7 scattered particles, four steps
+// 1379, 1274, 1163 and 1147 us.
+constexpr uint32_t kLaneBucket = 16;
 
 // Move entry of a column: bits 1-2 drift direction + 1, bits 8-31 the crossing
 // threshold on the offset word w (move_threshold).  A right-moving column's
@@ -194,10 +198,11 @@ struct RangeSchedule {
   uint32_t n_warps;
   uint32_t start, size, ticket;  // current round: first unit, units a range, first ticket
 
-  __device__ __forceinline__ RangeSchedule(uint32_t units, uint32_t warps, uint32_t most = kMaxRange)
+  __device__ __forceinline__ RangeSchedule(uint32_t units, uint32_t warps, uint32_t most = kMaxRange,
+                                           uint32_t single = kSingleRound)
       : total(units), n_warps(warps), start(0u), ticket(0u) {
-    size = units <= kSingleRound * warps ? (units + warps - 1u) / warps : most;
-    if (units > kSingleRound * warps) fit();
+    size = units <= single * warps ? (units + warps - 1u) / warps : most;
+    if (units > single * warps) fit();
   }
   // halves the range size while a round of it would take more than half of what is left
   __device__ __forceinline__ void fit() {
@@ -330,17 +335,18 @@ __device__ __forceinline__ void walk_ids(const C& c, uint32_t r0, uint32_t r1, i
         const int k = min((B.b << 5) + lane, c.n_M() - 1);
         uint32_t above = 0u;
 #pragma unroll
-        for (uint32_t t = 0; t < kLaneBucket / 2; ++t)
-          if (t < cnt) above += w[t] > th;
-        if (most > kLaneBucket / 2) {
+        for (uint32_t t0 = 0; t0 < kLaneBucket; t0 += 4) {
+          if (t0 && most <= t0) break;
 #pragma unroll
-          for (uint32_t t = kLaneBucket / 2; t < kLaneBucket; ++t)
+          for (uint32_t t = t0; t < t0 + 4; ++t)
             if (t < cnt) above += w[t] > th;
         }
         const uint32_t mv = (B.e & 6u) == 0u ? cnt - above : above;
         if (cnt) count(k, B.e, cnt - mv, mv);
+        // candidate quads with ids in this block: their ids in the lanes' buckets
+        const unsigned span = (0xffffffffu << ((x - a) >> 2)) & (0xffffffffu >> (31u - ((lim - 1u - a) >> 2)));
 #pragma unroll 1
-        for (unsigned cd = cand; cd; cd &= cd - 1u) {  // candidate quads: their ids in the lanes' buckets
+        for (unsigned cd = cand & span; cd; cd &= cd - 1u) {
           const uint32_t q0 = a + 4u * (uint32_t)(__ffs(cd) - 1);
           const uint32_t in = first_mask((int)(from + cnt - q0)) & ~first_mask((int)(from - q0));
           const bool me = cnt && in;
