@@ -533,15 +533,21 @@ __device__ __forceinline__ void a_run_window(const float* w, int h, int cell, in
 // of 64 K values, 32 columns each, at columns 0 .. 255), built once and used
 // by every column tile; two 128-column FP32 accumulator buffers at columns
 // 256 and 384 let the epilogue of tile j overlap the MMAs of tile j + 1; the
-// shared memory holds a ring of 11 B stages (one 128-column x 64-K image
-// each), so the tensor core reads only B from shared memory and the ring
+// shared memory holds a ring of kTaStages B stages (128 columns x two 64-K
+// blocks each), so the tensor core reads only B from shared memory and the ring
 // covers a copy round trip.  Builder warp w writes TMEM lanes 32 (w % 4) ..
 // + 31 (one row of the tile per thread) for the K blocks kb = w / 4 (mod 4):
 // its row's entries, packed in pairs, by tcgen05.st, then arrives on
-// a_ready[kb].  The MMA thread waits for a_ready (first tile), each B stage
-// and a drained accumulator buffer, commits each stage and each tile.  Every
-// wait is bounded; on a timeout an abort flag makes all roles drain to the
-// final barrier, after which TMEM is freed.
+// a_ready[kb].  Two threads issue the MMAs, one the even and one the odd column
+// tiles: each waits for a_ready (its first tile), each B stage and its drained
+// accumulator buffer, and commits each stage and each tile.  Every wait is
+// bounded; on a timeout an abort flag makes all roles drain to the final
+// barrier, after which TMEM is freed.
+// What bounds it: building A, then the commits between the MMAs (with one
+// issuing thread and a commit per K block they ran at a third of the pipe's
+// rate).  BF16, 16384 cells at Q = 1024: 22.8 -> 19.0 us with two issuers and
+// stages of two blocks; N = 2, FP16, 3600 cells: 57 -> 12.7 us, its terms no
+// longer chosen by divergent branches.
 constexpr int kTaStages = 5;        // stages of two 64-K blocks
 constexpr int kTaThreads = kWsBuilders + 96;
 constexpr uint32_t kTaStageBytes = 2 * kTileBytes;
