@@ -86,3 +86,45 @@ def test_a_gradient_that_is_not_finite_shows_in_every_parameter(wmc):
     gb[0, 7] = float("inf")
     got = wmc.potential_tanh_vjp(p, T, 16, 16, 0.5, gb)
     assert not torch.isfinite(got).any()
+
+
+def _fma32(a, b, c):
+    """a b + c of FP32 arrays, rounded once: the product is exact in FP64, the
+    FP64 sum is rounded to odd (by its TwoSum error), which rounds on correctly."""
+    p, c = a.astype(np.float64) * b.astype(np.float64), c.astype(np.float64)
+    s = p + c
+    t = s - p
+    err = (p - (s - t)) + (c - t)
+    even = (s.view(np.int64) & 1) == 0
+    s = np.where((err != 0) & even, np.nextafter(s, np.where(err > 0, np.inf, -np.inf)), s)
+    return s.astype(np.float32)
+
+
+@pytest.mark.parametrize("n_x,nb,ns", [(300, 2, 0), (700, 3, 5), (1000, 0, 300), (4096, 16, 16)])
+def test_potential_sums_each_window_by_one_rounding(wmc, n_x, nb, ns):
+    """V bit for bit: the windows' values (each by itself, with height one) times
+    their heights, added in turn with one rounding each, whether a window lies
+    within the reach of the exponentials or is passed over."""
+    p = _params(wmc, n_x, 64)
+    rng = np.random.Generator(np.random.PCG64(n_x + ns))
+    L, eps = n_x * 0.25, 0.5
+    heights = np.r_[rng.uniform(0.05, 0.3, nb), rng.uniform(-0.02, 0.02, ns)].astype(np.float32)
+    centres, widths = rng.uniform(0, L, nb), rng.uniform(1, 5, nb)
+    if nb:  # edges 52.9 and 53.1 eps from the centre of cell 0, where windows begin to be passed over
+        widths[0], centres[0] = 0.2 * eps, 0.125 + 53.0 * eps
+    place = np.r_[widths, centres].astype(np.float32)
+
+    def potential(hs):  # hs [n, nb + ns]
+        th = np.concatenate([hs[:, :nb], np.tile(place, (len(hs), 1)), hs[:, nb:]], 1).astype(np.float32)
+        return wmc.potential_tanh(p, torch.from_numpy(th).cuda(), nb, ns, eps).cpu().numpy()
+
+    w = potential(np.eye(nb + ns))
+    assert (w == 0).any() and ((w != 0) & (w < 1)).any()
+    ref = np.zeros(n_x, np.float32)
+    for k in range(nb + ns):
+        ref = _fma32(np.full(n_x, heights[k]), w[k], ref)
+    np.testing.assert_array_equal(potential(heights[None])[0], ref)
+    for k in {0, nb + ns - 1}:
+        bad = heights.copy()
+        bad[k] = np.inf
+        assert not np.isfinite(potential(bad[None])).any()
