@@ -31,6 +31,7 @@
 #include <cuda_fp16.h>
 
 #include "wmc_device.cuh"
+#include "wmc_ta_ring.cuh"
 
 namespace wmc {
 
@@ -539,19 +540,19 @@ __device__ __forceinline__ void a_run_window(const float* w, int h, int cell, in
 // + 31 (one row of the tile per thread) for the K blocks kb = w / 4 (mod 4):
 // its row's entries, packed in pairs, by tcgen05.st, then arrives on
 // a_ready[kb].  Two threads issue the MMAs, one the even and one the odd column
-// tiles: each waits for a_ready (its first tile), each B stage and its drained
-// accumulator buffer, and commits each stage and each tile.  Every wait is
-// bounded; on a timeout an abort flag makes all roles drain to the final
-// barrier, after which TMEM is freed.
+// tiles: each waits for a_ready (its first tile), each B stage of its tiles (by
+// the barrier of that filling, wmc_ta_ring.cuh) and its drained accumulator
+// buffer, and commits each stage and each tile.  Every wait is bounded; on a
+// timeout an abort flag makes all roles drain to the final barrier, after which
+// TMEM is freed.
 // What bounds it: building A, then the commits between the MMAs (with one
 // issuing thread and a commit per K block they ran at a third of the pipe's
 // rate).  BF16, 16384 cells at Q = 1024: 22.8 -> 19.0 us with two issuers and
 // stages of two blocks; N = 2, FP16, 3600 cells: 57 -> 12.7 us, its terms no
 // longer chosen by divergent branches.
-constexpr int kTaStages = 5;        // stages of two 64-K blocks
 constexpr int kTaThreads = kWsBuilders + 96;
 constexpr uint32_t kTaStageBytes = 2 * kTileBytes;
-constexpr int kTaMaxKB = 8;
+static_assert((kTaMaxKB * TK + 1 + TN - 1) / TN <= kTaMaxTiles, "h <= kTaMaxKB TK + 1 columns");
 constexpr uint32_t kTaAccCol = 256;
 
 __host__ __device__ constexpr size_t ta_window_floats(int h) {
@@ -580,7 +581,7 @@ __global__ __launch_bounds__(kTaThreads, 1) void k_kernel_eval_tc_ta(const float
   uint8_t* sB = smem;                                                     // STG stages of two 128 x 64 blocks
   float* sV = reinterpret_cast<float*>(sB + (size_t)STG * kTaStageBytes);  // window, then epilogue staging
   __shared__ __align__(8) uint64_t a_ready[kTaMaxKB];
-  __shared__ __align__(8) uint64_t b_full[kTaStages], b_empty[kTaStages];
+  __shared__ __align__(8) uint64_t b_full[kTaFills], b_empty[kTaStages];
   __shared__ __align__(8) uint64_t acc_full[2], acc_empty[2];
   __shared__ __align__(8) uint64_t drain[2];
   __shared__ int s_min[kWsBuilders / 32], s_max[kWsBuilders / 32];
@@ -600,10 +601,8 @@ __global__ __launch_bounds__(kTaThreads, 1) void k_kernel_eval_tc_ta(const float
   if (warp == 0) tmem_alloc(&tmem_slot, n_cols);
   if (tid == 0) {
     for (int q = 0; q < KB; ++q) mbar_init(&a_ready[q], 4);  // one arrival per lane-quarter warp
-    for (int q = 0; q < STG; ++q) {
-      mbar_init(&b_full[q], 1);
-      mbar_init(&b_empty[q], 1);
-    }
+    for (int q = 0; q < n_tiles; ++q) mbar_init(&b_full[q], 1);
+    for (int q = 0; q < STG; ++q) mbar_init(&b_empty[q], 1);
     for (int q = 0; q < 2; ++q) {
       mbar_init(&acc_full[q], 1);
       mbar_init(&acc_empty[q], kWsBuilders / 32);  // one arrival per epilogue warp
@@ -622,28 +621,29 @@ __global__ __launch_bounds__(kTaThreads, 1) void k_kernel_eval_tc_ta(const float
     if (lane == 0) {
       int issued = 0;
       for (int t = 0; t < n_tiles && !s_abort; ++t) {
-        const int st = t % STG;
-        if (t >= STG && !mbar_wait(&b_empty[st], (uint32_t)(((t / STG) - 1) & 1))) {
+        const int st = ta_stage(t);
+        uint64_t* full = &b_full[ta_full_bar(t)];
+        if (t >= STG && !mbar_wait(&b_empty[st], ta_empty_parity(t))) {
           atomicOr(flags, WMC_FLAG_TIMEOUT);
           s_abort = 1;
           break;
         }
         const int nt = nt_begin + t / KP, kb = 2 * (t % KP);
         const uint32_t bytes = kb + 1 < KB ? kTaStageBytes : kTileBytes;
-        mbar_expect_tx(&b_full[st], bytes);
-        bulk_g2s(sB + (size_t)st * kTaStageBytes, img_b + ((size_t)nt * KB + kb) * (kTileBytes / 2), bytes, &b_full[st]);
+        mbar_expect_tx(full, bytes);
+        bulk_g2s(sB + (size_t)st * kTaStageBytes, img_b + ((size_t)nt * KB + kb) * (kTileBytes / 2), bytes, full);
         issued = t + 1;
       }
       if (s_abort)  // let the copies still in flight land before the CTA exits (bounded)
         for (int t = max(0, issued - STG); t < issued; ++t)
-          (void)mbar_wait(&b_full[t % STG], (uint32_t)((t / STG) & 1));
+          (void)mbar_wait(&b_full[ta_full_bar(t)], ta_full_parity(t));
     }
   } else if (warp == kWsBuilders / 32 || warp == kWsBuilders / 32 + 2) {
     // ---- MMA issuers: one thread the even column tiles (accumulator 0), one the
     // odd ones, so that one's waits and commits pass behind the other's MMAs
     const int buf = warp == kWsBuilders / 32 ? 0 : 1;
     if (lane == 0) {
-      for (int j = buf; j < n_my && !s_abort; j += 2) {
+      for (int j = buf; j < n_my && !s_abort; j += kTaIssuers) {
         if (j >= 2 && !mbar_wait(&acc_empty[buf], (uint32_t)(((j - 2) >> 1) & 1))) {
           atomicOr(flags, WMC_FLAG_TIMEOUT);
           s_abort = 1;
@@ -652,9 +652,9 @@ __global__ __launch_bounds__(kTaThreads, 1) void k_kernel_eval_tc_ta(const float
         tc_fence_after();
         const uint32_t acc = tmem + kTaAccCol + (uint32_t)(buf * TN);
         for (int kb = 0; kb < KB; ++kb) {
-          const int t = j * KP + kb / 2, st = t % STG;
+          const int t = j * KP + kb / 2, st = ta_stage(t);
           if ((j < 2 && !mbar_wait(&a_ready[kb], 0u)) ||
-              ((kb & 1) == 0 && !mbar_wait(&b_full[st], (uint32_t)((t / STG) & 1)))) {
+              ((kb & 1) == 0 && !mbar_wait(&b_full[ta_full_bar(t)], ta_full_parity(t)))) {
             atomicOr(flags, WMC_FLAG_TIMEOUT);
             s_abort = 1;
             break;

@@ -219,3 +219,28 @@ def test_fp32_request_runs_the_stated_form(wmc, wl, form):
     a = wmc.kernel_eval(p, V, occ, ws, prec=wmc.FP32).cpu().numpy()
     b = wmc.kernel_eval(p, V, occ, ws, prec=wmc.PRECISIONS[form]).cpu().numpy()
     assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("form", ["bf16", "fp16"])
+@pytest.mark.parametrize("net,Q", [(1, 386), (1, 516), (1, 772), (1, 1026), (2, 642), (2, 1024)])
+def test_ring_of_b_stages_goes_round(wmc, net, Q, form):
+    """All column tiles in one CTA (a tile of rows for every SM, so the B stages
+    are filled up to twenty times) against calls of 128 rows, whose tiles are
+    split over CTAs that hardly reuse a stage: the same bits, call after call."""
+    n_x = 128 * torch.cuda.get_device_properties(0).multi_processor_count
+    wl = wi.DOUBLE_BARRIER_16384.replace(n_x=n_x, Q=Q, n_M=Q)
+    p = wmc.Params.of(wl)
+    ws = wmc.workspace(p)
+    wmc.init(p, ws)
+    V = torch.from_numpy(np.random.Generator(np.random.PCG64(Q)).uniform(-0.2, 0.3, n_x).astype(np.float32)).cuda()
+    f = wmc.kernel_eval if net == 1 else wmc.kernel_eval_n2
+    occ = torch.arange(n_x, dtype=torch.int32, device="cuda")
+    prec = wmc.PRECISIONS[form]
+    parts = [(r0, f(p, V, occ[r0:r0 + 128], ws, prec)) for r0 in range(0, n_x, 128 * 19)]
+    out = torch.empty((n_x, Q // 2), device="cuda")
+    for _ in range(20):
+        out.fill_(float("nan"))
+        f(p, V, occ, ws, prec, out)
+        for r0, ref in parts:
+            assert torch.equal(out[r0:r0 + 128], ref)
+    assert torch.isfinite(out).all() and wmc.get_counters(p, ws)["flags"] == 0
