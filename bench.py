@@ -605,7 +605,7 @@ def n2_train_rate(wmc, torch, dev, stream, n_examples=100, epochs=200, n_runs=15
     """The trained N = 2 network (Sec. 2.3): 100 Gaussian-bump potentials on
     256 cells (Q = n_M = 64), 200 epochs of SGD (one example per step), a sweep
     of n_runs learning rates log-spaced over [1e-5, 1e-2] (the paper's 1e-5,
-    1e-4, 1e-3 among them), one thread block per run, all in one launch; the
+    1e-4, 1e-3 among them), a cluster of thread blocks per run, all in one launch; the
     exact kernels from wmc_kernel_eval_rows.  The FP64 oracle's SGD step is
     timed on a bounded sample of steps."""
     from paper_1806_00082_gb300 import n2train

@@ -291,12 +291,16 @@ wmc_status wmc_kernel_eval_n2(const wmc_params* p, const float* V, const int32_t
  *          period (columns j = 0 .. h - 1, e.g. from wmc_kernel_eval_rows).
  *   order  [dev] int32[epochs][n_examples]: the examples of each epoch in turn.
  *   lr     [dev] float[n_runs]: runs train the same examples in the same order,
- *          one learning rate each (one thread block per run).
+ *          one learning rate each (a cluster of one to eight thread blocks per
+ *          run, as many as the SMs hold for all of them).
  *   params [dev] float[n_runs][Q + 4]: initial weights in, trained weights out.
  *   loss   [dev] float[n_runs][epochs] or NULL: mean loss of each epoch (each
  *          step's loss taken before its update).
  * n_x even; WMC_ERR_UNSUPPORTED if n_x (Q/2 + 1) + Q^2 floats exceed the shared
- * memory of one block (about 200 KB).  Deterministic for given inputs. */
+ * memory of one block (about 200 KB).  Deterministic: a run's result follows
+ * from its own inputs alone, whatever other runs the call has and on any GPU.
+ * The rounding of the parameters is carried from step to step within a call, so
+ * training cut into several calls may differ from one call in the last bits. */
 wmc_status wmc_n2_train(const wmc_params* p, int32_t n_examples, const float* V, const float* VW, int32_t epochs,
                         const int32_t* order, int32_t n_runs, const float* lr, float* params, float* loss,
                         wmc_stream_t stream);

@@ -18,11 +18,14 @@
 //
 // k_n2_train: one cluster of CTAs per training run (runs differ in learning
 // rate; they train on the same examples in the same order), the whole SGD loop
-// inside it.  The rows of an example are split over the CTAs; each builds the
-// phase tables (sincospif of the current wt) for itself, its residuals and its
-// share of the gradient; the shares are exchanged through distributed shared
-// memory with one cluster barrier per step and added in rank order by every
-// CTA, so all of them make the same update and a run is deterministic.
+// inside it.  The rows of an example are cut into up to eight parts, by n_x
+// alone, and the parts shared out over the CTAs; each CTA builds the phase tables
+// (sincospif of the current wt) for itself, its residuals and its share of the
+// gradient; the shares are exchanged through distributed shared memory with one
+// cluster barrier per step and every CTA adds them, so all of them make the same
+// update.  Every sum is taken within a part and then over the parts in pairs, in
+// an order that does not depend on the number of CTAs: a run's result is the same
+// beside any other runs and on any GPU.
 // k_n2_eval: the trained model's rows, in 1/s, for given parameters.
 #include <cooperative_groups.h>
 
@@ -35,26 +38,47 @@ namespace {
 constexpr float kPiF = 3.14159265358979f;  // pi rounded to FP32
 constexpr int kN2Threads = 512;
 constexpr int kN2Warps = kN2Threads / 32;
-constexpr int kN2MaxCluster = 8;
+constexpr int kN2MaxParts = 8;  // parts of the rows, and CTAs of a cluster
+
+// Parts of the rows: as many as hold four row pairs each.
+__host__ __device__ inline int n2_parts(int n_x) {
+  int P = 1;
+  while (2 * P <= kN2MaxParts && n_x / 2 >= 4 * 2 * P) P *= 2;
+  return P;
+}
 
 // Sizes of k_n2_train with the rows over C CTAs.  Rows and pair offsets are
 // held by parity (row i meets the offsets dd = d + h of parity (i + h) mod 2):
-// M row pairs per CTA and h offsets, both padded to fours for 16-byte loads.
+// G groups of four row pairs, part c of P the groups [G c / P, G (c + 1) / P), up
+// to Mp row pairs per CTA, and h offsets padded to hp, a multiple of four, for
+// 16-byte loads.
 struct N2Shape {
-  int h, hp, M, Mp;
+  int h, hp, G, Mp, parts;  // parts: of one CTA
   __host__ __device__ N2Shape(int n_x, int Q, int C)
-      : h(Q / 2), hp((Q / 2 + 3) & ~3), M((n_x / 2 + C - 1) / C), Mp(((n_x / 2 + C - 1) / C + 3) & ~3) {}
-  // sin and phi-weighted cos tables [h][2][hp]; W P [h][2][Mp], later the W
-  // gradient's parts [Mp / 4][2][hp]; residuals [2][h][Mp]; V of the rows'
-  // windows; cos(pi j / Q); parameters; the exchanged sums, two buffers;
-  // reduction scratch
+      : h(Q / 2), hp((Q / 2 + 3) & ~3), G((n_x / 2 + 3) / 4), Mp(4 * ((G + C - 1) / C)), parts(n2_parts(n_x) / C) {}
+  // sin and phi-weighted cos tables [h][2][hp]; W P [h][2][Mp], later the sums of
+  // the groups, [Mp / 4][2][hp] of the W gradient and as many of the other four;
+  // residuals [2][h][Mp]; V of the rows' windows; cos(pi j / Q); parameters; the
+  // exchanged sums, two buffers; the loss of the groups [Mp / 4][2][hp / 4]
   __host__ __device__ size_t table() const { return (size_t)h * 2 * hp; }
   __host__ __device__ size_t rows() const { return (size_t)h * 2 * Mp; }
   __host__ __device__ size_t window() const { return (size_t)2 * Mp + 2 * h + 4; }
+  __host__ __device__ size_t exchanged() const { return (size_t)2 * h + 5 * parts; }
+  __host__ __device__ size_t losses() const { return (size_t)(Mp / 4) * 2 * (hp / 4); }
   __host__ __device__ size_t floats() const {
-    return 2 * table() + 2 * rows() + ((window() + 3) & ~(size_t)3) + hp + (2 * h + 4) + 2 * (2 * h + 5) + 5 * kN2Warps;
+    return 2 * table() + 2 * rows() + ((window() + 3) & ~(size_t)3) + hp + (2 * h + 4) + 2 * exchanged() + losses();
   }
 };
+
+// Sum over the parts in pairs (entries past the last are zero): the sum of
+// aligned runs of parts, then of the runs' sums, is the same sum.
+__device__ __forceinline__ float n2_pairwise(float (&x)[kN2MaxParts]) {
+#pragma unroll
+  for (int w = 1; w < kN2MaxParts; w *= 2)
+#pragma unroll
+    for (int c = 0; c < kN2MaxParts; c += 2 * w) x[c] += x[c + w];
+  return x[0];
+}
 
 __device__ __forceinline__ float n2_pot(const float* __restrict__ V, int n_x, int bc, int l) {
   if (l >= 0 && l < n_x) return __ldg(V + l);
@@ -68,8 +92,12 @@ __device__ __forceinline__ float n2_pot(const float* __restrict__ V, int n_x, in
 // 4 rows x 4 offsets of the gradient sums: 16 and 32 FMAs for 5 and 3 loads of
 // shared memory (one load per FMA, 40 k shared-memory cycles a step, bound the
 // form with one output per thread at 36 us a step on one SM).  256 cells, Q =
-// 64, three runs: 6.9 us a step with eight CTAs per run, bound by the
-// barriers and the chain of phases.
+// 64, three runs: 6.9 us a step with eight CTAs per run.  There a CTA has 64
+// tiles, so two of its sixteen warps do the residuals and the gradient sums, with
+// little to hide their latency: by clock stamps 2800 and 4500 of 14600 cycles a
+// step, the tables 2800, W P 1500, the sums and their exchange 3000.  152 runs
+// of one CTA each: 20.8 us a step (19.8 with sums whose order followed the
+// number of CTAs).
 __global__ __launch_bounds__(kN2Threads) void k_n2_train(int n_x, int Q, int bc, int n_ex, const float* __restrict__ Vs,
                                                           const float* __restrict__ VW, float scale, int epochs,
                                                           const int* __restrict__ order, const float* __restrict__ lr,
@@ -80,7 +108,8 @@ __global__ __launch_bounds__(kN2Threads) void k_n2_train(int n_x, int Q, int bc,
   const int C = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
   const int run = blockIdx.x / C;
   const N2Shape z(n_x, Q, C);
-  const int h = z.h, hp = z.hp, M = z.M, Mp = z.Mp, NV = Q + 5;  // NV exchanged sums: dW, dwv, dwt, loss
+  // exchanged sums: dW, then dwv, dwt and the loss of each of the CTA's parts
+  const int h = z.h, hp = z.hp, Mp = z.Mp, n_parts = z.parts, NV = (int)z.exchanged();
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   float* sS = sm_n2;              // [h][2][hp]: sin of offset dd (parity, dd / 2) at column j
   float* sC = sS + z.table();     // phi_j times the cosines
@@ -90,23 +119,30 @@ __global__ __launch_bounds__(kN2Threads) void k_n2_train(int n_x, int Q, int bc,
   float* sCJ = sV + ((z.window() + 3) & ~(size_t)3);
   float* sP = sCJ + hp;           // parameters
   float* sX = sP + (Q + 4);       // exchanged sums, by step parity
-  float* red = sX + 2 * NV;       // [5][warps]
-  float* sGp = sWP;               // the W gradient's parts, once W P has been used
-  const int m0 = rank * M, m_n = max(0, min(M, n_x / 2 - m0));  // this CTA's row pairs
-  const int i0 = 2 * m0;
+  float* sL = sX + 2 * NV;        // the groups' losses
+  // this CTA's groups of row pairs, its row pairs and its first row
+  const int g0 = (int)((long long)z.G * rank / C), RG = (int)((long long)z.G * (rank + 1) / C) - g0;
+  const int m_n = min(4 * RG, n_x / 2 - 4 * g0), i0 = 8 * g0;
+  float* sGp = sWP;               // the W gradient of the groups, once W P has been used
+  // their sums for dwv1, dwv2, dwt1, dwt2 (one column: in the place of the residuals, which no sum reads)
+  float* sG4 = h > 1 ? sGp + (size_t)RG * 2 * hp : sR;
+  // first group of each of the CTA's parts (and the end of the last), and log2 of their number
+  __shared__ int s_first[kN2MaxParts + 1];
+  if (tid <= n_parts) s_first[tid] = (int)((long long)z.G * (rank * n_parts + tid) / (C * n_parts)) - g0;
+  const int log_parts = __ffs(n_parts) - 1;
   const float rate = __ldg(lr + run);
   float* prm = params + (size_t)run * (Q + 4);
   for (int q = tid; q < Q + 4; q += kN2Threads) sP[q] = prm[q];
   for (int j = tid; j < h; j += kN2Threads) sCJ[j] = cospif((float)j / (float)Q);
   for (size_t q = tid; q < 2 * z.table(); q += kN2Threads) sS[q] = 0.f;  // (the padding stays zero)
   const float inv_n = 2.f / (float)((long long)n_x * (h - 1));  // d(mean of squares)/dy = inv_n r
-  const int RG = Mp / 4, JG = hp / 4;  // groups of four row pairs, of four columns or offsets
+  const int JG = hp / 4;  // groups of four columns or offsets
   const int n_tasks = 2 * RG * JG;
   __syncthreads();
   int step = 0;
-  // what the rounding of this thread's parameter has left out so far (the sizes
-  // that are accepted have Q <= 226, so a thread holds one at most).  300 steps
-  // of 256 cells, Q = 64: parameters 4.4e-7 -> 2e-8 from FP64, no time.
+  // what the rounding of this thread's parameter has left out so far in this call
+  // (the sizes that are accepted have Q <= 222, so a thread holds one at most).
+  // 300 steps of 256 cells, Q = 64: parameters 4.4e-7 -> 2e-8 from FP64, no time.
   float low = 0.f;
   for (int ep = 0; ep < epochs; ++ep) {
     float ep_loss = 0.f;
@@ -133,7 +169,6 @@ __global__ __launch_bounds__(kN2Threads) void k_n2_train(int n_x, int Q, int bc,
       }
       __syncthreads();
       // residuals
-      float part = 0.f;
       for (int t = tid; t < n_tasks; t += kN2Threads) {
         const int rg = t % RG, jg = (t / RG) % JG, p = t / (RG * JG);
         const int pd = (i0 + p + h) & 1;  // parity of the rows' offsets
@@ -166,6 +201,7 @@ __global__ __launch_bounds__(kN2Threads) void k_n2_train(int n_x, int Q, int bc,
             for (int a = 0; a < 4; ++a) acc[a][b] = fmaf(wa[a], sv, acc[a][b]);
           }
         }
+        float part = 0.f;
 #pragma unroll
         for (int b = 0; b < 4; ++b) {
           const int j = 4 * jg + b;
@@ -182,10 +218,10 @@ __global__ __launch_bounds__(kN2Threads) void k_n2_train(int n_x, int Q, int bc,
             *reinterpret_cast<float4*>(sR + ((size_t)p * h + j) * Mp + 4 * rg) = r4;
           }
         }
+        sL[(rg * 2 + p) * JG + jg] = part;
       }
       __syncthreads();
       // gradient sums of 4 rows x 4 offsets
-      float gv1 = 0.f, gv2 = 0.f, gt1 = 0.f, gt2 = 0.f;
       for (int t = tid; t < n_tasks; t += kN2Threads) {
         const int rg = t % RG, dg = (t / RG) % JG, p = t / (RG * JG);
         const int pd = (i0 + p + h) & 1;
@@ -212,6 +248,7 @@ __global__ __launch_bounds__(kN2Threads) void k_n2_train(int n_x, int Q, int bc,
         }
         float4 g4;
         float* gw = reinterpret_cast<float*>(&g4);
+        float gv1 = 0.f, gv2 = 0.f, gt1 = 0.f, gt2 = 0.f;
 #pragma unroll
         for (int b = 0; b < 4; ++b) {
           const int dd = 2 * (4 * dg + b) + pd, d = dd - h;
@@ -235,36 +272,66 @@ __global__ __launch_bounds__(kN2Threads) void k_n2_train(int n_x, int Q, int bc,
         }
         // (each offset belongs to one row parity, so a slot has one writer)
         *reinterpret_cast<float4*>(sGp + ((size_t)rg * 2 + pd) * hp + 4 * dg) = g4;
-      }
-      float v5[5] = {gv1, gv2, gt1, gt2, part};
-#pragma unroll
-      for (int q = 0; q < 5; ++q) {
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) v5[q] += __shfl_down_sync(0xffffffffu, v5[q], off);
-        if (lane == 0) red[q * kN2Warps + wid] = v5[q];
+        *reinterpret_cast<float4*>(sG4 + ((size_t)rg * 2 + pd) * hp + 4 * dg) = make_float4(gv1, gv2, gt1, gt2);
       }
       __syncthreads();
+      // this CTA's sums: dW over its parts, an offset per thread, and the other
+      // five of each part by one warp
       float* mine = sX + (step & 1) * NV;
-      for (int q = tid; q < NV; q += kN2Threads) {
-        float v = 0.f;
-        if (q < Q)
-          for (int rg = 0; rg < RG; ++rg) v += sGp[((size_t)rg * 2 + (q & 1)) * hp + (q >> 1)];
-        else
-          for (int w = 0; w < kN2Warps; ++w) v += red[(q - Q) * kN2Warps + w];
+      if (const int q = tid; q < Q) {
+        const float* gp = sGp + (size_t)(q & 1) * hp + (q >> 1);
+        float v = 0.f, s1 = 0.f, s2 = 0.f, s4 = 0.f;  // runs of one, two and four parts waiting for their neighbours
+        int rg = 0;
+#pragma unroll 1
+        for (int c = 0; c < n_parts; ++c) {
+          v = 0.f;
+#pragma unroll 4
+          for (const int end = s_first[c + 1]; rg < end; ++rg) v += gp[(size_t)rg * 2 * hp];
+          if (!(c & 1)) {
+            s1 = v;
+            continue;
+          }
+          v = s1 + v;
+          if (!(c & 2)) {
+            s2 = v;
+            continue;
+          }
+          v = s2 + v;
+          if (!(c & 4)) s4 = v;
+          else v = s4 + v;
+        }
         mine[q] = v;
+      }
+      if (const int c = kN2Warps - 1 - wid; c < n_parts) {
+        float v5[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
+        for (int e = s_first[c] * 2 * JG + lane; e < s_first[c + 1] * 2 * JG; e += 32) {
+          const float4 v = *reinterpret_cast<const float4*>(sG4 + 4 * e);
+          v5[0] += v.x, v5[1] += v.y, v5[2] += v.z, v5[3] += v.w, v5[4] += sL[e];
+        }
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1)
+#pragma unroll
+          for (int u = 0; u < 5; ++u) v5[u] += __shfl_down_sync(0xffffffffu, v5[u], off);
+        if (lane == 0)
+          for (int u = 0; u < 5; ++u) mine[Q + 5 * c + u] = v5[u];
       }
       // every CTA's sums are there; the other buffer serves the next step, so
       // that no CTA overwrites sums another still reads
       if (C > 1) cluster.sync();
       else __syncthreads();
-      if (const int q = tid; q < NV) {
-        float x[kN2MaxCluster], v = 0.f;  // (all loads under way before the first sum)
+      if (const int q = tid; q < Q + 5) {
+        // dW from every CTA, the others from every part; without branches, so that
+        // all loads are under way before the first sum (700 cycles a step otherwise)
+        float x[kN2MaxParts];
+        const int n = q < Q ? C : C * n_parts, shift = q < Q ? 0 : log_parts;
 #pragma unroll
-        for (int c = 0; c < kN2MaxCluster; ++c)
-          x[c] = c < C ? (C > 1 ? *(cluster.map_shared_rank(mine, c) + q) : mine[q]) : 0.f;
+        for (int c = 0; c < kN2MaxParts; ++c) {
+          const int u = min(c, n - 1);
+          x[c] = *(cluster.map_shared_rank(mine, u >> shift) + q + 5 * (u & ((1 << shift) - 1)));
+        }
 #pragma unroll
-        for (int c = 0; c < kN2MaxCluster; ++c)
-          if (c < C) v += x[c];
+        for (int c = 0; c < kN2MaxParts; ++c) x[c] = c < n ? x[c] : 0.f;
+        const float v = n2_pairwise(x);
         if (q < Q + 4) {
           const float old = sP[q], up = fmaf(-rate, v, low);
           const float now = __fadd_rn(old, up), d = __fsub_rn(now, old);
@@ -276,7 +343,7 @@ __global__ __launch_bounds__(kN2Threads) void k_n2_train(int n_x, int Q, int bc,
       }
       __syncthreads();
     }
-    if (rank == 0 && tid == (Q + 4) % kN2Threads && loss_out) loss_out[(size_t)run * epochs + ep] = ep_loss / (float)n_ex;
+    if (rank == 0 && tid == Q + 4 && loss_out) loss_out[(size_t)run * epochs + ep] = ep_loss / (float)n_ex;
   }
   if (rank == 0)
     for (int q = tid; q < Q + 4; q += kN2Threads) prm[q] = sP[q];
@@ -335,10 +402,9 @@ wmc_status wmc_n2_train(const wmc_params* p, int32_t n_examples, const float* V,
                        (size_t)(2 * p->Q + 4) + 192) > 200 * 1024)
     return WMC_ERR_UNSUPPORTED;
   if (n_runs == 0 || epochs == 0) return WMC_OK;
-  // CTAs per run: as many as the SMs hold for all runs, with at least four row
-  // pairs each
+  // CTAs per run: as many as the SMs hold for all runs, with at least one part each
   int C = 1;
-  while (2 * C <= kN2MaxCluster && (long long)n_runs * 2 * C <= num_sms() && p->n_x / 2 >= 4 * 2 * C) C *= 2;
+  while (2 * C <= n2_parts(p->n_x) && (long long)n_runs * 2 * C <= num_sms()) C *= 2;
   const size_t sm = sizeof(float) * N2Shape(p->n_x, p->Q, C).floats();
   if (sm > 48 * 1024 && raise_smem_limit(reinterpret_cast<const void*>(k_n2_train), sm) != cudaSuccess)
     return WMC_ERR_CUDA;

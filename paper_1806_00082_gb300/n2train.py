@@ -1,8 +1,8 @@
 """Training of the N = 2 network of Sec. 2.3 (Eq. kernel_ML, N = 2) on the GPU:
 the exact kernels of the example potentials from wmc_kernel_eval_rows (the
-FP32-accuracy form), then stochastic gradient descent in wmc_n2_train, one
-thread block per learning rate.  The trained weights give kernel rows through
-wmc_n2_eval."""
+FP32-accuracy form), then stochastic gradient descent in wmc_n2_train, a
+cluster of thread blocks per learning rate.  The trained weights give kernel
+rows through wmc_n2_eval."""
 from __future__ import annotations
 
 import torch

@@ -118,3 +118,32 @@ def test_sgd_with_the_rows_split_over_ctas(wmc, n_x, q, runs):
         pf, hist = nt.train(p0, Vs, Ts, order, float(lrs[r]), w.Q)
         assert np.linalg.norm(got[r] - pf) <= 1e-2 * np.linalg.norm(pf - p0) + 1e-6
         assert np.all(np.abs(got_loss[r] - hist) <= 1e-4 * hist + 1e-12)
+
+
+@pytest.mark.parametrize("n_x,q,companions", [(256, 64, 2), (256, 64, 29), (256, 64, 59), (256, 64, 151), (66, 14, 151),
+                                              (98, 30, 39), (70, 190, 151), (4, 222, 151)])
+def test_a_run_does_not_depend_on_the_other_runs(wmc, n_x, q, companions):
+    """One learning rate alone (its rows over up to eight CTAs) and among others
+    (over fewer, down to one): the same weights and losses, bit for bit."""
+    w = _wl(n_x=n_x, q=q)
+    n_ex, epochs = 3, 2
+    rng = np.random.default_rng(n_x + companions)
+    Vs = torch.from_numpy(rng.uniform(-0.2, 0.3, (n_ex, n_x)).astype(np.float32)).cuda()
+    p = wmc.Params.of(w)
+    ws = wmc.workspace(p)
+    wmc.init(p, ws)
+    T = wmc.kernel_eval_rows(p, Vs, ws)
+    order = torch.from_numpy(wi.sgd_order(epochs, n_ex)).cuda()
+    lrs = torch.from_numpy(rng.uniform(1e-3, 1e-2, 1 + companions).astype(np.float32)).cuda()
+    start = torch.from_numpy((nt.initial_params(w.Q) + rng.normal(0.0, 0.02, w.Q + 4)).astype(np.float32)).cuda()
+
+    def train(rates):
+        prm, loss = start.repeat(rates.numel(), 1), torch.zeros((rates.numel(), epochs), device="cuda")
+        wmc.n2_train(p, Vs, T, order, rates, prm, loss)
+        return prm, loss
+
+    prm, loss = train(lrs)
+    assert torch.isfinite(prm).all() and torch.isfinite(loss).all()
+    for r in {0, companions // 2, companions}:
+        alone_p, alone_l = train(lrs[r:r + 1].contiguous())
+        assert torch.equal(alone_p[0], prm[r]) and torch.equal(alone_l[0], loss[r])
