@@ -400,16 +400,19 @@ wmc_status wmc_batch_init(const wmc_params* ps, int32_t n_sims, void* ws, size_t
 
 /* n_steps steps of every simulation from hist_a (state after step
  * t_first - 1), hist_b the second buffer, final state in hist_a.
- * per_thread: survivor ids per lane of a work item (4, 8, 16, 32, 64, 128 or
- * 256; 0 = 16), e.g. from wmc_batch_autotune; results do not depend on it.  use_graph
- * as for wmc_run. */
+ * per_thread: survivor ids per lane of the largest ranges a warp takes at a
+ * time (4, 8, 16, 32, 64, 128 or 256; 0 = 16; values up to 64 take the same
+ * ranges), e.g. from wmc_batch_autotune; the histograms do not depend on it.
+ * n_items counts runs of up to 32 per_thread ids of one cell, and a population of
+ * more than 2^23 + 2 x cells of them sets WMC_FLAG_CAPACITY.  use_graph as for
+ * wmc_run. */
 wmc_status wmc_batch_run(const wmc_params* ps, int32_t n_sims, const float* V, int32_t* hist_a, int32_t* hist_b,
                          uint32_t t_first, int32_t n_steps, int32_t per_thread, int32_t use_graph, void* ws,
                          wmc_stream_t stream);
 
 /* Times one batch step from hist (left unchanged; scratch [dev] receives the
- * output) for each candidate work-item size and writes the fastest to
- * *best_per_thread [host].  Synchronises. */
+ * output) for each range size that differs (per_thread 16, 128 and 256) and
+ * writes the fastest to *best_per_thread [host].  Synchronises. */
 wmc_status wmc_batch_autotune(const wmc_params* ps, int32_t n_sims, const float* V, int32_t* hist, int32_t* scratch,
                               uint32_t t, void* ws, int32_t* best_per_thread, wmc_stream_t stream);
 

@@ -929,9 +929,7 @@ cudaError_t b_one_step(const BatchLayout& L, const BatchView& v, int n, const fl
   a.NM = L.NM;
   a.NB = L.NB;
   a.n_cells = (int)nc;
-  // 32 per_thread ids in windows of 128; shorter ranges than the single
-  // simulation's only add their own cost
-  a.max_range = per_thread / 4 > (int)kMaxRange ? (uint32_t)per_thread / 4u : kMaxRange;
+  a.max_range = batch_max_range(per_thread);
   k_b_step<<<grid, kBStepWarps * 32, 0, s>>>(a);
   const unsigned pair_blocks = (L.pair_cap + kBStepWarps * 32 - 1) / (kBStepWarps * 32);
   const unsigned pair_most = 8u * (unsigned)num_sms();
@@ -960,8 +958,6 @@ struct BatchGraphs {
   BatchGraph slot[kBatchGraphs];
 };
 BatchGraphs g_bgraph;
-
-bool valid_per(int per) { return per == 4 || per == 8 || per == 16 || per == 32 || per == 64 || per == 128 || per == 256; }
 
 }  // namespace
 }  // namespace wmc
@@ -1042,7 +1038,7 @@ wmc_status wmc_batch_run(const wmc_params* ps, int32_t n_sims, const float* V, i
   if (!batch_ok(ps, n_sims) || !V || !hist_a || !hist_b || hist_a == hist_b || !ws || n_steps < 0 || t_first == 0)
     return WMC_ERR_ARG;
   if (per_thread == 0) per_thread = 16;
-  if (!valid_per(per_thread)) return WMC_ERR_ARG;
+  if (!valid_per_thread(per_thread)) return WMC_ERR_ARG;
   if (n_steps == 0) return WMC_OK;
   const BatchLayout L = batch_layout(ps, n_sims);
   const BatchView v = batch_view(L, ws);
@@ -1124,23 +1120,22 @@ wmc_status wmc_batch_autotune(const wmc_params* ps, int32_t n_sims, const float*
   const BatchView v = batch_view(L, ws);
   cudaStream_t s = (cudaStream_t)stream;
   const int grid = b_step_grid();
-  const int cands[5] = {16, 32, 64, 128, 256};
   cudaEvent_t e0, e1;
   if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess) return WMC_ERR_CUDA;
   float best = 1e30f;
-  int best_per = 16;
+  int best_per = kTuneCandidates[0];
   for (int r = 0; r < 2; ++r) {  // second round measures warm
-    for (int q = 0; q < 5; ++q) {
+    for (const int per : kTuneCandidates) {
       k_b_set_step<<<1, 1, 0, s>>>(v.hdr, t - 1u);
       cudaEventRecord(e0, s);
-      if (b_one_step(L, v, n_sims, V, hist, scratch, cands[q], grid, s) != cudaSuccess) return WMC_ERR_CUDA;
+      if (b_one_step(L, v, n_sims, V, hist, scratch, per, grid, s) != cudaSuccess) return WMC_ERR_CUDA;
       cudaEventRecord(e1, s);
       if (cudaEventSynchronize(e1) != cudaSuccess) return WMC_ERR_CUDA;
       float ms = 0.f;
       cudaEventElapsedTime(&ms, e0, e1);
       if (r == 1 && ms < best) {
         best = ms;
-        best_per = cands[q];
+        best_per = per;
       }
     }
   }

@@ -33,6 +33,7 @@
 // for these calls.
 #pragma once
 
+#include "wmc_batch_ranges.cuh"
 #include "wmc_device.cuh"
 
 namespace wmc {
@@ -193,7 +194,7 @@ __device__ __forceinline__ uint32_t window_of_unit(const CellWork& c, uint32_t t
 // 1e8 particles, took single warps up to 390 of 340 us: the SM favours its
 // older warps, which go on to new ranges while a starved one sits on its
 // share; a range of 16 costs 1 % more instructions than one of 32.)
-constexpr uint32_t kMinRange = 4, kMaxRange = 16, kSingleRound = 24;
+constexpr uint32_t kMinRange = 4, kSingleRound = 24;
 
 struct RangeSchedule {
   uint32_t total;     // units
