@@ -8,6 +8,7 @@
 
 #include <cuda.h>  // driver types only: the two driver calls below come through cudaGetDriverEntryPointByVersion
 
+#include "wmc_graph_slots.cuh"
 #include "wmc_internal.cuh"
 
 namespace wmc {
@@ -186,7 +187,7 @@ static cudaError_t kernel_and_cdf_occupied(const wmc_params& p, const View& v, c
 // id of the context that made them: after cudaDeviceReset the device has a
 // new context and those handles are dropped (not destroyed: they died with
 // their context) and made again.
-static unsigned long long current_context_id() {
+unsigned long long current_context_id() {
   using GetCurrent = CUresult (*)(CUcontext*);
   using GetId = CUresult (*)(CUcontext, unsigned long long*);
   static GetCurrent get_current = nullptr;
@@ -359,22 +360,16 @@ cudaError_t step_timing_record(cudaStream_t s, bool end) {
 // alternates between buffer sets (copies of the next state overlapping the
 // current step) reuses its graphs instead of recapturing.
 constexpr int kGraphSlots = 4;
-struct GraphSlot {
-  bool valid = false;
-  unsigned long long last_use = 0;
+struct GraphKey {
   wmc_params p;
   const void *V, *a, *b, *ws;
   int prec;
   cudaStream_t stream;
-  int device;
-  unsigned long long ctx;
   int timing;
-  cudaGraphExec_t exec = nullptr;
 };
 struct GraphCache {
   std::mutex mu;
-  unsigned long long uses = 0;
-  GraphSlot slot[kGraphSlots];
+  GraphSlots<GraphKey, cudaGraphExec_t, kGraphSlots> slots;
 };
 static GraphCache g_graph;   // the step pair a -> b -> a
 static GraphCache g_graph1;  // one step a -> b and the copy back to a (odd step counts)
@@ -389,28 +384,13 @@ static wmc_status launch_cached(GraphCache& gc, const wmc_params* p, const float
   int dev = 0;
   cudaGetDevice(&dev);
   const unsigned long long ctx = current_context_id();
-  const int timing = step_timing_on();
-  GraphSlot* hit = nullptr;
-  GraphSlot* victim = &gc.slot[0];
-  for (GraphSlot& g : gc.slot) {
-    if (g.valid && g.device == dev && g.ctx != ctx) {  // made in an earlier context of this device
-      g.valid = false;
-      g.exec = nullptr;
-    }
-    if (g.valid && memcmp(&g.p, p, sizeof(wmc_params)) == 0 && g.V == V && g.a == a && g.b == b && g.ws == ws &&
-        g.prec == (int)prec && g.stream == s && g.device == dev && g.timing == timing) {
-      hit = &g;
-      break;
-    }
-    if (!g.valid || (victim->valid && g.last_use < victim->last_use)) victim = &g;
-  }
+  const GraphKey key{*p, V, a, b, ws, (int)prec, s, step_timing_on()};
+  auto* hit = gc.slots.find(dev, ctx, [&](const GraphKey& k) {
+    return memcmp(&k.p, p, sizeof(wmc_params)) == 0 && k.V == key.V && k.a == key.a && k.b == key.b && k.ws == key.ws &&
+           k.prec == key.prec && k.stream == key.stream && k.timing == key.timing;
+  });
   if (!hit) {
-    GraphSlot& gs = *victim;
-    if (gs.exec) {
-      cudaGraphExecDestroy(gs.exec);
-      gs.exec = nullptr;
-    }
-    gs.valid = false;
+    auto& slot = gc.slots.take([](cudaGraphExec_t e) { cudaGraphExecDestroy(e); });
     cudaGraph_t graph = nullptr;
     if (cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal) != cudaSuccess) return WMC_ERR_CUDA;
     const wmc_status st = body();
@@ -419,23 +399,12 @@ static wmc_status launch_cached(GraphCache& gc, const wmc_params* p, const float
       if (graph) cudaGraphDestroy(graph);
       return st != WMC_OK ? st : WMC_ERR_CUDA;
     }
-    e = cudaGraphInstantiate(&gs.exec, graph, 0);
+    cudaGraphExec_t exec = nullptr;
+    e = cudaGraphInstantiate(&exec, graph, 0);
     cudaGraphDestroy(graph);
     if (e != cudaSuccess) return WMC_ERR_CUDA;
-    gs.valid = true;
-    gs.p = *p;
-    gs.V = V;
-    gs.a = a;
-    gs.b = b;
-    gs.ws = ws;
-    gs.prec = (int)prec;
-    gs.stream = s;
-    gs.device = dev;
-    gs.ctx = ctx;
-    gs.timing = timing;
-    hit = &gs;
+    hit = gc.slots.fill(slot, key, exec, dev, ctx);
   }
-  hit->last_use = ++gc.uses;
   for (int q = 0; q < launches; ++q)
     if (cudaGraphLaunch(hit->exec, s) != cudaSuccess) return WMC_ERR_CUDA;
   return WMC_OK;

@@ -19,6 +19,7 @@
 #include <type_traits>
 #include <vector>
 
+#include "wmc_graph_slots.cuh"
 #include "wmc_walk.cuh"
 
 namespace wmc {
@@ -942,20 +943,15 @@ cudaError_t b_one_step(const BatchLayout& L, const BatchView& v, int n, const fl
 // to another and back does not recapture (a pass over 58 small simulations,
 // three batches in turn: most of its 430 us was capture and instantiation).
 constexpr int kBatchGraphs = 4;
-struct BatchGraph {
-  bool valid = false;
-  unsigned long long last_use = 0;
+struct BatchGraphKey {
   std::vector<wmc_params> ps;
-  const void *V, *a, *b, *ws;
-  int per;
-  cudaStream_t stream;
-  int device;
-  cudaGraphExec_t exec = nullptr;
+  const void *V = nullptr, *a = nullptr, *b = nullptr, *ws = nullptr;
+  int per = 0;
+  cudaStream_t stream = nullptr;
 };
 struct BatchGraphs {
   std::mutex mu;
-  unsigned long long uses = 0;
-  BatchGraph slot[kBatchGraphs];
+  GraphSlots<BatchGraphKey, cudaGraphExec_t, kBatchGraphs> slots;
 };
 BatchGraphs g_bgraph;
 
@@ -1051,23 +1047,13 @@ wmc_status wmc_batch_run(const wmc_params* ps, int32_t n_sims, const float* V, i
     std::lock_guard<std::mutex> lock(g_bgraph.mu);
     int dev = 0;
     cudaGetDevice(&dev);
-    BatchGraph *hit = nullptr, *victim = &g_bgraph.slot[0];
-    for (BatchGraph& g : g_bgraph.slot) {
-      if (g.valid && (int)g.ps.size() == n_sims && g.V == V && g.a == hist_a && g.b == hist_b && g.ws == ws &&
-          g.per == per_thread && g.stream == s && g.device == dev &&
-          memcmp(g.ps.data(), ps, sizeof(wmc_params) * n_sims) == 0) {
-        hit = &g;
-        break;
-      }
-      if (!g.valid || (victim->valid && g.last_use < victim->last_use)) victim = &g;
-    }
+    const unsigned long long ctx = current_context_id();
+    auto* hit = g_bgraph.slots.find(dev, ctx, [&](const BatchGraphKey& k) {
+      return (int)k.ps.size() == n_sims && k.V == V && k.a == hist_a && k.b == hist_b && k.ws == ws &&
+             k.per == per_thread && k.stream == s && memcmp(k.ps.data(), ps, sizeof(wmc_params) * n_sims) == 0;
+    });
     if (!hit) {
-      BatchGraph& gs = *victim;
-      if (gs.exec) {
-        cudaGraphExecDestroy(gs.exec);
-        gs.exec = nullptr;
-      }
-      gs.valid = false;
+      auto& slot = g_bgraph.slots.take([](cudaGraphExec_t e) { cudaGraphExecDestroy(e); });
       cudaGraph_t graph = nullptr;
       if (cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal) != cudaSuccess) return WMC_ERR_CUDA;
       cudaError_t e = b_one_step(L, v, n_sims, V, hist_a, hist_b, per_thread, grid, s);
@@ -1077,24 +1063,12 @@ wmc_status wmc_batch_run(const wmc_params* ps, int32_t n_sims, const float* V, i
         if (graph) cudaGraphDestroy(graph);
         return WMC_ERR_CUDA;
       }
-      e = cudaGraphInstantiate(&gs.exec, graph, 0);
+      cudaGraphExec_t exec = nullptr;
+      e = cudaGraphInstantiate(&exec, graph, 0);
       cudaGraphDestroy(graph);
-      if (e != cudaSuccess) {
-        gs.exec = nullptr;
-        return WMC_ERR_CUDA;
-      }
-      gs.valid = true;
-      gs.ps.assign(ps, ps + n_sims);
-      gs.V = V;
-      gs.a = hist_a;
-      gs.b = hist_b;
-      gs.ws = ws;
-      gs.per = per_thread;
-      gs.stream = s;
-      gs.device = dev;
-      hit = &gs;
+      if (e != cudaSuccess) return WMC_ERR_CUDA;
+      hit = g_bgraph.slots.fill(slot, BatchGraphKey{{ps, ps + n_sims}, V, hist_a, hist_b, ws, per_thread, s}, exec, dev, ctx);
     }
-    hit->last_use = ++g_bgraph.uses;
     for (int q = 0; q < pairs; ++q)
       if (cudaGraphLaunch(hit->exec, s) != cudaSuccess) return WMC_ERR_CUDA;
   } else {

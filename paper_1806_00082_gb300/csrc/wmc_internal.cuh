@@ -291,6 +291,8 @@ cudaError_t launch_philox_throughput(uint32_t k0, uint32_t k1, int pairs_per_thr
                                      cudaStream_t s);
 
 int num_sms();
+// Id of the calling thread's current CUDA context (0 if the driver cannot say).
+unsigned long long current_context_id();
 // Raises a kernel's dynamic shared-memory limit (kept per kernel, device and
 // context; the runtime is called only when the limit has to grow).
 cudaError_t raise_smem_limit(const void* func, size_t bytes);
