@@ -866,15 +866,85 @@ __device__ __forceinline__ int grid_count_tc(int r, int Q, int a, int b, int r0)
 
 __host__ __device__ constexpr size_t split_window_floats(int h) { return (size_t)kWindowSpan + 2 * (size_t)h + 4; }
 
+// Tiles whose rows fit no window (cells too far apart, or of more than one
+// potential): in the STAGED form every builder warp fetches 16 terms of each of its
+// 32 rows at a time by coalesced loads and hands them to the rows' threads through
+// kRowStage floats of shared memory.  Where the windows leave no room for it, that
+// is the tile's own window buffer, which is then large enough.
+constexpr int kRowStage = 32 * 16;  // floats per builder warp
+constexpr int kRowStageOwn = 8 * kRowStage;
+__host__ __device__ constexpr bool split_row_stage_apart(int h) {
+  return kSmemAlignPad + (size_t)kSpStages * 2 * kTileBytes + sizeof(float) * 8 * kWsStageFloats +
+             sizeof(float) * (2 * split_window_floats(h) + kRowStageOwn) <=
+         226 * 1024;
+}
+static_assert([] {
+  for (int h = 1; h <= 2048; ++h)
+    if (!split_row_stage_apart(h) && split_window_floats(h) < kRowStageOwn + 4) return false;
+  return true;
+}(), "a window buffer holds the row stages where they have no room of their own");
+
 // NET = 3: the rows of gVW and VWh of a K block (128 x 32) pass through
 // kDenseStages buffers of shared memory each, padded to 36 floats a row; fewer
 // B stages make room.
 constexpr int kDenseStages = 3, kDensePitch = 36;
 __host__ __device__ constexpr int split_stages(int net) { return net == 3 ? 3 : kSpStages; }
 
-__host__ __device__ constexpr size_t split_smem_bytes(int h, int net) {
+__host__ __device__ constexpr size_t split_smem_bytes(int h, int net, bool staged) {
   return kSmemAlignPad + (size_t)split_stages(net) * 2 * kTileBytes + sizeof(float) * 8 * kWsStageFloats +
-         sizeof(float) * (net == 3 ? (size_t)2 * kDenseStages * TM * kDensePitch : 2 * split_window_floats(h));
+         sizeof(float) * (net == 3 ? (size_t)2 * kDenseStages * TM * kDensePitch
+                                   : 2 * split_window_floats(h) + (staged && split_row_stage_apart(h) ? kRowStageOwn : 0));
+}
+
+// N consecutive terms kk = k0 .. of the A operand for the 32 rows of a warp (cell,
+// and base = where its potential begins: the lane's row), dv those of the lane's
+// own row.  Lanes 0-15 load the 16 terms of one row and lanes 16-31 those of the
+// next, consecutive cells each; a row's 16-byte groups go to stg XOR-swizzled by
+// (row / 2) % 4, so that the row's thread reads them without bank conflicts.
+template <int NET, int N>
+__device__ __forceinline__ void a_run_rows(const float* __restrict__ V, int n_x, int bc, int h, int cell, int base,
+                                           int k0, float* stg, float (&dv)[N]) {
+  static_assert(N % 16 == 0, "");
+  const int lane = threadIdx.x & 31, l = lane & 15, second = lane >> 4;
+  const int last = NET == 1 ? h - 2 : h - 1;  // last term that is not zero
+#pragma unroll
+  for (int q = 0; q < N; q += 16) {
+    const int t = k0 + q + l;
+    if (k0 + q > last) {  // (uniform)
+#pragma unroll
+      for (int e = 0; e < 16; ++e) dv[q + e] = 0.f;
+      continue;
+    }
+    __syncwarp();  // the stage's last terms are read
+#pragma unroll 1
+    for (int j0 = 0; j0 < 16; j0 += 8) {
+      float va[8], vb[8];  // sixteen loads under way together, without branches
+      uint32_t left = 0u;
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const int row = 2 * (j0 + j) + second;
+        const int c = __shfl_sync(0xffffffffu, cell, row), b = __shfl_sync(0xffffffffu, base, row);
+        const bool right = NET == 1 || ((c + t) & 1) == 0;
+        const int a0 = NET == 1 ? c + t + 1 : (right ? c + t : c - t - 1), a1 = NET == 1 ? c - t - 1 : a0 + 1;
+        const float x0 = __ldg(V + (b + min(max(a0, 0), n_x - 1))), x1 = __ldg(V + (b + min(max(a1, 0), n_x - 1)));
+        va[j] = (unsigned)a0 < (unsigned)n_x || bc ? x0 : 0.f;
+        vb[j] = (unsigned)a1 < (unsigned)n_x || bc ? x1 : 0.f;
+        if (NET == 2) left |= (right ? 0u : 1u) << j;
+      }
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        float d = NET == 1 ? __fsub_rn(va[j], vb[j]) : __fadd_rn(va[j], vb[j]);
+        if (NET == 2 && ((left >> j) & 1u)) d = -d;
+        stg[(2 * (j0 + j) + second) * 16 + (((l >> 2) ^ ((j0 + j) & 3)) << 2) + (l & 3)] = t <= last ? d : 0.f;
+      }
+    }
+    __syncwarp();
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const float4 x = *reinterpret_cast<const float4*>(stg + lane * 16 + 4 * (e ^ ((lane >> 1) & 3)));
+      dv[q + 4 * e] = x.x, dv[q + 4 * e + 1] = x.y, dv[q + 4 * e + 2] = x.z, dv[q + 4 * e + 3] = x.w;
+    }
+  }
 }
 
 __device__ __forceinline__ void mma_tf32_ta(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc, uint32_t idesc,
@@ -918,7 +988,7 @@ struct SplitRows {
   int pot;
 };
 
-template <bool TF32, int NET>
+template <bool TF32, int NET, bool STAGED>
 __global__ __launch_bounds__(kSpThreads, 1) void k_rows_split(
     const float* __restrict__ V, int n_x, int bc, int Q, const int* __restrict__ occ,
     const int* __restrict__ n_occ_dev, int n_occ_host, const void* __restrict__ img_hi_v,
@@ -1219,6 +1289,9 @@ __global__ __launch_bounds__(kSpThreads, 1) void k_rows_split(
           }
         } else if (cur.window) {
           a_run_window<NET == 3 ? 1 : NET, EPT>(w, h, cur.cell, k0, dv);
+        } else if (STAGED) {
+          float* stg = s_win + (split_row_stage_apart(h) ? 2 * wf : ((wb * wf + 3) & ~(size_t)3)) + warp * kRowStage;
+          a_run_rows<NET == 3 ? 1 : NET, EPT>(V, n_x, bc, h, cur.cell, cur.pot * n_x, k0, stg, dv);
         } else {
 #pragma unroll
           for (int e = 0; e < EPT; ++e) dv[e] = a_term<NET == 3 ? 1 : NET>(Vr, n_x, bc, h, cur.cell, k0 + e);
@@ -1413,18 +1486,46 @@ cudaError_t launch_init_tc_images(const wmc_params& p, void* images, cudaStream_
 }
 
 // One persistent CTA per SM, fewer if there are fewer tiles.
+template <bool TF32, int NET, bool STAGED>
+static cudaError_t launch_split_as(const float* V, int n_x, int bc, int Q, const int* occ, const int* n_occ_dev,
+                                   int n_occ_host, int max_rows, const void* img_hi, const void* img_lo, int KB, int NT,
+                                   float c, float* out, unsigned int* flags, const DenseA& dense, cudaStream_t s) {
+  const size_t sm = split_smem_bytes(Q / 2, NET, STAGED);
+  const cudaError_t e = raise_smem_limit(reinterpret_cast<const void*>(k_rows_split<TF32, NET, STAGED>), sm);
+  if (e != cudaSuccess) return e;
+  const long long tiles = (long long)((max_rows + TM - 1) / TM) * NT;
+  const unsigned grid = (unsigned)(tiles < num_sms() ? tiles : num_sms());
+  k_rows_split<TF32, NET, STAGED><<<grid, kSpThreads, sm, s>>>(V, n_x, bc, Q, occ, n_occ_dev, n_occ_host, img_hi,
+                                                               img_lo, KB, NT, c, out, flags, dense);
+  return cudaGetLastError();
+}
+
+// The staged form where tiles may be without a window: lists from the host that
+// leave cells out, of domains that no window spans, and rows over several
+// potentials that tiles straddle.  With each thread reading its own row in such
+// tiles (the plain form), a load touched 32 lines, and they ran up to 1.75 times as
+// long as in the kernel that built passes of four K blocks: 37 random cells, Q =
+// 2048, 3xTF32: 108 us there, 118 us plain, 60 us staged; 9000 permuted cells of
+// 20000, Q = 1024, FP16 split: 240, 162 and 64 us, of the N = 2 network 172, 267 and
+// 70 us; 33 x 700 rows, FP16 split: 148, 202 and 97 us.  Where all tiles have windows
+// the staged form costs 3xTF32 more (16384 cells at Q = 1024 66.3 against 64.1 us,
+// FP16 split nothing), and in the step loop its shared memory costs the kernels
+// around it 20 us a step.  So the occupied lists of a step and lists of every cell
+// take the plain form, and 3xTF32 lists of at least a quarter of the cells too: if
+// they ascend, 128 of them span some 512 cells and have windows (in any order, 9000
+// of 20000: 157 us plain, 71 us staged).
 template <bool TF32, int NET>
 static cudaError_t launch_split(const float* V, int n_x, int bc, int Q, const int* occ, const int* n_occ_dev,
                                 int n_occ_host, int max_rows, const void* img_hi, const void* img_lo, int KB, int NT,
                                 float c, float* out, unsigned int* flags, const DenseA& dense, cudaStream_t s) {
-  const size_t sm = split_smem_bytes(Q / 2, NET);
-  const cudaError_t e = raise_smem_limit(reinterpret_cast<const void*>(k_rows_split<TF32, NET>), sm);
-  if (e != cudaSuccess) return e;
-  const long long tiles = (long long)((max_rows + TM - 1) / TM) * NT;
-  const unsigned grid = (unsigned)(tiles < num_sms() ? tiles : num_sms());
-  k_rows_split<TF32, NET><<<grid, kSpThreads, sm, s>>>(V, n_x, bc, Q, occ, n_occ_dev, n_occ_host, img_hi, img_lo, KB, NT,
-                                                       c, out, flags, dense);
-  return cudaGetLastError();
+  if (NET != 3) {
+    const bool left_out = (TF32 ? 4ll : 1ll) * n_occ_host < n_x;
+    if (occ ? !n_occ_dev && left_out && n_x > kWindowSpan : max_rows > n_x && n_x % TM != 0)
+      return launch_split_as<TF32, NET, NET != 3>(V, n_x, bc, Q, occ, n_occ_dev, n_occ_host, max_rows, img_hi, img_lo, KB,
+                                                  NT, c, out, flags, dense, s);
+  }
+  return launch_split_as<TF32, NET, false>(V, n_x, bc, Q, occ, n_occ_dev, n_occ_host, max_rows, img_hi, img_lo, KB, NT,
+                                           c, out, flags, dense, s);
 }
 
 // Abar = c Gbar S^T on the 3xTF32 split kernel (NET = 3), rows = n_pot n_x

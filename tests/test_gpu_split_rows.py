@@ -106,3 +106,46 @@ def test_split_rows_over_several_potentials(wmc, n_pot, n_x):
     for b in range(n_pot):
         ref = oracle.kernel_rows(oracle.params(wl), V[b], np.arange(n_x))[:, Q // 2:]
         assert normwise(got[b], ref) <= TOL
+
+
+@pytest.mark.parametrize("form,net", [("tf32x3", 1), ("fp16_split", 1), ("fp16_split", 2)])
+@pytest.mark.parametrize("bc", [0, 1])
+@pytest.mark.parametrize("Q", [2, 4, 34, 66, 258, 1024, 3580, 3582, 4096])
+def test_rows_without_a_window_are_the_windows_rows(wmc, form, net, bc, Q):
+    """Cells in any order, whose 128-row tiles fit no window, and rows over several
+    potentials: the bits of consecutive cells (Q = 3580 is the widest window beside
+    which the rows' stages have room of their own), at the domain's edges too and
+    with values that are not finite."""
+    n_x = 1300
+    wl = wi.DOUBLE_BARRIER_16384.replace(n_x=n_x, Q=Q, n_M=Q, bc_potential=bc)
+    p = wmc.Params.of(wl)
+    ws = wmc.workspace(p)
+    wmc.init(p, ws)
+    rng = np.random.Generator(np.random.PCG64(Q + bc))
+    f, prec = wmc.kernel_eval if net == 1 else wmc.kernel_eval_n2, wmc.PRECISIONS[form]
+    for bad in (False, True):
+        V = rng.uniform(-0.2, 0.3, n_x).astype(np.float32)
+        if bad:
+            V[700], V[3] = np.inf, np.nan
+        Vd = torch.from_numpy(V).cuda()
+        run = f(p, Vd, torch.arange(n_x, dtype=torch.int32, device="cuda"), ws, prec)
+        for n in (2, 129, n_x):
+            cells = np.r_[0, n_x - 1, rng.permutation(np.arange(1, n_x - 1))][:n]
+            got = f(p, Vd, torch.from_numpy(cells.astype(np.int32)).cuda(), ws, prec)
+            np.testing.assert_array_equal(got.cpu().numpy(), run[torch.from_numpy(cells).cuda()].cpu().numpy())
+    assert wmc.get_counters(p, ws)["flags"] == 0
+
+
+@pytest.mark.parametrize("form", ["tf32x3", "fp16_split"])
+@pytest.mark.parametrize("Q,n_pot,n_x", [(66, 300, 1), (258, 7, 37), (1024, 3, 333), (130, 2, 129)])
+def test_implicit_rows_are_the_rows_of_each_potential(wmc, form, Q, n_pot, n_x):
+    wl = wi.TANH_BARRIERS_4096.replace(n_x=n_x, Q=Q, n_M=Q)
+    p = wmc.Params.of(wl)
+    ws = wmc.workspace(p)
+    wmc.init(p, ws)
+    V = torch.from_numpy(np.random.Generator(np.random.PCG64(Q)).uniform(-0.2, 0.2, (n_pot, n_x)).astype(np.float32)).cuda()
+    prec = wmc.PRECISIONS[form]
+    got = wmc.kernel_eval_rows(p, V, ws, prec).view(n_pot, n_x, -1)
+    occ = torch.arange(n_x, dtype=torch.int32, device="cuda")
+    for b in range(n_pot):
+        assert torch.equal(got[b], wmc.kernel_eval(p, V[b].contiguous(), occ, ws, prec))
