@@ -812,8 +812,8 @@ __device__ __noinline__ void b_rewalk_events(const BatchStepArgs& a, uint32_t t,
   if (nq) flush();
 }
 
-// The queued quads of the step: one thread each.  The last block to finish
-// resets the queue and the range ticket for the next step.
+// The queued quads of the step, by ids or by quads as in the single form.  The last
+// block to finish resets the queue and the range ticket for the next step.
 __global__ __launch_bounds__(kBStepWarps * 32, 4) void k_b_pairs(const __grid_constant__ BatchStepArgs a) {
   __shared__ uint4 s_queue[kBStepWarps][kWalkQueue + 32];
   __shared__ BatchRow s_row[kBStepWarps];
@@ -821,13 +821,14 @@ __global__ __launch_bounds__(kBStepWarps * 32, 4) void k_b_pairs(const __grid_co
   const uint32_t t = a.hdr->step;
   const unsigned n = a.hdr->pair_count;
   // (blocks without work leave at once and are not counted)
-  const unsigned blocks = n > a.pair_cap ? gridDim.x : min(gridDim.x, max(1u, (n + blockDim.x - 1) / blockDim.x));
+  const unsigned split = pairs_split(n, gridDim.x * blockDim.x), items = n << split;
+  const unsigned blocks = n > a.pair_cap ? gridDim.x : min(gridDim.x, max(1u, (items + blockDim.x - 1) / blockDim.x));
   if (blockIdx.x >= blocks) return;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   PairCounters pc;
   if (n <= a.pair_cap) {
-    for (unsigned e = blockIdx.x * blockDim.x + threadIdx.x; e < n; e += blocks * blockDim.x)
-      b_quad_events(a, t, a.pairs[e], pc);
+    for (unsigned e = blockIdx.x * blockDim.x + threadIdx.x; e < items; e += blocks * blockDim.x)
+      b_quad_events(a, t, pairs_item(a.pairs, e, split), pc);
   } else {
     b_rewalk_events(a, t, s_queue[wid], s_row + wid, pc);
   }

@@ -257,21 +257,26 @@ __device__ __noinline__ void rewalk_events(const StepArgs& a, uint32_t t, uint4*
   if (nq) flush();
 }
 
-// The queued quads of the step: one thread each.  The last block to
-// finish resets the queue and the work-item ticket for the next step.
+// The queued quads of the step: a thread for each of a quad's four ids while the
+// grid has that many, so that no thread draws and samples two events one after
+// the other; one thread per quad beyond.  24 cells of 1026 columns, 18000 events
+// in 16000 quads: 24.5 us by quads, 15.1 us by ids.  The last block to finish resets
+// the queue and the work-item ticket for the next step.
 __global__ __launch_bounds__(kStepThreads, 4) void k_pairs(const __grid_constant__ StepArgs a) {
   const int rows_by_cell = (int)a.hdr->rows_by_cell;
   const uint32_t t = a.t_from_device ? a.hdr->step : a.t;
   const unsigned n = a.hdr->pair_count;
   // the blocks that have work (or block 0) count themselves done; the others
   // leave at once, whether they see the count or its reset
-  const unsigned blocks = n > a.pair_cap ? gridDim.x : min(gridDim.x, max(1u, (n + kStepThreads - 1) / kStepThreads));
+  const unsigned split = pairs_split(n, gridDim.x * kStepThreads), items = n << split;
+  const unsigned blocks =
+      n > a.pair_cap ? gridDim.x : min(gridDim.x, max(1u, (items + kStepThreads - 1) / kStepThreads));
   if (blockIdx.x >= blocks) return;
   unsigned long long pairs = 0, dropped = 0;
   long long drop_signed = 0;
   if (n <= a.pair_cap) {
-    for (unsigned e = blockIdx.x * kStepThreads + threadIdx.x; e < n; e += blocks * kStepThreads)
-      quad_events(a, rows_by_cell, t, a.pairs[e], pairs, dropped, drop_signed);
+    for (unsigned e = blockIdx.x * kStepThreads + threadIdx.x; e < items; e += blocks * kStepThreads)
+      quad_events(a, rows_by_cell, t, pairs_item(a.pairs, e, split), pairs, dropped, drop_signed);
   } else {
     __shared__ uint4 s_queue[kStepWarps][kWalkQueue + 32];
     rewalk_events(a, t, s_queue[threadIdx.x >> 5], pairs, dropped, drop_signed);

@@ -235,6 +235,15 @@ struct RangeSchedule {
 // drawn again and tested where the events are completed, 32 quads at a time.
 constexpr int kWalkQueue = 160;
 
+// The pair kernels' items: quads, or (split 2) their ids where the threads are
+// enough, item e then being id e % 4 of quad e / 4.
+__device__ __forceinline__ unsigned pairs_split(unsigned n, unsigned threads) { return n <= threads / 4u ? 2u : 0u; }
+__device__ __forceinline__ uint4 pairs_item(const uint4* pairs, unsigned e, unsigned split) {
+  uint4 ev = pairs[e >> split];
+  if (split) ev.z &= 0xffffu | (1u << (16u + (e & 3u)));
+  return ev;
+}
+
 // Walks the ids at offsets [r0, r1) of cell c (r0 a multiple of 4, ids before
 // the cell's first excluded).  draw(offset / 4, gen, wr, wg) gives the quad's
 // offset words and, if gen, its creation words; count(k, e, stay, move) takes

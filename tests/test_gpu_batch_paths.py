@@ -107,6 +107,28 @@ def test_more_event_quads_than_the_batch_queue(wmc):
     assert c["pairs"] == pairs > 4 * 2 ** 21 and c["flags"] == 0
 
 
+@pytest.mark.parametrize("scale", [3, 60, 1000])
+def test_events_by_ids_and_by_quads(wmc, scale):
+    """The pair kernels take a thread per id of a queued quad up to a quarter of
+    their threads, a thread per quad beyond (scale 1000: 4e5 quads and more): each
+    simulation against the oracle, the batch against each simulation."""
+    wls, Vs, hs = _busy(3, scale, scale)
+    B = _Batch(wmc, wls, Vs, hs)
+    got = B.run(5, 2, use_graph=False)
+    c = wmc.batch_get_counters(B.ps, B.ws)
+    pairs = 0
+    for q, w in enumerate(wls):
+        ref, ca = B.alone(q, 5, 2)
+        np.testing.assert_array_equal(got[B.ho[q]:B.ho[q + 1]].reshape(w.n_x, w.n_M), ref)
+        pairs += ca["pairs"]
+        full, half = oracle_tables(w, Vs[q])
+        want, st = oracle.simulate(oracle.params(w), hs[q], 5, 2, table=full)
+        out, co = gpu_run_table(wmc, torch, wmc.Params.of(w), half, hs[q], 5, 2)
+        np.testing.assert_array_equal(out, want)
+        assert co["pairs"] == st[oracle.ST_PAIRS] and co["flags"] == 0
+    assert c["pairs"] == pairs > 0 and c["flags"] == 0
+
+
 def test_more_event_quads_than_the_queue_of_one_simulation(wmc):
     """The same for one simulation, against the oracle."""
     wls, Vs, hs = _busy(1, 3, 30_000)
