@@ -15,22 +15,26 @@
 //     particle state with 450 non-empty buckets a cell): the stretch of such
 //     windows runs with the bucket's data in uniform values, two instructions
 //     per particle beside the generator, one warp reduction per stretch;
-//   - otherwise buckets of more than kLaneBucket ids in the window are counted
-//     under quad masks, bucket by bucket;
-//   - and each smaller one by the lane that holds its column, from the offset
-//     words in shared memory, with neighbouring columns' additions coalesced.
+//   - otherwise up to kFewBuckets buckets of more than kLaneBucket ids in the
+//     window are counted under quad masks, bucket by bucket;
+//   - and the others from the offset words in shared memory: each by the lane
+//     that holds its column, or, if one has more than kLaneBucket ids, by as many
+//     lanes as there are for each column.
+// The counts then go out together, with neighbouring columns' additions coalesced.
 //
 // What bounds it: instruction issue and the wide multiplier.  The two calls of a
 // quad take 34 wide multiplications (4 cycles each on a scheduler) and as many
 // XORs; a one-bucket window takes 104 instructions (with creation words), a
 // mixed one several hundred.  Measured (ncu, 1.08e8 particles, 3555 occupied
-// cells with 450 non-empty buckets each): k_step 372 -> 260 us, 275e6 -> 176e6
+// cells with 450 non-empty buckets each): k_step 372 -> 205 us, 275e6 -> 142e6
 // warp instructions, against the form that staged each row in shared memory
 // and gave every lane a run of ids of its own (nearly every warp iteration
 // then met a lane that changed its bucket); drift only, 1e7 particles on 2000
-// cells: 34 -> 20 us.  With kLaneBucket = 16 and candidates matched by block, in
-// the step graph at 1.06e8 particles, 237 us.  The generator alone takes 111 us
-// for these calls.
+// cells: 34 -> 20 us.  The generator alone takes 111 us for the calls of the first.
+// Rows of 64 columns that are all held by a few dozen ids are what that form did
+// best: 16384 such cells, two steps, drift only, mean bucket 20, 50 and 130: 213,
+// 368 and 675 us there, here 334, 478 and 805 us with every larger bucket under
+// masks and 228, 402 and 758 us as it is.
 #pragma once
 
 #include "wmc_batch_ranges.cuh"
@@ -43,6 +47,12 @@ namespace wmc {
 // 3286, 3263 and 3300 us; 38 simulations of 2.5e7 scattered particles, four steps
 // 1379, 1274, 1163 and 1147 us.
 constexpr uint32_t kLaneBucket = 16;
+// A bucket under masks takes some forty instructions of the whole warp, shared-out
+// lanes about as many for all buckets and five more for every four ids of a lane's:
+// with 1 instead of 2, buckets of 130 ids (above) 829 instead of 758 us; with all
+// windows' lanes shared out also where no bucket is large, 400 small simulations
+// 1148 instead of 1110 us.
+constexpr int kFewBuckets = 2;
 
 // Move entry of a column: bits 1-2 drift direction + 1, bits 8-31 the crossing
 // threshold on the offset word w (move_threshold).  A right-moving column's
@@ -306,71 +316,91 @@ __device__ __forceinline__ void walk_ids(const C& c, uint32_t r0, uint32_t r1, i
       if (lane == 0) count(k, e, all - mv, mv);
       continue;
     }
-    // a window with several buckets, or cut by the range's ends: its offset
-    // words go to shared memory, block by block the larger buckets are counted
-    // by the warp and each small one by the lane that holds its column
+    // a window with several buckets, or cut by the range's ends, block by block: one
+    // or two large buckets are counted by the warp, the others from the offset
+    // words in shared memory by the lane or lanes of each column
     const uint32_t qa = a + 4u * (uint32_t)lane;
     const uint32_t wend = a + 128u < r1 ? a + 128u : r1;
     uint4 wr, wg = make_uint4(0u, 0u, 0u, 0u);
     draw(qa >> 2, gen, wr, wg);
     const unsigned cand = __ballot_sync(0xffffffffu, gen && min(min(wg.x, wg.y), min(wg.z, wg.w)) <= rej);
-    words[lane] = wr;
-    __syncwarp();
     while (true) {
       const uint32_t lim = B.end < wend ? B.end : wend;
       // the ids [from, to) of this window in the lane's bucket
       uint32_t from = __shfl_up_sync(0xffffffffu, B.E, 1);
       from = lane && from > x ? from : x;
       const uint32_t to = B.E < lim ? B.E : lim;
-      uint32_t cnt = to > from ? to - from : 0u;
+      const uint32_t cnt = to > from ? to - from : 0u;
+      uint32_t own = cnt, mv = 0u, most = __reduce_max_sync(0xffffffffu, cnt);
       unsigned big = __ballot_sync(0xffffffffu, cnt > kLaneBucket);
-      if (cnt > kLaneBucket) cnt = 0u;
+      const int k = min((B.b << 5) + lane, c.n_M() - 1);
+      if (big && __popc(big) <= kFewBuckets) {
+        if (cnt > kLaneBucket) own = 0u;
 #pragma unroll 1
-      while (big) {
-        j = __ffs(big) - 1;
-        big &= big - 1u;
-        const uint32_t f = __shfl_sync(0xffffffffu, from, j), t = __shfl_sync(0xffffffffu, to, j),
-                       e = __shfl_sync(0xffffffffu, B.e, j);
-        const uint32_t inb = first_mask((int)(t - qa)) & ~first_mask((int)(f - qa));
-        const int k = min((B.b << 5) + j, c.n_M() - 1);
-        const uint32_t mv = __reduce_add_sync(0xffffffffu, (uint32_t)__popc(move_bits(wr, e) & inb));
-        if (cand) {
-          const bool me = (cand >> lane) & 1u && inb != 0u;
-          push(__ballot_sync(0xffffffffu, me), me, qa >> 2, k, e, inb);
+        while (big) {
+          j = __ffs(big) - 1;
+          big &= big - 1u;
+          const uint32_t f = __shfl_sync(0xffffffffu, from, j), t = __shfl_sync(0xffffffffu, to, j),
+                         e = __shfl_sync(0xffffffffu, B.e, j);
+          const uint32_t inb = first_mask((int)(t - qa)) & ~first_mask((int)(f - qa));
+          const uint32_t m = __reduce_add_sync(0xffffffffu, (uint32_t)__popc(move_bits(wr, e) & inb));
+          if (lane == j) mv = m;
+          if (cand) {
+            const bool me = (cand >> lane) & 1u && inb != 0u;
+            push(__ballot_sync(0xffffffffu, me), me, qa >> 2, min((B.b << 5) + j, c.n_M() - 1), e, inb);
+          }
         }
-        if (lane == 0) count(k, e, t - f - mv, mv);
+        most = __reduce_max_sync(0xffffffffu, own);
       }
-      const uint32_t most = __reduce_max_sync(0xffffffffu, cnt);
-      if (most) {
-        const uint32_t* w = reinterpret_cast<const uint32_t*>(words) + (from - a);
-        const uint32_t th = B.e | 255u;
-        const int k = min((B.b << 5) + lane, c.n_M() - 1);
+      if (most) {  // (what follows leaves the words read)
+        words[lane] = wr;
+        __syncwarp();
+        const uint32_t* w = reinterpret_cast<const uint32_t*>(words);
         uint32_t above = 0u;
+        if (most <= kLaneBucket) {
+          const uint32_t th = B.e | 255u;
+          w += from - a;
 #pragma unroll
-        for (uint32_t t0 = 0; t0 < kLaneBucket; t0 += 4) {
-          if (t0 && most <= t0) break;
+          for (uint32_t t0 = 0; t0 < kLaneBucket; t0 += 4) {
+            if (t0 && most <= t0) break;
 #pragma unroll
-          for (uint32_t t = t0; t < t0 + 4; ++t)
-            if (t < cnt) above += w[t] > th;
+            for (uint32_t t = t0; t < t0 + 4; ++t)
+              if (t < own) above += w[t] > th;
+          }
+        } else {
+          // columns j0 .. j0 + 2^(5 - s) - 1 hold them: 2^s lanes count each
+          const unsigned held = __ballot_sync(0xffffffffu, own != 0u);
+          const int j0 = __ffs(held) - 1, s = __clz(31 - __clz(held) - j0) - 27, src = j0 + (lane >> s);
+          const uint32_t n = __shfl_sync(0xffffffffu, own, src), th = __shfl_sync(0xffffffffu, B.e, src) | 255u;
+          w += __shfl_sync(0xffffffffu, from, src) - a;
+#pragma unroll 1
+          for (uint32_t t = (uint32_t)lane & ((1u << s) - 1u); t < n; t += 4u << s)
+#pragma unroll
+            for (uint32_t u = 0; u < 4; ++u)
+              if (t + (u << s) < n) above += w[t + (u << s)] > th;
+          __syncwarp();
+#pragma unroll 1
+          for (int o = 1 << s >> 1; o; o >>= 1) above += __shfl_xor_sync(0xffffffffu, above, o);
+          above = __shfl_sync(0xffffffffu, above, (lane - j0) << s);
         }
-        const uint32_t mv = (B.e & 6u) == 0u ? cnt - above : above;
-        if (cnt) count(k, B.e, cnt - mv, mv);
+        __syncwarp();
+        if (own) mv = (B.e & 6u) == 0u ? own - above : above;
         // candidate quads with ids in this block: their ids in the lanes' buckets
         const unsigned span = (0xffffffffu << ((x - a) >> 2)) & (0xffffffffu >> (31u - ((lim - 1u - a) >> 2)));
 #pragma unroll 1
         for (unsigned cd = cand & span; cd; cd &= cd - 1u) {
           const uint32_t q0 = a + 4u * (uint32_t)(__ffs(cd) - 1);
-          const uint32_t in = first_mask((int)(from + cnt - q0)) & ~first_mask((int)(from - q0));
-          const bool me = cnt && in;
+          const uint32_t in = first_mask((int)(from + own - q0)) & ~first_mask((int)(from - q0));
+          const bool me = own && in;
           const unsigned who = __ballot_sync(0xffffffffu, me);
           if (who) push(who, me, q0 >> 2, k, B.e, in);
         }
       }
+      if (cnt) count(k, B.e, cnt - mv, mv);
       if (lim == wend) break;
       x = lim;
       walk_load(c, x, B, lane);
     }
-    __syncwarp();  // the words are read before the next window's are written
     a += 128u;
   }
 }

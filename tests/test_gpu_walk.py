@@ -97,3 +97,21 @@ def test_snapshot_places_and_words(wmc, id_base, n_x, n_M):
         gid = int(i) + id_base
         w = int(oracle.philox((gid // 4, 5, 2, wl.sim), (wl.seed & 0xffffffff, wl.seed >> 32))[gid % 4])
         assert f[i] == np.float32((w >> 8) * 2.0 ** -24)
+
+
+@pytest.mark.parametrize("sizes", [(15, 16, 17, 18), (17, 19, 20, 21, 24), (12, 30, 33, 40, 43), (0, 0, 31, 48, 60, 63, 64),
+                                   (0, 16, 17, 90, 110, 127), (1, 2, 0, 0, 45, 80)])
+@pytest.mark.parametrize("n_x,Q,n_M", [(7, 2, 2), (33, 32, 30), (33, 32, 34), (33, 64, 64), (12, 64, 1026)])
+def test_windows_of_mid_sized_buckets(wmc, sizes, n_x, Q, n_M):
+    """Windows that hold one, two and more buckets of more than 16 ids, beside small
+    and empty ones, in columns that are few or all of a block: counted under masks, by
+    a lane each or by several lanes each; drift only and with pairs."""
+    wl, V = _workload(n_x, Q, n_M)
+    rng = np.random.Generator(np.random.PCG64(sum(sizes) + n_M))
+    h0 = (rng.choice(sizes, size=(n_x, n_M)) * rng.choice([-1, 1], size=(n_x, n_M))).astype(np.int32)
+    for v in (V, np.zeros_like(V)):
+        full, half = oracle_tables(wl, v)
+        ref, st = oracle.simulate(oracle.params(wl), h0, 3, 2, table=full)
+        got, c = gpu_run_table(wmc, torch, wmc.Params.of(wl), half, h0, 3, 2)
+        np.testing.assert_array_equal(got, ref)
+        assert c["pairs"] == st[oracle.ST_PAIRS] and c["flags"] == 0
