@@ -128,3 +128,26 @@ def test_potential_sums_each_window_by_one_rounding(wmc, n_x, nb, ns):
         bad = heights.copy()
         bad[k] = np.inf
         assert not np.isfinite(potential(bad[None])).any()
+
+
+@pytest.mark.parametrize("n_x", [64, 106, 107, 4096])
+@pytest.mark.parametrize("ns", [1, 255, 256, 257, 513])
+def test_segments_beyond_one_round_of_edges(wmc, n_x, ns):
+    """The edges are staged 256 segments at a time: each segment by itself at its
+    place, and all of them added in turn with one rounding each, on domains that
+    every window reaches (53 eps and less) and on wider ones."""
+    p = _params(wmc, n_x, 64)
+    rng = np.random.Generator(np.random.PCG64(n_x + ns))
+    eps, L = 0.5, n_x * 0.25
+    heights = rng.uniform(-0.02, 0.02, ns).astype(np.float32)
+    w = wmc.potential_tanh(p, torch.from_numpy(np.eye(ns, dtype=np.float32)).cuda(), 0, ns, eps).cpu().numpy()
+    x = (np.arange(n_x) + 0.5) * 0.25
+    s = np.arange(ns)[:, None]
+    exact = 0.5 * (np.tanh((x - L * s / ns) / eps) - np.tanh((x - L * (s + 1) / ns) / eps))
+    # an edge position is rounded at |x| <= 1024 nm: 2^-14 nm over eps in the argument of a window
+    assert np.abs(w - exact).max() <= 2.0 ** -13
+    ref = np.zeros(n_x, np.float32)
+    for k in range(ns):
+        ref = _fma32(np.full(n_x, heights[k]), w[k], ref)
+    got = wmc.potential_tanh(p, torch.from_numpy(heights[None]).cuda(), 0, ns, eps).cpu().numpy()[0]
+    np.testing.assert_array_equal(got, ref)
