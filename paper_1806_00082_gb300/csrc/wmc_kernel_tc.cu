@@ -1513,13 +1513,17 @@ static cudaError_t launch_split_as(const float* V, int n_x, int bc, int Q, const
 // around it 20 us a step.  So the occupied lists of a step and lists of every cell
 // take the plain form, and 3xTF32 lists of at least a quarter of the cells too: if
 // they ascend, 128 of them span some 512 cells and have windows (in any order, 9000
-// of 20000: 157 us plain, 71 us staged).
+// of 20000: 157 us plain, 71 us staged).  That exception ends where the kernel's
+// shared memory leaves an L1 that does not hold the potential: 4500 permuted cells
+// of 9001 at Q = 2048 took 240 us in the kernel before, 351 us plain, 127 us staged,
+// against 3 to 5 % on lists that ascend.
 template <bool TF32, int NET>
 static cudaError_t launch_split(const float* V, int n_x, int bc, int Q, const int* occ, const int* n_occ_dev,
                                 int n_occ_host, int max_rows, const void* img_hi, const void* img_lo, int KB, int NT,
                                 float c, float* out, unsigned int* flags, const DenseA& dense, cudaStream_t s) {
   if (NET != 3) {
-    const bool left_out = (TF32 ? 4ll : 1ll) * n_occ_host < n_x;
+    const bool uncached = split_smem_bytes(Q / 2, NET, false) > 192 * 1024 && n_x > 7 * 1024;
+    const bool left_out = (TF32 && !uncached ? 4ll : 1ll) * n_occ_host < n_x;
     if (occ ? !n_occ_dev && left_out && n_x > kWindowSpan : max_rows > n_x && n_x % TM != 0)
       return launch_split_as<TF32, NET, NET != 3>(V, n_x, bc, Q, occ, n_occ_dev, n_occ_host, max_rows, img_hi, img_lo, KB,
                                                   NT, c, out, flags, dense, s);

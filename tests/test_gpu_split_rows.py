@@ -149,3 +149,22 @@ def test_implicit_rows_are_the_rows_of_each_potential(wmc, form, Q, n_pot, n_x):
     occ = torch.arange(n_x, dtype=torch.int32, device="cuda")
     for b in range(n_pot):
         assert torch.equal(got[b], wmc.kernel_eval(p, V[b].contiguous(), occ, ws, prec))
+
+
+@pytest.mark.parametrize("n_x,Q", [(7168, 1276), (7169, 1276), (7169, 1280), (7400, 2048)])
+def test_permuted_cells_of_a_domain_beyond_the_cache(wmc, n_x, Q):
+    """Both sides of the line from which lists of many cells have their terms fetched
+    by coalesced loads: any order gives the bits of consecutive cells."""
+    wl = wi.DOUBLE_BARRIER_16384.replace(n_x=n_x, Q=Q, n_M=Q)
+    p = wmc.Params.of(wl)
+    ws = wmc.workspace(p)
+    wmc.init(p, ws)
+    rng = np.random.Generator(np.random.PCG64(n_x + Q))
+    V = torch.from_numpy(rng.uniform(-0.2, 0.3, n_x).astype(np.float32)).cuda()
+    run = wmc.kernel_eval(p, V, torch.arange(n_x, dtype=torch.int32, device="cuda"), ws, wmc.TF32X3)
+    for n in (n_x // 2, n_x - 1, n_x):
+        cells = rng.permutation(n_x)[:n]
+        for c in (cells, np.sort(cells)):
+            got = wmc.kernel_eval(p, V, torch.from_numpy(c.astype(np.int32)).cuda(), ws, wmc.TF32X3)
+            assert torch.equal(got, run[torch.from_numpy(c).cuda()])
+    assert wmc.get_counters(p, ws)["flags"] == 0
