@@ -360,6 +360,11 @@ cudaError_t launch_step(const wmc_params& p, const View& v, const int32_t* hist_
 // else id by id.  Bound by the 11 B written per particle; 1e7 particles on 2000
 // cells: 180 -> 45 us (one thread per run of ids, a call per id and single
 // stores before; the writes alone would take 16 us).
+// SPARSE: rows wide enough for a window in more than kManyBlocks column blocks. 3000
+// cells of 1026 columns, one in ten with a particle: 54 us with rows staged in shared
+// memory, 61 us from block to block, 21 us; the code costs denser states of such rows
+// up to 10 % (12 registers), so narrower ones do without.
+template <bool SPARSE>
 __global__ __launch_bounds__(kStepThreads) void k_materialize(const int32_t* __restrict__ hist,
                                                               const unsigned long long* __restrict__ R,
                                                               const uint32_t* __restrict__ U,
@@ -369,6 +374,7 @@ __global__ __launch_bounds__(kStepThreads) void k_materialize(const int32_t* __r
                                                               int32_t* __restrict__ cell, float* __restrict__ f,
                                                               int16_t* __restrict__ M, int8_t* __restrict__ sign,
                                                               long long capacity, int vec_ok) {
+  __shared__ uint4 s_words[SPARSE ? kStepWarps : 1][32];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   if ((long long)hdr->population > capacity) {
     if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(&hdr->flags, WMC_FLAG_CAPACITY);
@@ -431,7 +437,27 @@ __global__ __launch_bounds__(kStepThreads) void k_materialize(const int32_t* __r
             have |= 1u << j;
           }
         }
+        const uint32_t part = lim - x;
         x = lim;
+        if (WalkSparse sp; SPARSE && x < wend && part <= kFewIds && sparse_begin(c, x, wend, B, lane, sp)) {
+          s_words[wid][lane] = w;  // id by id, by the lane of its block
+          __syncwarp();
+          const uint32_t* words = reinterpret_cast<const uint32_t*>(s_words[wid]);
+          int k;
+          uint32_t e, q0, q1;
+#pragma unroll 1
+          while (sparse_next(c, sp, k, e, q0, q1)) {
+#pragma unroll 1
+            for (uint32_t q = q0; q < q1; ++q) {
+              const long long o = (long long)(A + q) - (long long)id_base;
+              cell[o] = cw.i;
+              f[o] = (float)(words[q - a] >> 8) * 0x1p-24f;
+              M[o] = (int16_t)(k - h);
+              sign[o] = (int8_t)(e & 1u ? -1 : 1);
+            }
+          }
+          __syncwarp();
+        }
       }
       const long long o = (long long)(A + qa) - (long long)id_base;
       const float fv[4] = {(float)(w.x >> 8) * 0x1p-24f, (float)(w.y >> 8) * 0x1p-24f, (float)(w.z >> 8) * 0x1p-24f,
@@ -463,7 +489,8 @@ cudaError_t launch_materialize(const wmc_params& p, const View& v, const int32_t
                                float* f, int16_t* M, int8_t* sign, long long capacity, cudaStream_t s) {
   const auto aligned = [](const void* q, uintptr_t n) { return (reinterpret_cast<uintptr_t>(q) & (n - 1)) == 0; };
   const int vec_ok = aligned(cell, 16) && aligned(f, 16) && aligned(M, 8) && aligned(sign, 4);
-  k_materialize<<<6 * num_sms(), kStepThreads, 0, s>>>(
+  const auto k = p.n_M > 32 * kManyBlocks ? k_materialize<true> : k_materialize<false>;
+  k<<<6 * num_sms(), kStepThreads, 0, s>>>(
       hist, v.R, v.U, v.bp, v.xm, v.hdr, p.n_x, p.n_M, p.sim,
       philox_keys((uint32_t)(p.seed & 0xffffffffu), (uint32_t)(p.seed >> 32)), t, cell, f, M, sign, capacity, vec_ok);
   return cudaGetLastError();

@@ -115,3 +115,37 @@ def test_windows_of_mid_sized_buckets(wmc, sizes, n_x, Q, n_M):
         got, c = gpu_run_table(wmc, torch, wmc.Params.of(wl), half, h0, 3, 2)
         np.testing.assert_array_equal(got, ref)
         assert c["pairs"] == st[oracle.ST_PAIRS] and c["flags"] == 0
+
+
+@pytest.mark.parametrize("one_in", [1, 3, 8, 30])
+@pytest.mark.parametrize("n_x,Q,n_M", [(5, 64, 386), (5, 64, 1026), (4, 64, 4096)])
+def test_sparse_rows(wmc, n_x, Q, n_M, one_in):
+    """Windows whose ids lie in more and in fewer than a dozen column blocks of a few
+    ids each, over the edges of 32 blocks, with a large bucket between them; the
+    step with and without pairs, and the snapshot."""
+    wl, V = _workload(n_x, Q, n_M)
+    if n_M > 2052:
+        wl = wl.replace(dt_s=wl.dt_s / 2)  # (a particle moves one cell at most)
+    rng = np.random.Generator(np.random.PCG64(one_in + n_M))
+    h0 = np.where(rng.random((n_x, n_M)) < 1 / one_in, rng.choice([-3, -1, -1, 1, 1, 2], size=(n_x, n_M)), 0).astype(np.int32)
+    h0[1, n_M // 2 + 5], h0[2, -1] = 333, -40
+    p = wmc.Params.of(wl)
+    for v in (V, np.zeros_like(V)):
+        full, half = oracle_tables(wl, v)
+        ref, st = oracle.simulate(oracle.params(wl), h0, 3, 2, table=full)
+        got, c = gpu_run_table(wmc, torch, p, half, h0, 3, 2)
+        np.testing.assert_array_equal(got, ref)
+        assert c["pairs"] == st[oracle.ST_PAIRS] and c["flags"] == 0
+    ws = wmc.workspace(p)
+    wmc.init(p, ws)
+    hd = torch.from_numpy(h0).cuda()
+    wmc.annihilate(p, hd, ws)
+    n = np.abs(h0).reshape(-1).astype(np.int64)
+    at = np.repeat(np.arange(n.size), n)
+    cell, f, M, s = (x.cpu().numpy() for x in wmc.materialize(p, hd, 5, ws, int(n.sum())))
+    np.testing.assert_array_equal(cell, at // n_M)
+    np.testing.assert_array_equal(M, at % n_M - n_M // 2)
+    np.testing.assert_array_equal(s, np.sign(h0.reshape(-1))[at])
+    for i in range(0, at.size, max(1, at.size // 300)):
+        w = int(oracle.philox((i // 4, 5, 2, wl.sim), (wl.seed & 0xffffffff, wl.seed >> 32))[i % 4])
+        assert f[i] == np.float32((w >> 8) * 2.0 ** -24)
