@@ -37,14 +37,14 @@ L2_BYTES = 129 * 2 ** 20
 
 # DRAM bytes (read + write) of one particle-step kernel launch from the ncu
 # capture named below; None until the current kernel has been captured.
-K_STEP_DRAM_BYTES = 18963712
+K_STEP_DRAM_BYTES = 18915840
 K_STEP_TRAFFIC_SOURCE = ("ncu --set full capture of k_step on double-barrier-16384 (5th launch): dram read "
-                         "18.96 MB + write 0 per launch (profiles/k_step_double-barrier-16384.md)")
+                         "18.92 MB + write 0 per launch (profiles/k_step_double-barrier-16384.md)")
 # DRAM bytes of one BF16 launch of k_kernel_eval_tc_ta on all 16384 cells (the sine image and the potential
 # come from L2 after the first touch; the 32 MB of output rows stay in L2)
-TC_TA_DRAM_BYTES = 714240 + 5376
+TC_TA_DRAM_BYTES = 715008 + 5888
 TC_TA_DRAM_SOURCE = ("ncu --set full capture of k_kernel_eval_tc_ta<BF16> on double-barrier-16384 (4th launch): "
-                     "dram read 714.2 KB + write 5.4 KB (profiles/k_kernel_eval_tc_ta_double-barrier-16384.md)")
+                     "dram read 715.0 KB + write 5.9 KB (profiles/k_kernel_eval_tc_ta_double-barrier-16384.md)")
 
 
 def _env_int(k, d):

@@ -127,7 +127,7 @@ typedef struct wmc_counters {
   uint64_t dropped;         /* children outside the momentum grid (drop mode) */
   int64_t dropped_signed;   /* sum of their signs */
   int32_t n_occ;            /* cells whose kernel the last step evaluated */
-  int32_t n_items;          /* work items of the last step */
+  int32_t n_items;          /* runs of ids of one cell, as counted for the limit */
   uint32_t flags;           /* WMC_FLAG_* */
   uint32_t step;            /* device step counter used by wmc_run */
 } wmc_counters;
@@ -339,7 +339,7 @@ wmc_status wmc_kernel_cdf(const wmc_params* p, const float* VWh, int32_t n_rows,
  * ------------------------------------------------------------------------- */
 
 /* Rule 2 rebuild: enumerates the survivors of the net histogram hist [dev]
- * int32[n_x][n_M] (row-major ids, work items of 512 to 2048 ids of one cell, sized from the previous population), marks the
+ * int32[n_x][n_M] (row-major ids, n_items runs of up to 2048 ids of one cell), marks the
  * cells the next drift can reach (occupied cells and their neighbour in each
  * drift direction present) as the occupied list for the kernel, and, if
  * rho [dev] int64[n_x] is not NULL, writes the density (rule 1) of hist.

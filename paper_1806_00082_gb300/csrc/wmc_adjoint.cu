@@ -58,7 +58,7 @@ __device__ __forceinline__ float window(float x, float a, float b, float inv_eps
 // ---------------------------------------------------------------- potential
 // One thread per cell.  Windows that do not reach the cell are passed over and the
 // segment edges are divided once per block, kEdges segments at a time: 64 x 4096
-// cells of 32 windows 42 -> 13 us, of 700 segments 881 -> 201 us (326 us with each
+// cells of 32 windows 42 -> 14 us, of 700 segments 881 -> 201 us (326 us with each
 // cell's own divisions where they are more than kEdges).  A domain that every
 // window reaches does without the test, so that the windows' exponentials overlap:
 // one potential of 64 cells, 300 segments 90 -> 79 us.  A window adds height x

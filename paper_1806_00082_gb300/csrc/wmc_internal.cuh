@@ -68,7 +68,7 @@ struct DevHeader {
   unsigned int step;    // device step counter (wmc_run)
   unsigned int magic;
   unsigned int item_ticket;  // id ranges handed out by the running step launch
-  unsigned int blocks_done;  // step blocks finished (the last one resets both)
+  unsigned int pad1;
   unsigned int rows_by_cell; // 1: the kernel stage wrote its rows at the cell index, 0: at the occupied-list index
   unsigned int pair_count;   // quads queued by the particle-step kernel (reset by the pair kernel)
   unsigned int pairs_done;   // pair-kernel blocks finished (the last one resets the queue and the ticket)
@@ -238,7 +238,7 @@ __host__ __device__ __forceinline__ uint32_t units_of_cell(unsigned long long t,
 cudaError_t launch_init_tables(const wmc_params& p, const View& v, cudaStream_t s);
 cudaError_t launch_plan(const wmc_params& p, const View& v, const int32_t* hist, int64_t* rho, int advance_step,
                         cudaStream_t s, int32_t* zero_out = nullptr);
-// the two halves of launch_plan: the per-cell scan, and the single-block plan
+// the two halves of launch_plan: the per-cell scan, and the plan
 // (clear_thr: also zero the event thresholds of every cell)
 cudaError_t launch_rows(const wmc_params& p, const View& v, const int32_t* hist, int64_t* rho, cudaStream_t s,
                         int32_t* zero_out);

@@ -261,7 +261,7 @@ __device__ __noinline__ void rewalk_events(const StepArgs& a, uint32_t t, uint4*
 // grid has that many, so that no thread draws and samples two events one after
 // the other; one thread per quad beyond.  24 cells of 1026 columns, 18000 events
 // in 16000 quads: 24.5 us by quads, 15.1 us by ids.  The last block to finish resets
-// the queue and the work-item ticket for the next step.
+// the queue and the range ticket for the next step.
 __global__ __launch_bounds__(kStepThreads, 4) void k_pairs(const __grid_constant__ StepArgs a) {
   const int rows_by_cell = (int)a.hdr->rows_by_cell;
   const uint32_t t = a.t_from_device ? a.hdr->step : a.t;

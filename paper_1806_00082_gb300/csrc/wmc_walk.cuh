@@ -26,7 +26,7 @@
 // quad take 34 wide multiplications (4 cycles each on a scheduler) and as many
 // XORs; a one-bucket window takes 104 instructions (with creation words), a
 // mixed one several hundred.  Measured (ncu, 1.08e8 particles, 3555 occupied
-// cells with 450 non-empty buckets each): k_step 372 -> 205 us, 275e6 -> 142e6
+// cells with 450 non-empty buckets each): k_step 352 -> 201 us, 275e6 -> 140e6
 // warp instructions, against the form that staged each row in shared memory
 // and gave every lane a run of ids of its own (nearly every warp iteration
 // then met a lane that changed its bucket); drift only, 1e7 particles on 2000
